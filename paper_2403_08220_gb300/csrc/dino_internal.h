@@ -159,6 +159,52 @@ cudaError_t gemm_field(int M, int N, int K, const T *A, int lda, const T *B, int
                        const int *acc_flag, double s, double c, T *m, const T *Mf, int ldm,
                        cudaStream_t st);
 
+// ---- FP64 GEMMs on the tensor cores (k_gemm64.cu) -------------------------
+// Operands as kDigits64 planes of signed base-128 digits in bf16 (plane s at
+// + s * plane elements, row pitch ldp a multiple of 8) and one exponent a row.
+constexpr int kDigits64 = 8;
+int digit_pitch(int K);
+struct DigitMat {              // an operand B laid out once (weights, basis)
+  const __nv_bfloat16 *d = nullptr;
+  const int *ex = nullptr;     // row exponents
+  const int *fk = nullptr;     // column exponents taken out of B (nullptr: none)
+  int ldp = 0;
+  size_t plane = 0;
+  const double *src = nullptr;  // B itself, rows x K (pitch ld)
+  int ld = 0;
+};
+// Digits of rows x K values: src (pitch ld), or with src == nullptr the
+// products W[(row0 + i) % g] .* der[(row0 + i) / g] (rows of K and pitch ldd).
+// fk (fsign 1 or -1 times) is added to the exponents of the columns.
+cudaError_t launch_split64(int rows, int K, const double *src, int ld, const double *W,
+                           const double *der, int g, int ldd, int row0, const int *fk, int fsign,
+                           __nv_bfloat16 *dst, int ldp, size_t plane,
+                           int *ex, cudaStream_t st);
+cudaError_t launch_col_exp(int rows, int K, const double *B, int ld, int *fk, cudaStream_t st);
+// out = epilogue(A B^T) for M rows of A (digits A, ea; the values Asrc, pitch
+// lda, or the product form, read only for rows that are not finite); the epilogue's row index
+// starts at row0.  err (device): bit 8 is set when a bounded wait gave up.
+struct Gemm64Args {
+  int M = 0, N = 0, K = 0, row0 = 0;
+  const __nv_bfloat16 *A = nullptr;
+  const int *ea = nullptr;
+  int ldp = 0;
+  size_t plane = 0;
+  const double *Asrc = nullptr, *W = nullptr, *der = nullptr;
+  int lda = 0, g = 1, ldd = 0;
+  DigitMat B;
+  int *err = nullptr;
+};
+cudaError_t gemm64_store(const Gemm64Args &a, double *out, int ldo, cudaStream_t st);
+cudaError_t gemm64_bias_act(const Gemm64Args &a, const double *bias, int act, double *out,
+                            double *der, int ldo, cudaStream_t st);
+cudaError_t gemm64_scale_group(const Gemm64Args &a, const double *scale, int lds, int group,
+                               double *out, int ldo, cudaStream_t st);
+cudaError_t gemm64_coef(const Gemm64Args &a, const double *coef, int ldc, double c, double *out,
+                        int ldo, cudaStream_t st);
+cudaError_t gemm64_field(const Gemm64Args &a, const int *acc_flag, double s, double c, double *m,
+                         const double *Mf, int ldm, cudaStream_t st);
+
 // ---- elementwise / per-chain helpers -------------------------------------
 // Shared memory of the prior draw of one chain on an n x n grid (elements of `elem` bytes).
 size_t prior_draw_smem_bytes(int n, int elem);

@@ -429,6 +429,9 @@ struct Surrogate {
   int ldE = 0, ldD = 0;
   size_t plE = 0, plD = 0;
   std::vector<double *> dW, dWT, db;
+  // digits of the FP64 products' right-hand operands (empty ones take the SIMT GEMM)
+  std::vector<DigitMat> gW, gWT;
+  DigitMat gE, gD;
   std::vector<float *> fb, fW;
   std::vector<__nv_bfloat16 *> bW, bWT;
   std::vector<int> ldW, ldWT;
@@ -443,6 +446,8 @@ struct Surrogate {
     std::vector<std::pair<void *, size_t>> allocs;
     double *dEt = nullptr, *dEtD = nullptr;  // E_t (r_t x N), E_t D (r_t x r)
     std::vector<double *> dW, db;
+    DigitMat gEt, gEtD;
+    std::vector<DigitMat> gW;
     // tensor path: three bf16 slices of E_t (r_t x ldE), E_t D (r_t x ldD)
     // and of each W_l (pitch ldW[l]); FP32 biases
     __nv_bfloat16 *bEt = nullptr, *bEtD = nullptr;
@@ -469,6 +474,150 @@ static T *sur_upload(dino_ctx *ctx, Surrogate *s, const T *host, size_t n) {
   T *p = sur_alloc<T>(ctx, s, n);
   CK(cudaMemcpyAsync(p, host, n * sizeof(T), cudaMemcpyHostToDevice, ctx->stream));
   return p;
+}
+
+// ---------------------------------------------------------------------------
+// FP64 products (out = epilogue(A B^T), B rows x K)
+//
+// B's digits are laid out once, and the product runs on the tensor cores, when
+// B has at least kDigitsMinWork entries and neither side is short (a tile has 32
+// columns, a stage 32 of the reduction); below that the SIMT GEMM is as fast or
+// faster (64 rows by 16 x 1089: 18 us against 70 us).  The rule looks at B alone, so that an output's bits do not depend
+// on how many chains share the product.
+constexpr long kDigitsMinWork = 16384;
+
+// Digits of a device matrix B.  Left empty where the rule above or the HBM
+// budget says no; its products then take the SIMT GEMM.
+static DigitMat make_digits(dino_ctx *ctx, std::vector<std::pair<void *, size_t>> &allocs,
+                            const double *B, int rows, int K) {
+  DigitMat m;
+  if ((long)rows * K < kDigitsMinWork || rows < 32 || K < 32) return m;
+  const int ldp = digit_pitch(K);
+  const size_t plane = (size_t)rows * ldp;
+  const size_t bytes = (plane * kDigits64 * 2 + ((size_t)rows + K) * 4 + 15) & ~(size_t)15;
+  if (ctx->used + bytes > ctx->budget) return m;
+  void *p = nullptr;
+  if (cudaMalloc(&p, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    return m;
+  }
+  ctx->used += bytes;
+  allocs.push_back({p, bytes});
+  auto *d = (__nv_bfloat16 *)p;
+  int *ex = (int *)(d + plane * kDigits64), *fk = ex + rows;
+  CK(launch_col_exp(rows, K, B, K, fk, ctx->stream));
+  CK(launch_split64(rows, K, B, K, nullptr, nullptr, 1, 0, 0, fk, -1, d, ldp, plane, ex,
+                    ctx->stream));
+  m.d = d;
+  m.ex = ex;
+  m.fk = fk;
+  m.ldp = ldp;
+  m.plane = plane;
+  m.src = B;
+  m.ld = K;
+  return m;
+}
+
+// The left-hand operand of a product: M x K values (pitch lda), or in product
+// form (A == nullptr) the rows W[i % g] .* der[i / g] (pitches K and ldd).
+struct Left64 {
+  const double *A = nullptr;
+  int lda = 0;
+  const double *W = nullptr, *der = nullptr;
+  int g = 1, ldd = 0;
+};
+
+// Scratch for the digits of A: free device memory of the caller's.
+struct Scratch64 {
+  void *p = nullptr;
+  size_t bytes = 0;
+  int *err = nullptr;
+};
+
+// Bytes of A's digits worked on at a time: they are written and read again
+// while still in L2 (129 MB).
+constexpr size_t kDigitsChunk = 96u << 20;
+
+static bool has_digits(const DigitMat &B, const Scratch64 &ws, int K) {
+  return B.d && ws.p && ws.bytes >= 16 * (size_t)digit_pitch(K) + 16;
+}
+
+// The product on the tensor cores in chunks of rows: digits of A into the
+// scratch, then tc(args) for those rows.
+template <class Tc>
+static void digit_product(dino_ctx *ctx, cudaStream_t st, const char *name, int M, int N, int K,
+                          const Left64 &a, const DigitMat &B, const Scratch64 &ws, Tc &&tc) {
+  const int ldp = digit_pitch(K);
+  const size_t per = 16 * (size_t)ldp + 4;
+  size_t rows = std::min<size_t>({(size_t)M, (ws.bytes - 16) / per,
+                                  std::max<size_t>(128, kDigitsChunk / per)});
+  if (rows < (size_t)M) {  // equal chunks of whole 128-row tiles
+    const size_t n = ((size_t)M + rows - 1) / rows, even = ((size_t)M + n - 1) / n;
+    const size_t up = (even + 127) / 128 * 128;
+    rows = up <= rows ? up : (rows >= 128 ? rows / 128 * 128 : rows);
+  }
+  auto *d = (__nv_bfloat16 *)ws.p;
+  const size_t plane = rows * ldp;
+  int *ex = (int *)(d + plane * kDigits64);
+  for (size_t r0 = 0; r0 < (size_t)M; r0 += rows) {
+    const int m = (int)std::min(rows, (size_t)M - r0);
+    const double *A = a.A ? a.A + r0 * a.lda : nullptr;
+    launch(ctx, st, "split_f64", [&] {
+      return launch_split64(m, K, A, a.lda, a.W, a.der, a.g, a.ldd, (int)r0, B.fk, 1, d, ldp,
+                            plane, ex, st);
+    });
+    Gemm64Args g;
+    g.M = m;
+    g.N = N;
+    g.K = K;
+    g.row0 = (int)r0;
+    g.A = d;
+    g.ea = ex;
+    g.ldp = ldp;
+    g.plane = plane;
+    g.Asrc = A;
+    g.lda = a.lda;
+    g.W = a.W;
+    g.der = a.der;
+    g.g = a.g;
+    g.ldd = a.ldd;
+    g.B = B;
+    g.err = ws.err;
+    launch(ctx, st, name, [&] { return tc(g); });
+  }
+}
+
+static void store64(dino_ctx *ctx, cudaStream_t st, const char *name, int M, int N, int K,
+                    const double *A, int lda, const double *B, int ldb, const DigitMat &gB,
+                    const Scratch64 &ws, double *out, int ldo) {
+  if (has_digits(gB, ws, K)) {
+    Left64 l;
+    l.A = A;
+    l.lda = lda;
+    digit_product(ctx, st, name, M, N, K, l, gB, ws,
+                  [&](const Gemm64Args &g) { return gemm64_store(g, out, ldo, st); });
+    return;
+  }
+  launch(ctx, st, name,
+         [&] { return gemm_store<double>(M, N, K, A, lda, B, ldb, out, ldo, st); });
+}
+
+static void bias_act64(dino_ctx *ctx, cudaStream_t st, const char *name, int M, int N, int K,
+                       const double *A, int lda, const double *B, int ldb, const DigitMat &gB,
+                       const Scratch64 &ws, const double *bias, int act, double *out, double *der,
+                       int ldo) {
+  if (has_digits(gB, ws, K)) {
+    Left64 l;
+    l.A = A;
+    l.lda = lda;
+    digit_product(ctx, st, name, M, N, K, l, gB, ws, [&](const Gemm64Args &g) {
+      return gemm64_bias_act(g, bias, act, out, der, ldo, st);
+    });
+    return;
+  }
+  launch(ctx, st, name, [&] {
+    return gemm_bias_act<double>(M, N, K, A, lda, B, ldb, bias, act, out, der, ldo, st);
+  });
 }
 
 static std::vector<float> to_f32(const std::vector<double> &v) {
@@ -565,8 +714,13 @@ static void set_true_model(dino_ctx *ctx, Surrogate *s, const dino_true_model_de
   try {
     t.dEt = tm_upload(ctx, s, Et.data(), Et.size());
     t.dEtD = tm_upload(ctx, s, EtD.data(), EtD.size());
+    t.gEt = make_digits(ctx, t.allocs, t.dEt, t.r_t, N);
+    t.gW.resize(t.L);
+    if (s->precision == DINO_PREC_FP64) t.gEtD = make_digits(ctx, t.allocs, t.dEtD, t.r_t, r);
     for (int l = 0; l < t.L; ++l) {
       t.dW.push_back(tm_upload(ctx, s, W[l].data(), W[l].size()));
+      if (s->precision == DINO_PREC_FP64)
+        t.gW[l] = make_digits(ctx, t.allocs, t.dW[l], t.widths[l + 1], t.widths[l]);
       t.db.push_back(tm_upload(ctx, s, b[l].data(), b[l].size()));
       if (s->precision == DINO_PREC_BF16) {
         const int wo = t.widths[l + 1], wi = t.widths[l], ldw = pad8(wi);
@@ -701,6 +855,10 @@ static int load_surrogate(dino_ctx *ctx, const dino_surrogate_desc *d) {
   s->dD = sur_upload(ctx, s.get(), s->D.data(), s->D.size());
   s->dS = sur_upload(ctx, s.get(), S.data(), S.size());
   s->dSqrtLam = sur_upload(ctx, s.get(), sqrtlam.data(), sqrtlam.size());
+  s->gE = make_digits(ctx, s->allocs, s->dE, r, N);  // both precisions encode in FP64
+  if (s->precision == DINO_PREC_FP64) s->gD = make_digits(ctx, s->allocs, s->dD, N, r);
+  s->gW.resize(s->L);
+  s->gWT.resize(s->L);
   for (int l = 0; l < s->L; ++l) {
     const int wo = s->widths[l + 1], wi = s->widths[l];
     std::vector<double> WT((size_t)wi * wo);
@@ -709,6 +867,10 @@ static int load_surrogate(dino_ctx *ctx, const dino_surrogate_desc *d) {
     s->dW.push_back(sur_upload(ctx, s.get(), s->W[l].data(), s->W[l].size()));
     s->dWT.push_back(sur_upload(ctx, s.get(), WT.data(), WT.size()));
     s->db.push_back(sur_upload(ctx, s.get(), s->b[l].data(), s->b[l].size()));
+    if (s->precision == DINO_PREC_FP64) {
+      s->gW[l] = make_digits(ctx, s->allocs, s->dW[l], wo, wi);
+      if (l + 1 < s->L) s->gWT[l] = make_digits(ctx, s->allocs, s->dWT[l], wi, wo);
+    }
     if (l >= 1) s->widest = std::max(s->widest, wi);
     if (s->precision == DINO_PREC_BF16) {
       const auto fb = to_f32(s->b[l]);
@@ -784,6 +946,7 @@ struct Work {
   // FP64 path
   std::vector<double *> act64, der64;
   double *f64 = nullptr, *P64[2] = {nullptr, nullptr}, *J64 = nullptr;
+  size_t p_bytes = 0, j_bytes = 0;  // of each P64 (or Pb) and of J64
   // tensor path
   __nv_bfloat16 *xb = nullptr;
   int ldx = 0;
@@ -834,10 +997,12 @@ static void layout_work(const Surrogate *s, int C, Arena &ar, Work &w, bool assi
     }
     w.f64 = (double *)take((size_t)C * dy * 8);
     if (L >= 2) {
-      w.P64[0] = (double *)take(prows * s->widest * 8);
-      w.P64[1] = (double *)take(prows * s->widest * 8);
+      w.p_bytes = prows * s->widest * 8;
+      w.P64[0] = (double *)take(w.p_bytes);
+      w.P64[1] = (double *)take(w.p_bytes);
     }
-    w.J64 = (double *)take(rows * s->r * 8);
+    w.j_bytes = rows * s->r * 8;
+    w.J64 = (double *)take(w.j_bytes);
     if (s->jac_fwd) w.Jt = take(rows * s->r * 8);
   } else {
     w.ldx = pad8(s->r);
@@ -854,8 +1019,9 @@ static void layout_work(const Surrogate *s, int C, Arena &ar, Work &w, bool assi
     if (L >= 2) {
       w.ldp = pad8(s->widest);
       w.plp = prows * w.ldp;
-      w.Pb[0] = (__nv_bfloat16 *)take(w.plp * s->jac_slices * 2);
-      w.Pb[1] = (__nv_bfloat16 *)take(w.plp * s->jac_slices * 2);
+      w.p_bytes = w.plp * s->jac_slices * 2;
+      w.Pb[0] = (__nv_bfloat16 *)take(w.p_bytes);
+      w.Pb[1] = (__nv_bfloat16 *)take(w.p_bytes);
     }
     w.J32 = (float *)take(rows * s->r * 4);
     if (s->jac_fwd) w.Jt = take(rows * s->r * 4);
@@ -875,77 +1041,89 @@ static void layout_work(const Surrogate *s, int C, Arena &ar, Work &w, bool assi
 
 // Forward pass and Jacobian at the C points in `x` (FP64 C x r; the tensor
 // path reads the bf16 planes in w.xb, which the caller has filled).
-// with_a: the pool's state pairs w.a_df are valid (a step, not the initial
-// geometry), so K a is formed beside K b.
-static void eval_surrogate(dino_ctx *ctx, const Surrogate *s, Work &w, const double *x,
+// err: the pool's error word.  with_a: the pool's state pairs w.a_df are valid
+// (a step, not the initial geometry), so K a is formed beside K b.
+static void eval_surrogate(dino_ctx *ctx, const Surrogate *s, Work &w, const double *x, int *err,
                            cudaStream_t st, bool with_a = false) {
   const int C = w.C, L = s->L, dy = s->d_y, r = s->r;
   if (s->precision == DINO_PREC_FP64) {
     const double *a = x;
     int lda = r;
+    // digits of the forward pass's inputs in the Jacobian's buffers, not yet in use
+    const Scratch64 p0{w.P64[0], w.p_bytes, err};
     for (int l = 0; l + 1 < L; ++l) {
       const int wo = s->widths[l + 1], wi = s->widths[l];
-      launch(ctx, st, "mlp_f64", [&] {
-        return gemm_bias_act<double>(C, wo, wi, a, lda, s->dW[l], wi, s->db[l], s->act,
-                                     w.act64[l], w.der64[l], wo, st);
-      });
+      bias_act64(ctx, st, "mlp_f64", C, wo, wi, a, lda, s->dW[l], wi, s->gW[l], p0, s->db[l],
+                 s->act, w.act64[l], w.der64[l], wo);
       a = w.act64[l];
       lda = wo;
     }
-    launch(ctx, st, "mlp_f64", [&] {
-      return gemm_bias_act<double>(C, dy, s->widths[L - 1], a, lda, s->dW[L - 1],
-                                   s->widths[L - 1], s->db[L - 1], 0, w.f64, nullptr, dy, st);
-    });
+    bias_act64(ctx, st, "mlp_f64", C, dy, s->widths[L - 1], a, lda, s->dW[L - 1],
+               s->widths[L - 1], s->gW[L - 1], p0, s->db[L - 1], 0, w.f64, nullptr, dy);
     if (L == 1) {
       launch(ctx, st, "jac_broadcast", [&] {
         return launch_broadcast<double>(C, (size_t)dy * r, s->dW[0], w.J64, st);
       });
       return;
     }
-    if (s->jac_fwd) {
-      // forward mode on J^T: T = W_0^T .* d_0 (r x w_1 per chain);
-      // T <- (T W_l^T) .* d_l; J^T = T W_{L-1}^T, then J per chain
-      const int w1 = s->widths[1];
-      launch(ctx, st, "jac_init_f64", [&] {
-        return launch_jac_init<double>(C, r, w1, s->dWT[0], w.der64[0], w1, w.P64[0], st);
-      });
-      int cur = 0;
-      for (int l = 1; l + 1 < L; ++l) {
-        const int wi = s->widths[l], wo = s->widths[l + 1];
+    // The stacked products P <- (P B^T) .* d, B the weights: reverse mode
+    // P = W_{L-1} .* d_{L-2} (d_y rows per chain), B = W_l^T down to J = P W_0;
+    // forward mode on J^T, T = W_0^T .* d_0 (r rows per chain), B = W_l up to
+    // J^T = T W_{L-1}^T, then J per chain.  Where B has digits the start P is
+    // not formed: its digits are taken straight from W and d.
+    const bool fwd = s->jac_fwd;
+    const int g = fwd ? r : dy, nprod = L - 1;
+    const double *W0 = fwd ? s->dWT[0] : s->dW[L - 1];
+    const double *d0 = fwd ? w.der64[0] : w.der64[L - 2];
+    const int w0 = fwd ? s->widths[1] : s->widths[L - 1];
+    int cur = 0;
+    for (int q = 0; q < nprod; ++q) {
+      const int l = fwd ? q + 1 : L - 2 - q;
+      const bool last = q + 1 == nprod;
+      const int K = fwd ? s->widths[l] : s->widths[l + 1];
+      const int n = fwd ? s->widths[l + 1] : s->widths[l];
+      const double *B = fwd ? s->dW[l] : s->dWT[l];
+      const DigitMat &gB = fwd ? s->gW[l] : s->gWT[l];
+      const double *scale = last ? nullptr : (fwd ? w.der64[l] : w.der64[l - 1]);
+      double *out = last ? (fwd ? (double *)w.Jt : w.J64) : w.P64[1 - cur];
+      // digits: in P[0] for the first product (it starts from W and d) and in
+      // the other P for the last; in J, not yet in use, in between
+      const Scratch64 ws = q == 0 ? Scratch64{w.P64[0], w.p_bytes, err}
+                           : last ? Scratch64{w.P64[1 - cur], w.p_bytes, err}
+                                  : Scratch64{w.J64, w.j_bytes, err};
+      if (has_digits(gB, ws, K)) {
+        Left64 lf;
+        if (q == 0) {
+          lf.W = W0;
+          lf.der = d0;
+          lf.g = g;
+          lf.ldd = w0;
+        } else {
+          lf.A = w.P64[cur];
+          lf.lda = K;
+        }
+        digit_product(ctx, st, "jac_gemm_f64", C * g, n, K, lf, gB, ws,
+                      [&](const Gemm64Args &ga) {
+                        return last ? gemm64_store(ga, out, n, st)
+                                    : gemm64_scale_group(ga, scale, n, g, out, n, st);
+                      });
+      } else {
+        if (q == 0)
+          launch(ctx, st, "jac_init_f64", [&] {
+            return launch_jac_init<double>(C, g, w0, W0, d0, w0, w.P64[0], st);
+          });
         launch(ctx, st, "jac_gemm_f64", [&] {
-          return gemm_scale_group<double>(C * r, wo, wi, w.P64[cur], wi, s->dW[l], wi,
-                                          w.der64[l], wo, r, w.P64[1 - cur], wo, st);
+          return last ? gemm_store<double>(C * g, n, K, w.P64[cur], K, B, K, out, n, st)
+                      : gemm_scale_group<double>(C * g, n, K, w.P64[cur], K, B, K, scale, n, g,
+                                                 out, n, st);
         });
-        cur = 1 - cur;
       }
-      const int wl = s->widths[L - 1];
-      launch(ctx, st, "jac_gemm_f64", [&] {
-        return gemm_store<double>(C * r, dy, wl, w.P64[cur], wl, s->dW[L - 1], wl,
-                                  (double *)w.Jt, dy, st);
-      });
+      cur = 1 - cur;
+    }
+    if (fwd)
       launch(ctx, st, "jac_transpose", [&] {
         return launch_batched_transpose(C, r, dy, w.Jt, 0, w.J64, st);
       });
-      return;
-    }
-    // reverse mode: P = W_{L-1} .* d_{L-2}; P <- (P W_l) .* d_{l-1}; J = P W_0
-    const int wl = s->widths[L - 1];
-    launch(ctx, st, "jac_init_f64", [&] {
-      return launch_jac_init<double>(C, dy, wl, s->dW[L - 1], w.der64[L - 2], wl, w.P64[0], st);
-    });
-    int cur = 0;
-    for (int l = L - 2; l >= 1; --l) {
-      const int wi = s->widths[l], wo = s->widths[l + 1];
-      launch(ctx, st, "jac_gemm_f64", [&] {
-        return gemm_scale_group<double>(C * dy, wi, wo, w.P64[cur], wo, s->dWT[l], wo,
-                                        w.der64[l - 1], wi, dy, w.P64[1 - cur], wi, st);
-      });
-      cur = 1 - cur;
-    }
-    launch(ctx, st, "jac_gemm_f64", [&] {
-      return gemm_store<double>(C * dy, r, s->widths[1], w.P64[cur], s->widths[1], s->dWT[0],
-                                s->widths[1], w.J64, r, st);
-    });
     return;
   }
   // tensor-core path
@@ -1309,6 +1487,13 @@ static void split_input(dino_ctx *ctx, const Surrogate *s, Work &w, const double
 
 static size_t pool_footprint(const Surrogate *s, int C);
 
+// Scratch for digits outside the surrogate's evaluation: the Jacobian's first
+// product buffer.
+static Scratch64 pool_scratch(const Pool &p) {
+  void *b = p.s->precision == DINO_PREC_FP64 ? (void *)p.w.P64[0] : (void *)p.w.Pb[0];
+  return Scratch64{b, b ? p.w.p_bytes : 0, p.err};
+}
+
 // The true map f_t at the C points x_t = p.xt (FP64 path) or its slices
 // p.xtb (tensor path), into p.ft.
 static void true_forward(dino_ctx *ctx, const Surrogate *s, Pool &p, cudaStream_t st) {
@@ -1321,10 +1506,8 @@ static void true_forward(dino_ctx *ctx, const Surrogate *s, Pool &p, cudaStream_
       const int wo = t.widths[l + 1], wi = t.widths[l];
       const bool last = l + 1 == L;
       double *out = last ? (double *)p.ft : p.tact64[l];
-      launch(ctx, st, "true_mlp_f64", [&] {
-        return gemm_bias_act<double>(C, wo, wi, a, lda, t.dW[l], wi, t.db[l], last ? 0 : t.act,
-                                     out, nullptr, wo, st);
-      });
+      bias_act64(ctx, st, "true_mlp_f64", C, wo, wi, a, lda, t.dW[l], wi, t.gW[l],
+                 pool_scratch(p), t.db[l], last ? 0 : t.act, out, nullptr, wo);
       a = out;
       lda = wo;
     }
@@ -1375,14 +1558,10 @@ static void da_stage(dino_ctx *ctx, Pool &p, double cs, cudaStream_t st) {
   const int C = p.C, r = s->r, N = s->N, rt = t.r_t;
   const bool tc = s->precision != DINO_PREC_FP64;
   if (!tc) {
-    launch(ctx, st, "da_proj_f64", [&] {
-      return gemm_store<double>(C, rt, N, (const double *)p.Mf, N, t.dEt, N, (double *)p.EtM, rt,
-                                st);
-    });
-    launch(ctx, st, "da_proj_f64", [&] {
-      return gemm_store<double>(C, rt, r, (const double *)p.coef2, r, t.dEtD, r,
-                                (double *)p.EtDc, rt, st);
-    });
+    store64(ctx, st, "da_proj_f64", C, rt, N, (const double *)p.Mf, N, t.dEt, N, t.gEt,
+            pool_scratch(p), (double *)p.EtM, rt);
+    store64(ctx, st, "da_proj_f64", C, rt, r, (const double *)p.coef2, r, t.dEtD, r, t.gEtD,
+            pool_scratch(p), (double *)p.EtDc, rt);
   } else {
     auto proj = [&](const __nv_bfloat16 *A, int lda, const __nv_bfloat16 *B, size_t bpl, int K,
                     void *out) {
@@ -1457,9 +1636,7 @@ static void da_init(dino_ctx *ctx, Pool &p, const double *m64, cudaStream_t st) 
   const auto &t = s->tm;
   const int C = p.C, N = s->N, rt = t.r_t;
   const bool tc = s->precision != DINO_PREC_FP64;
-  launch(ctx, st, "da_encode_f64", [&] {
-    return gemm_store<double>(C, rt, N, m64, N, t.dEt, N, p.mt, rt, st);
-  });
+  store64(ctx, st, "da_encode_f64", C, rt, N, m64, N, t.dEt, N, t.gEt, pool_scratch(p), p.mt, rt);
   launch(ctx, st, "da_assemble", [&] {
     return launch_da_assemble(C, rt, 1.0, 0.0, p.mt, nullptr, nullptr, tc ? 1 : 0, p.xt, p.xtb,
                               p.ldxt, (size_t)C * p.ldxt, kTrueSlices, st);
@@ -1517,9 +1694,7 @@ static Pool *create_pool_on(dino_ctx *ctx, int sid, int C, double dt, uint64_t s
       });
     }
     // m_r = E m0 (eq:projector), then the geometry at m_r
-    launch(ctx, st, "encode_f64", [&] {
-      return gemm_store<double>(C, r, N, m64, N, s->dE, N, p->b, r, st);
-    });
+    store64(ctx, st, "encode_f64", C, r, N, m64, N, s->dE, N, s->gE, pool_scratch(*p), p->b, r);
     if (s->precision == DINO_PREC_FP64) {
       CK(cudaMemcpyAsync(p->m, m64, (size_t)C * N * 8, cudaMemcpyDeviceToDevice, st));
     } else {
@@ -1532,7 +1707,7 @@ static Pool *create_pool_on(dino_ctx *ctx, int sid, int C, double dt, uint64_t s
       launch(ctx, st, "to_df", [&] {
         return launch_to_df((size_t)C * r, p->b, p->w.b_df, p->w.a_df, st);
       });
-    eval_surrogate(ctx, s, p->w, p->b, st);
+    eval_surrogate(ctx, s, p->w, p->b, p->err, st);
     ReducedArgs ra = reduced_args(*p);
     launch(ctx, st, "geometry_init", [&] {
       return p->eig ? launch_eig_geometry(ra, 0, st)
@@ -1581,7 +1756,7 @@ static void step_pool(dino_ctx *ctx, Pool &p) {
     return p.eig ? launch_eig_propose(ra, st) : p.wb ? launch_wb_propose(ra, st)
                                                      : launch_propose(ra, st);
   });
-  eval_surrogate(ctx, s, p.w, p.b, st, true);
+  eval_surrogate(ctx, s, p.w, p.b, p.err, st, true);
   launch(ctx, st, "geometry", [&] {
     return p.eig ? launch_eig_geometry(ra, 1, st)
            : p.wb ? launch_wb_geometry(ra, 1, st) : launch_geometry(ra, 1, st);
@@ -1594,13 +1769,32 @@ static void step_pool(dino_ctx *ctx, Pool &p) {
                                        STREAM_Z_ID, p.step, Mf, N, st, nullptr, 0, 0, 0, ext_z,
                                        p.da ? p.acc : nullptr);
     });
-    launch(ctx, st, "field_coef_f64", [&] {
-      return gemm_coef<double>(C, r, N, Mf, N, s->dE, N, p.coef, r, cs, coef2, r, st);
-    });
+    const Scratch64 ws = pool_scratch(p);
+    if (has_digits(s->gE, ws, N)) {
+      Left64 l;
+      l.A = Mf;
+      l.lda = N;
+      digit_product(ctx, st, "field_coef_f64", C, r, N, l, s->gE, ws, [&](const Gemm64Args &g) {
+        return gemm64_coef(g, p.coef, r, cs, coef2, r, st);
+      });
+    } else {
+      launch(ctx, st, "field_coef_f64", [&] {
+        return gemm_coef<double>(C, r, N, Mf, N, s->dE, N, p.coef, r, cs, coef2, r, st);
+      });
+    }
     if (p.da) da_stage(ctx, p, cs, st);
-    launch(ctx, st, "field_update_f64", [&] {
-      return gemm_field<double>(C, N, r, coef2, r, s->dD, r, p.acc, p.sc, cs, m, Mf, N, st);
-    });
+    if (has_digits(s->gD, ws, r)) {
+      Left64 l;
+      l.A = coef2;
+      l.lda = r;
+      digit_product(ctx, st, "field_update_f64", C, N, r, l, s->gD, ws, [&](const Gemm64Args &g) {
+        return gemm64_field(g, p.acc, p.sc, cs, m, Mf, N, st);
+      });
+    } else {
+      launch(ctx, st, "field_update_f64", [&] {
+        return gemm_field<double>(C, N, r, coef2, r, s->dD, r, p.acc, p.sc, cs, m, Mf, N, st);
+      });
+    }
   } else {
     // FP32 draw plus its bf16 slices; both projections on the tensor cores
     // with three slices (six products, FP32-level operands)
@@ -1714,11 +1908,14 @@ static void surrogate_eval(dino_ctx *ctx, int sid, int n, const double *x_host, 
     }
     CK(cudaMemcpyAsync(p.b, x_host, (size_t)n * r * 8, cudaMemcpyHostToDevice, st));
     split_input(ctx, s, p.w, p.b, st);
-    eval_surrogate(ctx, s, p.w, p.b, st);
+    eval_surrogate(ctx, s, p.w, p.b, p.err, st);
     ReducedArgs ra = reduced_args(p);
     ra.noise_var = s->has_data ? s->noise_var : 1.0;
     launch(ctx, st, "geometry_init", [&] { return launch_geometry(ra, 0, st); });
+    int err = 0;
+    CK(cudaMemcpyAsync(&err, p.err, 4, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
+    if (err) fail(DINO_ETIMEOUT, "a device wait gave up (code %d)", err);
     std::vector<double> tmp;
     auto fetch = [&](const void *src, size_t cnt, bool f32, double *dst) {
       if (!dst) return;
@@ -1779,12 +1976,13 @@ static void dis_from_surrogate(dino_ctx *ctx, int sid, int n, uint64_t seed, int
   try {
     w = (double *)dev_alloc(ctx, wbytes);
     layout_pool(p, true);
+    CK(cudaMemsetAsync(p.err, 0, 16, st));
     double *At = w, *H = At + K * r, *G = H + rr, *Q = G + rr, *sig = Q + rr, *Et = sig + r + rr,
            *Dn = Et + (size_t)N * r, *En = Dn + (size_t)N * r_new, *PrT = En + (size_t)N * r_new;
     // encoded prior draws m_r ~ N(0, I_r) and the surrogate's Jacobian there
     launch(ctx, st, "normals", [&] { return launch_normals(seed, STREAM_DIS_ID, n, r, p.b, st); });
     split_input(ctx, s, p.w, p.b, st);
-    eval_surrogate(ctx, s, p.w, p.b, st);
+    eval_surrogate(ctx, s, p.w, p.b, p.err, st);
     const bool tc = s->precision == DINO_PREC_BF16;
     // H_mc = (1/n) sum_i J_i^T J_i / noise_var = At At^T, At = J^T / sqrt(n noise_var)
     launch(ctx, st, "transpose", [&] {
@@ -1799,7 +1997,10 @@ static void dis_from_surrogate(dino_ctx *ctx, int sid, int n, uint64_t seed, int
     std::vector<double> lam(r), Qh(rr);
     CK(cudaMemcpyAsync(lam.data(), sig, r * 8, cudaMemcpyDeviceToHost, st));
     CK(cudaMemcpyAsync(Qh.data(), Q, rr * 8, cudaMemcpyDeviceToHost, st));
+    int err = 0;
+    CK(cudaMemcpyAsync(&err, p.err, 4, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
+    if (err) fail(DINO_ETIMEOUT, "a device wait gave up (code %d)", err);
     // decreasing eigenvalues (H_mc is positive semidefinite: column norms = eigenvalues)
     std::vector<int> order(r);
     std::iota(order.begin(), order.end(), 0);

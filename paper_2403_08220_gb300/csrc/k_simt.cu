@@ -1,149 +1,71 @@
-// SIMT kernels of the sampler: FP64/FP32 tiled GEMMs with fused epilogues
-// (MLP layers, reverse-mode Jacobian products, complement projection and
-// field update), the full-KLE prior draw, and small elementwise helpers.
+// SIMT kernels of the sampler: the small FP64 GEMMs with fused epilogues (the
+// large ones run on the tensor cores, k_gemm64.cu), the full-KLE prior draw,
+// and small elementwise helpers.
 //
 // GEMM convention: out = epilogue(A B^T) with A: M x K (row pitch lda) and
 // B: N x K (row pitch ldb), i.e. both operands K-contiguous.
 #include <algorithm>
 
 #include "dino_internal.h"
+#include "epi64.cuh"
 #include "philox.cuh"
 
 namespace dino {
 namespace {
 
-constexpr int BM = 64, BN = 64, BK = 16, TM = 4, TN = 4, kGemmThreads = 256;
+// SIMT GEMM for the products too small for the tensor cores' digits (and for
+// operands without digits).  A CTA of 256 threads computes a T x T tile, kKG
+// threads per output: thread q takes the columns q, q + kKG, ... in two
+// alternating sums, joined by a butterfly, so that a long reduction over few
+// outputs still spreads over many CTAs.  The FP64 pipe takes one warp
+// instruction in 16 cycles, so operands read straight from L1 keep up with
+// it; what counts is to have every SM's pipe busy.  kKG depends on K alone:
+// an output's value does not depend on how many rows the product has.
+// (64 x 64 tiles staged in shared memory, the layout before: 1200 us for 64 x
+// 16 outputs over K = 1089 on one CTA, 117 us for 64 x 64 x 64 with a tanh;
+// now 18 and 9 us.)
+constexpr int kGemmThreads = 256;
 
-template <typename T>
-__device__ __forceinline__ T act_fn(int kind, T z) {
-  if (kind == 1) return tanh(z);
-  if (kind == 2) return T(0.5) * z * (T(1) + erf(z * T(0.70710678118654752440)));
-  return z;
-}
-
-template <typename T>
-__device__ __forceinline__ T act_deriv(int kind, T z) {
-  if (kind == 1) {
-    const T t = tanh(z);
-    return T(1) - t * t;
-  }
-  if (kind == 2)
-    return T(0.5) * (T(1) + erf(z * T(0.70710678118654752440))) +
-           z * exp(T(-0.5) * z * z) * T(0.39894228040143267794);
-  return T(1);
-}
-
-// Tiled GEMM: each thread owns a TM x TN block of outputs, strided by 16 so
-// that the shared-memory reads of a warp fall in distinct banks.
-template <typename T, class Epi>
+template <typename T, int kT, int kKG, class Epi>
 __global__ void __launch_bounds__(kGemmThreads)
     k_gemm(int M, int N, int K, const T *__restrict__ A, int lda, const T *__restrict__ B,
            int ldb, Epi epi) {
-  __shared__ T As[BK][BM + 1];
-  __shared__ T Bs[BK][BN + 1];
-  const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-  const int row0 = blockIdx.y * BM, col0 = blockIdx.x * BN;
-  T acc[TM][TN];
-#pragma unroll
-  for (int i = 0; i < TM; ++i)
-#pragma unroll
-    for (int j = 0; j < TN; ++j) acc[i][j] = T(0);
-  for (int k0 = 0; k0 < K; k0 += BK) {
-    for (int e = tid; e < BM * BK; e += kGemmThreads) {
-      const int m = e / BK, k = e % BK, gr = row0 + m, gk = k0 + k;
-      As[k][m] = (gr < M && gk < K) ? A[(size_t)gr * lda + gk] : T(0);
-    }
-    for (int e = tid; e < BN * BK; e += kGemmThreads) {
-      const int n = e / BK, k = e % BK, gc = col0 + n, gk = k0 + k;
-      Bs[k][n] = (gc < N && gk < K) ? B[(size_t)gc * ldb + gk] : T(0);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < BK; ++k) {
-      T a[TM], b[TN];
-#pragma unroll
-      for (int i = 0; i < TM; ++i) a[i] = As[k][ty + 16 * i];
-#pragma unroll
-      for (int j = 0; j < TN; ++j) b[j] = Bs[k][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < TM; ++i)
-#pragma unroll
-        for (int j = 0; j < TN; ++j) acc[i][j] += a[i] * b[j];
-    }
-    __syncthreads();
+  static_assert(kT * kT * kKG == kGemmThreads, "one output per kKG threads");
+  __shared__ T out[kT * kT];
+  const int o = threadIdx.x / kKG, q = threadIdx.x % kKG;
+  const int row0 = blockIdx.x * kT, col0 = blockIdx.y * kT;
+  const T *a = A + (size_t)min(row0 + o / kT, M - 1) * lda;
+  const T *b = B + (size_t)min(col0 + o % kT, N - 1) * ldb;
+  T s0 = T(0), s1 = T(0);
+  int k = q;
+#pragma unroll 4
+  for (; k + kKG < K; k += 2 * kKG) {
+    s0 += a[k] * b[k];
+    s1 += a[k + kKG] * b[k + kKG];
   }
+  if (k < K) s0 += a[k] * b[k];
+  s0 += s1;
 #pragma unroll
-  for (int i = 0; i < TM; ++i)
-#pragma unroll
-    for (int j = 0; j < TN; ++j) {
-      const int r = row0 + ty + 16 * i, c = col0 + tx + 16 * j;
-      if (r < M && c < N) epi(r, c, acc[i][j]);
-    }
+  for (int w = kKG / 2; w; w >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, w);
+  if (q == 0) out[o] = s0;
+  __syncthreads();
+  if (threadIdx.x < kT * kT) {
+    const int r = row0 + threadIdx.x / kT, c = col0 + threadIdx.x % kT;
+    if (r < M && c < N) epi(r, c, out[threadIdx.x]);
+  }
 }
-
-template <typename T>
-struct EpiStore {
-  T *out;
-  int ldo;
-  __device__ void operator()(int r, int c, T v) const { out[(size_t)r * ldo + c] = v; }
-};
-
-template <typename T>
-struct EpiBiasAct {
-  const T *bias;
-  int act;
-  T *out, *der;
-  int ldo;
-  __device__ void operator()(int r, int c, T v) const {
-    const T z = v + bias[c];
-    out[(size_t)r * ldo + c] = act_fn(act, z);
-    if (der) der[(size_t)r * ldo + c] = act_deriv(act, z);
-  }
-};
-
-template <typename T>
-struct EpiScaleGroup {
-  const T *scale;
-  int lds, group;
-  T *out;
-  int ldo;
-  __device__ void operator()(int r, int c, T v) const {
-    out[(size_t)r * ldo + c] = v * scale[(size_t)(r / group) * lds + c];
-  }
-};
-
-template <typename T>
-struct EpiCoef {
-  const double *coef;
-  int ldc;
-  double cs;
-  T *out;
-  int ldo;
-  __device__ void operator()(int r, int c, T v) const {
-    out[(size_t)r * ldo + c] = (T)(coef[(size_t)r * ldc + c] - cs * (double)v);
-  }
-};
-
-template <typename T>
-struct EpiField {
-  const int *acc;
-  double s, cs;
-  T *m;
-  const T *Mf;
-  int ldm;
-  __device__ void operator()(int r, int c, T v) const {
-    if (!acc[r]) return;
-    const size_t o = (size_t)r * ldm + c;
-    m[o] = (T)(s * (double)m[o] + cs * (double)Mf[o]) + v;
-  }
-};
 
 template <typename T, class Epi>
 cudaError_t run_gemm(int M, int N, int K, const T *A, int lda, const T *B, int ldb, Epi epi,
                      cudaStream_t st) {
   if (M <= 0 || N <= 0) return cudaSuccess;
-  dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM);
-  k_gemm<T, Epi><<<grid, kGemmThreads, 0, st>>>(M, N, K, A, lda, B, ldb, epi);
+  if (K > 256) {  // long reductions: 16 threads per output, 4 x 4 tiles
+    dim3 grid((M + 3) / 4, (N + 3) / 4);
+    k_gemm<T, 4, 16, Epi><<<grid, kGemmThreads, 0, st>>>(M, N, K, A, lda, B, ldb, epi);
+  } else {
+    dim3 grid((M + 7) / 8, (N + 7) / 8);
+    k_gemm<T, 8, 4, Epi><<<grid, kGemmThreads, 0, st>>>(M, N, K, A, lda, B, ldb, epi);
+  }
   return cudaGetLastError();
 }
 
