@@ -5,8 +5,9 @@
 // device byte through its own pool, or a latency-critical loop in which the
 // device-wide synchronisation that cudaMalloc/cudaFree may imply is not
 // acceptable.  The entry point below therefore never allocates.  Inputs and
-// outputs are device buffers the caller owns.  The intermediate products of
-// the reverse-mode Jacobian live in one file-scope device array of fixed size.
+// outputs are device buffers the caller owns.  The activations and their
+// derivatives live in one file-scope device array of fixed size, the products
+// of the reverse-mode Jacobian in shared memory.
 // Every GPU that loads this library holds that array until the process exits.
 //
 // Set-up: the host cannot use the array's name as a device address (in host
@@ -24,6 +25,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <mutex>
 
 namespace dino {
@@ -31,7 +33,7 @@ namespace {
 
 constexpr int kMaxLayers = 16;
 constexpr int kMaxDevices = 64;
-constexpr int kThreads = 256;
+constexpr int kJacThreads = 512;
 
 static __device__ __align__(256) double g_noalloc_scratch[DINO_NOALLOC_SCRATCH_DOUBLES];
 
@@ -59,73 +61,80 @@ __device__ __forceinline__ double act_deriv(int kind, double z) {
   return 1.0;
 }
 
-// One CTA per point.  Shared memory holds the activations and the activation
-// derivatives; the d_y x w products of the reverse sweep go to a per-point
-// slab of the scratch array (two ping-pong buffers of d_y * wmax doubles).
-__global__ void __launch_bounds__(kThreads)
-    k_jac_noalloc(const Net net, int wmax, const double *__restrict__ x, double *__restrict__ f,
-                  double *__restrict__ J, double *__restrict__ scratch) {
+// One layer of the forward pass for every point of the chunk: a warp per
+// output, lanes along the weight row.  The activations ping-pong between two
+// halves of a point's slab of the scratch array; the activation derivatives of
+// all hidden layers follow them (offset der_off of layer l).
+__global__ void __launch_bounds__(256)
+    k_layer(const Net net, int l, int wmax, int der_off, size_t slab, const double *__restrict__ x,
+            double *__restrict__ f, double *__restrict__ scratch) {
+  const int p = blockIdx.y, o = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int wi = net.w[l], wo = net.w[l + 1], r = net.w[0], dy = net.w[net.L];
+  if (o >= wo) return;
+  double *s = scratch + (size_t)p * slab;
+  const double *a = l == 0 ? x + (size_t)p * r : s + ((l - 1) & 1) * (size_t)wmax;
+  const double *W = net.W[l] + (size_t)o * wi;
+  double z = 0.0;
+  for (int i = lane; i < wi; i += 32) z += W[i] * a[i];
+#pragma unroll
+  for (int q = 16; q; q >>= 1) z += __shfl_xor_sync(0xffffffffu, z, q);
+  if (lane) return;
+  z += net.b[l][o];
+  if (l + 1 < net.L) {
+    s[(l & 1) * (size_t)wmax + o] = act_fn(net.act, z);
+    s[2 * (size_t)wmax + der_off + o] = act_deriv(net.act, z);
+  } else {
+    f[(size_t)p * dy + o] = z;
+  }
+}
+
+// Reverse sweep, rows [i0, i0 + rows) of one point's Jacobian per CTA: the rows
+// of P = W_{L-1} .* d_{L-2}, P <- (P W_l) .* d_{l-1}, J = P W_0 are independent, so
+// they stay in the CTA's shared memory and the d_y rows of a point spread over
+// as many SMs as there are.  The FP64 pipe (2 multiply-adds a cycle and SM)
+// bounds it, so a thread per output with its operands from L1 and shared
+// memory keeps up.  Eight points of widths 200-400-400-100: 8.0 ms with a CTA
+// per point and the products in global scratch, 0.44 ms here (0.31 ms at the
+// rate of 152 FP64 pipes).
+__global__ void __launch_bounds__(kJacThreads)
+    k_jac_rows(const Net net, int wmax, int rows, size_t slab, double *__restrict__ J,
+               const double *__restrict__ scratch) {
   extern __shared__ double sm[];
-  const int p = blockIdx.x, L = net.L, r = net.w[0], dy = net.w[L];
-  double *a[kMaxLayers + 1];
-  double *d[kMaxLayers];
-  int off = 0;
-  for (int l = 0; l < L; ++l) {  // a[0..L-1]: layer inputs; d[0..L-2]: derivatives
-    a[l] = sm + off;
-    off += net.w[l];
-  }
-  for (int l = 0; l + 1 < L; ++l) {
-    d[l] = sm + off;
-    off += net.w[l + 1];
-  }
-  for (int i = threadIdx.x; i < r; i += blockDim.x) a[0][i] = x[(size_t)p * r + i];
-  __syncthreads();
-  for (int l = 0; l < L; ++l) {
-    const int wi = net.w[l], wo = net.w[l + 1];
-    const double *W = net.W[l];
-    for (int o = threadIdx.x; o < wo; o += blockDim.x) {
-      double z = net.b[l][o];
-      for (int i = 0; i < wi; ++i) z += W[(size_t)o * wi + i] * a[l][i];
-      if (l + 1 < L) {
-        a[l + 1][o] = act_fn(net.act, z);
-        d[l][o] = act_deriv(net.act, z);
-      } else {
-        f[(size_t)p * dy + o] = z;
-      }
-    }
-    __syncthreads();
-  }
-  double *Jp = J + (size_t)p * dy * r;
+  const int p = blockIdx.y, L = net.L, r = net.w[0], dy = net.w[L];
+  const int i0 = blockIdx.x * rows, nr = min(rows, dy - i0);
+  double *Jp = J + ((size_t)p * dy + i0) * r;
   if (L == 1) {
-    for (int e = threadIdx.x; e < dy * r; e += blockDim.x) Jp[e] = net.W[0][e];
+    for (int e = threadIdx.x; e < nr * r; e += blockDim.x)
+      Jp[e] = net.W[0][(size_t)i0 * r + e];
     return;
   }
-  double *P = scratch + (size_t)p * 2 * dy * wmax;
-  double *Q = P + (size_t)dy * wmax;
+  const double *der = scratch + (size_t)p * slab + 2 * (size_t)wmax;
+  int off = 0;  // of d_{l - 1} (layer widths w_1 .. w_{L - 1})
+  for (int l = 1; l < L - 1; ++l) off += net.w[l];
+  double *P = sm, *Q = sm + (size_t)rows * wmax;
   const int wl = net.w[L - 1];
-  for (int e = threadIdx.x; e < dy * wl; e += blockDim.x)
-    P[e] = net.W[L - 1][e] * d[L - 2][e % wl];
+  for (int e = threadIdx.x; e < nr * wl; e += blockDim.x)
+    P[e] = net.W[L - 1][(size_t)i0 * wl + e] * der[off + e % wl];
   __syncthreads();
-  for (int l = L - 2; l >= 1; --l) {  // P <- (P W_l) .* d_{l-1}
+  for (int l = L - 2; l >= 0; --l) {
     const int wi = net.w[l], wo = net.w[l + 1];
-    const double *W = net.W[l];
-    for (int e = threadIdx.x; e < dy * wi; e += blockDim.x) {
-      const int i = e / wi, j = e % wi;
+    const double *__restrict__ W = net.W[l];
+    if (l > 0) off -= wi;
+    for (int e = threadIdx.x; e < nr * wi; e += blockDim.x) {
+      const int i = e / wi, j = e - i * wi;
+      const double *Pi = P + (size_t)i * wo, *Wj = W + j;
       double acc = 0.0;
-      for (int k = 0; k < wo; ++k) acc += P[(size_t)i * wo + k] * W[(size_t)k * wi + j];
-      Q[e] = acc * d[l - 1][j];
+#pragma unroll 8
+      for (int k = 0; k < wo; ++k) acc += Pi[k] * Wj[(size_t)k * wi];
+      if (l > 0)
+        Q[e] = acc * der[off + j];
+      else
+        Jp[e] = acc;
     }
     __syncthreads();
     double *t = P;
     P = Q;
     Q = t;
-  }
-  const int w1 = net.w[1];
-  for (int e = threadIdx.x; e < dy * r; e += blockDim.x) {  // J = P W_0
-    const int i = e / r, j = e % r;
-    double acc = 0.0;
-    for (int k = 0; k < w1; ++k) acc += P[(size_t)i * w1 + k] * net.W[0][(size_t)k * r + j];
-    Jp[e] = acc;
   }
 }
 
@@ -183,10 +192,42 @@ extern "C" int dino_surrogate_jacobian_noalloc(int n, int n_layers, const int *w
     }
     scratch = g_addr[dev];
   }
-  if (smem > 48 * 1024 &&
-      cudaFuncSetAttribute(k_jac_noalloc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem) != cudaSuccess)
+  // a point's slab: two activation buffers and every hidden layer's derivatives
+  const cudaStream_t st = (cudaStream_t)stream;
+  size_t hidden = 0;
+  for (int l = 1; l < n_layers; ++l) hidden += widths[l];
+  const int r = widths[0], dy = widths[n_layers];
+  const size_t slab = 2 * (size_t)wmax + hidden;
+  const size_t most = slab ? (size_t)DINO_NOALLOC_SCRATCH_DOUBLES / slab : (size_t)n;
+  // blockIdx.y runs over the points of a chunk
+  const int chunk = (int)std::min({most, (size_t)n, (size_t)65535});
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
     return DINO_ECUDA;
-  k_jac_noalloc<<<n, kThreads, smem, (cudaStream_t)stream>>>(net, wmax, x, f, J, scratch);
-  return cudaGetLastError() == cudaSuccess ? DINO_OK : DINO_ECUDA;
+  // rows per CTA: one CTA on every SM, within the shared memory of one CTA
+  // (two buffers of rows x wmax; one row always fits, since the widths' sums do)
+  const size_t row_bytes = 2 * (size_t)wmax * sizeof(double);
+  size_t rows = ((size_t)std::min(n, chunk) * dy + sms - 1) / sms;
+  if (row_bytes) rows = std::min(rows, (size_t)(200 * 1024) / row_bytes);
+  rows = std::max<size_t>(1, std::min(rows, (size_t)dy));
+  const size_t jsm = rows * row_bytes;
+  if (jsm > 48 * 1024 &&
+      cudaFuncSetAttribute(k_jac_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)jsm) !=
+          cudaSuccess)
+    return DINO_ECUDA;
+  for (int p0 = 0; p0 < n; p0 += chunk) {
+    const int np = std::min(chunk, n - p0);
+    int off = 0;
+    for (int l = 0; l < n_layers; ++l) {
+      dim3 grid((widths[l + 1] + 7) / 8, np);
+      k_layer<<<grid, 256, 0, st>>>(net, l, wmax, off, slab, x + (size_t)p0 * r,
+                                    f + (size_t)p0 * dy, scratch);
+      if (l + 1 < n_layers) off += widths[l + 1];
+    }
+    dim3 grid((unsigned)((dy + rows - 1) / rows), np);
+    k_jac_rows<<<grid, kJacThreads, jsm, st>>>(net, wmax, (int)rows, slab,
+                                               J + (size_t)p0 * dy * r, scratch);
+    if (cudaGetLastError() != cudaSuccess) return DINO_ECUDA;
+  }
+  return DINO_OK;
 }

@@ -1,0 +1,45 @@
+"""The allocation-free Jacobian's row split and its chunks of points.
+
+Rows per CTA with a remainder, one row per CTA, fewer rows than SMs, more
+points than the fixed scratch holds slabs for (d_y = 1 and many layers: the
+call runs in several chunks), against the FP64 oracle at the FP64 parity bar.
+"""
+import numpy as np
+import pytest
+
+from helpers import rel_err
+from oracle import mlp
+from workloads import mlp_weights
+
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-10
+
+
+@pytest.mark.parametrize("widths,act,n", [
+    ([33, 41, 100], mlp.ACT_TANH, 1),
+    ([200, 400, 400, 101], mlp.ACT_GELU, 11),
+    ([7, 64, 200, 3, 90, 128], mlp.ACT_GELU, 20),
+    ([5] + [100] * 10 + [1], mlp.ACT_TANH, 5242),
+    ([12, 6000, 2], mlp.ACT_GELU, 40),
+])
+def test_rows_and_chunks(widths, act, n):
+    torch = pytest.importorskip("torch")
+    import paper_2403_08220_gb300 as dino
+
+    Ws, bs = mlp_weights(widths, 17)
+    dev = torch.device("cuda", 0)
+    Wt = [torch.tensor(W, dtype=torch.float64, device=dev).contiguous() for W in Ws]
+    bt = [torch.tensor(b, dtype=torch.float64, device=dev).contiguous() for b in bs]
+    x = np.random.default_rng(3).standard_normal((n, widths[0]))
+    f_ref, zs = mlp.forward(Ws, bs, act, x)
+    J_ref = mlp.jacobian_reverse(Ws, act, zs)
+    xt = torch.tensor(x, dtype=torch.float64, device=dev)
+    ft = torch.full((n, widths[-1]), float("nan"), dtype=torch.float64, device=dev)
+    Jt = torch.full((n, widths[-1], widths[0]), float("nan"), dtype=torch.float64, device=dev)
+    dino.dino_surrogate_jacobian_noalloc(
+        n, widths, act, [t.data_ptr() for t in Wt], [t.data_ptr() for t in bt], xt.data_ptr(),
+        ft.data_ptr(), Jt.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    assert rel_err(ft.cpu().numpy(), f_ref) <= TOL
+    assert rel_err(Jt.cpu().numpy(), J_ref) <= TOL
