@@ -293,11 +293,20 @@ cudaError_t launch_diag_center(int d, int n_c, int n_s, const double *traj, int 
                                const double *means, double *Xc, double *Mc, cudaStream_t st);
 cudaError_t launch_diag_wv(int d, int n_c, int n_s, const double *Wr, const double *Br, double *W,
                            double *V, cudaStream_t st);
-// one-sided Jacobi on the d columns of G (in place); Q (optional) gets the
-// accumulated rotations, sig the column norms, *sweeps the sweeps taken
-cudaError_t launch_jacobi(int d, double *G, double *Q, double *sig, int *sweeps, cudaStream_t st);
-cudaError_t launch_sym_sqrt(int d, const double *Q, const double *lam, double *S, cudaStream_t st);
-cudaError_t launch_small_mm(int d, const double *A, const double *B, double *C, cudaStream_t st);
+// One-sided Jacobi on the d columns of G (in place), Q (optional, I on entry)
+// accumulating the rotations: a sweep is jacobi_rounds(d) rounds, and *rotated
+// is set when a round turned any pair.
+constexpr int kMaxJacobiSweeps = 60;
+int jacobi_rounds(int d);
+cudaError_t launch_eye(int d, double *Q, cudaStream_t st);
+cudaError_t launch_jacobi_round(int d, int rnd, double *G, double *Q, int *rotated,
+                                cudaStream_t st);
+cudaError_t launch_col_norms(int d, const double *G, double *sig, cudaStream_t st);
+// W = F F^T, V = C C^T (positive semidefinite, lower triangular factors)
+cudaError_t launch_psd_chol(int d, const double *W, const double *V, double *F, double *C,
+                            cudaStream_t st);
+// G = C^T F by columns
+cudaError_t launch_ct_f(int d, const double *C, const double *F, double *G, cudaStream_t st);
 cudaError_t launch_mpsrf_final(int d, const double *W, const double *V, const double *sig,
                                double *out, cudaStream_t st);
 // out (n x r) = standard normals of Philox (seed, stream, step 0, chain i)

@@ -486,10 +486,11 @@ static T *sur_upload(dino_ctx *ctx, Surrogate *s, const T *host, size_t n) {
 // on how many chains share the product.
 constexpr long kDigitsMinWork = 16384;
 
-// Digits of a device matrix B.  Left empty where the rule above or the HBM
-// budget says no; its products then take the SIMT GEMM.
+// Digits of a device matrix B, with its column exponents taken out unless the
+// same digits are to serve as A too.  Left empty where the rule above or the
+// HBM budget says no; its products then take the SIMT GEMM.
 static DigitMat make_digits(dino_ctx *ctx, std::vector<std::pair<void *, size_t>> &allocs,
-                            const double *B, int rows, int K) {
+                            const double *B, int rows, int K, bool equilibrate = true) {
   DigitMat m;
   if ((long)rows * K < kDigitsMinWork || rows < 32 || K < 32) return m;
   const int ldp = digit_pitch(K);
@@ -504,8 +505,8 @@ static DigitMat make_digits(dino_ctx *ctx, std::vector<std::pair<void *, size_t>
   ctx->used += bytes;
   allocs.push_back({p, bytes});
   auto *d = (__nv_bfloat16 *)p;
-  int *ex = (int *)(d + plane * kDigits64), *fk = ex + rows;
-  CK(launch_col_exp(rows, K, B, K, fk, ctx->stream));
+  int *ex = (int *)(d + plane * kDigits64), *fk = equilibrate ? ex + rows : nullptr;
+  if (fk) CK(launch_col_exp(rows, K, B, K, fk, ctx->stream));
   CK(launch_split64(rows, K, B, K, nullptr, nullptr, 1, 0, 0, fk, -1, d, ldp, plane, ex,
                     ctx->stream));
   m.d = d;
@@ -1953,6 +1954,70 @@ static void surrogate_eval(dino_ctx *ctx, int sid, int n, const double *x_host, 
 }
 
 // ---------------------------------------------------------------------------
+// dense symmetric problems of the diagnostics and the DIS basis
+
+// One-sided Jacobi on the columns of G: sweeps until one turns no pair, at most
+// kMaxJacobiSweeps; sig gets the column norms.  Synchronises the stream once a
+// sweep (a sweep is one launch per round).  flags: kMaxJacobiSweeps device ints.
+static int jacobi(dino_ctx *ctx, int d, double *G, double *Q, double *sig, int *flags,
+                  cudaStream_t st) {
+  CK(cudaMemsetAsync(flags, 0, kMaxJacobiSweeps * sizeof(int), st));
+  if (Q) launch(ctx, st, "jacobi_eye", [&] { return launch_eye(d, Q, st); });
+  int sweep = 0;
+  for (; sweep < kMaxJacobiSweeps; ++sweep) {
+    for (int rnd = 0; rnd < jacobi_rounds(d); ++rnd)
+      launch(ctx, st, "jacobi",
+             [&] { return launch_jacobi_round(d, rnd, G, Q, flags + sweep, st); });
+    int any = 0;
+    CK(cudaMemcpyAsync(&any, flags + sweep, sizeof(int), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    if (!any) break;
+  }
+  launch(ctx, st, "jacobi_norms", [&] { return launch_col_norms(d, G, sig, st); });
+  return sweep + 1;
+}
+
+// H = X X^T for a row-major d x K matrix X of the device: on the tensor cores
+// when the rule of make_digits admits X and its digits (16 bytes an entry) fit
+// the budget for the time of the call.
+static void gram64(dino_ctx *ctx, const char *name, int d, int K, const double *X, double *H,
+                   cudaStream_t st) {
+  std::vector<std::pair<void *, size_t>> tmp;
+  const DigitMat g = make_digits(ctx, tmp, X, d, K, false);
+  try {
+    if (g.d) {
+      int *err = (int *)dev_alloc(ctx, 16);
+      tmp.push_back({err, 16});
+      CK(cudaMemsetAsync(err, 0, 16, st));
+      Gemm64Args a;
+      a.M = a.N = d;
+      a.K = K;
+      a.A = g.d;
+      a.ea = g.ex;
+      a.ldp = g.ldp;
+      a.plane = g.plane;
+      a.Asrc = X;
+      a.lda = K;
+      a.B = g;
+      a.err = err;
+      launch(ctx, st, name, [&] { return gemm64_store(a, H, d, st); });
+      int e = 0;
+      CK(cudaMemcpyAsync(&e, err, 4, cudaMemcpyDeviceToHost, st));
+      CK(cudaStreamSynchronize(st));
+      if (e) fail(DINO_ETIMEOUT, "a device wait gave up (code %d)", e);
+    } else {
+      launch(ctx, st, name,
+             [&] { return gemm_store<double>(d, d, K, X, K, X, K, H, d, st); });
+    }
+  } catch (...) {
+    cudaStreamSynchronize(st);
+    for (auto &x : tmp) dev_free(ctx, x.first, x.second);
+    throw;
+  }
+  for (auto &x : tmp) dev_free(ctx, x.first, x.second);
+}
+
+// ---------------------------------------------------------------------------
 // derivative-informed subspace from the surrogate's Jacobians (setup)
 
 static void dis_from_surrogate(dino_ctx *ctx, int sid, int n, uint64_t seed, int r_new,
@@ -1970,7 +2035,7 @@ static void dis_from_surrogate(dino_ctx *ctx, int sid, int n, uint64_t seed, int
   p.ar.bytes = p.ar.off;
   const size_t K = (size_t)n * dy, rr = (size_t)r * r;
   const size_t wbytes = (K * r + 4 * rr + r + (size_t)N * r + 2 * (size_t)N * r_new +
-                         (size_t)r_new * r) * 8;
+                         (size_t)r_new * r + kMaxJacobiSweeps) * 8;
   p.ar.base = (char *)dev_alloc(ctx, p.ar.bytes);
   double *w = nullptr;
   try {
@@ -1989,11 +2054,9 @@ static void dis_from_surrogate(dino_ctx *ctx, int sid, int n, uint64_t seed, int
       return launch_transpose((int)K, r, tc ? (const void *)p.w.J32 : (const void *)p.w.J64,
                               tc ? 1 : 0, r, 1.0 / std::sqrt((double)n * s->noise_var), At, st);
     });
-    launch(ctx, st, "dis_gram", [&] {
-      return gemm_store<double>(r, r, (int)K, At, (int)K, At, (int)K, H, r, st);
-    });
+    gram64(ctx, "dis_gram", r, (int)K, At, H, st);
     CK(cudaMemcpyAsync(G, H, rr * 8, cudaMemcpyDeviceToDevice, st));
-    launch(ctx, st, "jacobi", [&] { return launch_jacobi(r, G, Q, sig, nullptr, st); });
+    jacobi(ctx, r, G, Q, sig, (int *)(PrT + (size_t)r_new * r), st);
     std::vector<double> lam(r), Qh(rr);
     CK(cudaMemcpyAsync(lam.data(), sig, r * 8, cudaMemcpyDeviceToHost, st));
     CK(cudaMemcpyAsync(Qh.data(), Q, rr * 8, cudaMemcpyDeviceToHost, st));
@@ -2145,35 +2208,26 @@ static void diag_compute(dino_ctx *ctx, Diag *g, int want_mpsrf, double *ess_out
   int sweeps = 0;
   if (want_mpsrf) {
     const size_t K = (size_t)n_c * n_s, dd = (size_t)d * d;
-    const size_t bytes = ((size_t)d * K + (size_t)d * n_c + 9 * dd + d + 4) * 8;
+    const size_t bytes = ((size_t)d * K + (size_t)d * n_c + 7 * dd + d + 4 + kMaxJacobiSweeps) * 8;
     double *w = (double *)dev_alloc(ctx, bytes);
     try {
       double *Xc = w, *Mc = Xc + (size_t)d * K, *Wr = Mc + (size_t)d * n_c, *Br = Wr + dd,
-             *W = Br + dd, *V = W + dd, *G = V + dd, *Q = G + dd, *Wh = Q + dd, *T = Wh + dd,
-             *M = T + dd, *sig = M + dd, *o = sig + d;
+             *W = Br + dd, *V = W + dd, *F = V + dd, *Cv = F + dd, *G = Cv + dd, *sig = G + dd,
+             *o = sig + d;
       launch(ctx, st, "diag_center", [&] {
         return launch_diag_center(d, n_c, n_s, g->traj, g->max_s, g->means, Xc, Mc, st);
       });
-      launch(ctx, st, "diag_gram", [&] {
-        return gemm_store<double>(d, d, (int)K, Xc, (int)K, Xc, (int)K, Wr, d, st);
-      });
+      gram64(ctx, "diag_gram", d, (int)K, Xc, Wr, st);
       launch(ctx, st, "diag_gram", [&] {
         return gemm_store<double>(d, d, n_c, Mc, n_c, Mc, n_c, Br, d, st);
       });
       launch(ctx, st, "diag_wv", [&] { return launch_diag_wv(d, n_c, n_s, Wr, Br, W, V, st); });
-      // W = Q diag(lam) Q^T (W symmetric: its rows are its columns)
-      CK(cudaMemcpyAsync(G, W, dd * 8, cudaMemcpyDeviceToDevice, st));
-      launch(ctx, st, "jacobi", [&] { return launch_jacobi(d, G, Q, sig, nullptr, st); });
-      launch(ctx, st, "sym_sqrt", [&] { return launch_sym_sqrt(d, Q, sig, Wh, st); });
-      launch(ctx, st, "small_mm", [&] { return launch_small_mm(d, Wh, V, T, st); });
-      launch(ctx, st, "small_mm", [&] { return launch_small_mm(d, T, Wh, M, st); });
-      // eigenvalues of W^1/2 V W^1/2 (symmetric positive semidefinite)
-      launch(ctx, st, "jacobi", [&] {
-        return launch_jacobi(d, M, nullptr, sig, reinterpret_cast<int *>(o + 3), st);
-      });
+      // the singular values of C^T F, W = F F^T, V = C C^T (k_diag.cu)
+      launch(ctx, st, "psd_chol", [&] { return launch_psd_chol(d, W, V, F, Cv, st); });
+      launch(ctx, st, "ct_f", [&] { return launch_ct_f(d, Cv, F, G, st); });
+      sweeps = jacobi(ctx, d, G, nullptr, sig, (int *)(o + 4), st);
       launch(ctx, st, "mpsrf_final", [&] { return launch_mpsrf_final(d, W, V, sig, o, st); });
       CK(cudaMemcpyAsync(out, o, 24, cudaMemcpyDeviceToHost, st));
-      CK(cudaMemcpyAsync(&sweeps, o + 3, 4, cudaMemcpyDeviceToHost, st));
       CK(cudaStreamSynchronize(st));
     } catch (...) {
       cudaStreamSynchronize(st);

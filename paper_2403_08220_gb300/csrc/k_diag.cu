@@ -7,28 +7,32 @@
 //                   a caller buffer);
 //   k_diag_ess      one CTA per degree of freedom: chain means and variances,
 //                   w and v (the 1D covariance estimators), the multi-chain
-//                   autocorrelation MACT(t) = 1 - (w - mean_k AC(t,k)) / v lag
-//                   pair by lag pair until the pair sum is no longer positive
+//                   autocorrelation MACT(t) = 1 - (w - mean_k AC(t,k)) / v in
+//                   passes of kLags lags until a pair sum is no longer positive
 //                   (the initial positive sequence), ESS% = 1 / (1 + 2 sum_t
 //                   MACT(t)) (eq:ess), and the squared jumps of the MSJ;
 //   k_diag_center   centred samples and centred chain means (d x n_c n_s and
 //                   d x n_c) whose Gram products give W and V
 //                   (eq:covariance_estimator);
-//   k_jacobi        one-sided Jacobi (Hestenes) on a d x d matrix held by
-//                   columns: column pairs are rotated until orthogonal, in
-//                   round-robin order so that the d/2 pairs of a round are
-//                   disjoint and run on separate warps; for a symmetric
-//                   positive semidefinite matrix the final column norms are
-//                   its eigenvalues and the accumulated rotations its
-//                   eigenvectors;
-//   k_sym_sqrt, k_mm  the square root Q diag(sqrt(lambda)) Q^T and the small
-//                   products of the Wasserstein MPSRF
-//                   Tr(W + V - 2 (W^1/2 V W^1/2)^1/2);
+//   k_psd_chol      W = F F^T and V = C C^T (lower triangular, one CTA each);
+//                   the eigenvalues of W^1/2 V W^1/2 are those of F^T V F, the
+//                   squared singular values of C^T F, so the Wasserstein MPSRF
+//                   Tr(W + V - 2 (W^1/2 V W^1/2)^1/2) is Tr W + Tr V - 2 |C^T F|_*
+//                   without a square root of W;
+//   k_ct_f          C^T F by columns;
+//   k_jacobi_round  one-sided Jacobi (Hestenes) on a d x d matrix held by
+//                   columns: column pairs are rotated until orthogonal; a
+//                   launch is one round of a round-robin over blocks of
+//                   columns, whose pairs are disjoint and run on separate CTAs
+//                   (the host loops over rounds and sweeps).  The final column
+//                   norms are the singular values; for a symmetric positive
+//                   semidefinite matrix they are its eigenvalues and the
+//                   accumulated rotations its eigenvectors;
 //   k_normals, k_transpose  the encoded prior draws and the stacked transposed
 //                   Jacobian of the surrogate-driven DIS basis (eq:mc_ppgnh),
 //                   whose eigenproblem the same Jacobi kernel solves.
 // Every loop is bounded by the sizes (lags by n_s, Jacobi sweeps by
-// kMaxSweeps); no kernel waits on another CTA.
+// kMaxJacobiSweeps); no kernel waits on another CTA.
 #include <algorithm>
 
 #include "chol.cuh"
@@ -37,7 +41,6 @@ namespace dino {
 namespace {
 
 constexpr int kEssThreads = 256;
-constexpr int kJacobiThreads = 1024;
 
 template <typename T>
 __global__ void k_diag_record(int n_c, int d, const T *__restrict__ src, int ld_src,
@@ -79,36 +82,70 @@ __device__ void block_sum2(double &x, double &y, double *red) {
   y = red[65];
 }
 
-// Dynamic shared memory: n_c chain means.
+// Sums over the warp of eight values at once: three steps that halve the
+// values a lane carries (4 + 2 + 1 additions) and two that add what is left;
+// lane l returns the sum of v[l & 7] (9 additions for 40).
+__device__ __forceinline__ double warp_sum8(const double v[8]) {
+  const int lane = threadIdx.x & 31;
+  double a[4], b[2], c;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const double keep = (lane & 1) ? v[2 * q + 1] : v[2 * q];
+    const double give = (lane & 1) ? v[2 * q] : v[2 * q + 1];
+    a[q] = keep + __shfl_xor_sync(kFull, give, 1);  // value 2 q + (lane & 1)
+  }
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const double keep = (lane & 2) ? a[2 * q + 1] : a[2 * q];
+    const double give = (lane & 2) ? a[2 * q] : a[2 * q + 1];
+    b[q] = keep + __shfl_xor_sync(kFull, give, 2);  // value 4 q + (lane & 3)
+  }
+  const double keep = (lane & 4) ? b[1] : b[0], give = (lane & 4) ? b[0] : b[1];
+  c = keep + __shfl_xor_sync(kFull, give, 4);  // value lane & 7
+  c += __shfl_xor_sync(kFull, c, 8);
+  return c + __shfl_xor_sync(kFull, c, 16);
+}
+
+constexpr int kLags = 8;     // lags per pass over the samples
+constexpr int kSegment = 128;  // samples of one chain that a warp takes at a time
+
+// Dynamic shared memory: n_c chain means, then with kStaged the centred samples
+// (n_c x n_s).  A pass forms kLags lags: per sample one multiply-add for
+// each from consecutive shared-memory words, and one reduction per pass (one
+// pass per lag pair over global memory, with a division per sample to find
+// its chain, took 17.4 ms for 200 degrees of freedom, 10 chains of 1000
+// samples; 3.3 ms now, 1.6 ms at the FP64 pipes' rate for all 1000 lags).
+// Lags past the first non-positive pair are formed and not used.
+template <bool kStaged>
 __global__ void __launch_bounds__(kEssThreads)
     k_diag_ess(int n_c, int n_s, const double *__restrict__ traj, int max_s,
                double *__restrict__ means, double *__restrict__ ess, double *__restrict__ sqjump) {
   extern __shared__ double mk[];
-  __shared__ double red[72];
+  __shared__ double red[72], lagsum[kEssThreads / 32][kLags];
+  __shared__ bool more_s;
+  double *xs = mk + n_c;
   const int i = blockIdx.x;
   const double *X = traj + (size_t)i * n_c * max_s;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  // chain means (warp per chain)
-  for (int k = warp; k < n_c; k += nw) {
-    double s = 0.0;
-    for (int j = lane; j < n_s; j += 32) s += X[(size_t)k * max_s + j];
-    s = warp_sum(s);
-    if (lane == 0) mk[k] = s / n_s;
-  }
-  __syncthreads();
-  // within-chain sums of squares and squared jumps
+  // chain means, within-chain sums of squares and squared jumps (warp per chain)
   double ss = 0.0, jj = 0.0;
-  const size_t tot = (size_t)n_c * n_s;
-  for (size_t e = threadIdx.x; e < tot; e += blockDim.x) {
-    const int k = (int)(e / n_s), j = (int)(e - (size_t)k * n_s);
-    const double x = X[(size_t)k * max_s + j] - mk[k];
-    ss += x * x;
-    if (j + 1 < n_s) {
-      const double dx = X[(size_t)k * max_s + j + 1] - X[(size_t)k * max_s + j];
-      jj += dx * dx;
+  for (int k = warp; k < n_c; k += nw) {
+    const double *xk = X + (size_t)k * max_s;
+    double s = 0.0;
+    for (int j = lane; j < n_s; j += 32) s += xk[j];
+    const double m = warp_sum(s) / n_s;
+    if (lane == 0) mk[k] = m;
+    for (int j = lane; j < n_s; j += 32) {
+      const double v = xk[j], x = v - m;
+      ss += x * x;
+      if (kStaged) xs[(size_t)k * n_s + j] = x;
+      if (j + 1 < n_s) {
+        const double dx = xk[j + 1] - v;
+        jj += dx * dx;
+      }
     }
   }
-  block_sum2(ss, jj, red);
+  block_sum2(ss, jj, red);  // includes barriers
   double gm = 0.0;
   for (int k = 0; k < n_c; ++k) gm += mk[k];
   gm /= n_c;
@@ -117,25 +154,57 @@ __global__ void __launch_bounds__(kEssThreads)
   const double w = ss / ((double)n_c * (n_s - 1));
   const double v = (double)(n_s - 1) / n_s * w + (double)(n_c + 1) / ((double)n_c * (n_c - 1)) * bs;
   // MACT(t) for lag pairs (2m, 2m + 1), MACT(0) = 1, while the pair sum is positive
+  const double inv_n = 1.0 / ((double)n_s * n_c), inv_v = 1.0 / v;
+  const int segs = (n_s + kSegment - 1) / kSegment;
   double total = 0.0;
   int pairs = 0;
-  for (int m = 0; 2 * m + 1 < n_s; ++m) {
-    double a0 = 0.0, a1 = 0.0;
-    const int t0 = 2 * m, t1 = 2 * m + 1;
-    for (size_t e = threadIdx.x; e < tot; e += blockDim.x) {
-      const int k = (int)(e / n_s), j = (int)(e - (size_t)k * n_s);
-      const double *xs = X + (size_t)k * max_s;
-      const double x = xs[j] - mk[k];
-      if (t0 > 0 && j + t0 < n_s) a0 += x * (xs[j + t0] - mk[k]);
-      if (j + t1 < n_s) a1 += x * (xs[j + t1] - mk[k]);
+  bool more = true;
+  for (int t0 = 0; more && t0 + 1 < n_s; t0 += kLags) {
+    double acc[kLags] = {};
+    for (int it = warp; it < n_c * segs; it += nw) {
+      const int k = it / segs, j0 = (it - k * segs) * kSegment;
+      const double m = mk[k];
+      const double *xk = kStaged ? xs + (size_t)k * n_s : X + (size_t)k * max_s;
+      const int j1 = min(n_s - t0, j0 + kSegment);  // later samples have no partner
+      if (j1 + t0 + kLags - 1 <= n_s) {
+        for (int j = j0 + lane; j < j1; j += 32) {
+          const double x = kStaged ? xk[j] : xk[j] - m;
+#pragma unroll
+          for (int q = 0; q < kLags; ++q) acc[q] += x * (kStaged ? xk[j + t0 + q] : xk[j + t0 + q] - m);
+        }
+      } else {
+        for (int j = j0 + lane; j < j1; j += 32) {
+          const double x = kStaged ? xk[j] : xk[j] - m;
+#pragma unroll
+          for (int q = 0; q < kLags; ++q)
+            if (j + t0 + q < n_s) acc[q] += x * (kStaged ? xk[j + t0 + q] : xk[j + t0 + q] - m);
+        }
+      }
     }
-    block_sum2(a0, a1, red);
-    const double r0 = t0 == 0 ? 1.0 : 1.0 - (w - a0 / ((double)n_s * n_c)) / v;
-    const double r1 = 1.0 - (w - a1 / ((double)n_s * n_c)) / v;
-    const double pair = r0 + r1;
-    if (!(pair > 0.0)) break;
-    total += pair;
-    ++pairs;
+    const double s = warp_sum8(acc);
+    if (lane < kLags) lagsum[warp][lane] = s;
+    __syncthreads();
+    if (warp == 0) {  // lane q: MACT(t0 + q); then the pairs in order
+      double r = 0.0;
+      if (lane < kLags) {
+        for (int u = 0; u < nw; ++u) r += lagsum[u][lane];
+        r = t0 + lane == 0 ? 1.0 : 1.0 - (w - r * inv_n) * inv_v;
+      }
+      const double pair = r + __shfl_xor_sync(kFull, r, 1);
+      bool on = true;
+#pragma unroll
+      for (int q = 0; q < kLags; q += 2) {
+        const double pq = __shfl_sync(kFull, pair, q);
+        on = on && t0 + q + 1 < n_s && pq > 0.0;
+        if (on) {
+          total += pq;
+          ++pairs;
+        }
+      }
+      if (lane == 0) more_s = on;
+    }
+    __syncthreads();
+    more = more_s;
   }
   if (threadIdx.x == 0) {
     ess[i] = pairs > 0 ? 1.0 / (2.0 * total - 1.0) : 1.0;
@@ -173,69 +242,223 @@ __global__ void k_diag_wv(int d, int n_c, int n_s, const double *__restrict__ Wr
   }
 }
 
-constexpr int kMaxSweeps = 60;
+// The rotation (c, s) that makes columns with squared norms al, be and product
+// ga orthogonal: t = tan of the smaller angle.  The angle needs no more than
+// FP32 (what it leaves of ga, ~1e-7 of it, the next sweep takes); the rotation
+// has to be orthogonal in FP64, so c = (1 + t^2)^-1/2 is an FP32 estimate
+// refined by two Newton steps, and FP64 divisions and square roots, long chains
+// on a pipe of 16 cycles an instruction, are left out.
+__device__ __forceinline__ void jacobi_rotation(double al, double be, double ga, double &c,
+                                                double &s) {
+  const double dq = be - al;
+  // both scaled by the same power of two into FP32's range
+  const int e = max((__double2hiint(dq) >> 20) & 0x7ff, (__double2hiint(ga) >> 20) & 0x7ff);
+  const double sc = __hiloint2double(max(1, min(2046, 2046 - e)) << 20, 0);
+  const float fg = (float)(ga * sc);
+  c = 1.0;
+  s = 0.0;
+  if (fg == 0.0f) return;
+  const float z = (float)(dq * sc) / (2.0f * fg), az = fabsf(z);
+  const float ft = az > 1e8f ? 0.5f / az : 1.0f / (az + sqrtf(1.0f + az * az));
+  const double t = (double)copysignf(ft, z), w = 1.0 + t * t;
+  double y = (double)rsqrtf((float)w);
+  y = y * (1.5 - 0.5 * w * y * y);
+  y = y * (1.5 - 0.5 * w * y * y);
+  c = y;
+  s = y * t;
+}
 
-// One-sided Jacobi on the d columns of G (column i at G + i d); with Q the
-// rotations are applied to Q as well (Q = I on entry).  sig[i] = |column i|.
-__global__ void __launch_bounds__(kJacobiThreads)
-    k_jacobi(int d, double *__restrict__ G, double *__restrict__ Q, double *__restrict__ sig,
-             int *__restrict__ sweeps_out) {
-  __shared__ int rotated;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int n = d + (d & 1);  // players of the round-robin, one dummy if d is odd
-  int sweep = 0;
-  for (; sweep < kMaxSweeps; ++sweep) {
-    if (threadIdx.x == 0) rotated = 0;
+constexpr int kPairThreads = 128;  // threads of a column pair
+
+// One round of a sweep: CTA pi takes the pair (p, q) of blocks of kB columns of
+// the round-robin over nb blocks, holds them (and their columns of Q) in
+// shared memory and rotates the kB x kB column pairs across the blocks, kB
+// disjoint ones at a time, each by kPairThreads threads; in the first round
+// of a sweep also the pairs inside the blocks.  With Q the rotations are
+// applied to Q as well.  *rotated is set when any pair was.  What bounds it is
+// the chain of dependent FP64 operations of one rotation (about 5 us with the
+// launch): d = 200, 9 sweeps of 199 rounds, 12.7 ms, against 465 ms for two
+// solves (W's square root, then W^1/2 V W^1/2) by one CTA that looped over all
+// pairs; blocks of 2 and of 4 columns take the same time at d = 200.
+template <int kB>
+__global__ void __launch_bounds__(kB *kPairThreads)
+    k_jacobi_round(int d, int nb, int rnd, double *__restrict__ G, double *__restrict__ Q,
+                   int *__restrict__ rotated) {
+  extern __shared__ double sm[];  // columns 0 .. kB - 1 of block p, kB .. 2 kB - 1 of block q
+  __shared__ double part[kB][kPairThreads / 32][4];
+  const int n = nb + (nb & 1);  // players, one dummy if nb is odd
+  const int pi = blockIdx.x;
+  const int p = pi == 0 ? n - 1 : (rnd + pi) % (n - 1);
+  const int q = (rnd - pi + n - 1) % (n - 1);
+  const bool inside = kB > 1 && rnd == 0;
+  if ((p >= nb || q >= nb) && !inside) return;
+  const int lane = threadIdx.x & 31, grp = threadIdx.x / kPairThreads,
+            gt = threadIdx.x % kPairThreads, gw = gt >> 5;
+  auto column = [&](int u) { return u < kB ? p * kB + u : q * kB + u - kB; };
+  double *sq = sm + (size_t)2 * kB * d;
+  for (int u = grp; u < 2 * kB; u += kB) {
+    const int col = column(u);
+    for (int k = gt; k < d; k += kPairThreads) {
+      sm[(size_t)u * d + k] = col < d ? G[(size_t)col * d + k] : 0.0;
+      if (Q) sq[(size_t)u * d + k] = col < d ? Q[(size_t)col * d + k] : 0.0;
+    }
+  }
+  __syncthreads();
+  bool any = false;
+  // rotates columns u and v of this group's pair; every thread of the CTA calls it
+  auto rotate = [&](int u, int v) {
+    double *x = sm + (size_t)u * d, *y = sm + (size_t)v * d;
+    double al = 0.0, be = 0.0, ga = 0.0;
+    for (int k = gt; k < d; k += kPairThreads) {
+      al += x[k] * x[k];
+      be += y[k] * y[k];
+      ga += x[k] * y[k];
+    }
+    // three sums over the warp in six additions: lane l ends with value l & 3
+    const double k0 = (lane & 1) ? be : al, g0 = (lane & 1) ? al : be;
+    const double a0 = k0 + __shfl_xor_sync(kFull, g0, 1);
+    const double k1 = (lane & 1) ? 0.0 : ga, g1 = (lane & 1) ? ga : 0.0;
+    const double a1 = k1 + __shfl_xor_sync(kFull, g1, 1);
+    double z = ((lane & 2) ? a1 : a0) + __shfl_xor_sync(kFull, (lane & 2) ? a0 : a1, 2);
+    z += __shfl_xor_sync(kFull, z, 4);
+    z += __shfl_xor_sync(kFull, z, 8);
+    z += __shfl_xor_sync(kFull, z, 16);
+    if (lane < 4) part[grp][gw][lane] = z;
     __syncthreads();
-    for (int rnd = 0; rnd < n - 1; ++rnd) {
-      for (int pi = warp; pi < n / 2; pi += nw) {
-        const int p = pi == 0 ? n - 1 : (rnd + pi) % (n - 1);
-        const int q = (rnd - pi + n - 1) % (n - 1);
-        if (p >= d || q >= d) continue;
-        double *gp = G + (size_t)p * d, *gq = G + (size_t)q * d;
-        double al = 0.0, be = 0.0, ga = 0.0;
-        for (int r = lane; r < d; r += 32) {
-          const double x = gp[r], y = gq[r];
-          al += x * x;
-          be += y * y;
-          ga += x * y;
+    al = be = ga = 0.0;
+#pragma unroll
+    for (int w = 0; w < kPairThreads / 32; ++w) {
+      al += part[grp][w][0];
+      be += part[grp][w][1];
+      ga += part[grp][w][2];
+    }
+    // |ga| > 1e-15 sqrt(al be), by squares where those stay in range
+    const double ab = al * be;
+    const bool turn = al != 0.0 && be != 0.0 &&
+                      (ab > 1e-250 && ab < 1e250 ? ga * ga > 1e-30 * ab
+                                                 : fabs(ga) > 1e-15 * sqrt(al) * sqrt(be));
+    if (turn) {
+      double c, s;
+      jacobi_rotation(al, be, ga, c, s);
+      for (int k = gt; k < d; k += kPairThreads) {
+        const double a = x[k], b = y[k];
+        x[k] = c * a - s * b;
+        y[k] = s * a + c * b;
+      }
+      if (Q) {
+        double *xq = sq + (size_t)u * d, *yq = sq + (size_t)v * d;
+        for (int k = gt; k < d; k += kPairThreads) {
+          const double a = xq[k], b = yq[k];
+          xq[k] = c * a - s * b;
+          yq[k] = s * a + c * b;
         }
-        al = warp_sum(al);
-        be = warp_sum(be);
-        ga = warp_sum(ga);
-        if (!(fabs(ga) > 1e-15 * sqrt(al * be)) || al == 0.0 || be == 0.0) continue;
-        const double zeta = (be - al) / (2.0 * ga);
-        const double t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-        const double c = 1.0 / sqrt(1.0 + t * t), s = c * t;
-        for (int r = lane; r < d; r += 32) {
-          const double x = gp[r], y = gq[r];
-          gp[r] = c * x - s * y;
-          gq[r] = s * x + c * y;
-        }
-        if (Q) {
-          double *qp = Q + (size_t)p * d, *qq = Q + (size_t)q * d;
-          for (int r = lane; r < d; r += 32) {
-            const double x = qp[r], y = qq[r];
-            qp[r] = c * x - s * y;
-            qq[r] = s * x + c * y;
-          }
-        }
-        if (lane == 0) rotated = 1;
+      }
+      any = true;
+    }
+    __syncthreads();
+  };
+  if constexpr (kB > 1) {
+    if (inside) {  // round-robin inside each block: kB / 2 disjoint pairs each
+      const int blk = grp / (kB / 2), g = grp % (kB / 2);
+      for (int t = 0; t < kB - 1; ++t) {
+        const int u = g == 0 ? kB - 1 : (t + g) % (kB - 1), v = (t - g + kB - 1) % (kB - 1);
+        rotate(blk * kB + u, blk * kB + v);
+      }
+    }
+  }
+  for (int t = 0; t < kB; ++t) rotate(grp, kB + (grp + t) % kB);
+  for (int u = grp; u < 2 * kB; u += kB) {
+    const int col = column(u);
+    if (col >= d) continue;
+    for (int k = gt; k < d; k += kPairThreads) {
+      G[(size_t)col * d + k] = sm[(size_t)u * d + k];
+      if (Q) Q[(size_t)col * d + k] = sq[(size_t)u * d + k];
+    }
+  }
+  if (any && gt == 0) *rotated = 1;
+}
+
+// sig[i] = |column i|: a warp per column
+__global__ void k_col_norms(int d, const double *__restrict__ G, double *__restrict__ sig) {
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (i >= d) return;
+  double s = 0.0;
+  for (int k = lane; k < d; k += 32) s += G[(size_t)i * d + k] * G[(size_t)i * d + k];
+  s = warp_sum(s);
+  if (lane == 0) sig[i] = sqrt(s);
+}
+
+// Cholesky factors of symmetric positive semidefinite matrices, one CTA each
+// (blockIdx 0: W -> F, 1: V -> C, d x d row-major, the lower triangle; above
+// it zeros).  Right-looking in panels of kCholPanel columns held in shared
+// memory.  A pivot at or below the rounding level of its diagonal entry (4
+// eps) is a direction the matrix does not have: its column is zero.
+constexpr int kCholPanel = 8;
+constexpr int kCholThreads = 1024;
+
+__global__ void __launch_bounds__(kCholThreads)
+    k_psd_chol(int d, const double *__restrict__ W, const double *__restrict__ V,
+               double *__restrict__ F, double *__restrict__ C) {
+  extern __shared__ double sm[];
+  double *P = sm, *diag = sm + (size_t)d * (kCholPanel + 1);  // panel rows padded by one
+  constexpr int ldp = kCholPanel + 1;
+  const double *A = blockIdx.x ? V : W;
+  double *L = blockIdx.x ? C : F;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  for (int e = tid; e < d * d; e += blockDim.x) {
+    const int i = e / d, j = e - i * d;
+    L[e] = j <= i ? A[e] : 0.0;
+    if (i == j) diag[i] = A[e];
+  }
+  __syncthreads();
+  for (int kb = 0; kb < d; kb += kCholPanel) {
+    const int nb = min(kCholPanel, d - kb);
+    for (int e = tid; e < (d - kb) * nb; e += blockDim.x) {
+      const int i = e / nb, q = e - i * nb;
+      P[i * ldp + q] = L[(size_t)(kb + i) * d + kb + q];
+    }
+    __syncthreads();
+    for (int q = 0; q < nb; ++q) {
+      const double piv = P[q * ldp + q];
+      const bool has = piv > 4.4e-16 * diag[kb + q];
+      const double root = has ? sqrt(piv) : 0.0, inv = has ? 1.0 / root : 0.0;
+      __syncthreads();  // everyone has read the pivot
+      for (int i = q + tid; i < d - kb; i += blockDim.x)
+        P[i * ldp + q] = i == q ? root : P[i * ldp + q] * inv;
+      __syncthreads();
+      for (int i = q + 1 + tid; i < d - kb; i += blockDim.x) {
+        const double l = P[i * ldp + q];
+        for (int c = q + 1; c < nb && c <= i; ++c) P[i * ldp + c] -= l * P[c * ldp + q];
       }
       __syncthreads();
     }
-    const int any = rotated;
+    for (int e = tid; e < (d - kb) * nb; e += blockDim.x) {
+      const int i = e / nb, q = e - i * nb;
+      if (q <= i) L[(size_t)(kb + i) * d + kb + q] = P[i * ldp + q];
+    }
+    const int j1 = nb;  // trailing rows and columns, relative to kb
+    for (int i = j1 + warp; i < d - kb; i += nw) {
+      double *row = L + (size_t)(kb + i) * d + kb;
+      for (int j = j1 + lane; j <= i; j += 32) {
+        double s = row[j];
+        for (int q = 0; q < nb; ++q) s -= P[i * ldp + q] * P[j * ldp + q];
+        row[j] = s;
+      }
+    }
     __syncthreads();
-    if (!any) break;
   }
-  for (int i = warp; i < d; i += nw) {
-    const double *g = G + (size_t)i * d;
+}
+
+// Column j of C^T F at G + j d: (C^T F)(i, j) = sum_{k >= max(i, j)} C(k, i) F(k, j)
+__global__ void k_ct_f(int d, const double *__restrict__ C, const double *__restrict__ F,
+                       double *__restrict__ G) {
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < d * d; e += gridDim.x * blockDim.x) {
+    const int j = e / d, i = e - j * d;
     double s = 0.0;
-    for (int r = lane; r < d; r += 32) s += g[r] * g[r];
-    s = warp_sum(s);
-    if (lane == 0) sig[i] = sqrt(s);
+#pragma unroll 4
+    for (int k = max(i, j); k < d; ++k) s += C[(size_t)k * d + i] * F[(size_t)k * d + j];
+    G[e] = s;
   }
-  if (threadIdx.x == 0 && sweeps_out) *sweeps_out = sweep + 1;
 }
 
 __global__ void k_eye(int d, double *__restrict__ Q) {
@@ -243,29 +466,7 @@ __global__ void k_eye(int d, double *__restrict__ Q) {
     Q[e] = (e / d == e % d) ? 1.0 : 0.0;
 }
 
-// S[a][b] = sum_i sqrt(max(lam_i, 0)) Q(a, i) Q(b, i), Q by columns.
-__global__ void k_sym_sqrt(int d, const double *__restrict__ Q, const double *__restrict__ lam,
-                           double *__restrict__ S) {
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < d * d; e += gridDim.x * blockDim.x) {
-    const int a = e / d, b = e % d;
-    double s = 0.0;
-    for (int i = 0; i < d; ++i) s += sqrt(fmax(lam[i], 0.0)) * Q[(size_t)i * d + a] * Q[(size_t)i * d + b];
-    S[e] = s;
-  }
-}
-
-// C = A B (row-major d x d)
-__global__ void k_mm(int d, const double *__restrict__ A, const double *__restrict__ B,
-                     double *__restrict__ C) {
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < d * d; e += gridDim.x * blockDim.x) {
-    const int a = e / d, b = e % d;
-    double s = 0.0;
-    for (int i = 0; i < d; ++i) s += A[(size_t)a * d + i] * B[(size_t)i * d + b];
-    C[e] = s;
-  }
-}
-
-// R_w = Tr W + Tr V - 2 sum_i sqrt(sig_i); out = {R_w, Tr W, Tr V}
+// R_w = Tr W + Tr V - 2 sum_i sig_i; out = {R_w, Tr W, Tr V}
 __global__ void k_mpsrf_final(int d, const double *__restrict__ W, const double *__restrict__ V,
                               const double *__restrict__ sig, double *__restrict__ out) {
   __shared__ double red[40];
@@ -273,7 +474,7 @@ __global__ void k_mpsrf_final(int d, const double *__restrict__ W, const double 
   for (int i = threadIdx.x; i < d; i += blockDim.x) {
     tw += W[(size_t)i * d + i];
     tv += V[(size_t)i * d + i];
-    sq += sqrt(fmax(sig[i], 0.0));
+    sq += sig[i];
   }
   tw = block_sum(tw, red);
   tv = block_sum(tv, red);
@@ -330,7 +531,17 @@ cudaError_t launch_diag_ess(int d, int n_c, int n_s, const double *traj, int max
                             double *ess, double *sqjump, cudaStream_t st) {
   if (d <= 0) return cudaSuccess;
   if (n_c < 2 || n_s < 2 || (size_t)n_c * 8 > 48 * 1024) return cudaErrorInvalidValue;
-  k_diag_ess<<<d, kEssThreads, (size_t)n_c * 8, st>>>(n_c, n_s, traj, max_s, means, ess, sqjump);
+  // the centred samples in shared memory where they fit (two CTAs an SM up to 14000)
+  const size_t staged = ((size_t)n_c * n_s + n_c) * 8;
+  if (staged <= 200 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(k_diag_ess<true>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)staged);
+    if (e != cudaSuccess) return e;
+    k_diag_ess<true><<<d, kEssThreads, staged, st>>>(n_c, n_s, traj, max_s, means, ess, sqjump);
+  } else {
+    k_diag_ess<false><<<d, kEssThreads, (size_t)n_c * 8, st>>>(n_c, n_s, traj, max_s, means, ess,
+                                                               sqjump);
+  }
   return cudaGetLastError();
 }
 
@@ -347,26 +558,61 @@ cudaError_t launch_diag_wv(int d, int n_c, int n_s, const double *Wr, const doub
   return cudaGetLastError();
 }
 
-cudaError_t launch_jacobi(int d, double *G, double *Q, double *sig, int *sweeps,
-                          cudaStream_t st) {
-  if (d <= 0) return cudaSuccess;
-  if (Q) {
-    k_eye<<<grid_for((size_t)d * d), 256, 0, st>>>(d, Q);
-    cudaError_t e = cudaGetLastError();
+cudaError_t launch_eye(int d, double *Q, cudaStream_t st) {
+  k_eye<<<grid_for((size_t)d * d), 256, 0, st>>>(d, Q);
+  return cudaGetLastError();
+}
+
+// Blocks of 1, 2 or 4 columns: the fewest that leave at most 152 block pairs, so
+// that a round is one wave of CTAs.
+static int jacobi_block(int d) { return d <= 304 ? 1 : d <= 608 ? 2 : 4; }
+
+int jacobi_rounds(int d) {
+  const int nb = (d + jacobi_block(d) - 1) / jacobi_block(d);
+  return std::max(1, nb + (nb & 1) - 1);
+}
+
+template <int kB>
+static cudaError_t jacobi_round(int d, int rnd, double *G, double *Q, int *rotated,
+                                cudaStream_t st) {
+  const int nb = (d + kB - 1) / kB, n = nb + (nb & 1);
+  const size_t smem = (size_t)2 * kB * d * sizeof(double) * (Q ? 2 : 1);
+  if (smem > 48 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(k_jacobi_round<kB>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  k_jacobi<<<1, kJacobiThreads, 0, st>>>(d, G, Q, sig, sweeps);
+  k_jacobi_round<kB><<<n / 2, kB * kPairThreads, smem, st>>>(d, nb, rnd, G, Q, rotated);
   return cudaGetLastError();
 }
 
-cudaError_t launch_sym_sqrt(int d, const double *Q, const double *lam, double *S,
+cudaError_t launch_jacobi_round(int d, int rnd, double *G, double *Q, int *rotated,
+                                cudaStream_t st) {
+  if (d <= 1) return cudaSuccess;
+  switch (jacobi_block(d)) {
+    case 1: return jacobi_round<1>(d, rnd, G, Q, rotated, st);
+    case 2: return jacobi_round<2>(d, rnd, G, Q, rotated, st);
+    default: return jacobi_round<4>(d, rnd, G, Q, rotated, st);
+  }
+}
+
+cudaError_t launch_col_norms(int d, const double *G, double *sig, cudaStream_t st) {
+  k_col_norms<<<(d + 7) / 8, 256, 0, st>>>(d, G, sig);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_psd_chol(int d, const double *W, const double *V, double *F, double *C,
                             cudaStream_t st) {
-  k_sym_sqrt<<<grid_for((size_t)d * d), 256, 0, st>>>(d, Q, lam, S);
+  const size_t smem = (size_t)d * (kCholPanel + 2) * sizeof(double);
+  cudaError_t e = cudaFuncSetAttribute(k_psd_chol, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem);
+  if (e != cudaSuccess) return e;
+  k_psd_chol<<<2, kCholThreads, smem, st>>>(d, W, V, F, C);
   return cudaGetLastError();
 }
 
-cudaError_t launch_small_mm(int d, const double *A, const double *B, double *C, cudaStream_t st) {
-  k_mm<<<grid_for((size_t)d * d), 256, 0, st>>>(d, A, B, C);
+cudaError_t launch_ct_f(int d, const double *C, const double *F, double *G, cudaStream_t st) {
+  k_ct_f<<<grid_for((size_t)d * d), 256, 0, st>>>(d, C, F, G);
   return cudaGetLastError();
 }
 

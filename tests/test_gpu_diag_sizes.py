@@ -1,0 +1,80 @@
+"""Diagnostics at the edges of their kernels, against the FP64 oracle.
+
+Jacobi blocks of one, two and four columns with odd numbers of them, the
+staged and unstaged autocorrelation kernel, lag passes that end inside their
+eight lags or at the last sample, covariances with fewer samples than degrees
+of freedom (a positive semidefinite W), a degree of freedom that never moves,
+and the Gram matrix on the tensor cores (d >= 32).  Tolerances as in
+test_gpu_diag.py: 1e-9 relative for the effective sample sizes and 1e-9 of
+Tr V for the MPSRF, whose square roots turn a rounding error eps of a zero
+eigenvalue into sqrt(eps) = 1.5e-8 of its scale: 2e-8 where W is singular.
+"""
+import numpy as np
+import pytest
+
+from oracle import diagnostics as dg
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dino():
+    import paper_2403_08220_gb300 as d
+    return d
+
+
+@pytest.mark.parametrize("n_c,n_s,d,rho", [
+    (2, 2, 1, 0.0),
+    (3, 9, 2, 0.3),
+    (5, 64, 7, 0.9),
+    (4, 3000, 33, 0.99),       # long memory; 96 KB of staged samples
+    (7, 4100, 5, 0.5),         # 230 KB of samples: not staged
+    (10, 130, 305, 0.6),       # blocks of two columns, an odd number of blocks
+    (6, 20, 40, 0.5),          # fewer samples than degrees of freedom
+    (12, 160, 613, 0.4),       # blocks of four columns
+])
+def test_sizes(dino, n_c, n_s, d, rho):
+    rng = np.random.default_rng(n_c + d)
+    X = np.empty((n_c, n_s, d))
+    x = rng.standard_normal((n_c, d))
+    for j in range(n_s):
+        x = rho * x + np.sqrt(1 - rho ** 2) * rng.standard_normal((n_c, d))
+        X[:, j] = x + 0.3 * np.arange(n_c)[:, None] / n_c
+    X *= np.exp(-3.0 * np.arange(d) / d)
+    ctx = dino.dino_init(0)
+    try:
+        g = dino.dino_diag_create(ctx, n_c, d, n_s)
+        for j in range(n_s):
+            dino.dino_diag_push(ctx, g, X[:, j, :])
+        out = dino.dino_diag_compute(ctx, g, d, mpsrf=True)
+    finally:
+        ctx.close()
+    ess = dg.ess_fractions(X)
+    W, V = dg.covariance_estimators(X)
+    singular = n_c * (n_s - 1) < d + 5
+    assert np.max(np.abs(out["ess"] - ess) / np.abs(ess)) <= 1e-9
+    assert abs(out["msj"] - dg.mean_squared_jump(X)) <= 1e-12 * dg.mean_squared_jump(X)
+    assert abs(out["trace_w"] - np.trace(W)) <= 1e-12 * np.trace(W)
+    assert abs(out["trace_v"] - np.trace(V)) <= 1e-12 * np.trace(V)
+    tol = (2e-8 * np.sqrt(d) if singular else 1e-9) * np.trace(V)
+    assert abs(out["mpsrf_w"] - dg.wasserstein_mpsrf(W, V)) <= tol
+
+
+def test_a_still_degree_of_freedom_and_repeated_columns(dino):
+    """A zero column of W and exactly dependent ones: no NaN, the oracle's MPSRF."""
+    rng = np.random.default_rng(4)
+    n_c, n_s, d = 4, 50, 36
+    X = rng.standard_normal((n_c, n_s, d)) + 0.2 * rng.standard_normal((n_c, 1, d))
+    X[:, :, 5] = X[:, :, 9]
+    X[:, :, 20] = 2.0 * X[:, :, 1] - X[:, :, 30]
+    X[:, :, 11] = 1.5
+    ctx = dino.dino_init(0)
+    try:
+        g = dino.dino_diag_create(ctx, n_c, d, n_s)
+        for j in range(n_s):
+            dino.dino_diag_push(ctx, g, X[:, j, :])
+        out = dino.dino_diag_compute(ctx, g, d, mpsrf=True)
+    finally:
+        ctx.close()
+    W, V = dg.covariance_estimators(X)
+    assert abs(out["mpsrf_w"] - dg.wasserstein_mpsrf(W, V)) <= 2e-8 * 6 * np.trace(V)
