@@ -549,6 +549,32 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// The rotation (c, s) that makes columns with squared norms al, be and product
+// ga orthogonal: t = s / c = tan of the smaller angle.  The angle needs no more
+// than FP32 (what it leaves of ga, ~1e-7 of it, the next sweep takes); the
+// rotation has to be orthogonal in FP64, so c = (1 + t^2)^-1/2 is an FP32
+// estimate y with one third-order step y + y (e / 2 + 3 e^2 / 8), e = 1 - w y^2,
+// and FP64 divisions and square roots, long chains on a pipe of 16 cycles an
+// instruction, are left out.
+__device__ __forceinline__ void jacobi_rotation(double al, double be, double ga, double &c,
+                                                double &s, double &t) {
+  const double dq = be - al;
+  // both scaled by the same power of two into FP32's range
+  const int e = max((__double2hiint(dq) >> 20) & 0x7ff, (__double2hiint(ga) >> 20) & 0x7ff);
+  const double sc = __hiloint2double(max(1, min(2046, 2046 - e)) << 20, 0);
+  const float fg = (float)(ga * sc);
+  c = 1.0;
+  s = t = 0.0;
+  if (fg == 0.0f) return;
+  const float z = (float)(dq * sc) / (2.0f * fg), az = fabsf(z);
+  const float ft =
+      copysignf(az > 1e8f ? 0.5f / az : 1.0f / (az + sqrtf(1.0f + az * az)), z);
+  t = (double)ft;
+  const double w = fma(t, t, 1.0), y = (double)rsqrtf(fmaf(ft, ft, 1.0f));
+  const double err = fma(-w * y, y, 1.0);
+  c = fma(y * err, fma(0.375, err, 0.5), y);
+  s = c * t;
+}
 
 // Gram products.  X(k, i), k < m (reduction), i < n: element X[k * ldx + i]
 // (kRedContig = false: X^T X of a row-major m x n matrix, the r-sized path's

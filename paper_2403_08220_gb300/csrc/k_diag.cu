@@ -242,32 +242,6 @@ __global__ void k_diag_wv(int d, int n_c, int n_s, const double *__restrict__ Wr
   }
 }
 
-// The rotation (c, s) that makes columns with squared norms al, be and product
-// ga orthogonal: t = tan of the smaller angle.  The angle needs no more than
-// FP32 (what it leaves of ga, ~1e-7 of it, the next sweep takes); the rotation
-// has to be orthogonal in FP64, so c = (1 + t^2)^-1/2 is an FP32 estimate
-// refined by two Newton steps, and FP64 divisions and square roots, long chains
-// on a pipe of 16 cycles an instruction, are left out.
-__device__ __forceinline__ void jacobi_rotation(double al, double be, double ga, double &c,
-                                                double &s) {
-  const double dq = be - al;
-  // both scaled by the same power of two into FP32's range
-  const int e = max((__double2hiint(dq) >> 20) & 0x7ff, (__double2hiint(ga) >> 20) & 0x7ff);
-  const double sc = __hiloint2double(max(1, min(2046, 2046 - e)) << 20, 0);
-  const float fg = (float)(ga * sc);
-  c = 1.0;
-  s = 0.0;
-  if (fg == 0.0f) return;
-  const float z = (float)(dq * sc) / (2.0f * fg), az = fabsf(z);
-  const float ft = az > 1e8f ? 0.5f / az : 1.0f / (az + sqrtf(1.0f + az * az));
-  const double t = (double)copysignf(ft, z), w = 1.0 + t * t;
-  double y = (double)rsqrtf((float)w);
-  y = y * (1.5 - 0.5 * w * y * y);
-  y = y * (1.5 - 0.5 * w * y * y);
-  c = y;
-  s = y * t;
-}
-
 constexpr int kPairThreads = 128;  // threads of a column pair
 
 // One round of a sweep: CTA pi takes the pair (p, q) of blocks of kB columns of
@@ -338,8 +312,8 @@ __global__ void __launch_bounds__(kB *kPairThreads)
                       (ab > 1e-250 && ab < 1e250 ? ga * ga > 1e-30 * ab
                                                  : fabs(ga) > 1e-15 * sqrt(al) * sqrt(be));
     if (turn) {
-      double c, s;
-      jacobi_rotation(al, be, ga, c, s);
+      double c, s, t;
+      jacobi_rotation(al, be, ga, c, s, t);
       for (int k = gt; k < d; k += kPairThreads) {
         const double a = x[k], b = y[k];
         x[k] = c * a - s * b;

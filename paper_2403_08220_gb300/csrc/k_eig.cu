@@ -15,17 +15,18 @@
 // log det(I + H) = sum_i log nu_i and w^T (I + H)^-1 w = |u|^2 - u^T v, so
 // log rho_{0,r} (Sec. 5.4) again needs only d_y-vectors.
 //
-// M is eigendecomposed per chain by one-sided Jacobi in shared memory (the
-// columns of M V are rotated until orthogonal; their norms are nu and V = U),
-// in FP64 on both precision paths.  The state slot holds U (d_y x d_y, by
-// columns), nu, u, v and t1 = |u|^2 - u^T v; J at the state is kept in Js as
-// on the perturbation-map path.
+// M is eigendecomposed per chain in FP64 on both precision paths: its Cholesky
+// factor M = L L^T, then one-sided Jacobi on the columns of L in shared memory
+// (rotated until orthogonal: L V = U diag(sqrt(nu)), so the normalised columns
+// are U; L's condition is the root of M's, and no V has to be carried).  The
+// state slot holds U (d_y x d_y, by columns), nu, u, v and t1 = |u|^2 - u^T v;
+// J at the state is kept in Js as on the perturbation-map path.
 #include "chol.cuh"
 
 namespace dino {
 namespace {
 
-constexpr int kEigThreads = 256;
+constexpr int kEigThreads = 256;  // proposal
 constexpr int kEigSweeps = 40;
 
 struct EigSlot {
@@ -39,14 +40,16 @@ struct EigSlot {
   }
 };
 
-// shared layout (doubles): Md[d^2] Vd[d^2] nu, Kb, Ka, u, w, vv, ys[d] | vb va [r] | red, flag
+// Odd pitch of the columns in shared memory.
+__host__ __device__ inline int eig_ld(int dy) { return dy | 1; }
+
+// shared layout (doubles): Md[d ld] kz, nu, Kb, Ka, u, w, vv, ys[d] | vb va [r] | red, flag
 struct EigLayout {
-  size_t Md, Vd, nu, Kb, Ka, u, w, vv, ys, vb, va, red, flag, tail;
+  size_t Md, kz, nu, Kb, Ka, u, w, vv, ys, vb, va, red, flag, tail;
   __host__ __device__ EigLayout(int r, int dy) {
-    const size_t dd = (size_t)dy * dy;
     Md = 0;
-    Vd = dd;
-    nu = 2 * dd;
+    kz = (size_t)dy * eig_ld(dy);
+    nu = kz + dy;
     Kb = nu + dy;
     Ka = Kb + dy;
     u = Ka + dy;
@@ -75,43 +78,107 @@ __device__ void k_times(const TJ *J, int dy, int r, double inv_sigma, const doub
   __syncthreads();
 }
 
-// One-sided Jacobi on the dense d x d matrix Md (by columns) with the
-// rotations accumulated in Vd (= I on entry); nu[i] = |column i of Md V|.
-__device__ void eig_jacobi(int d, double *Md, double *Vd, double *nu, int *flag) {
+// In-place Cholesky factor of the d x d matrix held by columns (pitch ld; the
+// lower triangle is read), zeros above the diagonal.  False, in every thread,
+// when a pivot was not positive.
+__device__ bool eig_cholesky(int d, int ld, double *A) {
+  bool ok = true;
+  for (int q = 0; q < d; ++q) {
+    const double piv = A[(size_t)q * ld + q];
+    ok = ok && piv > 0.0;
+    double root, inv;
+    F64::pivot(piv, root, inv);
+    __syncthreads();  // everyone has read the pivot
+    for (int i = q + threadIdx.x; i < d; i += blockDim.x)
+      A[(size_t)q * ld + i] = i == q ? root : A[(size_t)q * ld + i] * inv;
+    __syncthreads();
+    // columns right of q: a warp per column, lanes along it
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int j = q + 1 + warp; j < d; j += nw) {
+      const double l = A[(size_t)q * ld + j];
+      for (int i = j + lane; i < d; i += 32) A[(size_t)j * ld + i] -= l * A[(size_t)q * ld + i];
+    }
+    __syncthreads();
+  }
+  for (int e = threadIdx.x; e < d * d; e += blockDim.x) {
+    const int j = e / d, i = e - j * d;
+    if (i < j) A[(size_t)j * ld + i] = 0.0;
+  }
+  __syncthreads();
+  return ok;
+}
+
+// One-sided Jacobi on the columns of A (d x d, pitch ld); nrm: d doubles for
+// their squared norms.  Four lanes take a column pair, so that a warp
+// instruction of the FP64 pipe, which takes the SM 16 cycles whatever its lanes
+// do, serves eight pairs: E + 2 instructions for the product of the columns
+// (their norms are carried along, al - t ga and be + t ga, and formed anew
+// every sweep), about 15 for the rotation (its angle in FP32) and 4 E to apply
+// it, E = ceil(d / 4) entries per lane.  1024 chains at d = 25: 12.1 ms with a
+// warp per pair, three products, and FP64 divisions and square roots (about 90
+// instructions a pair), 2.6 ms with eight lanes per pair and three products,
+// 1.54 ms here.
+template <int E>
+__device__ void eig_jacobi(int d, int ld, double *A, double *nrm, int *flag) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int n = d + (d & 1);
+  const int g = lane >> 2, q = lane & 3;
+  const int n = d + (d & 1);  // players of the round-robin, one dummy if d is odd
   for (int sweep = 0; sweep < kEigSweeps; ++sweep) {
     if (threadIdx.x == 0) *flag = 0;
+    for (int base = 8 * warp; base < d; base += 8 * nw) {  // whole warps: shuffles inside
+      const int col = min(base + g, d - 1);
+      double s = 0.0;
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const int k = q + 4 * e;
+        const double x = k < d ? A[(size_t)col * ld + k] : 0.0;
+        s += x * x;
+      }
+      s += __shfl_xor_sync(kFull, s, 1);
+      s += __shfl_xor_sync(kFull, s, 2);
+      if (q == 0 && base + g < d) nrm[col] = s;
+    }
     __syncthreads();
     for (int rnd = 0; rnd < n - 1; ++rnd) {
-      for (int pi = warp; pi < n / 2; pi += nw) {
-        const int p = pi == 0 ? n - 1 : (rnd + pi) % (n - 1);
-        const int q = (rnd - pi + n - 1) % (n - 1);
-        if (p >= d || q >= d) continue;
-        double *gp = Md + (size_t)p * d, *gq = Md + (size_t)q * d;
-        double al = 0.0, be = 0.0, ga = 0.0;
-        for (int k = lane; k < d; k += 32) {
-          al += gp[k] * gp[k];
-          be += gq[k] * gq[k];
-          ga += gp[k] * gq[k];
+      // every lane of a warp makes the same passes
+      for (int base = 8 * warp; base < n / 2; base += 8 * nw) {
+        const int pi = base + g;
+        const int pc = pi == 0 ? n - 1 : (rnd + pi) % (n - 1);
+        const int qc = (rnd - pi + n - 1) % (n - 1);
+        const bool have = pi < n / 2 && pc < d && qc < d;
+        double *x = A + (size_t)(have ? pc : 0) * ld, *y = A + (size_t)(have ? qc : 0) * ld;
+        double xv[E], yv[E], ga = 0.0;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          const int k = q + 4 * e;
+          xv[e] = k < d ? x[k] : 0.0;
+          yv[e] = k < d ? y[k] : 0.0;
+          ga += xv[e] * yv[e];
         }
-        al = warp_sum(al);
-        be = warp_sum(be);
-        ga = warp_sum(ga);
-        if (!(fabs(ga) > 1e-15 * sqrt(al * be))) continue;
-        const double zeta = (be - al) / (2.0 * ga);
-        const double t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-        const double c = 1.0 / sqrt(1.0 + t * t), sn = c * t;
-        double *vp = Vd + (size_t)p * d, *vq = Vd + (size_t)q * d;
-        for (int k = lane; k < d; k += 32) {
-          const double x = gp[k], y = gq[k];
-          gp[k] = c * x - sn * y;
-          gq[k] = sn * x + c * y;
-          const double a = vp[k], b = vq[k];
-          vp[k] = c * a - sn * b;
-          vq[k] = sn * a + c * b;
+        ga += __shfl_xor_sync(kFull, ga, 1);
+        ga += __shfl_xor_sync(kFull, ga, 2);
+        const double al = have ? nrm[pc] : 0.0, be = have ? nrm[qc] : 0.0, ab = al * be;
+        const bool turn =
+            have && (ab > 1e-250 && ab < 1e250 ? ga * ga > 1e-30 * ab
+                                               : fabs(ga) > 1e-15 * sqrt(al) * sqrt(be));
+        if (!__any_sync(kFull, turn)) continue;
+        double c, s, t;
+        jacobi_rotation(al, be, ga, c, s, t);
+        if (turn) {
+#pragma unroll
+          for (int e = 0; e < E; ++e) {
+            const int k = q + 4 * e;
+            if (k < d) {
+              x[k] = c * xv[e] - s * yv[e];
+              y[k] = s * xv[e] + c * yv[e];
+            }
+          }
+          if (q == 0) {
+            nrm[pc] = al - t * ga;
+            nrm[qc] = be + t * ga;
+            *flag = 1;
+          }
         }
-        if (lane == 0) *flag = 1;
       }
       __syncthreads();
     }
@@ -119,40 +186,33 @@ __device__ void eig_jacobi(int d, double *Md, double *Vd, double *nu, int *flag)
     __syncthreads();
     if (!any) break;
   }
-  for (int i = warp; i < d; i += nw) {
-    double s = 0.0;
-    for (int k = lane; k < d; k += 32) s += Md[(size_t)i * d + k] * Md[(size_t)i * d + k];
-    s = warp_sum(s);
-    if (lane == 0) nu[i] = sqrt(s);
-  }
-  __syncthreads();
 }
 
-// out = U diag(f) U^T x over d-vectors (U by columns in Vd); tmp: d doubles
-__device__ void u_diag_ut(int d, const double *Vd, const double *f, const double *x, double *tmp,
-                          double *out) {
+// out = U diag(f) U^T x over d-vectors (U by columns, pitch ld); tmp: d doubles
+__device__ void u_diag_ut(int d, int ld, const double *U, const double *f, const double *x,
+                          double *tmp, double *out) {
   for (int i = threadIdx.x; i < d; i += blockDim.x) {
     double acc = 0.0;
-    for (int k = 0; k < d; ++k) acc += Vd[(size_t)i * d + k] * x[k];  // (U^T x)_i
+    for (int k = 0; k < d; ++k) acc += U[(size_t)i * ld + k] * x[k];  // (U^T x)_i
     tmp[i] = acc * f[i];
   }
   __syncthreads();
   for (int k = threadIdx.x; k < d; k += blockDim.x) {
     double acc = 0.0;
-    for (int i = 0; i < d; ++i) acc += Vd[(size_t)i * d + k] * tmp[i];
+    for (int i = 0; i < d; ++i) acc += U[(size_t)i * ld + k] * tmp[i];
     out[k] = acc;
   }
   __syncthreads();
 }
 
-template <typename TJ>
-__global__ void __launch_bounds__(kEigThreads) k_eig_geometry(ReducedArgs a, int mode) {
+template <typename TJ, int NT, int E>
+__global__ void __launch_bounds__(NT) k_eig_geometry(ReducedArgs a, int mode) {
   extern __shared__ __align__(16) double sm[];
   const int c = blockIdx.x, r = a.r, dy = a.d_y;
   const EigLayout lay(r, dy);
   const EigSlot sl(dy);
-  double *Md = sm + lay.Md, *Vd = sm + lay.Vd, *nu = sm + lay.nu, *Kb = sm + lay.Kb,
-         *Ka = sm + lay.Ka, *u = sm + lay.u, *wv = sm + lay.w, *vv = sm + lay.vv,
+  const int ld = eig_ld(dy);
+  double *Md = sm + lay.Md, *nu = sm + lay.nu, *Kb = sm + lay.Kb, *Ka = sm + lay.Ka, *u = sm + lay.u, *wv = sm + lay.w, *vv = sm + lay.vv,
          *ys = sm + lay.ys, *vb = sm + lay.vb, *va = sm + lay.va, *red = sm + lay.red;
   int *flag = reinterpret_cast<int *>(sm + lay.flag);
   const size_t ldS = (((size_t)dy * dy + 3 * (size_t)dy + 1) + 1) & ~(size_t)1;
@@ -183,39 +243,62 @@ __global__ void __launch_bounds__(kEigThreads) k_eig_geometry(ReducedArgs a, int
     k_times<TJ>(J, dy, r, inv_sigma, vb, Kb);
     k_times<TJ>(J, dy, r, inv_sigma, va, Ka);
   }
-  // M = I + K K^T (dense, by columns; symmetric), V = I
-  for (int e = threadIdx.x; e < dy * dy; e += blockDim.x) {
-    const int i = e / dy, j = e - i * dy;
-    double g;
-    if (a.G) {
-      const int hi = i > j ? i : j, lo = i > j ? j : i;  // the lower triangle is stored
-      g = (double)a.G[((size_t)c * dy + hi) * a.ldg + lo] * inv_nv;
-    } else {
-      double acc = 0.0;
-      for (int k = 0; k < r; ++k) acc += (double)J[(size_t)i * r + k] * (double)J[(size_t)j * r + k];
-      g = acc * inv_nv;
+  // M = I + K K^T (dense, by columns; symmetric)
+  auto form_m = [&]() {
+    for (int e = threadIdx.x; e < dy * dy; e += blockDim.x) {
+      const int i = e / dy, j = e - i * dy;
+      double g;
+      if (a.G) {
+        const int hi = i > j ? i : j, lo = i > j ? j : i;  // the lower triangle is stored
+        g = (double)a.G[((size_t)c * dy + hi) * a.ldg + lo] * inv_nv;
+      } else {
+        double acc = 0.0;
+        for (int k = 0; k < r; ++k)
+          acc += (double)J[(size_t)i * r + k] * (double)J[(size_t)j * r + k];
+        g = acc * inv_nv;
+      }
+      Md[(size_t)i * ld + j] = g + (i == j ? 1.0 : 0.0);
     }
-    Md[e] = g + (i == j ? 1.0 : 0.0);
-    Vd[e] = i == j ? 1.0 : 0.0;
+    __syncthreads();
+  };
+  form_m();
+  // M is at least I but for rounding; where a pivot fails all the same (data
+  // beyond the precision of the Gram matrix), Jacobi runs on M itself and the
+  // column norms are nu
+  const bool factored = eig_cholesky(dy, ld, Md);
+  if (!factored) form_m();
+  eig_jacobi<E>(dy, ld, Md, wv, flag);
+  {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int i = warp; i < dy; i += nw) {  // nu, and U: the columns over their norms
+      double *col = Md + (size_t)i * ld, s = 0.0;
+      for (int k = lane; k < dy; k += 32) s += col[k] * col[k];
+      s = warp_sum(s);
+      const double root = sqrt(s), inv = 1.0 / root;
+      if (lane == 0) nu[i] = factored ? s : root;
+      for (int k = lane; k < dy; k += 32) col[k] *= inv;
+    }
   }
   __syncthreads();
-  eig_jacobi(dy, Md, Vd, nu, flag);
-  double uu = 0.0, ld = 0.0;
+  double uu = 0.0, lgd = 0.0;
   for (int i = threadIdx.x; i < dy; i += blockDim.x) {
     u[i] = Kb[i] - ys[i];
     uu += u[i] * u[i];
-    ld += log(nu[i]);
+    lgd += log(nu[i]);
     wv[i] = 1.0 / nu[i];
   }
   uu = block_sum(uu, red);
-  const double hld_b = 0.5 * block_sum(ld, red);
-  u_diag_ut(dy, Vd, wv, u, ys, vv);  // v = M^-1 u
+  const double hld_b = 0.5 * block_sum(lgd, red);
+  u_diag_ut(dy, ld, Md, wv, u, ys, vv);  // v = M^-1 u
   double uv = 0.0;
   for (int i = threadIdx.x; i < dy; i += blockDim.x) uv += u[i] * vv[i];
   const double t1 = uu - block_sum(uv, red);
 
   auto store_slot = [&]() {
-    for (int e = threadIdx.x; e < dy * dy; e += blockDim.x) Sg[sl.U + e] = Vd[e];
+    for (int e = threadIdx.x; e < dy * dy; e += blockDim.x) {
+      const int i = e / dy;
+      Sg[sl.U + e] = Md[(size_t)i * ld + e - i * dy];
+    }
     for (int i = threadIdx.x; i < dy; i += blockDim.x) {
       Sg[sl.nu + i] = nu[i];
       Sg[sl.u + i] = u[i];
@@ -271,10 +354,10 @@ __global__ void __launch_bounds__(kEigThreads) k_eig_propose(ReducedArgs a) {
   const EigSlot sl(dy);
   const size_t ldS = (((size_t)dy * dy + 3 * (size_t)dy + 1) + 1) & ~(size_t)1;
   const double *Sg = a.L + (size_t)a.cur[c] * a.L_slot + (size_t)c * ldS;
-  double *Vd = sm + lay.Vd, *nu = sm + lay.nu, *Kx = sm + lay.Kb, *zd = sm + lay.Ka,
+  double *Vd = sm + lay.Md, *nu = sm + lay.nu, *Kx = sm + lay.Kb, *zd = sm + lay.Ka,
          *u = sm + lay.u, *fv = sm + lay.w, *vv = sm + lay.vv, *tmp = sm + lay.ys,
          *xa = sm + lay.vb, *xi = sm + lay.va, *red = sm + lay.red;
-  double *kz = sm + lay.Md;  // d_y-vector: U diag(nu^-1/2) U^T K xi
+  double *kz = sm + lay.kz;  // d_y-vector: U diag(nu^-1/2) U^T K xi
   const TJ *J = reinterpret_cast<const TJ *>(a.Js) + (size_t)c * dy * r;
   const double inv_sigma = sqrt(1.0 / a.noise_var);
   const double s = a.s, cs = sqrt(1.0 - s * s);
@@ -304,10 +387,10 @@ __global__ void __launch_bounds__(kEigThreads) k_eig_propose(ReducedArgs a) {
     fv[i] = -1.0 / (sq * (1.0 + sq));  // phi_i
   }
   __syncthreads();
-  u_diag_ut(dy, Vd, fv, Kx, tmp, zd);  // z = U diag(phi) U^T K xi
+  u_diag_ut(dy, dy, Vd, fv, Kx, tmp, zd);  // z = U diag(phi) U^T K xi
   for (int i = threadIdx.x; i < dy; i += blockDim.x) fv[i] = 1.0 / sqrt(nu[i]);
   __syncthreads();
-  u_diag_ut(dy, Vd, fv, Kx, tmp, kz);  // K (I + H)^-1/2 xi
+  u_diag_ut(dy, dy, Vd, fv, Kx, tmp, kz);  // K (I + H)^-1/2 xi
   // K^T z and K^T v: thread per column of J (coalesced across threads)
   for (int k = threadIdx.x; k < r; k += blockDim.x) {
     double az = 0.0, av = 0.0;
@@ -343,20 +426,24 @@ size_t eig_slot_stride(int d_y) {
 
 size_t eig_smem_bytes(int r, int d_y) { return EigLayout(r, d_y).tail * sizeof(double); }
 
-cudaError_t launch_eig_geometry(const ReducedArgs &a, int mode, cudaStream_t st) {
+template <typename TJ>
+static cudaError_t eig_geometry(const ReducedArgs &a, int mode, cudaStream_t st) {
   const size_t smem = eig_smem_bytes(a.r, a.d_y);
-  if (a.jf_f32) {
-    cudaError_t e = cudaFuncSetAttribute(k_eig_geometry<float>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  auto go = [&](auto kernel, int threads) {
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
     if (e != cudaSuccess) return e;
-    k_eig_geometry<float><<<a.C, kEigThreads, smem, st>>>(a, mode);
-  } else {
-    cudaError_t e = cudaFuncSetAttribute(k_eig_geometry<double>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k_eig_geometry<double><<<a.C, kEigThreads, smem, st>>>(a, mode);
-  }
-  return cudaGetLastError();
+    kernel<<<a.C, threads, smem, st>>>(a, mode);
+    return cudaGetLastError();
+  };
+  // entries per lane of a column pair: ceil(d_y / 4); 16 or 32 pairs of 4 lanes
+  if (a.d_y <= 16) return go(k_eig_geometry<TJ, 64, 4>, 64);
+  if (a.d_y <= 32) return go(k_eig_geometry<TJ, 64, 8>, 64);
+  return go(k_eig_geometry<TJ, 128, 16>, 128);
+}
+
+cudaError_t launch_eig_geometry(const ReducedArgs &a, int mode, cudaStream_t st) {
+  return a.jf_f32 ? eig_geometry<float>(a, mode, st) : eig_geometry<double>(a, mode, st);
 }
 
 cudaError_t launch_eig_propose(const ReducedArgs &a, cudaStream_t st) {
