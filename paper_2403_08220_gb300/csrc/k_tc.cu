@@ -42,7 +42,7 @@ namespace {
 constexpr int kBlockM = 128;
 constexpr int kBlockK = 64;  // 128 bytes of bf16: one swizzle row
 constexpr int kThreads = 192;
-constexpr int kMaxStages = 4;
+constexpr int kMaxStages = 8;  // small tiles: eight 20 KB stages in flight
 constexpr int kStageTiles = 4 * 32 * 128;  // epilogue staging: 32 rows x 128 B per warp
 constexpr int kStageTilesTma = 2 * kStageTiles;  // two such tiles per warp (bulk stores)
 
@@ -934,12 +934,17 @@ cudaError_t launch_tc_gemm(const TcGemmArgs &a, cudaStream_t st) {
   p.M = a.M;
   p.N = a.N;
   p.K = a.K;
-  // the complement's three-slice products (long K, many tiles): at most 128
-  // columns, so that a stage with a k-block of every slice of A and B (at
-  // most 96 KB) fits twice and each slice is loaded once per k-block
+  int dev = 0, sms = 0;  // persistent grid: one CTA per SM (its shared memory allows one)
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+    return cudaErrorInvalidValue;
+  // Widest column tile: 256, and 128 for the complement's three-slice products
+  // (long K, many tiles), whose stage with a k-block of every slice of A and B
+  // (at most 96 KB) then fits twice and loads each slice once per k-block.
+  const int mt = (a.M + kBlockM - 1) / kBlockM;
   const bool narrow = a.nslice == 3 && (a.epi == TC_EPI_COEF || a.epi == TC_EPI_FIELD_T);
   const int bn_max = narrow ? 128 : 256;
-  const int ntiles = (a.N + bn_max - 1) / bn_max;
+  int ntiles = (a.N + bn_max - 1) / bn_max;
   p.BN = ((a.N + ntiles - 1) / ntiles + 15) / 16 * 16;
   p.nkb = (a.K + kBlockK - 1) / kBlockK;
   static const int pa[6] = {0, 0, 1, 0, 1, 2}, pb[6] = {0, 1, 0, 2, 1, 0};
@@ -948,12 +953,23 @@ cudaError_t launch_tc_gemm(const TcGemmArgs &a, cudaStream_t st) {
     p.pair_a[i] = pa[i];
     p.pair_b[i] = pb[i];
   }
-  // group the slices of a k-block into one stage when two such stages fit
-  // (the two-slice Jacobian products: each A and B tile loaded once per
-  // k-block instead of once per slice pair)
-  const int pair_bytes = kBlockM * kBlockK * 2 + p.BN * kBlockK * 2;
+  // group the slices of a k-block into one stage when two such stages of the
+  // widest tile fit (the two-slice Jacobian products: each A and B tile loaded
+  // once per k-block instead of once per slice pair).  This sets the order of
+  // the FP32 sums, so it depends on N alone and not on the tile taken below.
+  int pair_bytes = kBlockM * kBlockK * 2 + p.BN * kBlockK * 2;
   p.nslice = a.nslice;
   p.grouped = a.nslice > 1 && 2 * pair_bytes * a.nslice <= 200 * 1024;
+  // Where the row tiles leave SMs idle, the columns are cut further, down to
+  // 32, until the tiles fill the SMs once: the MLP's layers of 400 columns
+  // over 64 chains as 13 tiles instead of 2 (39 -> 23 us a layer).
+  // The complement's products split K instead, or have many row tiles.
+  if (!narrow && mt * ntiles < sms) {
+    ntiles = std::max(ntiles, std::min(sms / mt, (a.N + 31) / 32));
+    p.BN = ((a.N + ntiles - 1) / ntiles + 15) / 16 * 16;
+    ntiles = (a.N + p.BN - 1) / p.BN;
+    pair_bytes = kBlockM * kBlockK * 2 + p.BN * kBlockK * 2;
+  }
   const int stage_bytes = p.grouped ? pair_bytes * a.nslice : pair_bytes;
   p.stages = (200 * 1024) / stage_bytes;
   if (p.stages > kMaxStages) p.stages = kMaxStages;
@@ -988,11 +1004,7 @@ cudaError_t launch_tc_gemm(const TcGemmArgs &a, cudaStream_t st) {
   if (!make_map(&tmA, a.A, a.K, a.M, a.lda, a.a_plane, a.nslice, kBlockM) ||
       !make_map(&tmB, a.B, a.K, a.N, a.ldb, a.b_plane, a.nslice, p.BN))
     return cudaErrorInvalidValue;
-  int dev = 0, sms = 0;  // persistent grid: one CTA per SM (its shared memory allows one)
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
-    return cudaErrorInvalidValue;
-  const int total = ((a.M + kBlockM - 1) / kBlockM) * ntiles;
+  const int total = mt * ntiles;
   // split K when the tiles fill fewer than two CTAs per SM (the projections
   // of small pools: M = chains, K = field nodes)
   p.ksplit = 1;
