@@ -15,7 +15,6 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kJChunk = 16;    // rows of an FP64 matrix staged per pass when forming a Gram matrix
-constexpr int kJChunkF = 32;   // rows of an FP32 matrix staged per pass
 constexpr int kNB = 8;         // Cholesky panel width
 constexpr int kHT = 4;         // FP32 register tile edge of the Gram products
 constexpr int kHMaxTiles = 3;  // tiles per thread: ceil(52*53/2 / 512) for n <= 208
@@ -623,131 +622,6 @@ __device__ void form_gram_f64(const double *X, int m, int n, int ldx, double inv
     }
     __syncthreads();
   }
-}
-
-// From an FP32 X into double-float entries: each thread accumulates up to
-// kHMaxTiles 4 x 4 tiles in FP32 registers (chunks of kJChunkF reduction rows
-// staged in shared memory, padded to a multiple of 4 columns); every
-// kGramFlush rows the FP32 tile sums are added exactly into double-float sums
-// held in Ls (each entry owned by one thread) and restart from zero, so the
-// FP32 rounding error grows with kGramFlush rather than with m.  At the end
-// each entry is multiplied by 1 / noise_var as a double-float and 1 is added
-// on the diagonal.  Large n takes several rounds of tiles.
-constexpr int kGramFlush = 2 * kJChunkF;
-
-template <bool kRedContig>
-__device__ void form_gram_f32(const float *X, int m, int n, int ldx, double inv_nv, float2 *Ls,
-                              float *Jc) {
-  const int r = n, dy = m;
-  const int nt = (r + kHT - 1) / kHT, rp = nt * kHT;
-  const int ntiles = nt * (nt + 1) / 2;
-  if (dy == 0) {
-    for (int e = threadIdx.x; e < tri(r); e += blockDim.x) Ls[e] = make_float2(0.0f, 0.0f);
-    __syncthreads();
-    for (int i = threadIdx.x; i < r; i += blockDim.x) Ls[tri(i) + i] = make_float2(1.0f, 0.0f);
-    __syncthreads();
-    return;
-  }
-  const float nh = __double2float_rn(inv_nv), nl = __double2float_rn(inv_nv - (double)nh);
-  const bool vec16 = !kRedContig && (ldx & 3) == 0 && ((uintptr_t)X & 15) == 0;
-  for (int t0 = 0; t0 < ntiles; t0 += kHMaxTiles * blockDim.x) {
-    int ti[kHMaxTiles], tj[kHMaxTiles];
-    float acc[kHMaxTiles][kHT][kHT];
-#pragma unroll
-    for (int s = 0; s < kHMaxTiles; ++s) {
-      const int t = t0 + threadIdx.x + s * blockDim.x;
-      if (t < ntiles) {
-        tri_pos(t, ti[s], tj[s]);
-      } else {
-        ti[s] = -1;
-        tj[s] = 0;
-      }
-#pragma unroll
-      for (int p = 0; p < kHT; ++p)
-#pragma unroll
-        for (int q = 0; q < kHT; ++q) acc[s][p][q] = 0.0f;
-    }
-    bool first = true;
-    for (int i0 = 0; i0 < dy; i0 += kJChunkF) {
-      const int nr = min(kJChunkF, dy - i0);
-      // unrolled so that each thread has several independent loads in flight
-      if (kRedContig) {
-#pragma unroll 8
-        for (int e = threadIdx.x; e < nr * rp; e += blockDim.x) {
-          const int j = e / nr, k = e % nr;
-          Jc[k * rp + j] = j < r ? X[(size_t)j * ldx + i0 + k] : 0.0f;
-        }
-      } else if (vec16) {  // 16-byte rows: asynchronous 16-byte copies, all in flight at once
-        const int q4 = rp / 4;
-        for (int e = threadIdx.x; e < nr * q4; e += blockDim.x) {
-          const int k = e / q4, j = 4 * (e - k * q4);
-          const int left = r - j;
-          const int bytes = left >= 4 ? 16 : (left > 0 ? 4 * left : 0);
-          cp_async16(Jc + k * rp + j, X + (size_t)(i0 + k) * ldx + (left > 0 ? j : 0), bytes);
-        }
-        cp_async_commit();
-        cp_async_wait<0>();
-      } else {
-#pragma unroll 8
-        for (int e = threadIdx.x; e < nr * rp; e += blockDim.x) {
-          const int k = e / rp, j = e % rp;
-          Jc[e] = j < r ? X[(size_t)(i0 + k) * ldx + j] : 0.0f;
-        }
-      }
-      __syncthreads();
-      for (int k = 0; k < nr; ++k) {
-        const float *row = Jc + k * rp;
-#pragma unroll
-        for (int s = 0; s < kHMaxTiles; ++s) {
-          if (ti[s] < 0) continue;
-          const float4 x = *reinterpret_cast<const float4 *>(row + kHT * ti[s]);
-          const float4 y = *reinterpret_cast<const float4 *>(row + kHT * tj[s]);
-          const float xa[4] = {x.x, x.y, x.z, x.w}, ya[4] = {y.x, y.y, y.z, y.w};
-#pragma unroll
-          for (int p = 0; p < kHT; ++p)
-#pragma unroll
-            for (int q = 0; q < kHT; ++q) acc[s][p][q] = fmaf(xa[p], ya[q], acc[s][p][q]);
-        }
-      }
-      __syncthreads();
-      if ((i0 + nr) % kGramFlush == 0 || i0 + nr >= dy) {
-#pragma unroll
-        for (int s = 0; s < kHMaxTiles; ++s) {
-          if (ti[s] < 0) continue;
-#pragma unroll
-          for (int p = 0; p < kHT; ++p)
-#pragma unroll
-            for (int q = 0; q < kHT; ++q) {
-              const int i = kHT * ti[s] + p, j = kHT * tj[s] + q;
-              if (i < r && j <= i) {
-                float2 *e = Ls + tri(i) + j;
-                const float2 x = make_float2(acc[s][p][q], 0.0f);
-                *e = first ? x : DF::add(*e, x);
-              }
-              acc[s][p][q] = 0.0f;
-            }
-        }
-        first = false;
-      }
-    }
-    // scale by 1 / noise_var and add the identity (the entries this thread owns)
-#pragma unroll
-    for (int s = 0; s < kHMaxTiles; ++s) {
-      if (ti[s] < 0) continue;
-#pragma unroll
-      for (int p = 0; p < kHT; ++p)
-#pragma unroll
-        for (int q = 0; q < kHT; ++q) {
-          const int i = kHT * ti[s] + p, j = kHT * tj[s] + q;
-          if (i < r && j <= i) {
-            float2 v = DF::mul(Ls[tri(i) + j], make_float2(nh, nl));
-            if (i == j) v = DF::add(make_float2(1.0f, 0.0f), v);
-            Ls[tri(i) + j] = v;
-          }
-        }
-    }
-  }
-  __syncthreads();
 }
 
 // log u of the accept test: caller-supplied, or from the chain's Philox

@@ -123,6 +123,8 @@ cudaError_t launch_propose(const ReducedArgs &a, cudaStream_t st);
 // mode 0: initialise the state at b; mode 1: geometry at the proposal b,
 // log-acceptance, accept test and state update
 cudaError_t launch_geometry(const ReducedArgs &a, int mode, cudaStream_t st);
+// FP32 Jacobian: I + J^T J / noise_var into the slot, before launch_geometry
+cudaError_t launch_gram_f32(const ReducedArgs &a, int mode, cudaStream_t st);
 // The Woodbury path (d_y < r): the same two steps with the d_y x d_y factor
 // of I + K K^T (K = J / sigma) and the perturbation noise map.
 size_t wb_smem_bytes(int r, int d_y, int jf_f32);

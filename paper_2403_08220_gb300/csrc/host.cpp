@@ -1478,6 +1478,12 @@ static ReducedArgs reduced_args(const Pool &p) {
   return a;
 }
 
+// r-sized path: I + H of the tensor path into the slot that launch_geometry factors
+static void gram_of(dino_ctx *ctx, const ReducedArgs &a, int mode, cudaStream_t st) {
+  if (!a.jf_f32) return;
+  launch(ctx, st, "gram_f32", [&] { return launch_gram_f32(a, mode, st); });
+}
+
 static void split_input(dino_ctx *ctx, const Surrogate *s, Work &w, const double *x,
                         cudaStream_t st) {
   if (s->precision != DINO_PREC_BF16) return;
@@ -1710,6 +1716,7 @@ static Pool *create_pool_on(dino_ctx *ctx, int sid, int C, double dt, uint64_t s
       });
     eval_surrogate(ctx, s, p->w, p->b, p->err, st);
     ReducedArgs ra = reduced_args(*p);
+    if (!p->wb) gram_of(ctx, ra, 0, st);
     launch(ctx, st, "geometry_init", [&] {
       return p->eig ? launch_eig_geometry(ra, 0, st)
              : p->wb ? launch_wb_geometry(ra, 0, st) : launch_geometry(ra, 0, st);
@@ -1758,6 +1765,7 @@ static void step_pool(dino_ctx *ctx, Pool &p) {
                                                      : launch_propose(ra, st);
   });
   eval_surrogate(ctx, s, p.w, p.b, p.err, st, true);
+  if (!p.wb) gram_of(ctx, ra, 1, st);
   launch(ctx, st, "geometry", [&] {
     return p.eig ? launch_eig_geometry(ra, 1, st)
            : p.wb ? launch_wb_geometry(ra, 1, st) : launch_geometry(ra, 1, st);
@@ -1912,6 +1920,7 @@ static void surrogate_eval(dino_ctx *ctx, int sid, int n, const double *x_host, 
     eval_surrogate(ctx, s, p.w, p.b, p.err, st);
     ReducedArgs ra = reduced_args(p);
     ra.noise_var = s->has_data ? s->noise_var : 1.0;
+    gram_of(ctx, ra, 0, st);
     launch(ctx, st, "geometry_init", [&] { return launch_geometry(ra, 0, st); });
     int err = 0;
     CK(cudaMemcpyAsync(&err, p.err, 4, cudaMemcpyDeviceToHost, st));

@@ -26,10 +26,15 @@
 // L^T mhat = ((1-s)(p - t) + sqrt(1-s^2) xi) / sqrt(1-s^2); on the reverse
 // side the geometry kernel forms L^T z and L^T x from the factor it holds.
 //
-// The FP64 pipe bounds these kernels (1/64 of the FP32 rate on GB300), so the
-// Cholesky is blocked (8-column panels with lookahead) to keep the FP64 units
-// fed from shared memory, and on the tensor-core path the product J^T J is
-// formed from the FP32 Jacobian in FP32 register tiles, off the FP64 pipe.
+//   k_gram_f32  on the tensor-core path, I + J^T J / noise_var in double-float
+//               from the FP32 Jacobian, into the slot that k_geometry factors.
+//
+// The FP64 pipe bounds the FP64 instantiations (1/64 of the FP32 rate on
+// GB300), so the Cholesky is blocked (8-column panels with lookahead) to keep
+// the FP64 units fed from shared memory; the tensor-core path factors in
+// double-float on the FP32 pipe.
+#include <algorithm>
+
 #include "chol.cuh"
 
 namespace dino {
@@ -274,6 +279,116 @@ __global__ void __launch_bounds__(32 * kPropWarps) k_propose_warp(ReducedArgs a)
     a.lq_fwd[c] = -a.dt / 8.0 * t1 + sqrt(a.dt) / 2.0 * t2 + a.hld[c] - 0.5 * t3;
 }
 
+// I + J^T J / noise_var of every chain in double-float, packed (tri(r) entries)
+// at the start of the slot that k_geometry factors (the spare one in mode 1).
+//
+// A CTA of 128 threads takes a 64 x 64 block of one chain's lower triangle,
+// 8 x 4 entries a thread; J (d_y x r, FP32) streams through two buffers of 32
+// rows x (64 + 64) columns by asynchronous copies.  The sums are FP32
+// multiply-adds over kGramFlush rows, added into double-float sums in
+// registers, so that the FP32 rounding error grows with kGramFlush rather
+// than with d_y.  What bounds it: FP32 multiply-adds, 32 for three 16-byte
+// shared-memory loads.  Inside k_geometry (one CTA per chain, 4 x 4 tiles in
+// several rounds over J, the sums flushed to the factor in shared or global
+// memory, and the registers of the tiles halving the warps of the
+// factorisation) both together took 9.85 ms for 512 chains at r = d_y = 400 and
+// 2.95 ms for 4096 at r = 128, d_y = 200; apart, 1.40 + 5.70 ms and 0.65 + 2.02 ms.
+constexpr int kGramB = 64, kGramK = 32, kGramThreads = 128;
+constexpr int kGramFlush = 64;  // rows per FP32 partial sum
+
+__global__ void __launch_bounds__(kGramThreads, 4) k_gram_f32(ReducedArgs a, int mode) {
+  __shared__ __align__(16) float stage[2][kGramK][2 * kGramB];
+  const int c = blockIdx.y, r = a.r, dy = a.d_y;
+  int bi, bj;  // block row and column, bj <= bi
+  tri_pos(blockIdx.x, bi, bj);
+  const float *J = reinterpret_cast<const float *>(a.J) + (size_t)c * dy * r;
+  const int slot = mode == 0 ? a.cur[c] : 1 - a.cur[c];
+  float2 *M = reinterpret_cast<float2 *>(a.L + (size_t)slot * a.L_slot +
+                                         (size_t)c * slot_stride(r));
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const bool vec = (r & 3) == 0;  // rows of J start on 16 bytes
+  const int nch = (dy + kGramK - 1) / kGramK;
+  auto issue = [&](int ch) {
+    float(*dst)[2 * kGramB] = stage[ch & 1];
+    const int k0 = ch * kGramK;
+    if (vec) {
+      for (int e = tid; e < kGramK * (2 * kGramB / 4); e += kGramThreads) {
+        const int k = e / (2 * kGramB / 4), q = 4 * (e % (2 * kGramB / 4));
+        const int col = q < kGramB ? bi * kGramB + q : bj * kGramB + q - kGramB;
+        const bool in = k0 + k < dy && col < r;
+        cp_async16(&dst[k][q], J + (in ? (size_t)(k0 + k) * r + col : 0), in ? 16 : 0);
+      }
+    } else {
+      for (int e = tid; e < kGramK * 2 * kGramB; e += kGramThreads) {
+        const int k = e / (2 * kGramB), q = e % (2 * kGramB);
+        const int col = q < kGramB ? bi * kGramB + q : bj * kGramB + q - kGramB;
+        const bool in = k0 + k < dy && col < r;
+        cp_async4(&dst[k][q], J + (in ? (size_t)(k0 + k) * r + col : 0), in ? 4 : 0);
+      }
+    }
+    cp_async_commit();
+  };
+  float acc[8][4];
+  float2 sum[8][4];
+#pragma unroll
+  for (int p = 0; p < 8; ++p)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      acc[p][q] = 0.0f;
+      sum[p][q] = make_float2(0.0f, 0.0f);
+    }
+  issue(0);
+  for (int ch = 0; ch < nch; ++ch) {
+    if (ch + 1 < nch)
+      issue(ch + 1);
+    else
+      cp_async_commit();
+    cp_async_wait<1>();
+    __syncthreads();
+    const float(*x)[2 * kGramB] = stage[ch & 1];
+    const int nr = min(kGramK, dy - ch * kGramK);
+#pragma unroll 4
+    for (int k = 0; k < nr; ++k) {
+      const float4 x0 = *reinterpret_cast<const float4 *>(&x[k][8 * ty]);
+      const float4 x1 = *reinterpret_cast<const float4 *>(&x[k][8 * ty + 4]);
+      const float4 y = *reinterpret_cast<const float4 *>(&x[k][kGramB + 4 * tx]);
+      const float xa[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+      const float ya[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+      for (int p = 0; p < 8; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[p][q] = fmaf(xa[p], ya[q], acc[p][q]);
+    }
+    __syncthreads();
+    const int done = ch * kGramK + nr;
+    if (done % kGramFlush == 0 || done >= dy) {
+#pragma unroll
+      for (int p = 0; p < 8; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float2 v = make_float2(acc[p][q], 0.0f);
+          sum[p][q] = done <= kGramFlush ? v : DF::add(sum[p][q], v);
+          acc[p][q] = 0.0f;
+        }
+    }
+  }
+  const double inv_nv = 1.0 / a.noise_var;
+  const float nh = __double2float_rn(inv_nv), nl = __double2float_rn(inv_nv - (double)nh);
+#pragma unroll
+  for (int p = 0; p < 8; ++p) {
+    const int i = bi * kGramB + 8 * ty + p;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int j = bj * kGramB + 4 * tx + q;
+      if (i < r && j <= i) {
+        float2 v = DF::mul(sum[p][q], make_float2(nh, nl));
+        if (i == j) v = DF::add(make_float2(1.0f, 0.0f), v);
+        M[tri(i) + j] = v;
+      }
+    }
+  }
+}
+
 // One CTA per chain at the point b.  G = false: the factor is built in shared
 // memory; G = true (large r): directly in the other global slot.
 //
@@ -288,8 +403,12 @@ __global__ void __launch_bounds__(32 * kPropWarps) k_propose_warp(ReducedArgs a)
 // an accepted chain to b: its factor slot (written only then, into the other
 // slot, which becomes current) and its state vectors.  The complement
 // coefficient b - s a is written for every chain.
+// The FP32-Jacobian instantiations find I + H in the slot (k_gram_f32) and run
+// at 64 registers a thread, 32 warps an SM where shared memory allows.
 template <typename TJ, bool G, int NT>
-__global__ void __launch_bounds__(NT, NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)) k_geometry(ReducedArgs a, int mode) {
+__global__ void __launch_bounds__(NT, sizeof(TJ) == 4 ? 1024 / NT
+                                                      : (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
+    k_geometry(ReducedArgs a, int mode) {
   // FP32 Jacobian (tensor-core path): double-float Cholesky; FP64 Jacobian: FP64
   using A = std::conditional_t<sizeof(TJ) == 4, DF, F64>;
   using E = typename A::T;
@@ -310,6 +429,14 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)) k_geo
   const TJ *J = reinterpret_cast<const TJ *>(a.J) + (size_t)c * dy * r;
   const TJ *f = reinterpret_cast<const TJ *>(a.f) + (size_t)c * dy;
   const double inv_nv = 1.0 / a.noise_var;
+  if constexpr (sizeof(TJ) == 4 && !G) {  // the packed I + H by 16-byte copies, all in flight
+    const size_t ne = tri_size(r);
+    const E *src = reinterpret_cast<const E *>(Lg);
+    for (size_t q = threadIdx.x; q < ne / 2; q += blockDim.x)
+      cp_async16(Ls + 2 * q, src + 2 * q, 16);
+    cp_async_commit();
+    if (threadIdx.x == 0 && (ne & 1)) Ls[ne - 1] = src[ne - 1];
+  }
 
   for (int i = threadIdx.x; i < r; i += blockDim.x) {
     vb[i] = a.b[(size_t)c * r + i];
@@ -324,14 +451,32 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)) k_geo
     ph += rs * rs;
   }
   const double phi_b = 0.5 * block_sum(ph, red) * inv_nv;  // includes a barrier
-  for (int j = threadIdx.x; j < r; j += blockDim.x) {
+  // g = J^T (f - y) / noise_var: thread per column (coalesced), and where there
+  // are threads for it two per column, each half of the rows
+  const int half = blockDim.x / 2;
+  const bool two = r <= half;
+  E *ge = reinterpret_cast<E *>(vp);  // the second halves' sums
+  if (two) {
+    const int h = threadIdx.x >= half ? 1 : 0, j = threadIdx.x - h * half;
     typename A::Acc acc = A::begin(E{});
-    for (int i = 0; i < dy; ++i) A::sub(acc, A::from_j(J[(size_t)i * r + j]), res[i]);
-    vg[j] = A::to(A::end(acc)) * inv_nv;  // g = J^T (f - y) / noise_var
+    if (j < r) {
+      const int i1 = h ? dy : dy / 2;
+      for (int i = h ? dy / 2 : 0; i < i1; ++i)
+        A::sub(acc, A::from_j(J[(size_t)i * r + j]), res[i]);
+      if (h) ge[j] = A::end(acc);
+    }
+    __syncthreads();
+    if (!h && j < r) vg[j] = A::to(A::add(A::end(acc), ge[j])) * inv_nv;
+  } else {
+    for (int j = threadIdx.x; j < r; j += blockDim.x) {
+      typename A::Acc acc = A::begin(E{});
+      for (int i = 0; i < dy; ++i) A::sub(acc, A::from_j(J[(size_t)i * r + j]), res[i]);
+      vg[j] = A::to(A::end(acc)) * inv_nv;
+    }
   }
   if constexpr (sizeof(TJ) == 4) {
-    form_gram_f32<false>(reinterpret_cast<const float *>(J), dy, r, r, inv_nv,
-                         reinterpret_cast<float2 *>(Ls), reinterpret_cast<float *>(sm + lay.tail));
+    if constexpr (!G) cp_async_wait<0>();
+    __syncthreads();
   } else {
     double *Ld = reinterpret_cast<double *>(Ls);
     form_gram_f64<false>(reinterpret_cast<const double *>(J), dy, r, r, inv_nv, Ld, sm + lay.tail);
@@ -416,7 +561,7 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)) k_geo
 
 bool uses_global_factor(int r, int d_y) {
   const Layout lay(r, d_y, false);
-  const size_t jc = (size_t)kJChunkF * ((r + kHT - 1) / kHT * kHT) * sizeof(float);
+  const size_t jc = (size_t)kJChunk * r * sizeof(double);
   return r > kMaxRSmem || lay.tail * sizeof(double) + jc > kSmemLimit;
 }
 
@@ -428,8 +573,7 @@ size_t propose_smem_bytes(int r) {
 size_t geometry_smem_bytes(int r, int d_y, int jf_f32) {
   const bool G = uses_global_factor(r, d_y);
   const Layout lay(r, d_y, G);
-  const size_t jc = jf_f32 ? (size_t)kJChunkF * ((r + kHT - 1) / kHT * kHT) * sizeof(float)
-                           : (size_t)kJChunk * r * sizeof(double);
+  const size_t jc = jf_f32 ? 0 : (size_t)kJChunk * r * sizeof(double);
   return lay.tail * sizeof(double) + jc;
 }
 
@@ -461,15 +605,39 @@ static cudaError_t launch_geometry_nt(const ReducedArgs &a, int mode, size_t sme
 }
 
 // CTA size by r: a small factor keeps few threads busy, and smaller CTAs let
-// more chains share an SM (the kernel's loops stride over blockDim); the
-// 128- and 256-thread kernels are held to 128 registers so that four and two
-// of them fit an SM.
+// more chains share an SM (the kernel's loops stride over blockDim).  FP64:
+// 128 and 256 threads are held to 128 registers so that four and two CTAs fit
+// an SM.  FP32 Jacobian: the size that fills 32 warps with as many CTAs as the
+// shared memory of the factor lets in (r = 100: four of 256 threads; r = 128:
+// two of 512).
 template <typename TJ, bool G>
 static cudaError_t launch_geometry_t(const ReducedArgs &a, int mode, size_t smem,
                                      cudaStream_t st) {
+  if constexpr (sizeof(TJ) == 4) {
+    const size_t ctas = kSmemLimit / (smem + 1024);
+    if (a.r <= 64) return launch_geometry_nt<TJ, G, 128>(a, mode, smem, st);
+    if (ctas >= 4 && a.r <= 128) return launch_geometry_nt<TJ, G, 256>(a, mode, smem, st);
+    return launch_geometry_nt<TJ, G, kThreads>(a, mode, smem, st);
+  }
   if (a.r <= 64) return launch_geometry_nt<TJ, G, 128>(a, mode, smem, st);
   if (a.r <= 128) return launch_geometry_nt<TJ, G, 256>(a, mode, smem, st);
   return launch_geometry_nt<TJ, G, kThreads>(a, mode, smem, st);
+}
+
+cudaError_t launch_gram_f32(const ReducedArgs &a, int mode, cudaStream_t st) {
+  const int nb = (a.r + kGramB - 1) / kGramB;
+  for (int c0 = 0; c0 < a.C; c0 += 65535) {  // the grid's second dimension ends there
+    ReducedArgs b = a;
+    const size_t o = c0;
+    b.C = std::min(65535, a.C - c0);
+    b.cur = a.cur + o;
+    b.L = a.L + o * slot_stride(a.r);
+    b.J = reinterpret_cast<const float *>(a.J) + o * a.d_y * a.r;
+    k_gram_f32<<<dim3(nb * (nb + 1) / 2, b.C), kGramThreads, 0, st>>>(b, mode);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t launch_geometry(const ReducedArgs &a, int mode, cudaStream_t st) {
