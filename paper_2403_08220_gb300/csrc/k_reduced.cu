@@ -42,32 +42,49 @@ namespace {
 
 constexpr int kThreads = 512;
 
-// x <- L^-T x (back substitution on the upper factor L^T).
-__device__ void cta_upper_solve(const double *Ls, const double *inv, int r, double *x) {
+// [x, z] <- L^-T [x, z] (back substitution on the upper factor L^T, read from
+// global memory): per 32-row diagonal block, staged in shared memory (blk, 32 x
+// 33) with the block's rows of the update loads in flight, warp 0 solves for x
+// and warp 1 for z; then both take the update from one read of the rows.  (One
+// right-hand side after the other, the block's entries read by the solving
+// warp: 1.10 ms for 512 chains at r = 400; 0.37 ms here.)
+__device__ void cta_upper_solve2(const double *Ls, const double *inv, int r, double *x, double *z,
+                                 double *blk) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int jb = ((r - 1) / 32) * 32; jb >= 0; jb -= 32) {
     const int nb = min(32, r - jb);
-    if (warp == 0) {
-      double xl = lane < nb ? x[jb + lane] : 0.0;
+    for (int e = threadIdx.x; e < 32 * 32; e += blockDim.x) {
+      const int k = e >> 5, i = e & 31;
+      if (k < nb && i <= k) blk[k * 33 + i] = Ls[tri(jb + k) + jb + i];
+    }
+    __syncthreads();
+    if (warp < 2) {
+      double *v = warp == 0 ? x : z;
+      double xl = lane < nb ? v[jb + lane] : 0.0;
       for (int k = nb - 1; k >= 0; --k) {
         const double yk = __shfl_sync(kFull, xl, k) * inv[jb + k];
         if (lane == k)
           xl = yk;
         else if (lane < k)
-          xl -= Ls[tri(jb + k) + jb + lane] * yk;
+          xl -= blk[k * 33 + lane] * yk;
       }
-      if (lane < nb) x[jb + lane] = xl;
+      if (lane < nb) v[jb + lane] = xl;
     }
     __syncthreads();
     for (int i = threadIdx.x; i < jb; i += blockDim.x) {
-      double acc = x[i];
-      for (int k = 0; k < nb; ++k) acc -= Ls[tri(jb + k) + i] * x[jb + k];
-      x[i] = acc;
+      double ax = x[i], az = z[i];
+#pragma unroll 8
+      for (int k = 0; k < nb; ++k) {
+        const double l = Ls[tri(jb + k) + i];
+        ax -= l * x[jb + k];
+        az -= l * z[jb + k];
+      }
+      x[i] = ax;
+      z[i] = az;
     }
     __syncthreads();
   }
 }
-
 
 // y1 = L^T x1 and, when `two`, y2 = L^T x2 over the leading r rows of L
 // (y_j = sum_{j <= i < r} L_ij x_i): column j by thread j, rows in order.
@@ -77,6 +94,7 @@ __device__ void cta_upper_matvec2(const typename A::T *Ls, int r, const typename
   using E = typename A::T;
   for (int j = threadIdx.x; j < r; j += blockDim.x) {
     typename A::Acc a1 = A::begin(E{}), a2 = A::begin(E{});
+#pragma unroll 4
     for (int i = j; i < r; ++i) {
       const E l = Ls[tri(i) + j];
       A::sub(a1, l, A::neg(x1[i]));
@@ -111,6 +129,7 @@ struct Layout {
 // processed), the vectors live in shared memory.
 __global__ void __launch_bounds__(kThreads) k_propose(ReducedArgs a) {
   extern __shared__ __align__(16) double sm[];
+  __shared__ double blk[32 * 33];
   const int c = blockIdx.x, r = a.r;
   const Layout lay(r, 0, true);
   const double *Ls = a.L + (size_t)a.cur[c] * a.L_slot + (size_t)c * slot_stride(r);
@@ -137,8 +156,8 @@ __global__ void __launch_bounds__(kThreads) k_propose(ReducedArgs a) {
       if (4 * blk + q < r) vx[4 * blk + q] = z2[4 * blk + q] = n4[q];
   }
   __syncthreads();
-  cta_upper_solve(Ls, inv, r, z1);  // z1 = L^-T t = (I+H)^-1 (a + g)
-  cta_upper_solve(Ls, inv, r, z2);  // z2 = L^-T xi
+  // z1 = L^-T t = (I+H)^-1 (a + g), z2 = L^-T xi
+  cta_upper_solve2(Ls, inv, r, z1, z2, blk);
   const double s = a.s, cs = sqrt(1.0 - s * s);
   double t1 = 0.0, t2 = 0.0, t3 = 0.0;
   for (int i = threadIdx.x; i < r; i += blockDim.x) {
@@ -405,10 +424,13 @@ __global__ void __launch_bounds__(kGramThreads, 4) k_gram_f32(ReducedArgs a, int
 // coefficient b - s a is written for every chain.
 // The FP32-Jacobian instantiations find I + H in the slot (k_gram_f32) and run
 // at 64 registers a thread, 32 warps an SM where shared memory allows.
+// G: `panel` (elements from the start of shared memory, 0 if it does not fit)
+// places the blocked factorisation's panel.
 template <typename TJ, bool G, int NT>
-__global__ void __launch_bounds__(NT, sizeof(TJ) == 4 ? 1024 / NT
-                                                      : (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
-    k_geometry(ReducedArgs a, int mode) {
+__global__ void __launch_bounds__(NT, sizeof(TJ) == 4 && !G
+                                          ? 1024 / NT
+                                          : (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
+    k_geometry(ReducedArgs a, int mode, int panel) {
   // FP32 Jacobian (tensor-core path): double-float Cholesky; FP64 Jacobian: FP64
   using A = std::conditional_t<sizeof(TJ) == 4, DF, F64>;
   using E = typename A::T;
@@ -496,7 +518,10 @@ __global__ void __launch_bounds__(NT, sizeof(TJ) == 4 ? 1024 / NT
   vv = block_sum(vv, red);
   if (threadIdx.x == 0) Ls[tri(r) + r] = A::from(1.0 + vv);
   __syncthreads();
-  cta_cholesky_panels<A>(Ls, inv, r + 1);
+  if (G && panel)
+    cta_cholesky_global<A>(Ls, inv, r + 1, reinterpret_cast<E *>(sm + panel));
+  else
+    cta_cholesky_panels<A>(Ls, inv, r + 1);
   double ld = 0.0;
   for (int i = threadIdx.x; i < r; i += blockDim.x) ld += log(A::to(Ls[tri(i) + i]));
   const double hld_b = block_sum(ld, red);
@@ -577,6 +602,17 @@ size_t geometry_smem_bytes(int r, int d_y, int jf_f32) {
   return lay.tail * sizeof(double) + jc;
 }
 
+// A factor in global memory: where its panel lies (after the vectors; the
+// staged rows of an FP64 J are done with by then), 0 where it does not fit.
+static int geometry_panel(int r, int d_y, size_t &smem) {
+  if (!uses_global_factor(r, d_y)) return 0;
+  const size_t at = Layout(r, d_y, true).tail;
+  const size_t need = (at + (size_t)(r + 1) * kPanelLd) * sizeof(double);
+  if (need > kSmemLimit) return 0;
+  smem = std::max(smem, need);
+  return (int)at;
+}
+
 cudaError_t launch_propose(const ReducedArgs &a, cudaStream_t st) {
   if (a.r <= 32 * 7) {
     const int grid = (a.C + kPropWarps - 1) / kPropWarps;
@@ -595,12 +631,12 @@ cudaError_t launch_propose(const ReducedArgs &a, cudaStream_t st) {
 }
 
 template <typename TJ, bool G, int NT>
-static cudaError_t launch_geometry_nt(const ReducedArgs &a, int mode, size_t smem,
+static cudaError_t launch_geometry_nt(const ReducedArgs &a, int mode, size_t smem, int panel,
                                       cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(k_geometry<TJ, G, NT>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_geometry<TJ, G, NT><<<a.C, NT, smem, st>>>(a, mode);
+  k_geometry<TJ, G, NT><<<a.C, NT, smem, st>>>(a, mode, panel);
   return cudaGetLastError();
 }
 
@@ -609,19 +645,22 @@ static cudaError_t launch_geometry_nt(const ReducedArgs &a, int mode, size_t sme
 // 128 and 256 threads are held to 128 registers so that four and two CTAs fit
 // an SM.  FP32 Jacobian: the size that fills 32 warps with as many CTAs as the
 // shared memory of the factor lets in (r = 100: four of 256 threads; r = 128:
-// two of 512).
+// two of 512).  A factor in global memory with its panel in shared memory: 256
+// threads at 128 registers, two CTAs an SM up to r of about 500.
 template <typename TJ, bool G>
 static cudaError_t launch_geometry_t(const ReducedArgs &a, int mode, size_t smem,
                                      cudaStream_t st) {
-  if constexpr (sizeof(TJ) == 4) {
+  const int panel = G ? geometry_panel(a.r, a.d_y, smem) : 0;
+  if (panel) return launch_geometry_nt<TJ, G, 256>(a, mode, smem, panel, st);
+  if constexpr (sizeof(TJ) == 4 && !G) {
     const size_t ctas = kSmemLimit / (smem + 1024);
-    if (a.r <= 64) return launch_geometry_nt<TJ, G, 128>(a, mode, smem, st);
-    if (ctas >= 4 && a.r <= 128) return launch_geometry_nt<TJ, G, 256>(a, mode, smem, st);
-    return launch_geometry_nt<TJ, G, kThreads>(a, mode, smem, st);
+    if (a.r <= 64) return launch_geometry_nt<TJ, G, 128>(a, mode, smem, 0, st);
+    if (ctas >= 4 && a.r <= 128) return launch_geometry_nt<TJ, G, 256>(a, mode, smem, 0, st);
+    return launch_geometry_nt<TJ, G, kThreads>(a, mode, smem, 0, st);
   }
-  if (a.r <= 64) return launch_geometry_nt<TJ, G, 128>(a, mode, smem, st);
-  if (a.r <= 128) return launch_geometry_nt<TJ, G, 256>(a, mode, smem, st);
-  return launch_geometry_nt<TJ, G, kThreads>(a, mode, smem, st);
+  if (a.r <= 64) return launch_geometry_nt<TJ, G, 128>(a, mode, smem, 0, st);
+  if (a.r <= 128) return launch_geometry_nt<TJ, G, 256>(a, mode, smem, 0, st);
+  return launch_geometry_nt<TJ, G, kThreads>(a, mode, smem, 0, st);
 }
 
 cudaError_t launch_gram_f32(const ReducedArgs &a, int mode, cudaStream_t st) {

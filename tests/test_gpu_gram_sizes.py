@@ -18,6 +18,8 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("r,d_y", [
     (1, 1), (3, 5), (32, 63), (63, 64), (64, 65), (65, 31), (66, 129), (127, 96), (128, 200),
     (129, 32), (160, 33), (209, 70), (260, 301),
+    # factors in global memory: the last 16-column panel with 16, 1 and 9 columns
+    (239, 40), (240, 17), (600, 50),
 ])
 def test_factor_of_the_librarys_own_jacobian(r, d_y):
     import paper_2403_08220_gb300 as dino
@@ -27,7 +29,7 @@ def test_factor_of_the_librarys_own_jacobian(r, d_y):
     ctx = dino.dino_init(0)
     try:
         sid = dino.dino_load_surrogate(
-            ctx, n_grid=17, prior_gamma=0.1, prior_delta=1.0, r=r, widths=widths, activation=1,
+            ctx, n_grid=17 if r <= 289 else 25, prior_gamma=0.1, prior_delta=1.0, r=r, widths=widths, activation=1,
             W=Ws, b=bs, basis_kind=dino.DINO_BASIS_KLE, y=np.zeros(d_y), noise_var=0.37,
             precision=dino.DINO_PREC_BF16, noise_map=dino.DINO_NOISE_CHOLESKY)
         x = np.random.default_rng(1).standard_normal((3, r))
