@@ -71,14 +71,19 @@ cudaError_t run_gemm(int M, int N, int K, const T *A, int lda, const T *B, int l
 
 // Prior draw: one CTA per chain; X = sqrt(Lambda) .* Z (spectral), Y = X S,
 // M = S^T Y, all n x n in shared memory with rows padded to a multiple of 4
-// (zero-filled).  Each product is computed in 4 x 4 register tiles: per step
-// of the reduction a tile reads one float4 (or double4-as-two-loads) row
-// segment of the right operand and four broadcast values of the left one.
-// FP32 draws with at most kPriorWide tiles use a CTA of kPriorWide threads
-// (four CTAs per SM), so that each product takes a single round; otherwise
-// kPriorThreads threads loop over the tiles.
-constexpr int kPriorThreads = 256;
-constexpr int kPriorWide = 320;
+// (zero-filled).  The sine matrix is symmetric in its nodes, S[k][n - 1 - i] =
+// (-1)^k S[k][i] (k from 0), so of each product only the first h = ceil(n / 2)
+// node rows or columns are formed, the even k into U and the odd k into V:
+// the node is U + V and its mirror image U - V, half the multiply-adds.  U
+// and V of a 4 x 4 tile are the work of two threads (one half of the CTA
+// each), V handed over through the destination; per step of the reduction a
+// tile reads one float4 (or double4-as-two-loads) row segment of the right
+// operand and one of the left.  FP64 is bound by its pipe (16 cycles a warp
+// instruction), FP32 by shared-memory reads and the transforms' latency.
+// kPriorThreads threads hold the tiles of n = 65 in one round.  (All n x n
+// nodes formed, n = 65: 0.84 ms for 16384 chains in FP32, 1.53 ms for 1024 in
+// FP64; 0.70 and 0.93 ms now.)
+constexpr int kPriorThreads = 320;
 
 __host__ __device__ inline int prior_ld(int n) { return (n + 3) / 4 * 4; }
 
@@ -102,8 +107,29 @@ __device__ __forceinline__ void load4(const T *p, T v[4]) {
   }
 }
 
-template <typename T, int NT>
-__global__ void __launch_bounds__(NT, NT == kPriorWide ? 4 : 1)
+// A 4 x 4 tile of sum_k a[k][0..3] b[k][0..3] over k = k0, k0 + 2, ... < n (rows
+// of pitch ld)
+template <typename T>
+__device__ __forceinline__ void half_tile(const T *a, const T *b, int ld, int k0, int n,
+                                          T acc[4][4]) {
+#pragma unroll
+  for (int p = 0; p < 4; ++p)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[p][q] = T(0);
+#pragma unroll 3
+  for (int k = k0; k < n; k += 2) {
+    T x[4], y[4];
+    load4(a + k * ld, x);
+    load4(b + k * ld, y);
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[p][q] += x[p] * y[q];
+  }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kPriorThreads, sizeof(T) == 4 ? 4 : 2)
     k_prior_draw(int n, const T *__restrict__ sqrtlam, const T *__restrict__ S, uint64_t seed,
                  uint64_t id_base, uint32_t stream, uint32_t step, T *out, int ldo,
                  __nv_bfloat16 *ms, int ldms, size_t ms_plane, int ms_slices,
@@ -111,6 +137,7 @@ __global__ void __launch_bounds__(NT, NT == kPriorWide ? 4 : 1)
   if (only && !only[blockIdx.x]) return;  // the whole CTA: this chain draws nothing
   extern __shared__ __align__(16) unsigned char smraw[];
   const int ld = prior_ld(n), nt = ld / 4, NN = ld * ld;
+  const int h = (n + 1) / 2, ht = (h + 3) / 4;  // nodes formed, and their tiles
   T *X = reinterpret_cast<T *>(smraw);
   T *Ss = X + NN;
   T *Y = Ss + NN;
@@ -152,24 +179,38 @@ __global__ void __launch_bounds__(NT, NT == kPriorWide ? 4 : 1)
     }
   }
   __syncthreads();
+  const int team = blockDim.x / 2, odd = threadIdx.x >= team ? 1 : 0,
+            mate = threadIdx.x - odd * team;
   // Y[ky][i] = sum_kx X[ky][kx] S[kx][i], with X held transposed (X[kx][ky]
   // at kx * ld + ky) so that both operands are read as row segments
-  for (int tt = threadIdx.x; tt < nt * nt; tt += blockDim.x) {
-    const int r0 = 4 * (tt / nt), c0 = 4 * (tt % nt);
-    T acc[4][4] = {};
-    for (int k = 0; k < n; ++k) {
-      T a[4], b[4];
-      load4(X + k * ld + r0, a);
-      load4(Ss + k * ld + c0, b);
+  for (int t0 = 0; t0 < nt * ht; t0 += team) {  // the same passes in every thread
+    const int tt = t0 + mate, r0 = 4 * (tt / ht), c0 = 4 * (tt % ht);
+    const bool on = tt < nt * ht;
+    T acc[4][4];
+    if (on) {
+      half_tile(X + r0, Ss + c0, ld, odd, n, acc);
+      if (odd)
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (c0 + q < h) Y[(r0 + p) * ld + c0 + q] = acc[p][q];
+    }
+    __syncthreads();
+    if (on && !odd) {
 #pragma unroll
       for (int p = 0; p < 4; ++p)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[p][q] += a[p] * b[q];
+        for (int q = 0; q < 4; ++q) {
+          const int i = c0 + q;
+          if (i < h) {
+            T *row = Y + (r0 + p) * ld;
+            const T v = row[i];
+            row[i] = acc[p][q] + v;
+            if (n - 1 - i != i) row[n - 1 - i] = acc[p][q] - v;
+          }
+        }
     }
-#pragma unroll
-    for (int p = 0; p < 4; ++p)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) Y[(r0 + p) * ld + c0 + q] = acc[p][q];
   }
   __syncthreads();
   // M[j][i] = sum_ky S[ky][j] Y[ky][i]; node p = i + n j.  The tiles land in
@@ -177,23 +218,33 @@ __global__ void __launch_bounds__(NT, NT == kPriorWide ? 4 : 1)
   // nodes in order), and the CTA then writes M and its slices with
   // consecutive threads on consecutive nodes.
   T *Mo = X;
-  for (int tt = threadIdx.x; tt < nt * nt; tt += blockDim.x) {
-    const int r0 = 4 * (tt / nt), c0 = 4 * (tt % nt);
-    T acc[4][4] = {};
-    for (int k = 0; k < n; ++k) {
-      T a[4], b[4];
-      load4(Ss + k * ld + r0, a);
-      load4(Y + k * ld + c0, b);
+  for (int t0 = 0; t0 < ht * nt; t0 += team) {
+    const int tt = t0 + mate, r0 = 4 * (tt / nt), c0 = 4 * (tt % nt);
+    const bool on = tt < ht * nt;
+    T acc[4][4];
+    if (on) {
+      half_tile(Ss + r0, Y + c0, ld, odd, n, acc);
+      if (odd)
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (r0 + p < h && c0 + q < n) Mo[(r0 + p) * n + c0 + q] = acc[p][q];
+    }
+    __syncthreads();
+    if (on && !odd) {
 #pragma unroll
       for (int p = 0; p < 4; ++p)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[p][q] += a[p] * b[q];
+        for (int q = 0; q < 4; ++q) {
+          const int j = r0 + p, i = c0 + q;
+          if (j < h && i < n) {
+            const T v = Mo[j * n + i];
+            Mo[j * n + i] = acc[p][q] + v;
+            if (n - 1 - j != j) Mo[(n - 1 - j) * n + i] = acc[p][q] - v;
+          }
+        }
     }
-#pragma unroll
-    for (int p = 0; p < 4; ++p)
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (r0 + p < n && c0 + q < n) Mo[(r0 + p) * n + c0 + q] = acc[p][q];
   }
   __syncthreads();
   T *o = out + (size_t)c * ldo;
@@ -381,18 +432,12 @@ cudaError_t launch_prior_draw(int C, int n, const T *sqrtlam, const T *S, uint64
   if (C <= 0) return cudaSuccess;
   if (ms && (sizeof(T) != 4 || ms_slices < 1 || ldms < n * n)) return cudaErrorInvalidValue;
   const size_t smem = prior_draw_smem_bytes(n, (int)sizeof(T));
-  const int nt = prior_ld(n) / 4;
-  auto go = [&](auto kernel, int threads) {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-    kernel<<<C, threads, smem, st>>>(n, sqrtlam, S, seed, id_base, stream, step, out, ldo, ms,
-                                     ldms, ms_plane, ms_slices, ext_z, only);
-    return cudaGetLastError();
-  };
-  if constexpr (sizeof(T) == 4)
-    if (nt * nt <= kPriorWide) return go(k_prior_draw<T, kPriorWide>, kPriorWide);
-  return go(k_prior_draw<T, kPriorThreads>, kPriorThreads);
+  cudaError_t e = cudaFuncSetAttribute(k_prior_draw<T>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k_prior_draw<T><<<C, kPriorThreads, smem, st>>>(n, sqrtlam, S, seed, id_base, stream, step, out,
+                                                  ldo, ms, ldms, ms_plane, ms_slices, ext_z, only);
+  return cudaGetLastError();
 }
 
 template <typename T>
