@@ -75,6 +75,8 @@ struct ReducedArgs {
   // Woodbury path, FP32 J: the Gram matrices J J^T formed beforehand (C x
   // d_y x ldg), or nullptr to form them in the geometry kernel
   const float *G = nullptr;
+  // FP64 J: J J^T formed beforehand, packed, in the slot to be factored
+  int gram_in_slot = 0;
   int ldg = 0;
   // Woodbury path with the tensor-core Gram: the proposal b and the state m_r
   // as double-float pairs (C x r), from which a warp-per-row kernel forms K b
@@ -197,6 +199,14 @@ struct Gemm64Args {
   DigitMat B;
   int *err = nullptr;
 };
+// Per-chain Gram matrices: for each of `groups` blocks J_c of g consecutive rows
+// of J (K columns, pitch ldj; their digits laid out without column exponents)
+// the packed lower triangle of J_c J_c^T at L + s slot + c stride, s = cur[c]
+// (mode 0) or the other slot.
+cudaError_t gram64_slots(int groups, int g, int K, const double *J, int ldj,
+                         const __nv_bfloat16 *digits, const int *ex, int ldp, size_t plane,
+                         double *L, size_t slot, size_t stride, const int *cur, int mode, int *err,
+                         cudaStream_t st);
 cudaError_t gemm64_store(const Gemm64Args &a, double *out, int ldo, cudaStream_t st);
 cudaError_t gemm64_bias_act(const Gemm64Args &a, const double *bias, int act, double *out,
                             double *der, int ldo, cudaStream_t st);

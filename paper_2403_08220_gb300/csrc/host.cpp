@@ -1478,10 +1478,44 @@ static ReducedArgs reduced_args(const Pool &p) {
   return a;
 }
 
-// r-sized path: I + H of the tensor path into the slot that launch_geometry factors
-static void gram_of(dino_ctx *ctx, const ReducedArgs &a, int mode, cudaStream_t st) {
-  if (!a.jf_f32) return;
-  launch(ctx, st, "gram_f32", [&] { return launch_gram_f32(a, mode, st); });
+// The Gram matrices that the geometry kernel finds in the slot it factors.
+// Tensor path, r-sized: I + J^T J / noise_var.  FP64 Woodbury path: J J^T on the
+// tensor cores, J's digits in the Jacobian's two product buffers (not in use any
+// more) for as many chains at a time as they hold; below 24 observations the
+// geometry kernel forms it as fast itself, and where the hidden layers are not
+// wider than r the buffers hold less than one chain.  The rule looks at the
+// surrogate alone, so that a chain's bits do not depend on the pool.
+static void gram_of(dino_ctx *ctx, const Pool &p, ReducedArgs &a, int mode, cudaStream_t st) {
+  const Surrogate *s = p.s;
+  if (!p.wb) {
+    if (a.jf_f32)
+      launch(ctx, st, "gram_f32", [&] { return launch_gram_f32(a, mode, st); });
+    return;
+  }
+  const int C = p.C, dy = s->d_y, r = s->r, ldp = digit_pitch(r);
+  if (a.jf_f32 || p.eig || s->L < 2 || dy < 24 || r < 32 || s->widest <= ldp) return;
+  // 16 ldp + 4 bytes a row and 16 to align: at most 2 x 8 widest bytes a row
+  const size_t per = ((size_t)16 * ldp + 4) * dy + 16;
+  char *base = (char *)p.w.P64[0];
+  const size_t bytes = (char *)p.w.P64[1] + p.w.p_bytes - base;
+  const int chunk = (int)std::min<size_t>(
+      {(size_t)C, bytes / per, std::max<size_t>(1, kDigitsChunk / per)});
+  auto *d = (__nv_bfloat16 *)base;
+  const size_t plane = (size_t)chunk * dy * ldp, ss = wb_slot_stride(dy);
+  int *ex = (int *)(d + plane * kDigits64);
+  for (int c0 = 0; c0 < C; c0 += chunk) {
+    const int n = std::min(chunk, C - c0);
+    const double *J = p.w.J64 + (size_t)c0 * dy * r;
+    launch(ctx, st, "split_f64", [&] {
+      return launch_split64(n * dy, r, J, r, nullptr, nullptr, 1, 0, 0, nullptr, 1, d, ldp, plane,
+                            ex, st);
+    });
+    launch(ctx, st, "gram_f64", [&] {
+      return gram64_slots(n, dy, r, J, r, d, ex, ldp, plane, a.L + (size_t)c0 * ss, a.L_slot, ss,
+                          a.cur + c0, mode, a.err, st);
+    });
+  }
+  a.gram_in_slot = 1;
 }
 
 static void split_input(dino_ctx *ctx, const Surrogate *s, Work &w, const double *x,
@@ -1716,7 +1750,7 @@ static Pool *create_pool_on(dino_ctx *ctx, int sid, int C, double dt, uint64_t s
       });
     eval_surrogate(ctx, s, p->w, p->b, p->err, st);
     ReducedArgs ra = reduced_args(*p);
-    if (!p->wb) gram_of(ctx, ra, 0, st);
+    gram_of(ctx, *p, ra, 0, st);
     launch(ctx, st, "geometry_init", [&] {
       return p->eig ? launch_eig_geometry(ra, 0, st)
              : p->wb ? launch_wb_geometry(ra, 0, st) : launch_geometry(ra, 0, st);
@@ -1757,15 +1791,15 @@ static void step_pool(dino_ctx *ctx, Pool &p) {
   const int C = p.C, r = s->r, N = s->N;
   cudaStream_t st = p.st;
   const double cs = std::sqrt(1.0 - p.sc * p.sc);
-  ReducedArgs ra = reduced_args(p);
   const double *ext_z =
       p.ext && p.ext_z ? p.ext + (size_t)C * (r + s->d_y) : nullptr;
+  ReducedArgs ra = reduced_args(p);
   launch(ctx, st, "propose", [&] {
     return p.eig ? launch_eig_propose(ra, st) : p.wb ? launch_wb_propose(ra, st)
                                                      : launch_propose(ra, st);
   });
   eval_surrogate(ctx, s, p.w, p.b, p.err, st, true);
-  if (!p.wb) gram_of(ctx, ra, 1, st);
+  gram_of(ctx, p, ra, 1, st);
   launch(ctx, st, "geometry", [&] {
     return p.eig ? launch_eig_geometry(ra, 1, st)
            : p.wb ? launch_wb_geometry(ra, 1, st) : launch_geometry(ra, 1, st);
@@ -1920,7 +1954,7 @@ static void surrogate_eval(dino_ctx *ctx, int sid, int n, const double *x_host, 
     eval_surrogate(ctx, s, p.w, p.b, p.err, st);
     ReducedArgs ra = reduced_args(p);
     ra.noise_var = s->has_data ? s->noise_var : 1.0;
-    gram_of(ctx, ra, 0, st);
+    gram_of(ctx, p, ra, 0, st);
     launch(ctx, st, "geometry_init", [&] { return launch_geometry(ra, 0, st); });
     int err = 0;
     CK(cudaMemcpyAsync(&err, p.err, 4, cudaMemcpyDeviceToHost, st));

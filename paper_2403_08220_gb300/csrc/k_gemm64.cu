@@ -215,6 +215,7 @@ __global__ void k_col_exp(int rows, int K, const double *__restrict__ B, int ld,
 
 struct Gemm64Params {
   int M, N, K, row0, nkb;
+  int grp;  // Gram products: rows of a group (0: one plain product)
   const int *ea, *eb;
   const double *A, *W, *der, *B;  // the FP64 operands, for rows of A that are not finite
   int lda, g, ldd, ldb;
@@ -264,6 +265,17 @@ __device__ __forceinline__ void tmem_wait_ld() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// The FP64 dot product of one element whose row or column is not finite.
+__device__ __noinline__ double plain_dot(const Gemm64Params &p, int g0, int row, int col) {
+  const double *y = p.B + (size_t)(g0 + col) * p.ldb;
+  const int gr = p.row0 + row;
+  const double *x = p.A ? p.A + (size_t)(g0 + row) * p.lda : p.W + (size_t)(gr % p.g) * p.K;
+  const double *d = p.A ? nullptr : p.der + (size_t)(gr / p.g) * p.ldd;
+  double v = 0.0;
+  for (int k = 0; k < p.K; ++k) v += (d ? x[k] * d[k] : x[k]) * y[k];
+  return v;
+}
+
 __device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t addr) {
   return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(512 >> 4) << 32) |
          ((uint64_t)1 << 46) | ((uint64_t)4 << 61);
@@ -273,7 +285,11 @@ __device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t addr) {
 // the MMA issue, warps 2-9 the epilogue (four lane quarters x two halves of
 // the tile's columns).  One set of accumulators: the MMAs of the next chunk or
 // tile start once the epilogue has read the previous one out of TMEM.
-template <int BN, class Epi>
+//
+// kGram: the Gram matrices of the groups of p.grp consecutive rows of A (both
+// operands are A's digits, N = grp): tile t is a block of one group, and blocks
+// above the diagonal are left out.
+template <int BN, bool kGram, class Epi>
 __global__ void __launch_bounds__(kGemm64Threads, 1)
     k_gemm64(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
              const Gemm64Params p, const Epi epi) {
@@ -293,7 +309,17 @@ __global__ void __launch_bounds__(kGemm64Threads, 1)
   const uint32_t acc_full = smem_u32(&bars[2 * kStages]), acc_empty = acc_full + 8,
                  drain = acc_full + 16;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int ntn = (p.N + BN - 1) / BN, ntiles = ((p.M + kBM - 1) / kBM) * ntn;
+  const int ntn = (p.N + BN - 1) / BN;
+  const int mpg = kGram ? (p.grp + kBM - 1) / kBM : 0;  // row tiles of a group
+  const int ntiles = kGram ? p.M / p.grp * mpg * ntn : ((p.M + kBM - 1) / kBM) * ntn;
+  // tile t: first row (of A) and first column, both within the group g0 .. for kGram
+  auto tile = [&](int t, int &g0, int &m0, int &n0) {
+    n0 = (t % ntn) * BN;
+    t /= ntn;
+    g0 = kGram ? (t / mpg) * p.grp : 0;
+    m0 = (kGram ? t % mpg : t) * kBM;
+    return !kGram || n0 < m0 + kBM;  // false: above the diagonal
+  };
   constexpr int kChunkB = kChunkK / kKB;           // stages per exact accumulation
 
   if (threadIdx.x == 0) {
@@ -325,7 +351,8 @@ __global__ void __launch_bounds__(kGemm64Threads, 1)
       int g = 0;
       bool ok = true;
       for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-        const int m0 = (t / ntn) * kBM, n0 = (t % ntn) * BN;
+        int g0, m0, n0;
+        if (!tile(t, g0, m0, n0)) continue;
         for (int kb = 0; kb < p.nkb; ++kb, ++g) {
           const int s = g % kStages;
           if (!mbar_wait(smem_u32(&bars[kStages + s]), ((uint32_t)(g / kStages) & 1u) ^ 1u,
@@ -337,8 +364,8 @@ __global__ void __launch_bounds__(kGemm64Threads, 1)
           }
           const uint32_t full = smem_u32(&bars[s]), sa = base + s * kStage;
           mbar_expect_tx(full, kStage);
-          tma_load_3d(sa, &tmA, kb * kKB, m0, 0, full);
-          tma_load_3d(sa + kABytes, &tmB, kb * kKB, n0, 0, full);
+          tma_load_3d(sa, &tmA, kb * kKB, g0 + m0, 0, full);
+          tma_load_3d(sa + kABytes, &tmB, kb * kKB, g0 + n0, 0, full);
         }
       }
       if (*abort_flag)  // let the copies already issued land
@@ -350,6 +377,8 @@ __global__ void __launch_bounds__(kGemm64Threads, 1)
       bool ok = true;
       int g = 0, j = 0;  // stages consumed, accumulations started
       for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+        int g0, m0, n0;
+        if (!tile(t, g0, m0, n0)) continue;
         for (int kb0 = 0; kb0 < p.nkb && ok; kb0 += kChunkB, ++j) {
           if (!mbar_wait(acc_empty, ((uint32_t)j & 1u) ^ 1u, abort_flag)) {
             *abort_flag = 1;
@@ -402,7 +431,10 @@ __global__ void __launch_bounds__(kGemm64Threads, 1)
     int j = 0;
     bool ok = true;
     for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-      const int m0 = (t / ntn) * kBM, n0 = (t % ntn) * BN + half * NC;
+      int g0, m0, n0;
+      if (!tile(t, g0, m0, n0)) continue;
+      n0 += half * NC;
+      const int rows = kGram ? p.grp : p.M;  // rows and columns are the group's
       const int row0 = m0 + quarter * 32, row = row0 + lane;
       long long acc[NC];  // the sum in units of level 3, and 28 bits below
       uint32_t low[NC];
@@ -447,34 +479,29 @@ __global__ void __launch_bounds__(kGemm64Threads, 1)
           asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(acc_empty) : "memory");
       }
       if (!ok) break;
-      const int ea = row < p.M ? p.ea[row] : 0;
-      const bool bad = ea == kBadRow;
+      const int ea = row < rows ? p.ea[g0 + row] : 0;
+      bool odd = ea == kBadRow;  // a row or (Gram products) a column that is not finite
       constexpr int kS = NC < 16 ? NC : 16;  // columns staged at a time
 #pragma unroll
       for (int c0 = 0; c0 < NC; c0 += kS) {
         if (n0 + c0 >= p.N) break;
 #pragma unroll
         for (int c = 0; c < kS; ++c) {
-          const int col = n0 + c0 + c;
-          double v = 0.0;
-          if (col < p.N) {
-            if (!bad) {
-              v = scaled_to_f64(acc[c0 + c], low[c0 + c], ea + p.eb[col] - 35);
-            } else {
-              const double *y = p.B + (size_t)col * p.ldb;
-              const int gr = p.row0 + row;
-              const double *x = p.A ? p.A + (size_t)row * p.lda : p.W + (size_t)(gr % p.g) * p.K;
-              const double *d = p.A ? nullptr : p.der + (size_t)(gr / p.g) * p.ldd;
-              for (int k = 0; k < p.K; ++k) v += (d ? x[k] * d[k] : x[k]) * y[k];
-            }
-          }
-          stg[lane * 16 + ((((c >> 1) ^ (lane & 7)) << 1) | (c & 1))] = v;
+          const int eb = n0 + c0 + c < p.N ? p.eb[g0 + n0 + c0 + c] : 0;
+          if (kGram) odd |= eb == kBadRow;
+          stg[lane * 16 + ((((c >> 1) ^ (lane & 7)) << 1) | (c & 1))] =
+              scaled_to_f64(acc[c0 + c], low[c0 + c], ea + eb - 35);
         }
+        const bool plain = __any_sync(0xffffffffu, odd);
         __syncwarp();
         for (int q = lane; q < 32 * kS; q += 32) {
           const int r = q / kS, c = q % kS, col = n0 + c0 + c;
-          if (row0 + r < p.M && col < p.N)
-            epi(p.row0 + row0 + r, col, stg[r * 16 + ((((c >> 1) ^ (r & 7)) << 1) | (c & 1))]);
+          if (row0 + r < rows && col < p.N && (!kGram || col <= row0 + r)) {
+            double v = stg[r * 16 + ((((c >> 1) ^ (r & 7)) << 1) | (c & 1))];
+            if (plain && (p.ea[g0 + row0 + r] == kBadRow || p.eb[g0 + col] == kBadRow))
+              v = plain_dot(p, g0, row0 + r, col);
+            epi(p.row0 + g0 + row0 + r, col, v);
+          }
         }
         __syncwarp();
       }
@@ -489,6 +516,20 @@ __global__ void __launch_bounds__(kGemm64Threads, 1)
                  : "memory");
   }
 }
+
+// Entry (row of all groups, column <= row within the group) of a packed triangle
+// in the chain's factor slot.
+struct EpiSlot {
+  double *L;
+  size_t slot, stride;
+  const int *cur;
+  int mode, g;
+  __device__ void operator()(int r, int c, double v) const {
+    const int chain = r / g, i = r - chain * g;
+    const int s = mode == 0 ? cur[chain] : 1 - cur[chain];
+    L[(size_t)s * slot + (size_t)chain * stride + (size_t)i * (i + 1) / 2 + c] = v;
+  }
+};
 
 // 3D map over digit planes: dims (K, rows, planes), box (32, box_rows, planes).
 bool make_digit_map(CUtensorMap *tm, const __nv_bfloat16 *ptr, int K, int rows, int ldp,
@@ -512,9 +553,10 @@ bool make_digit_map(CUtensorMap *tm, const __nv_bfloat16 *ptr, int K, int rows, 
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int BN, class Epi>
-cudaError_t run_gemm64(const Gemm64Args &a, const Epi &epi, cudaStream_t st) {
+template <int BN, bool kGram, class Epi>
+cudaError_t run_gemm64_t(const Gemm64Args &a, const Epi &epi, cudaStream_t st) {
   Gemm64Params p{};
+  p.grp = kGram ? a.N : 0;
   p.M = a.M;
   p.N = a.N;
   p.K = a.K;
@@ -534,7 +576,7 @@ cudaError_t run_gemm64(const Gemm64Args &a, const Epi &epi, cudaStream_t st) {
   p.tmem_cols = kDigits * BN;
   CUtensorMap tmA, tmB;
   if (!make_digit_map(&tmA, a.A, a.K, a.M, a.ldp, a.plane, kBM) ||
-      !make_digit_map(&tmB, a.B.d, a.K, a.N, a.B.ldp, a.B.plane, BN))
+      !make_digit_map(&tmB, a.B.d, a.K, kGram ? a.M : a.N, a.B.ldp, a.B.plane, BN))
     return cudaErrorInvalidValue;
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -542,10 +584,12 @@ cudaError_t run_gemm64(const Gemm64Args &a, const Epi &epi, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   const size_t smem = 1024 + kStages * (kABytes + (size_t)kDigits * BN * kKB * 2) + kStgBytes +
                       (2 * kStages + 5) * 8;
-  auto k = k_gemm64<BN, Epi>;
+  auto k = k_gemm64<BN, kGram, Epi>;
   e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const int tiles = ((a.M + kBM - 1) / kBM) * ((a.N + BN - 1) / BN);
+  const int ntn = (a.N + BN - 1) / BN;
+  const int tiles = kGram ? a.M / a.N * ((a.N + kBM - 1) / kBM) * ntn
+                          : ((a.M + kBM - 1) / kBM) * ntn;
   k<<<std::min(tiles, sms), kGemm64Threads, smem, st>>>(tmA, tmB, p, epi);
   return cudaGetLastError();
 }
@@ -558,8 +602,8 @@ cudaError_t run_gemm64(const Gemm64Args &a, const Epi &epi, cudaStream_t st) {
     return cudaErrorInvalidValue;
   // 64 columns a tile; 32 where those tiles would leave SMs idle
   const long t64 = (long)((a.M + kBM - 1) / kBM) * ((a.N + 63) / 64);
-  if (a.N <= 32 || t64 < 100) return run_gemm64<32>(a, epi, st);
-  return run_gemm64<64>(a, epi, st);
+  if (a.N <= 32 || t64 < 100) return run_gemm64_t<32, false>(a, epi, st);
+  return run_gemm64_t<64, false>(a, epi, st);
 }
 
 }  // namespace
@@ -588,6 +632,35 @@ cudaError_t launch_split64(int rows, int K, const double *src, int ld, const dou
 cudaError_t launch_col_exp(int rows, int K, const double *B, int ld, int *fk, cudaStream_t st) {
   k_col_exp<<<(K + 127) / 128, 128, 0, st>>>(rows, K, B, ld, fk);
   return cudaGetLastError();
+}
+
+cudaError_t gram64_slots(int groups, int g, int K, const double *J, int ldj,
+                         const __nv_bfloat16 *digits, const int *ex, int ldp, size_t plane,
+                         double *L, size_t slot, size_t stride, const int *cur, int mode, int *err,
+                         cudaStream_t st) {
+  if (groups <= 0) return cudaSuccess;
+  if (g < 1 || K <= 0 || (long long)groups * g > 0x7fffffffLL || (ldp & 7) || (plane & 7) ||
+      ((uintptr_t)digits & 15) || !err)
+    return cudaErrorInvalidValue;
+  Gemm64Args a;
+  a.M = groups * g;
+  a.N = g;
+  a.K = K;
+  a.A = digits;
+  a.ea = ex;
+  a.ldp = ldp;
+  a.plane = plane;
+  a.Asrc = J;
+  a.lda = ldj;
+  a.B.d = digits;
+  a.B.ex = ex;
+  a.B.ldp = ldp;
+  a.B.plane = plane;
+  a.B.src = J;
+  a.B.ld = ldj;
+  a.err = err;
+  const EpiSlot epi{L, slot, stride, cur, mode, g};
+  return g <= 32 ? run_gemm64_t<32, true>(a, epi, st) : run_gemm64_t<64, true>(a, epi, st);
 }
 
 cudaError_t gemm64_store(const Gemm64Args &a, double *out, int ldo, cudaStream_t st) {

@@ -503,8 +503,16 @@ __global__ void __launch_bounds__(NT, kWbMinBlocks) k_wb_geometry(ReducedArgs a,
     }
   } else {
     rows_times<A, TJ>(J, dy, r, inv_sigma, be, ae, mode == 1, Kb, Ka);  // K b, K a
-    form_gram_f64<true>(reinterpret_cast<const double *>(J), r, dy, r, inv_nv,
-                        reinterpret_cast<double *>(Ms), sm + lay.tail);
+    if (a.gram_in_slot) {  // formed on the tensor cores, packed in the slot
+      double *Md = reinterpret_cast<double *>(Ms);
+      for (int e = threadIdx.x; e < tri(dy); e += blockDim.x) Md[e] = Lg[e] * inv_nv;
+      __syncthreads();
+      for (int i = threadIdx.x; i < dy; i += blockDim.x) Md[tri(i) + i] += 1.0;
+      __syncthreads();
+    } else {
+      form_gram_f64<true>(reinterpret_cast<const double *>(J), r, dy, r, inv_nv,
+                          reinterpret_cast<double *>(Ms), sm + lay.tail);
+    }
   }
   double uu = 0.0;
   for (int i = threadIdx.x; i < dy; i += blockDim.x) {
@@ -802,7 +810,8 @@ size_t wb_geometry_smem(int r, int dy) {
 
 template <typename TJ, bool kPre, int NT>
 cudaError_t launch_wb_geometry_k(const ReducedArgs &a, int mode, cudaStream_t st) {
-  const size_t smem = wb_geometry_smem<TJ>(a.r, a.d_y);
+  const size_t smem = a.gram_in_slot ? WbLayout(a.r, a.d_y).tail * sizeof(double)  // no rows of J staged
+                            : wb_geometry_smem<TJ>(a.r, a.d_y);
   cudaError_t e = cudaFuncSetAttribute(k_wb_geometry<TJ, kPre, NT>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;

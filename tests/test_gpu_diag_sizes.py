@@ -78,3 +78,27 @@ def test_a_still_degree_of_freedom_and_repeated_columns(dino):
         ctx.close()
     W, V = dg.covariance_estimators(X)
     assert abs(out["mpsrf_w"] - dg.wasserstein_mpsrf(W, V)) <= 2e-8 * 6 * np.trace(V)
+
+
+def test_a_nan_sample_stays_in_its_degree_of_freedom(dino):
+    """One NaN among d = 40 (Gram matrix on the tensor cores): the other degrees
+    of freedom keep their bits, traces and MPSRF are NaN, as in plain arithmetic."""
+    rng = np.random.default_rng(9)
+    n_c, n_s, d = 3, 40, 40
+    X = rng.standard_normal((n_c, n_s, d))
+    res = []
+    for bad in (False, True):
+        if bad:
+            X[1, 7, 5] = np.nan
+        ctx = dino.dino_init(0)
+        try:
+            g = dino.dino_diag_create(ctx, n_c, d, n_s)
+            for j in range(n_s):
+                dino.dino_diag_push(ctx, g, X[:, j, :])
+            res.append(dino.dino_diag_compute(ctx, g, d, mpsrf=True))
+        finally:
+            ctx.close()
+    keep = np.arange(d) != 5
+    assert np.array_equal(res[0]["ess"][keep], res[1]["ess"][keep])
+    for k in ("msj", "trace_w", "trace_v", "mpsrf_w"):
+        assert np.isfinite(res[0][k]) and np.isnan(res[1][k]), k
