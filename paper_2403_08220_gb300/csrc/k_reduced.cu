@@ -35,7 +35,7 @@
 // double-float on the FP32 pipe.
 #include <algorithm>
 
-#include "chol.cuh"
+#include "chol_mma.cuh"
 
 namespace dino {
 namespace {
@@ -113,11 +113,12 @@ __device__ void cta_upper_matvec2(const typename A::T *Ls, int r, const typename
 // factor lives in its global slot and takes no shared memory.
 struct Layout {
   size_t Ls, inv, v0, res, red, flag, tail;
-  __host__ __device__ Layout(int r, int dy, bool global) {
+  // lean: without the last four vectors (vp, vq, be, ae)
+  __host__ __device__ Layout(int r, int dy, bool global, bool lean = false) {
     Ls = 0;
     inv = global ? 0 : slot_stride(r);
     v0 = inv + r + 1;
-    res = v0 + 7 * (size_t)r;
+    res = v0 + (lean ? 3 : 7) * (size_t)r;
     red = res + dy;
     flag = red + kRed;
     tail = (flag + 1 + 1) & ~(size_t)1;  // 16-byte aligned start of the J chunk
@@ -422,12 +423,13 @@ __global__ void __launch_bounds__(kGramThreads, 4) k_gram_f32(ReducedArgs a, int
 // an accepted chain to b: its factor slot (written only then, into the other
 // slot, which becomes current) and its state vectors.  The complement
 // coefficient b - s a is written for every chain.
-// The FP32-Jacobian instantiations find I + H in the slot (k_gram_f32) and run
-// at 64 registers a thread, 32 warps an SM where shared memory allows.
-// G: `panel` (elements from the start of shared memory, 0 if it does not fit)
-// places the blocked factorisation's panel.
-template <typename TJ, bool G, int NT>
-__global__ void __launch_bounds__(NT, sizeof(TJ) == 4 && !G
+// The FP32-Jacobian instantiations find I + H in the slot (k_gram_f32).  kBlk: a
+// blocked factorisation, whose digits or panel lie at sm + panel (FP32
+// Jacobian: trailing updates on the tensor cores; FP64: factors in global
+// memory).  Otherwise 8-column panels, and with an FP32 Jacobian 64 registers a
+// thread, 32 warps an SM where shared memory allows.
+template <typename TJ, bool G, int NT, bool kBlk>
+__global__ void __launch_bounds__(NT, sizeof(TJ) == 4 && !kBlk
                                           ? 1024 / NT
                                           : (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
     k_geometry(ReducedArgs a, int mode, int panel) {
@@ -438,7 +440,8 @@ __global__ void __launch_bounds__(NT, sizeof(TJ) == 4 && !G
   extern __shared__ __align__(16) double sm[];
   const int c = blockIdx.x, r = a.r, dy = a.d_y;
   const size_t ldL = slot_stride(r), lsz = tri_size(r + 1);
-  const Layout lay(r, dy, G);
+  constexpr bool kLean = G && sizeof(TJ) == 4 && kBlk;
+  const Layout lay(r, dy, G, kLean);
   const int slot = mode == 0 ? a.cur[c] : 1 - a.cur[c];
   double *Lg = a.L + (size_t)slot * a.L_slot + (size_t)c * ldL;
   E *Ls = reinterpret_cast<E *>(G ? Lg : sm + lay.Ls);
@@ -463,8 +466,10 @@ __global__ void __launch_bounds__(NT, sizeof(TJ) == 4 && !G
   for (int i = threadIdx.x; i < r; i += blockDim.x) {
     vb[i] = a.b[(size_t)c * r + i];
     va[i] = mode == 1 ? a.mr[(size_t)c * r + i] : 0.0;
-    be[i] = A::from(vb[i]);
-    ae[i] = A::from(va[i]);
+    if constexpr (!kLean) {
+      be[i] = A::from(vb[i]);
+      ae[i] = A::from(va[i]);
+    }
   }
   double ph = 0.0;
   for (int i = threadIdx.x; i < dy; i += blockDim.x) {
@@ -477,7 +482,8 @@ __global__ void __launch_bounds__(NT, sizeof(TJ) == 4 && !G
   // are threads for it two per column, each half of the rows
   const int half = blockDim.x / 2;
   const bool two = r <= half;
-  E *ge = reinterpret_cast<E *>(vp);  // the second halves' sums
+  // the second halves' sums (the lean layout has no vp yet: the panel's place)
+  E *ge = reinterpret_cast<E *>(kLean ? sm + panel : vp);
   if (two) {
     const int h = threadIdx.x >= half ? 1 : 0, j = threadIdx.x - h * half;
     typename A::Acc acc = A::begin(E{});
@@ -518,10 +524,25 @@ __global__ void __launch_bounds__(NT, sizeof(TJ) == 4 && !G
   vv = block_sum(vv, red);
   if (threadIdx.x == 0) Ls[tri(r) + r] = A::from(1.0 + vv);
   __syncthreads();
-  if (G && panel)
-    cta_cholesky_global<A>(Ls, inv, r + 1, reinterpret_cast<E *>(sm + panel));
-  else
+  if constexpr (!kBlk)
     cta_cholesky_panels<A>(Ls, inv, r + 1);
+  else if constexpr (sizeof(TJ) == 8)
+    cta_cholesky_global<A>(Ls, inv, r + 1, reinterpret_cast<E *>(sm + panel));
+  else if constexpr (G)
+    cta_cholesky_global_mma(Ls, inv, r + 1, reinterpret_cast<char *>(sm + panel));
+  else
+    cta_cholesky_mma(Ls, inv, r + 1, reinterpret_cast<char *>(sm + panel));
+  if constexpr (kLean) {  // vp, vq, and b, a as factor elements, over the panel
+    __syncthreads();
+    vp = sm + panel;
+    vq = vp + r;
+    be = reinterpret_cast<E *>(vq + r);
+    ae = be + r;
+    for (int i = threadIdx.x; i < r; i += blockDim.x) {
+      be[i] = A::from(vb[i]);
+      ae[i] = A::from(va[i]);
+    }
+  }
   double ld = 0.0;
   for (int i = threadIdx.x; i < r; i += blockDim.x) ld += log(A::to(Ls[tri(i) + i]));
   const double hld_b = block_sum(ld, red);
@@ -602,22 +623,13 @@ size_t geometry_smem_bytes(int r, int d_y, int jf_f32) {
   return lay.tail * sizeof(double) + jc;
 }
 
-// A factor in global memory: where its panel lies (after the vectors; the
-// staged rows of an FP64 J are done with by then), 0 where it does not fit.
-static int geometry_panel(int r, int d_y, size_t &smem) {
-  if (!uses_global_factor(r, d_y)) return 0;
-  const size_t at = Layout(r, d_y, true).tail;
-  const size_t need = (at + (size_t)(r + 1) * kPanelLd) * sizeof(double);
-  if (need > kSmemLimit) return 0;
-  smem = std::max(smem, need);
-  return (int)at;
-}
-
 cudaError_t launch_propose(const ReducedArgs &a, cudaStream_t st) {
   if (a.r <= 32 * 7) {
     const int grid = (a.C + kPropWarps - 1) / kPropWarps;
     if (a.r <= 32 * 2)
       k_propose_warp<2><<<grid, 32 * kPropWarps, 0, st>>>(a);
+    else if (a.r <= 32 * 4)
+      k_propose_warp<4><<<grid, 32 * kPropWarps, 0, st>>>(a);
     else
       k_propose_warp<7><<<grid, 32 * kPropWarps, 0, st>>>(a);
     return cudaGetLastError();
@@ -630,37 +642,67 @@ cudaError_t launch_propose(const ReducedArgs &a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-template <typename TJ, bool G, int NT>
+// r from which the smem-resident factor of an FP32 Jacobian takes the blocked
+// factorisation: at r = 128 it is the faster (1.60 against 2.02 ms for 4096 chains),
+// at r = 73 the slower (the four CTAs an SM of the plain one hide its chains of
+// dependent operations better: 2.85 against 2.60 ms for a step of 4089 chains).
+constexpr int kBlkMinR = 112;
+
+// Where the blocked factorisations keep their digits or panel (elements from the
+// start of shared memory; 0 where they do not apply or fit), with smem raised
+// to hold them.  FP32 Jacobian: behind the layout; for a factor in global memory
+// the vectors vp, vq, be, ae, formed after it, take the panel's place.  FP64 with
+// the factor in global memory: after the vectors (the staged rows of J are done
+// with by then).
+static int geometry_panel(int r, int d_y, int jf_f32, size_t &smem) {
+  const bool G = uses_global_factor(r, d_y);
+  if (!G && (!jf_f32 || r < kBlkMinR)) return 0;
+  const size_t at = Layout(r, d_y, G, G && jf_f32).tail;
+  const size_t bytes = !jf_f32 ? (size_t)(r + 1) * kPanelLd * sizeof(double)
+                       : G     ? std::max(mma_panel_bytes(r + 1), (size_t)32 * r)
+                               : mma_digit_bytes(r + 1);
+  const size_t need = at * sizeof(double) + bytes;
+  if (need > kSmemLimit) return 0;
+  smem = G && jf_f32 ? need : std::max(smem, need);
+  return (int)at;
+}
+
+template <typename TJ, bool G, int NT, bool kBlk>
 static cudaError_t launch_geometry_nt(const ReducedArgs &a, int mode, size_t smem, int panel,
                                       cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute(k_geometry<TJ, G, NT>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  auto k = k_geometry<TJ, G, NT, kBlk>;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_geometry<TJ, G, NT><<<a.C, NT, smem, st>>>(a, mode, panel);
+  k<<<a.C, NT, smem, st>>>(a, mode, panel);
   return cudaGetLastError();
 }
 
-// CTA size by r: a small factor keeps few threads busy, and smaller CTAs let
-// more chains share an SM (the kernel's loops stride over blockDim).  FP64:
-// 128 and 256 threads are held to 128 registers so that four and two CTAs fit
-// an SM.  FP32 Jacobian: the size that fills 32 warps with as many CTAs as the
-// shared memory of the factor lets in (r = 100: four of 256 threads; r = 128:
-// two of 512).  A factor in global memory with its panel in shared memory: 256
-// threads at 128 registers, two CTAs an SM up to r of about 500.
+// CTA size: smaller CTAs let more chains share an SM (the kernel's loops stride
+// over blockDim).  FP64: 128 threads up to r = 64 and 256 up to r = 128, held to 128
+// registers so that four and two CTAs fit an SM.  FP32 Jacobian, plain: the size
+// that fills 32 warps with as many CTAs as the shared memory of the factor lets
+// in (r = 100: four of 256 threads).  Blocked: 256 threads at 128 registers while
+// two CTAs fit an SM (r = 128; factors in global memory up to r = 400), else 512.
 template <typename TJ, bool G>
 static cudaError_t launch_geometry_t(const ReducedArgs &a, int mode, size_t smem,
                                      cudaStream_t st) {
-  const int panel = G ? geometry_panel(a.r, a.d_y, smem) : 0;
-  if (panel) return launch_geometry_nt<TJ, G, 256>(a, mode, smem, panel, st);
-  if constexpr (sizeof(TJ) == 4 && !G) {
-    const size_t ctas = kSmemLimit / (smem + 1024);
-    if (a.r <= 64) return launch_geometry_nt<TJ, G, 128>(a, mode, smem, 0, st);
-    if (ctas >= 4 && a.r <= 128) return launch_geometry_nt<TJ, G, 256>(a, mode, smem, 0, st);
-    return launch_geometry_nt<TJ, G, kThreads>(a, mode, smem, 0, st);
+  const int panel = geometry_panel(a.r, a.d_y, a.jf_f32, smem);
+  const size_t ctas = kSmemLimit / (smem + 1024);
+  if constexpr (G) {
+    if (panel) return launch_geometry_nt<TJ, G, 256, true>(a, mode, smem, panel, st);
+    return launch_geometry_nt<TJ, G, kThreads, false>(a, mode, smem, 0, st);
+  } else if constexpr (sizeof(TJ) == 4) {
+    if (panel)
+      return ctas >= 2 ? launch_geometry_nt<TJ, G, 256, true>(a, mode, smem, panel, st)
+                       : launch_geometry_nt<TJ, G, kThreads, true>(a, mode, smem, panel, st);
+    if (a.r <= 64) return launch_geometry_nt<TJ, G, 128, false>(a, mode, smem, 0, st);
+    if (ctas >= 4) return launch_geometry_nt<TJ, G, 256, false>(a, mode, smem, 0, st);
+    return launch_geometry_nt<TJ, G, kThreads, false>(a, mode, smem, 0, st);
+  } else {
+    if (a.r <= 64) return launch_geometry_nt<TJ, G, 128, false>(a, mode, smem, 0, st);
+    if (a.r <= 128) return launch_geometry_nt<TJ, G, 256, false>(a, mode, smem, 0, st);
+    return launch_geometry_nt<TJ, G, kThreads, false>(a, mode, smem, 0, st);
   }
-  if (a.r <= 64) return launch_geometry_nt<TJ, G, 128>(a, mode, smem, 0, st);
-  if (a.r <= 128) return launch_geometry_nt<TJ, G, 256>(a, mode, smem, 0, st);
-  return launch_geometry_nt<TJ, G, kThreads>(a, mode, smem, 0, st);
 }
 
 cudaError_t launch_gram_f32(const ReducedArgs &a, int mode, cudaStream_t st) {

@@ -1,0 +1,49 @@
+"""The double-float factorisation with tensor-core trailing updates, against FP64.
+
+Small-integer weights and the identity activation make J exact, so I + J^T J is
+exact in FP32 and the factor of the r-sized path must agree with an FP64
+Cholesky.  Sizes around the 8- and 16-column panels, the 16-row and 32-column
+work items, and each place of the factor (shared memory with 128, 256 and 512
+threads, global memory); columns of J scaled by powers of two spread the
+diagonal over twelve binary orders.  The double-float entries carry 48 bits
+relative to the diagonal, so L L^T must reproduce the matrix to 2^-44 n of
+sqrt(M_ii M_jj) (one rounding per column, a factor 16 for the worst case); that
+error E moves half log det by at most sum |M^-1| |E| / 2.
+"""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("r", [1, 7, 8, 9, 15, 16, 17, 23, 24, 31, 32, 33, 47, 64, 65, 100, 127,
+                               130, 160, 195, 207, 209, 240, 255, 400])
+def test_factor_reproduces_the_matrix(r):
+    import paper_2403_08220_gb300 as dino
+
+    rng = np.random.default_rng(r)
+    h, dy = 30, r + 11
+    W1 = rng.integers(-1, 2, size=(h, r)) * 2.0 ** rng.integers(-6, 7, size=r)
+    W2 = rng.integers(-1, 2, size=(dy, h)).astype(float)
+    n = int(np.ceil(np.sqrt(r))) + 1
+    ctx = dino.dino_init(0)
+    try:
+        sid = dino.dino_load_surrogate(
+            ctx, n_grid=n, prior_gamma=0.1, prior_delta=1.0, r=r, widths=[r, h, dy],
+            activation=0, W=[W1, W2], b=[np.zeros(h), np.zeros(dy)],
+            basis_kind=dino.DINO_BASIS_KLE, y=np.zeros(dy), noise_var=1.0,
+            precision=dino.DINO_PREC_BF16, noise_map=dino.DINO_NOISE_CHOLESKY)
+        o = dino.dino_surrogate_eval(ctx, sid, rng.standard_normal((2, r)), dy)
+    finally:
+        ctx.close()
+    for c in range(2):
+        J = o["J"][c]
+        assert np.array_equal(J, W2 @ W1)
+        M = np.eye(r) + J.T @ J
+        s = np.sqrt(np.diag(M))
+        L = o["L"][c].astype(np.longdouble)
+        err = np.abs((L @ L.T).astype(np.float64) - M) / np.outer(s, s)
+        assert err.max() <= 2.0 ** -44 * max(r, 4), err.max()
+        ref = np.linalg.slogdet(M)[1] / 2
+        tol = 2.0 ** -45 * max(r, 4) * np.sum(np.abs(np.linalg.inv(M)) * np.outer(s, s))
+        assert abs(o["hld"][c] - ref) <= tol + 1e-13 * abs(ref)
