@@ -139,20 +139,19 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float &a, float &b) {
   return u;
 }
 
-__device__ __forceinline__ float act_fn(int kind, float z) {
-  if (kind == 1) return tanhf(z);
-  if (kind == 2) return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f));
-  return z;
-}
-__device__ __forceinline__ float act_deriv(int kind, float z) {
+// The activation of z and its derivative, one erf or tanh for both (a layer of 400
+// over 4096 chains: 46 us with two, 39 us).
+__device__ __forceinline__ void act_both(int kind, float z, float &a, float &d) {
+  a = z;
+  d = 1.0f;
   if (kind == 1) {
-    const float t = tanhf(z);
-    return 1.0f - t * t;
+    a = tanhf(z);
+    d = 1.0f - a * a;
+  } else if (kind == 2) {
+    const float e = 1.0f + erff(z * 0.70710678118654752f);
+    a = 0.5f * z * e;
+    d = 0.5f * e + z * __expf(-0.5f * z * z) * 0.39894228040143267794f;
   }
-  if (kind == 2)
-    return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) +
-           z * __expf(-0.5f * z * z) * 0.39894228040143267794f;
-  return 1.0f;
 }
 
 __device__ __forceinline__ void store_slices(float x, __nv_bfloat16 *dst, size_t plane,
@@ -459,7 +458,11 @@ __global__ void __launch_bounds__(kThreads, 1)
               for (int h = 0; h < 2; ++h) {
                 uint32_t w[32];
 #pragma unroll
-                for (int j = 0; j < 32; ++j) w[j] = __float_as_uint(act_deriv(p.act, v[32 * h + j]));
+                for (int j = 0; j < 32; ++j) {  // the derivative out, the activation in v
+                  float d;
+                  act_both(p.act, v[32 * h + j], v[32 * h + j], d);
+                  w[j] = __float_as_uint(d);
+                }
                 if (p.tma)  // tmO maps the derivative here
                   store_rows_tma(stg, sbuf, w, &tmO, false, n0 + c0 + 32 * h, row0, 0, nrows,
                                  lane);
@@ -469,8 +472,6 @@ __global__ void __launch_bounds__(kThreads, 1)
                       reinterpret_cast<char *>(p.der + (size_t)row0 * p.N + n0 + c0 + 32 * h),
                       (size_t)p.N * 4, nrows, lane);
               }
-#pragma unroll
-              for (int j = 0; j < 64; ++j) v[j] = act_fn(p.act, v[j]);
             }
             for (int sl = 0; sl < p.out_slices; ++sl) {
               uint32_t w[32];
@@ -533,8 +534,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
               const float z = v[j] + (j < ncols ? p.bias[col0 + j] : 0.0f);
-              x[j] = act_fn(p.act, z);
-              v[j] = act_deriv(p.act, z);
+              act_both(p.act, z, x[j], v[j]);
             }
             if (ncols == 16 && (p.N & 3) == 0) {
 #pragma unroll
@@ -603,15 +603,16 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
-// Per-group Gram matrices G_c = J_c J_c^T (persistent, one CTA per SM, groups
-// c = blockIdx.x, + gridDim.x, ...).  A stage holds one 64-wide k-block of
-// all slices of the 128 rows starting at row c g (the rows past the group
-// belong to the next group or are zero-filled past the end, and are never
-// stored); both MMA operands are views of the same staged tile, B its first
-// BN = ceil16(g) rows.  Roles and bounded waits as in k_tc_gemm; the
-// epilogue writes rows i < g, columns j < g.
+// Per-group Gram matrices G_c = J_c J_c^T (persistent, one CTA per SM, tiles of
+// `batch` groups from c on).  A stage holds one 64-wide k-block of
+// all slices of the 128 rows starting at row c g: `batch` = 128 / g whole groups
+// (rows past them belong to the next tile's or are zero-filled past the end);
+// both MMA operands are views of the same staged tile, B its first
+// ceil16(batch g) rows, and the epilogue writes the groups' diagonal blocks.
+// Roles and bounded waits as in k_tc_gemm.
 struct GramParams {
   int C, g, K, BN, nkb, nslice, npairs, stages;
+  int batch;  // groups per tile
   int pair_a[6], pair_b[6];
   float *out;
   int ldo;
@@ -665,7 +666,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (lane == 0) {
       int g = 0;
       bool ok = true;
-      for (int c = blockIdx.x; c < p.C && ok; c += gridDim.x) {
+      for (int c = blockIdx.x * p.batch; c < p.C && ok; c += gridDim.x * p.batch) {
         for (int kb = 0; kb < p.nkb; ++kb, ++g) {
           const int s = g % S;
           const uint32_t ph = (uint32_t)(g / S) & 1u;
@@ -692,7 +693,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint32_t idesc = idesc_bf16(kBlockM, p.BN);
       bool ok = true;
       int g = 0, j = 0;
-      for (int c = blockIdx.x; c < p.C && ok; c += gridDim.x, ++j) {
+      for (int c = blockIdx.x * p.batch; c < p.C && ok; c += gridDim.x * p.batch, ++j) {
         const int b = j & 1;
         if (!mbar_wait(smem_u32(&bars[2 * S + 2 + b]), (((uint32_t)j >> 1) & 1u) ^ 1u,
                        abort_flag)) {
@@ -736,7 +737,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int i0 = quarter * 32, nrows = min(32, p.g - i0);  // rows of this warp in the group
     uint4 *stg = stg_all + quarter * 256;
     int j = 0;
-    for (int c = blockIdx.x; c < p.C; c += gridDim.x, ++j) {
+    for (int c = blockIdx.x * p.batch; c < p.C; c += gridDim.x * p.batch, ++j) {
       const int b = j & 1;
       int okl = 0;
       if (lane == 0)
@@ -750,8 +751,22 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       fence_after();
       const uint32_t tacc = tmem + ((uint32_t)(i0) << 16) + (uint32_t)(b * p.BN);
+      if (p.batch > 1) {
+        // lane: row i0 + lane of the tile, of group row / g; its own group's columns
+        const int row = i0 + lane, grp = row / p.g, lo = grp * p.g;
+        const bool in = grp < p.batch && c + grp < p.C;
+        float *o = p.out + ((size_t)c * p.g + row) * p.ldo - lo;
+        for (int c0 = 0; c0 < p.batch * p.g; c0 += 16) {
+          float v[16];
+          tmem_ld16(tacc + (uint32_t)c0, v);
+          if (in && c0 + 16 > lo && c0 < lo + p.g)
+#pragma unroll
+            for (int q = 0; q < 16; ++q)
+              if (c0 + q >= lo && c0 + q < lo + p.g) o[c0 + q] = v[q];
+        }
+      }
       float *orow = p.out + ((size_t)c * p.g + i0) * p.ldo;
-      int c0 = 0;
+      int c0 = p.batch > 1 ? p.g : 0;
       if ((p.ldo & 3) == 0) {
         for (; c0 + 32 <= p.g; c0 += 32) {
           float v[32];
@@ -1064,7 +1079,10 @@ cudaError_t launch_tc_gram(int C, int g, int K, const __nv_bfloat16 *J, int ldj,
   p.C = C;
   p.g = g;
   p.K = K;
-  p.BN = (g + 15) / 16 * 16;
+  // as many groups as fit the 128 rows of a tile; each entry is the same sum in
+  // the same order (d_y = 25, 4096 groups: 150 us with a group a tile, 54 us)
+  p.batch = kBlockM / g;
+  p.BN = (p.batch * g + 15) / 16 * 16;
   p.nkb = (K + kBlockK - 1) / kBlockK;
   p.nslice = nslice;
   static const int pa[6] = {0, 0, 1, 0, 1, 2}, pb[6] = {0, 1, 0, 2, 1, 0};
@@ -1094,7 +1112,7 @@ cudaError_t launch_tc_gram(int C, int g, int K, const __nv_bfloat16 *J, int ldj,
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
     return cudaErrorInvalidValue;
-  k_tc_gram<<<std::min(C, sms), kThreads, smem, st>>>(tm, p);
+  k_tc_gram<<<std::min((C + p.batch - 1) / p.batch, sms), kThreads, smem, st>>>(tm, p);
   return cudaGetLastError();
 }
 

@@ -37,8 +37,13 @@ namespace dino {
 namespace {
 
 constexpr int kWbThreads = 128;
-constexpr int kWbPreThreads = 256;  // geometry with the Gram matrix and K b, K a formed beforehand
-constexpr int kWbMinBlocks = 4;     // CTAs per SM the register budget is sized for
+constexpr int kWbMinBlocks = 4;  // CTAs per SM the register budget is sized for
+
+// Threads of the double-float kernels' CTA by d_y (64 registers each): a small
+// factor keeps few threads busy, and its chains of dependent operations are
+// hidden by more chains on the SM (d_y = 25, 4096 chains, 256 and 64 threads:
+// geometry 234 and 120 us, proposal 142 and 99 us).
+inline int wb_pre_threads(int dy) { return dy <= 32 ? 64 : dy <= 64 ? 128 : 256; }
 
 // Slot offsets (8-byte elements).
 struct WbSlot {
@@ -360,10 +365,11 @@ __device__ void wb_store_factor(double *Lg, const typename A::T *Ms, const typen
 
 // One CTA of NT threads per chain at the point b (see the file comment).
 // kPre: the Gram matrix J J^T and K b, K a come formed (the tensor-core
-// path); this instantiation is kept lean in registers so that NT = 256
-// threads (64 registers each) fit four CTAs on an SM.
+// path); this instantiation is kept lean in registers so that 1024 threads (64
+// registers each) fit an SM.
 template <typename TJ, bool kPre, int NT>
-__global__ void __launch_bounds__(NT, kWbMinBlocks) k_wb_geometry(ReducedArgs a, int mode) {
+__global__ void __launch_bounds__(NT, kPre ? 1024 / NT : kWbMinBlocks)
+    k_wb_geometry(ReducedArgs a, int mode) {
   using A = std::conditional_t<sizeof(TJ) == 4, DF, F64>;
   using E = typename A::T;
   static_assert(sizeof(E) == sizeof(double), "one factor element per double of the slot");
@@ -591,7 +597,8 @@ __global__ void __launch_bounds__(NT, kWbMinBlocks) k_wb_geometry(ReducedArgs a,
 
 // One CTA per chain at the state x = m_r (see the file comment).
 template <typename TJ, int NT>
-__global__ void __launch_bounds__(NT, kWbMinBlocks) k_wb_propose(ReducedArgs a) {
+__global__ void __launch_bounds__(NT, sizeof(TJ) == 4 ? 1024 / NT : kWbMinBlocks)
+    k_wb_propose(ReducedArgs a) {
   using A = std::conditional_t<sizeof(TJ) == 4, DF, F64>;
   using E = typename A::T;
   extern __shared__ __align__(16) double sm[];
@@ -822,7 +829,7 @@ cudaError_t launch_wb_geometry_k(const ReducedArgs &a, int mode, cudaStream_t st
 }
 
 // The in-place conversion of the staged Gram matrix (kPre) is safe when, at
-// every chunk boundary E (entries of 8 per thread of kWbPreThreads), the
+// every chunk boundary E (8 entries per thread of the CTA), the
 // double-float writes below it (bytes [0, 8E)) end at or below the staged
 // FP32 entry E, the first one not yet read.
 bool wb_pre_stage_fits(int dy, int ldg) {
@@ -830,7 +837,7 @@ bool wb_pre_stage_fits(int dy, int ldg) {
   const size_t gbytes = (size_t)dy * ldg * 4;
   if (gbytes > region || gbytes % 16) return false;
   const size_t S = region - gbytes;
-  const long ntri = (long)dy * (dy + 1) / 2, step = 8L * kWbPreThreads;
+  const long ntri = (long)dy * (dy + 1) / 2, step = 8L * wb_pre_threads(dy);
   for (long E = step; E < ntri; E += step) {
     long i = 0;
     while ((i + 1) * (i + 2) / 2 <= E) ++i;
@@ -843,16 +850,18 @@ bool wb_pre_stage_fits(int dy, int ldg) {
 template <typename TJ>
 cudaError_t launch_wb_geometry_t(const ReducedArgs &a, int mode, cudaStream_t st) {
   if constexpr (sizeof(TJ) == 4)
-    if (a.G && a.Kb_pre && wb_pre_stage_fits(a.d_y, a.ldg))
-      return launch_wb_geometry_k<TJ, true, kWbPreThreads>(a, mode, st);
+    if (a.G && a.Kb_pre && wb_pre_stage_fits(a.d_y, a.ldg)) {
+      const int nt = wb_pre_threads(a.d_y);
+      return nt == 64    ? launch_wb_geometry_k<TJ, true, 64>(a, mode, st)
+             : nt == 128 ? launch_wb_geometry_k<TJ, true, 128>(a, mode, st)
+                         : launch_wb_geometry_k<TJ, true, 256>(a, mode, st);
+    }
   return launch_wb_geometry_k<TJ, false, kWbThreads>(a, mode, st);
 }
 
-template <typename TJ>
-cudaError_t launch_wb_propose_t(const ReducedArgs &a, cudaStream_t st) {
+template <typename TJ, int NT>
+cudaError_t launch_wb_propose_k(const ReducedArgs &a, cudaStream_t st) {
   const size_t smem = WbLayout(a.r, a.d_y).tail * sizeof(double);
-  // the double-float path at 256 threads (64 registers, 32 warps per SM)
-  constexpr int NT = sizeof(TJ) == 4 ? kWbPreThreads : kWbThreads;
   cudaError_t e = cudaFuncSetAttribute(k_wb_propose<TJ, NT>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -860,6 +869,17 @@ cudaError_t launch_wb_propose_t(const ReducedArgs &a, cudaStream_t st) {
   b.derive();
   k_wb_propose<TJ, NT><<<a.C, NT, smem, st>>>(b);
   return cudaGetLastError();
+}
+
+template <typename TJ>
+cudaError_t launch_wb_propose_t(const ReducedArgs &a, cudaStream_t st) {
+  if constexpr (sizeof(TJ) == 4) {
+    const int nt = wb_pre_threads(a.d_y);
+    return nt == 64    ? launch_wb_propose_k<TJ, 64>(a, st)
+           : nt == 128 ? launch_wb_propose_k<TJ, 128>(a, st)
+                       : launch_wb_propose_k<TJ, 256>(a, st);
+  }
+  return launch_wb_propose_k<TJ, kWbThreads>(a, st);
 }
 
 }  // namespace
