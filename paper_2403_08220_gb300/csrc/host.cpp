@@ -528,20 +528,23 @@ struct Left64 {
   int g = 1, ldd = 0;
 };
 
-// Scratch for the digits of A: free device memory of the caller's.
+// Scratch for the digits of A: free device memory of the caller's, and the
+// pool's own for a single row, taken where the other does not hold one (a few
+// chains with few observations), so that no product changes its route, and
+// with it its last bits, with the number of chains.
 struct Scratch64 {
   void *p = nullptr;
   size_t bytes = 0;
   int *err = nullptr;
+  void *row = nullptr;
 };
+static size_t digit_row_bytes(int K) { return 16 * (size_t)digit_pitch(K) + 32; }
 
 // Bytes of A's digits worked on at a time: they are written and read again
 // while still in L2 (129 MB).
 constexpr size_t kDigitsChunk = 96u << 20;
 
-static bool has_digits(const DigitMat &B, const Scratch64 &ws, int K) {
-  return B.d && ws.p && ws.bytes >= 16 * (size_t)digit_pitch(K) + 16;
-}
+static bool has_digits(const DigitMat &B, const Scratch64 &ws) { return B.d && ws.p && ws.row; }
 
 // The product on the tensor cores in chunks of rows: digits of A into the
 // scratch, then tc(args) for those rows.
@@ -549,15 +552,17 @@ template <class Tc>
 static void digit_product(dino_ctx *ctx, cudaStream_t st, const char *name, int M, int N, int K,
                           const Left64 &a, const DigitMat &B, const Scratch64 &ws, Tc &&tc) {
   const int ldp = digit_pitch(K);
-  const size_t per = 16 * (size_t)ldp + 4;
-  size_t rows = std::min<size_t>({(size_t)M, (ws.bytes - 16) / per,
+  const size_t per = 16 * (size_t)ldp + 4, one = digit_row_bytes(K);
+  char *scratch = (char *)(ws.bytes >= one ? ws.p : ws.row);
+  const size_t bytes = std::max(ws.bytes, one);
+  size_t rows = std::min<size_t>({(size_t)M, (bytes - 16) / per,
                                   std::max<size_t>(128, kDigitsChunk / per)});
   if (rows < (size_t)M) {  // equal chunks of whole 128-row tiles
     const size_t n = ((size_t)M + rows - 1) / rows, even = ((size_t)M + n - 1) / n;
     const size_t up = (even + 127) / 128 * 128;
     rows = up <= rows ? up : (rows >= 128 ? rows / 128 * 128 : rows);
   }
-  auto *d = (__nv_bfloat16 *)ws.p;
+  auto *d = (__nv_bfloat16 *)scratch;
   const size_t plane = rows * ldp;
   int *ex = (int *)(d + plane * kDigits64);
   for (size_t r0 = 0; r0 < (size_t)M; r0 += rows) {
@@ -591,7 +596,7 @@ static void digit_product(dino_ctx *ctx, cudaStream_t st, const char *name, int 
 static void store64(dino_ctx *ctx, cudaStream_t st, const char *name, int M, int N, int K,
                     const double *A, int lda, const double *B, int ldb, const DigitMat &gB,
                     const Scratch64 &ws, double *out, int ldo) {
-  if (has_digits(gB, ws, K)) {
+  if (has_digits(gB, ws)) {
     Left64 l;
     l.A = A;
     l.lda = lda;
@@ -607,7 +612,7 @@ static void bias_act64(dino_ctx *ctx, cudaStream_t st, const char *name, int M, 
                        const double *A, int lda, const double *B, int ldb, const DigitMat &gB,
                        const Scratch64 &ws, const double *bias, int act, double *out, double *der,
                        int ldo) {
-  if (has_digits(gB, ws, K)) {
+  if (has_digits(gB, ws)) {
     Left64 l;
     l.A = A;
     l.lda = lda;
@@ -948,6 +953,7 @@ struct Work {
   std::vector<double *> act64, der64;
   double *f64 = nullptr, *P64[2] = {nullptr, nullptr}, *J64 = nullptr;
   size_t p_bytes = 0, j_bytes = 0;  // of each P64 (or Pb) and of J64
+  void *digit_row = nullptr;        // digits of one row of any FP64 product
   // tensor path
   __nv_bfloat16 *xb = nullptr;
   int ldx = 0;
@@ -1051,7 +1057,7 @@ static void eval_surrogate(dino_ctx *ctx, const Surrogate *s, Work &w, const dou
     const double *a = x;
     int lda = r;
     // digits of the forward pass's inputs in the Jacobian's buffers, not yet in use
-    const Scratch64 p0{w.P64[0], w.p_bytes, err};
+    const Scratch64 p0{w.P64[0], w.p_bytes, err, w.digit_row};
     for (int l = 0; l + 1 < L; ++l) {
       const int wo = s->widths[l + 1], wi = s->widths[l];
       bias_act64(ctx, st, "mlp_f64", C, wo, wi, a, lda, s->dW[l], wi, s->gW[l], p0, s->db[l],
@@ -1089,10 +1095,10 @@ static void eval_surrogate(dino_ctx *ctx, const Surrogate *s, Work &w, const dou
       double *out = last ? (fwd ? (double *)w.Jt : w.J64) : w.P64[1 - cur];
       // digits: in P[0] for the first product (it starts from W and d) and in
       // the other P for the last; in J, not yet in use, in between
-      const Scratch64 ws = q == 0 ? Scratch64{w.P64[0], w.p_bytes, err}
-                           : last ? Scratch64{w.P64[1 - cur], w.p_bytes, err}
-                                  : Scratch64{w.J64, w.j_bytes, err};
-      if (has_digits(gB, ws, K)) {
+      const Scratch64 ws = q == 0 ? p0
+                           : last ? Scratch64{w.P64[1 - cur], w.p_bytes, err, w.digit_row}
+                                  : Scratch64{w.J64, w.j_bytes, err, w.digit_row};
+      if (has_digits(gB, ws)) {
         Left64 lf;
         if (q == 0) {
           lf.W = W0;
@@ -1372,6 +1378,10 @@ static void layout_pool(Pool &p, bool assign) {
     p.coef2s = (__nv_bfloat16 *)take((size_t)C * s->ldD * kFieldSlices * 2);
   }
   layout_work(s, C, ar, p.w, assign, p.wb && s->tc_gram);
+  int kmax = N;
+  for (int x : s->widths) kmax = std::max(kmax, x);
+  for (int x : s->tm.widths) kmax = std::max(kmax, x);
+  if (s->L >= 2) p.w.digit_row = take(digit_row_bytes(kmax));
   p.da = s->tm.on;
   if (p.da) {
     const auto &t = s->tm;
@@ -1532,7 +1542,7 @@ static size_t pool_footprint(const Surrogate *s, int C);
 // product buffer.
 static Scratch64 pool_scratch(const Pool &p) {
   void *b = p.s->precision == DINO_PREC_FP64 ? (void *)p.w.P64[0] : (void *)p.w.Pb[0];
-  return Scratch64{b, b ? p.w.p_bytes : 0, p.err};
+  return Scratch64{b, b ? p.w.p_bytes : 0, p.err, p.w.digit_row};
 }
 
 // The true map f_t at the C points x_t = p.xt (FP64 path) or its slices
@@ -1813,7 +1823,7 @@ static void step_pool(dino_ctx *ctx, Pool &p) {
                                        p.da ? p.acc : nullptr);
     });
     const Scratch64 ws = pool_scratch(p);
-    if (has_digits(s->gE, ws, N)) {
+    if (has_digits(s->gE, ws)) {
       Left64 l;
       l.A = Mf;
       l.lda = N;
@@ -1826,7 +1836,7 @@ static void step_pool(dino_ctx *ctx, Pool &p) {
       });
     }
     if (p.da) da_stage(ctx, p, cs, st);
-    if (has_digits(s->gD, ws, r)) {
+    if (has_digits(s->gD, ws)) {
       Left64 l;
       l.A = coef2;
       l.lda = r;
@@ -2913,9 +2923,13 @@ int dino_chains_read(dino_ctx *ctx, int pool_id, double *m, double *m_r, double 
       if (p->s->precision == DINO_PREC_FP64) {
         CK(cudaMemcpy(m, p->m, (size_t)C * N * 8, cudaMemcpyDeviceToHost));
       } else {
-        std::vector<float> t((size_t)C * N);
-        CK(cudaMemcpy(t.data(), p->m, t.size() * 4, cudaMemcpyDeviceToHost));
-        for (size_t i = 0; i < t.size(); ++i) m[i] = t[i];
+        // widened on the device, in the prior draw's buffer (C N doubles, written
+        // anew by every transition)
+        launch(ctx, p->st, "field_out", [&] {
+          return launch_f32_to_f64((size_t)C * N, (const float *)p->m, (double *)p->Mf, p->st);
+        });
+        CK(cudaMemcpyAsync(m, p->Mf, (size_t)C * N * 8, cudaMemcpyDeviceToHost, p->st));
+        CK(cudaStreamSynchronize(p->st));
       }
     }
     if (m_r) CK(cudaMemcpy(m_r, p->mr, (size_t)C * r * 8, cudaMemcpyDeviceToHost));

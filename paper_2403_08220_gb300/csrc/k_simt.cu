@@ -458,6 +458,11 @@ cudaError_t launch_copy_f64(size_t n, const double *src, double *dst, cudaStream
   return cudaGetLastError();
 }
 
+cudaError_t launch_f32_to_f64(size_t n, const float *src, double *dst, cudaStream_t st) {
+  k_convert<float, double><<<grid_for(n), 256, 0, st>>>(n, src, dst);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_f64_to_f32(size_t n, const double *src, float *dst, cudaStream_t st) {
   k_convert<double, float><<<grid_for(n), 256, 0, st>>>(n, src, dst);
   return cudaGetLastError();
