@@ -361,8 +361,9 @@ int dino_dis_from_surrogate(dino_ctx *ctx, int surrogate_id, int n_samples, uint
  *     initial positive sequence (MACT(0) = 1, pairs MACT(2i) + MACT(2i+1) > 0);
  *     returned as a fraction;
  *   the Wasserstein MPSRF Tr(W + V - 2 (W^1/2 V W^1/2)^1/2) of the within-
- *     chain and pooled covariance estimators (eq:covariance_estimator), with
- *     the symmetric square roots from a one-sided Jacobi eigensolver
+ *     chain and pooled covariance estimators (eq:covariance_estimator), whose
+ *     last term is the nuclear norm of C^T F for V = C C^T, W = F F^T: from the
+ *     polar factor, or one-sided Jacobi where that is nearly singular
  *     (n_dof <= 1024);
  *   the mean squared jump MSJ = 1/(n_s - 1) sum_j |x_{j+1} - x_j|^2, averaged
  *     over chains (the acceptance rate comes with dino_chains_step's stats).
@@ -376,7 +377,7 @@ typedef struct {
   double msj;
   double mpsrf_w;        /* NaN unless requested */
   double trace_w, trace_v;
-  int jacobi_sweeps;     /* sweeps of the last eigensolve */
+  int jacobi_sweeps;     /* Jacobi sweeps of the MPSRF; 0 where it needed none */
 } dino_diag_result;
 
 /* Errors: EINVAL (n_chains < 2 or > 6144, n_dof < 1, max_samples < 2), ENOMEM. */

@@ -318,6 +318,16 @@ cudaError_t launch_col_norms(int d, const double *G, double *sig, cudaStream_t s
 // W = F F^T, V = C C^T (positive semidefinite, lower triangular factors)
 cudaError_t launch_psd_chol(int d, const double *W, const double *V, double *F, double *C,
                             cudaStream_t st);
+// Newton-Schulz on X = A / |A|_F, Y = X^T (d x d, FP64): P = (3 I - X^T X) / 2 with
+// *res, if given, = max |X^T X - I| (bits of a double, zero on entry); Y = P X^T, X2 = Y^T;
+// out[i] = sum_k Y[i][k] At[i][k], whose sum is tr(X^T A)
+cudaError_t launch_ns_start(int d, const double *At, double *Y, double *X, cudaStream_t st);
+cudaError_t launch_ns_poly(int d, const double *Y, double *P, unsigned long long *res,
+                           cudaStream_t st);
+cudaError_t launch_ns_update(int d, const double *P, const double *X, double *Y, double *X2,
+                             cudaStream_t st);
+cudaError_t launch_row_dots(int d, const double *Y, const double *At, double *out,
+                            cudaStream_t st);
 // G = C^T F by columns
 cudaError_t launch_ct_f(int d, const double *C, const double *F, double *G, cudaStream_t st);
 cudaError_t launch_mpsrf_final(int d, const double *W, const double *V, const double *sig,

@@ -84,5 +84,29 @@ struct EpiField {
   }
 };
 
+// Newton-Schulz: P = (3 I - S) / 2 from S = X^T X, and the largest |S - I| (as the
+// bits of a nonnegative double; a NaN is larger than every number) where res is
+// given
+struct EpiPoly {
+  double *P;
+  int ld;
+  unsigned long long *res;
+  __device__ void operator()(int r, int c, double v) const {
+    const double e = v - (r == c ? 1.0 : 0.0);
+    P[(size_t)r * ld + c] = (r == c ? 1.0 : 0.0) - 0.5 * e;
+    if (res) atomicMax(res, (unsigned long long)__double_as_longlong(fabs(e)));
+  }
+};
+
+// ... and the new Y = X^T = P X^T, kept both ways
+struct EpiBoth {
+  double *Y, *X;
+  int ld;
+  __device__ void operator()(int r, int c, double v) const {
+    Y[(size_t)r * ld + c] = v;
+    X[(size_t)c * ld + r] = v;
+  }
+};
+
 }  // namespace
 }  // namespace dino

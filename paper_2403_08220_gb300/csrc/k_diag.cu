@@ -20,6 +20,13 @@
 //                   Tr(W + V - 2 (W^1/2 V W^1/2)^1/2) is Tr W + Tr V - 2 |C^T F|_*
 //                   without a square root of W;
 //   k_ct_f          C^T F by columns;
+//   k_ns_start, k_row_dots  the nuclear norm |A|_* = tr(U^T A) of A = C^T F from its
+//                   polar factor U, the limit of the Newton-Schulz iteration
+//                   X <- X (3 I - X^T X) / 2 from A / |A|_F (two d x d products a
+//                   step, k_simt.cu).  Every singular value of X grows by up to
+//                   1.5 a step until it reaches 1, so about log_1.5(|A|_F /
+//                   sigma_min) + 5 steps do; where A is singular or nearly so
+//                   they do not, and the one-sided Jacobi below takes over;
 //   k_jacobi_round  one-sided Jacobi (Hestenes) on a d x d matrix held by
 //                   columns: column pairs are rotated until orthogonal; a
 //                   launch is one round of a round-robin over blocks of
@@ -529,6 +536,45 @@ cudaError_t launch_diag_center(int d, int n_c, int n_s, const double *traj, int 
 cudaError_t launch_diag_wv(int d, int n_c, int n_s, const double *Wr, const double *Br, double *W,
                            double *V, cudaStream_t st) {
   k_diag_wv<<<grid_for((size_t)d * d), 256, 0, st>>>(d, n_c, n_s, Wr, Br, W, V);
+  return cudaGetLastError();
+}
+
+// Y = A^T / |A|_F and X = Y^T, At = A^T row-major (one CTA: |A|_F first)
+__global__ void __launch_bounds__(1024)
+    k_ns_start(int d, const double *__restrict__ At, double *__restrict__ Y,
+               double *__restrict__ X) {
+  __shared__ double red[40];
+  double s = 0.0;
+  for (int e = threadIdx.x; e < d * d; e += blockDim.x) s += At[e] * At[e];
+  s = block_sum(s, red);
+  const double scale = 1.0 / sqrt(s);
+  for (int e = threadIdx.x; e < d * d; e += blockDim.x) {
+    const int i = e / d, j = e - i * d;
+    const double v = At[e] * scale;
+    Y[e] = v;
+    X[(size_t)j * d + i] = v;
+  }
+}
+
+// out[i] = sum_k Y[i][k] At[i][k]: a warp per row
+__global__ void k_row_dots(int d, const double *__restrict__ Y, const double *__restrict__ At,
+                           double *__restrict__ out) {
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (i >= d) return;
+  double s = 0.0;
+  for (int k = lane; k < d; k += 32) s += Y[(size_t)i * d + k] * At[(size_t)i * d + k];
+  s = warp_sum(s);
+  if (lane == 0) out[i] = s;
+}
+
+cudaError_t launch_ns_start(int d, const double *At, double *Y, double *X, cudaStream_t st) {
+  k_ns_start<<<1, 1024, 0, st>>>(d, At, Y, X);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_row_dots(int d, const double *Y, const double *At, double *out,
+                            cudaStream_t st) {
+  k_row_dots<<<(d + 7) / 8, 256, 0, st>>>(d, Y, At, out);
   return cudaGetLastError();
 }
 

@@ -334,6 +334,16 @@ cudaError_t gemm_field(int M, int N, int K, const T *A, int lda, const T *B, int
   return run_gemm(M, N, K, A, lda, B, ldb, EpiField<T>{acc_flag, s, c, m, Mf, ldm}, st);
 }
 
+cudaError_t launch_ns_poly(int d, const double *Y, double *P, unsigned long long *res,
+                           cudaStream_t st) {
+  return run_gemm(d, d, d, Y, d, Y, d, EpiPoly{P, d, res}, st);
+}
+
+cudaError_t launch_ns_update(int d, const double *P, const double *X, double *Y, double *X2,
+                             cudaStream_t st) {
+  return run_gemm(d, d, d, P, d, X, d, EpiBoth{Y, X2, d}, st);
+}
+
 // Tiles of 32 x 32 through shared memory (rows padded by one), so that reads
 // and writes are both along rows: HBM-bound (4096 blocks of 128 x 200 FP32, 839
 // MB: 361 us with strided reads, 168 us).

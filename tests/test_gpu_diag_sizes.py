@@ -102,3 +102,27 @@ def test_a_nan_sample_stays_in_its_degree_of_freedom(dino):
     assert np.array_equal(res[0]["ess"][keep], res[1]["ess"][keep])
     for k in ("msj", "trace_w", "trace_v", "mpsrf_w"):
         assert np.isfinite(res[0][k]) and np.isnan(res[1][k]), k
+
+
+@pytest.mark.parametrize("d,span,polar", [
+    (7, 2.0, False), (8, 2.0, True), (9, 4.0, True),   # from d = 8 on the polar factor
+    (61, 6.0, True), (257, 1.0, True), (512, 1.0, True), (513, 1.0, False),
+    (64, 26.0, False),    # scales down to 5e-12: the iteration gives up, Jacobi solves
+])
+def test_nuclear_norm_by_polar_factor_or_jacobi(dino, d, span, polar):
+    rng = np.random.default_rng(d)
+    n_c, n_s = 4, max(24, d)
+    X = rng.standard_normal((n_c, n_s, d)) + 0.3 * rng.standard_normal((n_c, 1, d))
+    X *= np.exp(-span * np.arange(d) / d)
+    ctx = dino.dino_init(0)
+    try:
+        g = dino.dino_diag_create(ctx, n_c, d, n_s)
+        for j in range(n_s):
+            dino.dino_diag_push(ctx, g, X[:, j, :])
+        out = dino.dino_diag_compute(ctx, g, d, mpsrf=True)
+    finally:
+        ctx.close()
+    W, V = dg.covariance_estimators(X)
+    assert (out["jacobi_sweeps"] == 0) == polar
+    tol = (1e-9 if span < 10 else 2e-8 * np.sqrt(d)) * np.trace(V)
+    assert abs(out["mpsrf_w"] - dg.wasserstein_mpsrf(W, V)) <= tol
