@@ -5,7 +5,7 @@
 //
 //   k_diag_record   appends one sample of every chain (from a pool's state or
 //                   a caller buffer);
-//   k_diag_ess      one CTA per degree of freedom: chain means and variances,
+//   k_diag_ess      a cluster of 1 to 8 CTAs per degree of freedom: chain means and variances,
 //                   w and v (the 1D covariance estimators), the multi-chain
 //                   autocorrelation MACT(t) = 1 - (w - mean_k AC(t,k)) / v in
 //                   passes of kLags lags until a pair sum is no longer positive
@@ -39,13 +39,19 @@
 //                   Jacobian of the surrogate-driven DIS basis (eq:mc_ppgnh),
 //                   whose eigenproblem the same Jacobi kernel solves.
 // Every loop is bounded by the sizes (lags by n_s, Jacobi sweeps by
-// kMaxJacobiSweeps); no kernel waits on another CTA.
+// kMaxJacobiSweeps); CTAs wait on one another only at the barriers of a cluster,
+// which all of its CTAs reach the same number of times (every CTA walks the same
+// MACT values).
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "chol.cuh"
 
 namespace dino {
 namespace {
+
+namespace cg = cooperative_groups;
 
 constexpr int kEssThreads = 256;
 
@@ -114,14 +120,18 @@ __device__ __forceinline__ double warp_sum8(const double v[8]) {
 }
 
 constexpr int kLags = 8;     // lags per pass over the samples
+constexpr int kEssMaxCluster = 8;  // CTAs that share a degree of freedom's lags
 constexpr int kSegment = 128;  // samples of one chain that a warp takes at a time
 
 // Dynamic shared memory: n_c chain means, then with kStaged the centred samples
-// (n_c x n_s).  A pass forms kLags lags: per sample one multiply-add for
-// each from consecutive shared-memory words, and one reduction per pass (one
-// pass per lag pair over global memory, with a division per sample to find
-// its chain, took 17.4 ms for 200 degrees of freedom, 10 chains of 1000
-// samples; 3.3 ms now, 1.6 ms at the FP64 pipes' rate for all 1000 lags).
+// (n_c x n_s).  A pass forms kLags lags in each CTA of the cluster: per sample
+// one multiply-add for each from consecutive shared-memory words, and one
+// reduction per pass.  The CTAs exchange MACT through each other's shared memory
+// and each walks the pairs in order.  Bound by the FP64 pipes; degrees of
+// freedom differ in their lags, up to all n_s.  (One pass per lag pair over
+// global memory, with a division per sample to find its chain, took 17.4 ms for
+// 200 degrees of freedom, 10 chains of 1000 samples, of which some run all 1000
+// lags; a CTA each 3.3 ms; clusters of four 1.84 ms.)
 // Lags past the first non-positive pair are formed and not used.
 template <bool kStaged>
 __global__ void __launch_bounds__(kEssThreads)
@@ -129,9 +139,12 @@ __global__ void __launch_bounds__(kEssThreads)
                double *__restrict__ means, double *__restrict__ ess, double *__restrict__ sqjump) {
   extern __shared__ double mk[];
   __shared__ double red[72], lagsum[kEssThreads / 32][kLags];
+  __shared__ double mact[2][kEssMaxCluster * kLags];  // a pass's MACT, by its parity
   __shared__ bool more_s;
   double *xs = mk + n_c;
-  const int i = blockIdx.x;
+  const cg::cluster_group cluster = cg::this_cluster();
+  const int cs = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  const int i = blockIdx.x / cs;
   const double *X = traj + (size_t)i * n_c * max_s;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   // chain means, within-chain sums of squares and squared jumps (warp per chain)
@@ -166,7 +179,9 @@ __global__ void __launch_bounds__(kEssThreads)
   double total = 0.0;
   int pairs = 0;
   bool more = true;
-  for (int t0 = 0; more && t0 + 1 < n_s; t0 += kLags) {
+  cluster.sync();  // every CTA runs before one writes into another's mact
+  for (int base = 0, buf = 0; more && base + 1 < n_s; base += cs * kLags, buf ^= 1) {
+    const int t0 = base + rank * kLags;
     double acc[kLags] = {};
     for (int it = warp; it < n_c * segs; it += nw) {
       const int k = it / segs, j0 = (it - k * segs) * kSegment;
@@ -191,18 +206,19 @@ __global__ void __launch_bounds__(kEssThreads)
     const double s = warp_sum8(acc);
     if (lane < kLags) lagsum[warp][lane] = s;
     __syncthreads();
-    if (warp == 0) {  // lane q: MACT(t0 + q); then the pairs in order
+    if (warp == 0 && lane < kLags) {  // MACT(t0 + lane), to every CTA
       double r = 0.0;
-      if (lane < kLags) {
-        for (int u = 0; u < nw; ++u) r += lagsum[u][lane];
-        r = t0 + lane == 0 ? 1.0 : 1.0 - (w - r * inv_n) * inv_v;
-      }
-      const double pair = r + __shfl_xor_sync(kFull, r, 1);
+      for (int u = 0; u < nw; ++u) r += lagsum[u][lane];
+      r = t0 + lane == 0 ? 1.0 : 1.0 - (w - r * inv_n) * inv_v;
+      for (int p = 0; p < cs; ++p)
+        *cluster.map_shared_rank(&mact[buf][rank * kLags + lane], p) = r;
+    }
+    cluster.sync();  // the other buffer is written until the next one
+    if (warp == 0) {  // the pairs in order
       bool on = true;
-#pragma unroll
-      for (int q = 0; q < kLags; q += 2) {
-        const double pq = __shfl_sync(kFull, pair, q);
-        on = on && t0 + q + 1 < n_s && pq > 0.0;
+      for (int q = 0; on && q < cs * kLags; q += 2) {
+        const double pq = mact[buf][q] + mact[buf][q + 1];
+        on = base + q + 1 < n_s && pq > 0.0;
         if (on) {
           total += pq;
           ++pairs;
@@ -213,6 +229,7 @@ __global__ void __launch_bounds__(kEssThreads)
     __syncthreads();
     more = more_s;
   }
+  if (rank) return;  // the last write into another CTA's memory came before a barrier
   if (threadIdx.x == 0) {
     ess[i] = pairs > 0 ? 1.0 / (2.0 * total - 1.0) : 1.0;
     sqjump[i] = jj;
@@ -514,16 +531,32 @@ cudaError_t launch_diag_ess(int d, int n_c, int n_s, const double *traj, int max
   if (n_c < 2 || n_s < 2 || (size_t)n_c * 8 > 48 * 1024) return cudaErrorInvalidValue;
   // the centred samples in shared memory where they fit (two CTAs an SM up to 14000)
   const size_t staged = ((size_t)n_c * n_s + n_c) * 8;
-  if (staged <= 200 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_diag_ess<true>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)staged);
-    if (e != cudaSuccess) return e;
-    k_diag_ess<true><<<d, kEssThreads, staged, st>>>(n_c, n_s, traj, max_s, means, ess, sqjump);
-  } else {
-    k_diag_ess<false><<<d, kEssThreads, (size_t)n_c * 8, st>>>(n_c, n_s, traj, max_s, means, ess,
-                                                               sqjump);
-  }
-  return cudaGetLastError();
+  const bool fits = staged <= 200 * 1024;
+  auto kernel = fits ? k_diag_ess<true> : k_diag_ess<false>;
+  // More CTAs for a degree of freedom while the chip (two CTAs an SM) has room: the
+  // slowest one, which may run all n_s lags, sets the time.  Each CTA of a cluster
+  // stages all samples and a pass forms 8 lags in each, so a cluster costs where
+  // the lags are few: 10 chains of 1000 samples, 1 / 2 / 4 / 8 CTAs, correlation
+  // 0.9: d = 8 0.51 / 0.31 / 0.21 / 0.16 ms, d = 200 1.23 / 0.85 / 0.70 / 0.77,
+  // d = 2000 3.80 / 3.61 / 4.74 / 6.95; correlation 0.5, d = 200: 0.25 / 0.25 /
+  // 0.35 / 0.65; 50 samples, d = 100: 0.08 / 0.09 / 0.09 / 0.13.
+  int cs = d * 8 <= 304 ? kEssMaxCluster : d * 4 <= 800 ? 4 : d <= 1000 ? 2 : 1;
+  while (cs > 1 && n_s < 64 * cs) cs /= 2;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = cs;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(d * cs);
+  cfg.blockDim = dim3(kEssThreads);
+  cfg.dynamicSmemBytes = fits ? staged : (size_t)n_c * 8;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)cfg.dynamicSmemBytes);
+  if (e != cudaSuccess) return e;
+  return cudaLaunchKernelEx(&cfg, kernel, n_c, n_s, traj, max_s, means, ess, sqjump);
 }
 
 cudaError_t launch_diag_center(int d, int n_c, int n_s, const double *traj, int max_s,
