@@ -226,14 +226,16 @@ size_t prior_draw_smem_bytes(int n, int elem);
 // (row pitch ldms, plane stride ms_plane) for the tensor-core projections.
 // With ext_z (C x N doubles, nullptr for Philox) the normals Z_c are the
 // caller's, indexed like the Philox ones.  With `only`, chains c with
-// only[c] == 0 draw nothing (their rows keep earlier contents).
+// only[c] == 0 draw nothing (their rows keep earlier contents).  With `overlap`
+// the draw may run while the kernel before it on the stream still does (pdl.cuh;
+// it stores after that kernel's end): sqrtlam, S and ext_z must not come from it.
 template <typename T>
 cudaError_t launch_prior_draw(int C, int n, const T *sqrtlam, const T *S, uint64_t seed,
                               uint64_t id_base, uint32_t stream, uint32_t step, T *out,
                               int ldo, cudaStream_t st,
                               __nv_bfloat16 *ms = nullptr, int ldms = 0, size_t ms_plane = 0,
                               int ms_slices = 0, const double *ext_z = nullptr,
-                              const int *only = nullptr);
+                              const int *only = nullptr, bool overlap = false);
 // P[(c d_y + i) w + k] = WL[i w + k] * der[c ldd + k]
 template <typename T>
 cudaError_t launch_jac_init(int C, int d_y, int w, const T *WL, const T *der, int ldd, T *P,

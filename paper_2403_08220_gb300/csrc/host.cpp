@@ -1820,7 +1820,7 @@ static void step_pool(dino_ctx *ctx, Pool &p) {
     launch(ctx, st, "prior_draw_f64", [&] {
       return launch_prior_draw<double>(C, s->n_grid, s->dSqrtLam, s->dS, p.seed, p.id_base,
                                        STREAM_Z_ID, p.step, Mf, N, st, nullptr, 0, 0, 0, ext_z,
-                                       p.da ? p.acc : nullptr);
+                                       p.da ? p.acc : nullptr, true);
     });
     const Scratch64 ws = pool_scratch(p);
     if (has_digits(s->gE, ws)) {
@@ -1856,7 +1856,7 @@ static void step_pool(dino_ctx *ctx, Pool &p) {
       return launch_prior_draw<float>(C, s->n_grid, s->fSqrtLam, s->fS, p.seed, p.id_base,
                                       STREAM_Z_ID, p.step, Mf, N, st, p.Ms, s->ldE,
                                       (size_t)C * s->ldE, kFieldSlices, ext_z,
-                                      p.da ? p.acc : nullptr);
+                                      p.da ? p.acc : nullptr, true);
     });
     launch(ctx, st, "field_coef_tc", [&] {
       // coef2 (C x r) = coef - cs M E^T, written as bf16 slices

@@ -22,6 +22,7 @@
 // state slot holds U (d_y x d_y, by columns), nu, u, v and t1 = |u|^2 - u^T v;
 // J at the state is kept in Js as on the perturbation-map path.
 #include "chol.cuh"
+#include "pdl.cuh"
 
 namespace dino {
 namespace {
@@ -207,6 +208,7 @@ __device__ void u_diag_ut(int d, int ld, const double *U, const double *f, const
 
 template <typename TJ, int NT, int E>
 __global__ void __launch_bounds__(NT) k_eig_geometry(ReducedArgs a, int mode) {
+  pdl_begin();
   extern __shared__ __align__(16) double sm[];
   const int c = blockIdx.x, r = a.r, dy = a.d_y;
   const EigLayout lay(r, dy);
@@ -348,6 +350,7 @@ __global__ void __launch_bounds__(NT) k_eig_geometry(ReducedArgs a, int mode) {
 
 template <typename TJ>
 __global__ void __launch_bounds__(kEigThreads) k_eig_propose(ReducedArgs a) {
+  pdl_begin();
   extern __shared__ __align__(16) double sm[];
   const int c = blockIdx.x, r = a.r, dy = a.d_y;
   const EigLayout lay(r, dy);
@@ -433,8 +436,7 @@ static cudaError_t eig_geometry(const ReducedArgs &a, int mode, cudaStream_t st)
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
-    kernel<<<a.C, threads, smem, st>>>(a, mode);
-    return cudaGetLastError();
+    return launch_pdl_n(chain_ctas(a.C), kernel, a.C, threads, smem, st, a, mode);
   };
   // entries per lane of a column pair: ceil(d_y / 4); 16 or 32 pairs of 4 lanes
   if (a.d_y <= 16) return go(k_eig_geometry<TJ, 64, 4>, 64);
@@ -448,18 +450,11 @@ cudaError_t launch_eig_geometry(const ReducedArgs &a, int mode, cudaStream_t st)
 
 cudaError_t launch_eig_propose(const ReducedArgs &a, cudaStream_t st) {
   const size_t smem = eig_smem_bytes(a.r, a.d_y);
-  if (a.jf_f32) {
-    cudaError_t e = cudaFuncSetAttribute(k_eig_propose<float>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k_eig_propose<float><<<a.C, kEigThreads, smem, st>>>(a);
-  } else {
-    cudaError_t e = cudaFuncSetAttribute(k_eig_propose<double>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k_eig_propose<double><<<a.C, kEigThreads, smem, st>>>(a);
-  }
-  return cudaGetLastError();
+  auto k = a.jf_f32 ? k_eig_propose<float> : k_eig_propose<double>;
+  const cudaError_t e =
+      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl_n(chain_ctas(a.C), k, a.C, kEigThreads, smem, st, a);
 }
 
 }  // namespace dino

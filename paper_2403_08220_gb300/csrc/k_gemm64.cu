@@ -48,6 +48,7 @@
 
 #include "dino_internal.h"
 #include "epi64.cuh"
+#include "pdl.cuh"
 #include "tcgen05.cuh"
 
 namespace dino {
@@ -91,6 +92,7 @@ __device__ __forceinline__ int exp_field(double x) {
 // 60 us against 37 us for 19456 rows of 400).
 template <int kQ>
 __global__ void __launch_bounds__(256) k_split64(const SplitArgs a) {
+  pdl_begin();
   const int lane = threadIdx.x & 31;
   const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (row >= a.rows) return;
@@ -345,6 +347,7 @@ __global__ void __launch_bounds__(kGemm64Threads, 1)
   __syncthreads();
   fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_begin();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -590,8 +593,7 @@ cudaError_t run_gemm64_t(const Gemm64Args &a, const Epi &epi, cudaStream_t st) {
   const int ntn = (a.N + BN - 1) / BN;
   const int tiles = kGram ? a.M / a.N * ((a.N + kBM - 1) / kBM) * ntn
                           : ((a.M + kBM - 1) / kBM) * ntn;
-  k<<<std::min(tiles, sms), kGemm64Threads, smem, st>>>(tmA, tmB, p, epi);
-  return cudaGetLastError();
+  return launch_pdl_n(tiles, k, std::min(tiles, sms), kGemm64Threads, smem, st, tmA, tmB, p, epi);
 }
 
 template <class Epi>
@@ -618,15 +620,9 @@ cudaError_t launch_split64(int rows, int K, const double *src, int ld, const dou
   if (K <= 0 || ldp < K || (ldp & 7) || (plane & 7)) return cudaErrorInvalidValue;
   SplitArgs a{rows, K, ldp, plane, src, ld, W, der, g, ldd, row0, fk, fsign, dst, ex};
   const int grid = (rows + 7) / 8;
-  if (ldp <= 128)
-    k_split64<1><<<grid, 256, 0, st>>>(a);
-  else if (ldp <= 256)
-    k_split64<2><<<grid, 256, 0, st>>>(a);
-  else if (ldp <= 512)
-    k_split64<4><<<grid, 256, 0, st>>>(a);
-  else
-    k_split64<0><<<grid, 256, 0, st>>>(a);
-  return cudaGetLastError();
+  auto k = ldp <= 128 ? k_split64<1> : ldp <= 256 ? k_split64<2> : ldp <= 512 ? k_split64<4>
+                                                                              : k_split64<0>;
+  return launch_pdl(k, grid, 256, 0, st, a);
 }
 
 cudaError_t launch_col_exp(int rows, int K, const double *B, int ld, int *fk, cudaStream_t st) {

@@ -36,6 +36,7 @@
 #include <algorithm>
 
 #include "chol_mma.cuh"
+#include "pdl.cuh"
 
 namespace dino {
 namespace {
@@ -129,6 +130,7 @@ struct Layout {
 // factor is read from its global slot (L2-resident while the chain is
 // processed), the vectors live in shared memory.
 __global__ void __launch_bounds__(kThreads) k_propose(ReducedArgs a) {
+  pdl_begin();
   extern __shared__ __align__(16) double sm[];
   __shared__ double blk[32 * 33];
   const int c = blockIdx.x, r = a.r;
@@ -238,6 +240,7 @@ __device__ __forceinline__ void warp_upper_solve2(const double *__restrict__ L, 
 
 template <int S>
 __global__ void __launch_bounds__(32 * kPropWarps) k_propose_warp(ReducedArgs a) {
+  pdl_begin();
   __shared__ double xi_s[kPropWarps][32 * S];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int c = blockIdx.x * kPropWarps + w;
@@ -317,6 +320,7 @@ constexpr int kGramB = 64, kGramK = 32, kGramThreads = 128;
 constexpr int kGramFlush = 64;  // rows per FP32 partial sum
 
 __global__ void __launch_bounds__(kGramThreads, 4) k_gram_f32(ReducedArgs a, int mode) {
+  pdl_begin();
   __shared__ __align__(16) float stage[2][kGramK][2 * kGramB];
   const int c = blockIdx.y, r = a.r, dy = a.d_y;
   int bi, bj;  // block row and column, bj <= bi
@@ -433,6 +437,7 @@ __global__ void __launch_bounds__(NT, sizeof(TJ) == 4 && !kBlk
                                           ? 1024 / NT
                                           : (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
     k_geometry(ReducedArgs a, int mode, int panel) {
+  pdl_begin();
   // FP32 Jacobian (tensor-core path): double-float Cholesky; FP64 Jacobian: FP64
   using A = std::conditional_t<sizeof(TJ) == 4, DF, F64>;
   using E = typename A::T;
@@ -626,20 +631,16 @@ size_t geometry_smem_bytes(int r, int d_y, int jf_f32) {
 cudaError_t launch_propose(const ReducedArgs &a, cudaStream_t st) {
   if (a.r <= 32 * 7) {
     const int grid = (a.C + kPropWarps - 1) / kPropWarps;
-    if (a.r <= 32 * 2)
-      k_propose_warp<2><<<grid, 32 * kPropWarps, 0, st>>>(a);
-    else if (a.r <= 32 * 4)
-      k_propose_warp<4><<<grid, 32 * kPropWarps, 0, st>>>(a);
-    else
-      k_propose_warp<7><<<grid, 32 * kPropWarps, 0, st>>>(a);
-    return cudaGetLastError();
+    auto k = a.r <= 32 * 2   ? k_propose_warp<2>
+             : a.r <= 32 * 4 ? k_propose_warp<4>
+                             : k_propose_warp<7>;
+    return launch_pdl(k, grid, 32 * kPropWarps, 0, st, a);
   }
   const size_t smem = propose_smem_bytes(a.r);
   cudaError_t e =
       cudaFuncSetAttribute(k_propose, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_propose<<<a.C, kThreads, smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_pdl_n(chain_ctas(a.C), k_propose, a.C, kThreads, smem, st, a);
 }
 
 // r from which the smem-resident factor of an FP32 Jacobian takes the blocked
@@ -673,8 +674,7 @@ static cudaError_t launch_geometry_nt(const ReducedArgs &a, int mode, size_t sme
   auto k = k_geometry<TJ, G, NT, kBlk>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k<<<a.C, NT, smem, st>>>(a, mode, panel);
-  return cudaGetLastError();
+  return launch_pdl_n(chain_ctas(a.C), k, a.C, NT, smem, st, a, mode, panel);
 }
 
 // CTA size: smaller CTAs let more chains share an SM (the kernel's loops stride
@@ -714,8 +714,8 @@ cudaError_t launch_gram_f32(const ReducedArgs &a, int mode, cudaStream_t st) {
     b.cur = a.cur + o;
     b.L = a.L + o * slot_stride(a.r);
     b.J = reinterpret_cast<const float *>(a.J) + o * a.d_y * a.r;
-    k_gram_f32<<<dim3(nb * (nb + 1) / 2, b.C), kGramThreads, 0, st>>>(b, mode);
-    const cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_pdl(k_gram_f32, dim3(nb * (nb + 1) / 2, b.C), kGramThreads, 0, st, b,
+                                     mode);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

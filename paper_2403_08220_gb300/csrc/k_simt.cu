@@ -8,6 +8,7 @@
 
 #include "dino_internal.h"
 #include "epi64.cuh"
+#include "pdl.cuh"
 #include "philox.cuh"
 
 namespace dino {
@@ -28,9 +29,11 @@ constexpr int kGemmThreads = 256;
 
 template <typename T, int kT, int kKG, class Epi>
 __global__ void __launch_bounds__(kGemmThreads)
-    k_gemm(int M, int N, int K, const T *__restrict__ A, int lda, const T *__restrict__ B,
-           int ldb, Epi epi) {
+    k_gemm(int M, int N, int K, const T *A, int lda, const T *B, int ldb, Epi epi) {
   static_assert(kT * kT * kKG == kGemmThreads, "one output per kKG threads");
+  pdl_begin();
+  A = pdl_after(A);
+  B = pdl_after(B);
   __shared__ T out[kT * kT];
   const int o = threadIdx.x / kKG, q = threadIdx.x % kKG;
   const int row0 = blockIdx.x * kT, col0 = blockIdx.y * kT;
@@ -40,10 +43,10 @@ __global__ void __launch_bounds__(kGemmThreads)
   int k = q;
 #pragma unroll 4
   for (; k + kKG < K; k += 2 * kKG) {
-    s0 += a[k] * b[k];
-    s1 += a[k + kKG] * b[k + kKG];
+    s0 += __ldg(a + k) * __ldg(b + k);
+    s1 += __ldg(a + k + kKG) * __ldg(b + k + kKG);
   }
-  if (k < K) s0 += a[k] * b[k];
+  if (k < K) s0 += __ldg(a + k) * __ldg(b + k);
   s0 += s1;
 #pragma unroll
   for (int w = kKG / 2; w; w >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, w);
@@ -61,12 +64,11 @@ cudaError_t run_gemm(int M, int N, int K, const T *A, int lda, const T *B, int l
   if (M <= 0 || N <= 0) return cudaSuccess;
   if (K > 256) {  // long reductions: 16 threads per output, 4 x 4 tiles
     dim3 grid((M + 3) / 4, (N + 3) / 4);
-    k_gemm<T, 4, 16, Epi><<<grid, kGemmThreads, 0, st>>>(M, N, K, A, lda, B, ldb, epi);
+    return launch_pdl(k_gemm<T, 4, 16, Epi>, grid, kGemmThreads, 0, st, M, N, K, A, lda, B, ldb, epi);
   } else {
     dim3 grid((M + 7) / 8, (N + 7) / 8);
-    k_gemm<T, 8, 4, Epi><<<grid, kGemmThreads, 0, st>>>(M, N, K, A, lda, B, ldb, epi);
+    return launch_pdl(k_gemm<T, 8, 4, Epi>, grid, kGemmThreads, 0, st, M, N, K, A, lda, B, ldb, epi);
   }
-  return cudaGetLastError();
 }
 
 // Prior draw: one CTA per chain; X = sqrt(Lambda) .* Z (spectral), Y = X S,
@@ -134,7 +136,10 @@ __global__ void __launch_bounds__(kPriorThreads, sizeof(T) == 4 ? 4 : 2)
                  uint64_t id_base, uint32_t stream, uint32_t step, T *out, int ldo,
                  __nv_bfloat16 *ms, int ldms, size_t ms_plane, int ms_slices,
                  const double *__restrict__ ext_z, const int *__restrict__ only) {
-  if (only && !only[blockIdx.x]) return;  // the whole CTA: this chain draws nothing
+  if (only) {
+    pdl_wait();
+    if (!only[blockIdx.x]) return;  // the whole CTA: this chain draws nothing
+  }
   extern __shared__ __align__(16) unsigned char smraw[];
   const int ld = prior_ld(n), nt = ld / 4, NN = ld * ld;
   const int h = (n + 1) / 2, ht = (h + 3) / 4;  // nodes formed, and their tiles
@@ -247,6 +252,7 @@ __global__ void __launch_bounds__(kPriorThreads, sizeof(T) == 4 ? 4 : 2)
     }
   }
   __syncthreads();
+  pdl_begin();  // the draw needs nothing of the kernels before; its outputs may be in use
   T *o = out + (size_t)c * ldo;
   for (int e = threadIdx.x; e < N; e += blockDim.x) {
     const T v = Mo[e];
@@ -267,8 +273,10 @@ __global__ void __launch_bounds__(kPriorThreads, sizeof(T) == 4 ? 4 : 2)
 }
 
 template <typename T>
-__global__ void k_jac_init(int C, int d_y, int w, const T *__restrict__ WL,
-                           const T *__restrict__ der, int ldd, T *__restrict__ P) {
+__global__ void k_jac_init(int C, int d_y, int w, const T *__restrict__ WL, const T *der, int ldd,
+                           T *__restrict__ P) {
+  pdl_begin();
+  der = pdl_after(der);
   const size_t total = (size_t)C * d_y * w;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total;
        e += (size_t)gridDim.x * blockDim.x) {
@@ -276,7 +284,7 @@ __global__ void k_jac_init(int C, int d_y, int w, const T *__restrict__ WL,
     const int k = (int)(e % w);
     const size_t c = row / d_y;
     const int i = (int)(row % d_y);
-    P[e] = WL[(size_t)i * w + k] * der[c * ldd + k];
+    P[e] = WL[(size_t)i * w + k] * __ldg(der + c * ldd + k);
   }
 }
 
@@ -349,7 +357,9 @@ cudaError_t launch_ns_update(int d, const double *P, const double *X, double *Y,
 // MB: 361 us with strided reads, 168 us).
 template <typename T>
 __global__ void __launch_bounds__(256)
-    k_batched_transpose(int a, int b, const T *__restrict__ src, T *__restrict__ dst) {
+    k_batched_transpose(int a, int b, const T *src, T *__restrict__ dst) {
+  pdl_begin();
+  src = pdl_after(src);
   __shared__ T tile[32][33];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int nb = (b + 31) / 32;
@@ -357,7 +367,7 @@ __global__ void __launch_bounds__(256)
   const size_t off = (size_t)blockIdx.y * a * b;
 #pragma unroll
   for (int k = 0; k < 32; k += 8)
-    if (i0 + ty + k < a && j0 + tx < b) tile[ty + k][tx] = src[off + (size_t)(i0 + ty + k) * b + j0 + tx];
+    if (i0 + ty + k < a && j0 + tx < b) tile[ty + k][tx] = __ldg(src + off + (size_t)(i0 + ty + k) * b + j0 + tx);
   __syncthreads();
 #pragma unroll
   for (int k = 0; k < 32; k += 8)
@@ -370,13 +380,11 @@ cudaError_t launch_batched_transpose(int C, int a, int b, const void *src, int f
   const size_t blk = (size_t)a * b;
   for (int c0 = 0; c0 < C; c0 += 65535) {  // the grid's second dimension ends there
     const dim3 grid(((a + 31) / 32) * ((b + 31) / 32), std::min(65535, C - c0));
-    if (f32)
-      k_batched_transpose<float><<<grid, 256, 0, st>>>(a, b, (const float *)src + c0 * blk,
-                                                       (float *)dst + c0 * blk);
-    else
-      k_batched_transpose<double><<<grid, 256, 0, st>>>(a, b, (const double *)src + c0 * blk,
-                                                        (double *)dst + c0 * blk);
-    const cudaError_t e = cudaGetLastError();
+    const cudaError_t e =
+        f32 ? launch_pdl(k_batched_transpose<float>, grid, 256, 0, st, a, b,
+                         (const float *)src + c0 * blk, (float *)dst + c0 * blk)
+            : launch_pdl(k_batched_transpose<double>, grid, 256, 0, st, a, b,
+                         (const double *)src + c0 * blk, (double *)dst + c0 * blk);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -438,13 +446,19 @@ template <typename T>
 cudaError_t launch_prior_draw(int C, int n, const T *sqrtlam, const T *S, uint64_t seed,
                               uint64_t id_base, uint32_t stream, uint32_t step, T *out, int ldo,
                               cudaStream_t st, __nv_bfloat16 *ms, int ldms, size_t ms_plane,
-                              int ms_slices, const double *ext_z, const int *only) {
+                              int ms_slices, const double *ext_z, const int *only,
+                              bool overlap) {
   if (C <= 0) return cudaSuccess;
   if (ms && (sizeof(T) != 4 || ms_slices < 1 || ldms < n * n)) return cudaErrorInvalidValue;
   const size_t smem = prior_draw_smem_bytes(n, (int)sizeof(T));
   cudaError_t e = cudaFuncSetAttribute(k_prior_draw<T>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
+  // beside the geometry kernel: 64 chains, n = 65, 19 us of 317 hidden
+  if (overlap)
+    return launch_pdl_n(chain_ctas(C), k_prior_draw<T>, C, kPriorThreads, smem, st, n, sqrtlam, S,
+                        seed, id_base, stream, step, out, ldo, ms, ldms, ms_plane, ms_slices, ext_z,
+                        only);
   k_prior_draw<T><<<C, kPriorThreads, smem, st>>>(n, sqrtlam, S, seed, id_base, stream, step, out,
                                                   ldo, ms, ldms, ms_plane, ms_slices, ext_z, only);
   return cudaGetLastError();
@@ -453,8 +467,8 @@ cudaError_t launch_prior_draw(int C, int n, const T *sqrtlam, const T *S, uint64
 template <typename T>
 cudaError_t launch_jac_init(int C, int d_y, int w, const T *WL, const T *der, int ldd, T *P,
                             cudaStream_t st) {
-  k_jac_init<T><<<grid_for((size_t)C * d_y * w), 256, 0, st>>>(C, d_y, w, WL, der, ldd, P);
-  return cudaGetLastError();
+  return launch_pdl(k_jac_init<T>, grid_for((size_t)C * d_y * w), 256, 0, st, C, d_y, w, WL, der, ldd,
+                    P);
 }
 
 template <typename T>
@@ -500,7 +514,7 @@ template cudaError_t launch_broadcast<double>(int, size_t, const double *, doubl
   template cudaError_t launch_prior_draw<T>(int, int, const T *, const T *, uint64_t,         \
                                             uint64_t, uint32_t, uint32_t, T *, int,           \
                                             cudaStream_t, __nv_bfloat16 *, int, size_t, int, \
-                                            const double *, const int *);
+                                            const double *, const int *, bool);
 DINO_INST_DRAW(double)
 DINO_INST_DRAW(float)
 

@@ -34,6 +34,7 @@
 #include <cstring>
 
 #include "dino_internal.h"
+#include "pdl.cuh"
 #include "tcgen05.cuh"
 
 namespace dino {
@@ -227,6 +228,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_begin();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -661,6 +663,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_begin();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -803,10 +806,13 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 // Split-K finish of TC_EPI_COEF: out slices = coef - cs * (sum of the K
 // chunks' FP32 partials), in chunk order.
-__global__ void k_coef_finish(uint32_t total, int N, int ksplit, const float *__restrict__ ws,
-                              const double *__restrict__ coef, int ldc, double cs,
-                              __nv_bfloat16 *__restrict__ out, int ldo, size_t plane,
-                              int nslice) {
+__global__ void k_coef_finish(uint32_t total, int N, int ksplit, const float *ws,
+                              const double *coef, int ldc, double cs,
+                              __nv_bfloat16 *__restrict__ out, int ldo,
+                              size_t plane, int nslice) {
+  pdl_begin();
+  ws = pdl_after(ws);
+  coef = pdl_after(coef);
   for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += gridDim.x * blockDim.x) {
     const uint32_t row = e / (uint32_t)N, col = e - row * (uint32_t)N;
@@ -817,8 +823,10 @@ __global__ void k_coef_finish(uint32_t total, int N, int ksplit, const float *__
   }
 }
 
-__global__ void k_split_bf16(int rows, int cols, const double *__restrict__ src, int lds,
+__global__ void k_split_bf16(int rows, int cols, const double *src, int lds,
                              __nv_bfloat16 *__restrict__ dst, int ldd, size_t plane, int nslice) {
+  pdl_begin();
+  src = pdl_after(src);
   const size_t total = (size_t)rows * cols;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total;
        e += (size_t)gridDim.x * blockDim.x) {
@@ -829,9 +837,10 @@ __global__ void k_split_bf16(int rows, int cols, const double *__restrict__ src,
 }
 
 __global__ void k_jac_init_bf16(int C, int d_y, int w, const float *__restrict__ WL,
-                                const float *__restrict__ der, int ldd,
-                                __nv_bfloat16 *__restrict__ P, int ldp, size_t plane,
-                                int nslice) {
+                                const float *der, int ldd, __nv_bfloat16 *__restrict__ P, int ldp,
+                                size_t plane, int nslice) {
+  pdl_begin();
+  der = pdl_after(der);
   // P = W_L .* der (per chain).  Work items are groups of 8 consecutive
   // columns of one row (c, i), enumerated row-major over all rows, so that
   // consecutive threads write consecutive 16-byte pieces and every thread
@@ -1059,14 +1068,13 @@ cudaError_t launch_tc_gemm(const TcGemmArgs &a, cudaStream_t st) {
   cudaError_t e =
       cudaFuncSetAttribute(k_tc_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_tc_gemm<<<std::min(total * p.ksplit, sms), kThreads, smem, st>>>(tmA, tmB, tmO, tmS, p);
-  cudaError_t e2 = cudaGetLastError();
+  const cudaError_t e2 = launch_pdl_n((long)total * p.ksplit, k_tc_gemm, std::min(total * p.ksplit, sms), kThreads, smem, st,
+                                    tmA, tmB, tmO, tmS, p);
   if (e2 != cudaSuccess || p.ksplit == 1) return e2;
   const size_t n = (size_t)a.M * a.N;
   const int grid = (int)std::min<size_t>((n + 255) / 256, 152 * 32);
-  k_coef_finish<<<grid, 256, 0, st>>>((uint32_t)n, a.N, p.ksplit, p.ws, a.coef, a.ldc, a.cs,
-                                      a.out_bf, a.ldo, a.out_plane, a.out_slices);
-  return cudaGetLastError();
+  return launch_pdl(k_coef_finish, grid, 256, 0, st, (uint32_t)n, a.N, p.ksplit, p.ws, a.coef, a.ldc,
+                    a.cs, a.out_bf, a.ldo, a.out_plane, a.out_slices);
 }
 
 cudaError_t launch_tc_gram(int C, int g, int K, const __nv_bfloat16 *J, int ldj, size_t plane,
@@ -1112,8 +1120,7 @@ cudaError_t launch_tc_gram(int C, int g, int K, const __nv_bfloat16 *J, int ldj,
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
     return cudaErrorInvalidValue;
-  k_tc_gram<<<std::min((C + p.batch - 1) / p.batch, sms), kThreads, smem, st>>>(tm, p);
-  return cudaGetLastError();
+  return launch_pdl_n(C / p.batch, k_tc_gram, std::min((C + p.batch - 1) / p.batch, sms), kThreads, smem, st, tm, p);
 }
 
 cudaError_t launch_split_bf16_f64(int rows, int cols, const double *src, int lds,
@@ -1121,8 +1128,8 @@ cudaError_t launch_split_bf16_f64(int rows, int cols, const double *src, int lds
                                   cudaStream_t st) {
   const size_t n = (size_t)rows * cols;
   const int grid = (int)std::min<size_t>((n + 255) / 256, 152 * 32);
-  k_split_bf16<<<grid > 0 ? grid : 1, 256, 0, st>>>(rows, cols, src, lds, dst, ldd, plane, nslice);
-  return cudaGetLastError();
+  return launch_pdl(k_split_bf16, grid > 0 ? grid : 1, 256, 0, st, rows, cols, src, lds, dst, ldd,
+                    plane, nslice);
 }
 
 cudaError_t launch_jac_init_bf16(int C, int d_y, int w, const float *WL, const float *der,
@@ -1131,9 +1138,8 @@ cudaError_t launch_jac_init_bf16(int C, int d_y, int w, const float *WL, const f
   const size_t items = (size_t)C * d_y * ((w + 7) / 8);  // 8 columns per thread
   if (items >= 0xffffffffull - 152ull * 16 * 256) return cudaErrorInvalidValue;
   const int grid = (int)std::min<size_t>((items + 255) / 256, 152 * 16);
-  k_jac_init_bf16<<<grid > 0 ? grid : 1, 256, 0, st>>>(C, d_y, w, WL, der, ldd, P, ldp, plane,
-                                                       nslice);
-  return cudaGetLastError();
+  return launch_pdl(k_jac_init_bf16, grid > 0 ? grid : 1, 256, 0, st, C, d_y, w, WL, der, ldd, P, ldp,
+                    plane, nslice);
 }
 
 }  // namespace dino

@@ -32,6 +32,7 @@
 // The tensor-core path (FP32 J) computes in double-float arithmetic on the
 // FP32 pipe, the FP64 path in FP64.
 #include "chol.cuh"
+#include "pdl.cuh"
 
 namespace dino {
 namespace {
@@ -370,6 +371,7 @@ __device__ void wb_store_factor(double *Lg, const typename A::T *Ms, const typen
 template <typename TJ, bool kPre, int NT>
 __global__ void __launch_bounds__(NT, kPre ? 1024 / NT : kWbMinBlocks)
     k_wb_geometry(ReducedArgs a, int mode) {
+  pdl_begin();
   using A = std::conditional_t<sizeof(TJ) == 4, DF, F64>;
   using E = typename A::T;
   static_assert(sizeof(E) == sizeof(double), "one factor element per double of the slot");
@@ -599,6 +601,7 @@ __global__ void __launch_bounds__(NT, kPre ? 1024 / NT : kWbMinBlocks)
 template <typename TJ, int NT>
 __global__ void __launch_bounds__(NT, sizeof(TJ) == 4 ? 1024 / NT : kWbMinBlocks)
     k_wb_propose(ReducedArgs a) {
+  pdl_begin();
   using A = std::conditional_t<sizeof(TJ) == 4, DF, F64>;
   using E = typename A::T;
   extern __shared__ __align__(16) double sm[];
@@ -824,8 +827,7 @@ cudaError_t launch_wb_geometry_k(const ReducedArgs &a, int mode, cudaStream_t st
   if (e != cudaSuccess) return e;
   ReducedArgs b = a;
   b.derive();
-  k_wb_geometry<TJ, kPre, NT><<<a.C, NT, smem, st>>>(b, mode);
-  return cudaGetLastError();
+  return launch_pdl_n(chain_ctas(a.C), k_wb_geometry<TJ, kPre, NT>, a.C, NT, smem, st, b, mode);
 }
 
 // The in-place conversion of the staged Gram matrix (kPre) is safe when, at
@@ -867,8 +869,7 @@ cudaError_t launch_wb_propose_k(const ReducedArgs &a, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   ReducedArgs b = a;
   b.derive();
-  k_wb_propose<TJ, NT><<<a.C, NT, smem, st>>>(b);
-  return cudaGetLastError();
+  return launch_pdl_n(chain_ctas(a.C), k_wb_propose<TJ, NT>, a.C, NT, smem, st, b);
 }
 
 template <typename TJ>
