@@ -488,17 +488,18 @@ int dino_kernel_times(dino_ctx *ctx, char *names, double *total_ms, uint64_t *la
  * It is meant for host code that must not call cudaMalloc: for example a
  * plugin inside a framework that owns every device byte through its own
  * pool, or a latency-critical loop in which the synchronisation that
- * cudaMalloc/cudaFree can imply is not acceptable.  The intermediate
- * d_y x width products live in a fixed device array of
+ * cudaMalloc/cudaFree can imply is not acceptable.  The layers'
+ * activations and derivatives live in a fixed device array of
  * DINO_NOALLOC_SCRATCH_DOUBLES doubles (8 MiB) that every GPU loading the
- * library keeps until the process exits.
+ * library keeps until the process exits; the rows of the Jacobian's products
+ * in shared memory.
  *
  * widths: host array of n_layers + 1 entries (widths[0] = r, widths[n_layers]
  *   = d_y), 1 <= n_layers <= 16; activation as in dino_surrogate_desc.
  * W, b: host arrays of n_layers DEVICE pointers; W[l] is widths[l+1] x
  *   widths[l] row-major, b[l] has widths[l+1] entries.
  * x: device, n x r; f: device, n x d_y; J: device, n x d_y x r (row-major).
- *   All buffers belong to the caller; results are written before the kernel
+ *   All buffers belong to the caller; results are written before the last kernel
  *   ends on `stream` (a cudaStream_t, or NULL for the legacy default stream).
  * Limit: n * 2 * d_y * (largest hidden width) must not exceed
  *   DINO_NOALLOC_SCRATCH_DOUBLES, and the activations must fit in 200 KB of
@@ -509,7 +510,7 @@ int dino_kernel_times(dino_ctx *ctx, char *names, double *total_ms, uint64_t *la
  *   before any stream capture on the device.
  * Every call shares the one array: calls whose kernels can overlap on the GPU
  *   (unordered streams) race on it, so order them on one stream.
- * Returns DINO_OK once the kernel is queued, DINO_ECUDA if the launch fails. */
+ * Returns DINO_OK once the kernels are queued, DINO_ECUDA if a launch fails. */
 #define DINO_NOALLOC_SCRATCH_DOUBLES (1u << 20)
 
 int dino_surrogate_jacobian_noalloc(int n, int n_layers, const int *widths, int activation,

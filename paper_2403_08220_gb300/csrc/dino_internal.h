@@ -1,5 +1,5 @@
 // Internal interfaces between the host runtime (host.cpp) and the kernels.
-// Every launcher issues exactly one kernel on the given stream.
+// Every launcher issues its kernel or kernels on the given stream.
 #pragma once
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
