@@ -349,51 +349,74 @@ struct PanelAt {
 // Factor the 8 x 8 diagonal block at kb (size nb) by one warp, in registers.
 // Lane 4 i + s holds the entries (i, s) and (i, s + 4) of the lower block;
 // rows and columns >= nb are padded with the identity, which leaves the rows
-// < nb unchanged and is never stored.  Column q: every lane takes the pivot
-// A::pivot of the broadcast diagonal entry, the owners of column q scale it,
-// and each entry (i, k), q < k <= i, takes the rank-1 update with the scaled
-// values of rows i and k fetched by shuffles.  The arithmetic per entry is the
-// column-at-a-time sequence; inv[k] = 1 / L_kk, and lsc (packed, 8 x 8)
-// receives the strictly lower block scaled by row, L_ij / L_ii.
-template <class A, class At>
+// < nb unchanged and is never stored.  With kUpd the block first takes the
+// rank-8 update by the panel at kp, A_ij -= sum_{k < 8} L_{i,kp+k} L_{j,kp+k}.
+// Column q: every lane takes the pivot A::pivot of the broadcast diagonal
+// entry, and each entry (i, k), q < k <= i, the rank-1 update with the scaled
+// values of rows i and k.  The arithmetic per entry is the column-at-a-time
+// sequence; inv[k] = 1 / L_kk, and lsc (packed, 8 x 8) receives the strictly
+// lower block scaled by row, L_ij / L_ii.
+//
+// This is the serial path of the factorisation, all latency: the values of
+// column q are fetched by shuffles while the pivot is formed and scaled by
+// every lane that uses them, and entries are chosen by selects, not branches.
+// (One chain an SM, d_y = 100, cycles a panel: update 1850 and factor 3650 of
+// 10,800 before, with the corner's 36 entries over 32 lanes; geometry of 64
+// chains 89 -> 70 us, of 4096 at r = 128 1.60 -> 1.52 ms.)
+template <class A, bool kUpd, class At>
 __device__ __noinline__ void warp_factor_diag(At Ls, typename A::T *inv, int kb, int nb, int lane,
-                                              typename A::T *lsc) {
+                                              typename A::T *lsc, int kp = 0) {
   using E = typename A::T;
   const int i = lane >> 2, s = lane & 3;
   const E one = A::from_j(1.0f);
-  E c0 = E{}, c1 = E{};  // (i, s) and (i, s + 4)
-  E id_i = one;          // 1 / L_ii of this lane's row
-  if (s <= i) c0 = i < nb ? Ls(kb + i, kb + s) : (i == s ? one : E{});
-  if (s + 4 <= i) c1 = i < nb ? Ls(kb + i, kb + s + 4) : (i == s + 4 ? one : E{});
+  const int ri = kb + min(i, nb - 1), rs = kb + min(s, nb - 1), rs4 = kb + min(s + 4, nb - 1);
+  const bool in0 = s <= i, in1 = s + 4 <= i;  // entries of the lower block
+  // (i, s) and (i, s + 4); outside the lower block any value of it, never used
+  E c0 = Ls(ri, min(rs, ri)), c1 = Ls(ri, min(rs4, ri));
+  E id_i = one;  // 1 / L_ii of this lane's row
+  if constexpr (kUpd) {
+    typename A::Acc a0 = A::begin(c0), a1 = A::begin(c1);
+    const E *x = &Ls(ri, kp), *y0 = &Ls(rs, kp), *y1 = &Ls(rs4, kp);
+#pragma unroll
+    for (int k = 0; k < kNB; ++k) {
+      A::sub(a0, x[k], y0[k]);
+      A::sub(a1, x[k], y1[k]);
+    }
+    c0 = A::end(a0);
+    c1 = A::end(a1);
+  }
+  if (i >= nb) {
+    c0 = i == s ? one : E{};
+    c1 = i == s + 4 ? one : E{};
+  }
 #pragma unroll
   for (int q = 0; q < kNB; ++q) {
     const int sq = q & 3;
     E &own = q < 4 ? c0 : c1;  // this lane's entry in column q, if any
+    E uiq = shfl_elt(own, 4 * i + sq), us = uiq, us4 = uiq;  // A_iq, A_sq, A_{s+4,q}
+    if (q < 3) us = shfl_elt(own, 4 * s + sq);
+    if (q < kNB - 1) us4 = shfl_elt(own, 4 * (s + 4) + sq);
     E d, id;
     A::pivot(shfl_elt(own, 4 * q + sq), d, id);
     if (lane == 0 && q < nb) inv[kb + q] = id;
-    if (i == q) id_i = id;
-    if (s == sq && i > q) own = A::mul(own, id);
-    if (s == sq && i == q) own = d;
-    if (q == kNB - 1) break;  // nothing right of the last column
-    const E ciq = shfl_elt(own, 4 * i + sq);  // L_iq
-    if (q < 3) {                              // entries (i, s) with s > q exist
-      const E csq = shfl_elt(own, 4 * s + sq);  // L_sq
-      if (s > q && s <= i) {
-        typename A::Acc acc = A::begin(c0);
-        A::sub(acc, ciq, csq);
-        c0 = A::end(acc);
-      }
+    id_i = i == q ? id : id_i;
+    const E liq = A::mul(uiq, id);  // L_iq
+    if (s == sq) own = i > q ? liq : i == q ? d : own;
+    if (q < 3) {  // entries (i, s) with s > q exist
+      typename A::Acc acc = A::begin(c0);
+      A::sub(acc, liq, A::mul(us, id));
+      const E v = A::end(acc);
+      c0 = s > q && in0 ? v : c0;
     }
-    const E cs4q = shfl_elt(own, 4 * (s + 4) + sq);  // L_{s+4,q}
-    if (s + 4 > q && s + 4 <= i) {
+    if (q < kNB - 1) {
       typename A::Acc acc = A::begin(c1);
-      A::sub(acc, ciq, cs4q);
-      c1 = A::end(acc);
+      A::sub(acc, liq, A::mul(us4, id));
+      const E v = A::end(acc);
+      c1 = s + 4 > q && in1 ? v : c1;
     }
   }
-  if (i < nb && s <= i) Ls(kb + i, kb + s) = c0;
-  if (i < nb && s + 4 <= i) Ls(kb + i, kb + s + 4) = c1;
+  if (i < nb && in0) Ls(kb + i, kb + s) = c0;
+  if (i < nb && in1) Ls(kb + i, kb + s + 4) = c1;
   // the rows of the block scaled by their inverse pivots, L_ij / L_ii (j < i),
   // for the row solves
   if (s < i) lsc[tri(i) + s] = A::mul(c0, id_i);
@@ -404,28 +427,25 @@ __device__ __noinline__ void warp_factor_diag(At Ls, typename A::T *inv, int kb,
 // Row i of the panel at kb (width nb): L[i, kb:kb+nb] <- L[i, kb:kb+nb] L_bb^-T,
 // by forward substitution with the row-scaled block lsc (L_qp / L_qq):
 // x_q = b_q / L_qq - sum_{p<q} x_p (L_qp / L_qq), so that each step of the
-// dependent chain is one multiply-subtract.
+// dependent chain is one multiply-subtract.  The panel is kNB wide: only the last
+// one can be narrower, and it has no rows below.
 template <class A, class At>
 __device__ __noinline__ void panel_row(At Ls, const typename A::T *inv, const typename A::T *lsc,
-                                       int kb, int nb, int i) {
+                                       int kb, int i) {
   using E = typename A::T;
-  E *row = &Ls(i, 0);
+  E *row = &Ls(i, kb);
   E x[kNB];
 #pragma unroll
-  for (int q = 0; q < kNB; ++q)
-    if (q < nb) x[q] = A::mul(row[kb + q], inv[kb + q]);
+  for (int q = 0; q < kNB; ++q) x[q] = A::mul(row[q], inv[kb + q]);
 #pragma unroll
   for (int q = 1; q < kNB; ++q) {
-    if (q < nb) {
-      typename A::Acc acc = A::begin(x[q]);
+    typename A::Acc acc = A::begin(x[q]);
 #pragma unroll
-      for (int p = 0; p < q; ++p) A::sub(acc, x[p], lsc[tri(q) + p]);
-      x[q] = A::end(acc);
-    }
+    for (int p = 0; p < q; ++p) A::sub(acc, x[p], lsc[tri(q) + p]);
+    x[q] = A::end(acc);
   }
 #pragma unroll
-  for (int q = 0; q < kNB; ++q)
-    if (q < nb) row[kb + q] = x[q];
+  for (int q = 0; q < kNB; ++q) row[q] = x[q];
 }
 
 // Trailing update of a right-looking Cholesky step: every entry (i, j) with
@@ -444,8 +464,8 @@ __device__ __noinline__ void panel_row(At Ls, const typename A::T *inv, const ty
 // Every entry is written by one lane and only panel columns are read, so the
 // items need no synchronisation.  The first item (the corner of the first
 // block) is the 8 x 8 diagonal block of the next panel at c0; with
-// `factor_next` the warp that takes it factors that block right after, a
-// short serial path that the other warps' items overlap.
+// `factor_next` the warp that takes it updates and factors that block in
+// registers, a short serial path that the other warps' items overlap.
 constexpr int kColRows = 16;
 
 template <class A>
@@ -465,6 +485,10 @@ __device__ void trailing_cols(typename A::T *Ls, typename A::T *inv, typename A:
       q -= chunks;
     }
     if (b == nblk) return;
+    if (factor_next && item == 0) {  // the next panel's diagonal block
+      warp_factor_diag<A, true>(PackedAt<E>{Ls}, inv, c0, min(kNB, n - c0), lane, lsc, kb);
+      continue;
+    }
     if (q < 3) {  // the diagonal triangle: its 8 x 8 corner, then two halves of the rest
       const int m = min(32, n - jb), ne = m * (m + 1) / 2, nc = min(ne, tri(kNB));
       const int half = (ne - nc + 1) / 2;
@@ -479,10 +503,6 @@ __device__ void trailing_cols(typename A::T *Ls, typename A::T *inv, typename A:
 #pragma unroll
         for (int k = 0; k < kNB; ++k) A::sub(acc, x[k], y[k]);
         *p = A::end(acc);
-      }
-      if (factor_next && item == 0) {  // the next panel's diagonal block is final
-        __syncwarp();
-        warp_factor_diag<A>(PackedAt<E>{Ls}, inv, c0, min(kNB, n - c0), lane, lsc);
       }
       continue;
     }
@@ -530,14 +550,14 @@ __device__ void cta_cholesky_panels(typename A::T *Ls, typename A::T *inv, int n
   __shared__ typename A::T lsc[kNB * (kNB + 1) / 2];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const PackedAt<typename A::T> at{Ls};
-  if (warp == blockIdx.x % nw) warp_factor_diag<A>(at, inv, 0, min(kNB, n), lane, lsc);
+  if (warp == blockIdx.x % nw) warp_factor_diag<A, false>(at, inv, 0, min(kNB, n), lane, lsc);
   __syncthreads();
   for (int kb = 0; kb < n; kb += kNB) {
     const int nb = min(kNB, n - kb), j1 = kb + nb;
     const int rot = (kb / kNB + blockIdx.x) % nw;
     if (threadIdx.x == 0) next_item = 0;
     const int t = (threadIdx.x + 32 * rot) % blockDim.x;
-    for (int i = j1 + t; i < n; i += blockDim.x) panel_row<A>(at, inv, lsc, kb, nb, i);
+    for (int i = j1 + t; i < n; i += blockDim.x) panel_row<A>(at, inv, lsc, kb, i);
     __syncthreads();
     if (j1 < n) {
       trailing_cols<A>(Ls, inv, lsc, n, kb, j1, &next_item, true);
@@ -577,10 +597,10 @@ __device__ void cta_cholesky_global(typename A::T *Lg, typename A::T *inv, int n
     __syncthreads();
     for (int kk = 0; kk < w; kk += kNB) {
       const int nb = min(kNB, w - kk);
-      if (warp == (kb / kNB + kk / kNB) % nw) warp_factor_diag<A>(at, inv + kb, kk, nb, lane, lsc);
+      if (warp == (kb / kNB + kk / kNB) % nw) warp_factor_diag<A, false>(at, inv + kb, kk, nb, lane, lsc);
       __syncthreads();
       for (int i = kk + nb + tid; i < m; i += blockDim.x)
-        panel_row<A>(at, inv + kb, lsc, kk, nb, i);
+        panel_row<A>(at, inv + kb, lsc, kk, i);
       __syncthreads();
       const int rest = w - kk - nb, c0 = kk + nb;  // panel columns still to come
       if (rest > 0) {

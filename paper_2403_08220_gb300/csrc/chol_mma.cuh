@@ -19,7 +19,7 @@
 // scheduler; here 28 mma.sync.m16n8k16 per 128 entries (8 cycles each on
 // GB300) run beside about 42 instructions per entry that join the levels.
 // Geometry of 512 chains at r = 400 (factor in global memory): 4.61 -> 3.44 ms;
-// of 4096 chains at r = 128: 2.02 -> 1.60 ms.  The d_y-sized factors of the Woodbury path (101
+// of 4096 chains at r = 128: 2.02 -> 1.60 ms (3.40 and 1.52 since the diagonal blocks take less).  The d_y-sized factors of the Woodbury path (101
 // rows, four chains an SM) gain nothing: 3.32 against 3.20 ms for 16384 chains,
 // their time is in the panels and barriers.
 #pragma once
@@ -209,13 +209,13 @@ __device__ void cta_cholesky_mma(float2 *Ls, float2 *inv, int n, char *dig) {
   float *scl = reinterpret_cast<float *>(dig + (size_t)max(0, n - kMmaW) * kDigPitch);
   for (int i = tid; i < n; i += blockDim.x) scl[i] = row_scale(Ls[tri(i) + i].x);
   __syncthreads();  // the scales are taken before the first block is factored
-  if (warp == blockIdx.x % nw) warp_factor_diag<A>(at, inv, 0, min(kNB, n), lane, lsc);
+  if (warp == blockIdx.x % nw) warp_factor_diag<A, false>(at, inv, 0, min(kNB, n), lane, lsc);
   __syncthreads();
   for (int kb = 0; kb < n; kb += kMmaW) {
     const int rot = (kb / kMmaW + blockIdx.x) % nw, t = (tid + 32 * rot) % blockDim.x;
     const int nb1 = min(kNB, n - kb), k2 = kb + nb1, nb2 = min(kNB, n - k2), j0 = k2 + nb2;
     if (tid == 0) next_item = 0;
-    for (int i = k2 + t; i < n; i += blockDim.x) panel_row<A>(at, inv, lsc, kb, nb1, i);
+    for (int i = k2 + t; i < n; i += blockDim.x) panel_row<A>(at, inv, lsc, kb, i);
     __syncthreads();
     if (nb2 <= 0) return;
     auto update = [&](int i, int c) {  // entry (i, c) of the second eight columns
@@ -225,13 +225,7 @@ __device__ void cta_cholesky_mma(float2 *Ls, float2 *inv, int n, char *dig) {
       at(i, c) = A::end(acc);
     };
     if (warp == rot) {
-      for (int e = lane; e < nb2 * (nb2 + 1) / 2; e += 32) {
-        int i, c;
-        tri_pos(e, i, c);
-        update(k2 + i, k2 + c);
-      }
-      __syncwarp();
-      warp_factor_diag<A>(at, inv, k2, nb2, lane, lsc);
+      warp_factor_diag<A, true>(at, inv, k2, nb2, lane, lsc, kb);
     } else {
       const int w = (warp - rot + nw) % nw - 1;  // 0 .. nw - 2
       for (int e = 32 * w + lane; e < (n - j0) * kNB; e += 32 * (nw - 1))
@@ -239,7 +233,7 @@ __device__ void cta_cholesky_mma(float2 *Ls, float2 *inv, int n, char *dig) {
     }
     __syncthreads();
     if (j0 >= n) return;
-    for (int i = j0 + t; i < n; i += blockDim.x) panel_row<A>(at, inv, lsc, k2, kNB, i);
+    for (int i = j0 + t; i < n; i += blockDim.x) panel_row<A>(at, inv, lsc, k2, i);
     __syncthreads();
     for (int e = tid; e < (n - j0) * (kMmaW / 2); e += blockDim.x) {
       const int i = j0 + e / (kMmaW / 2), q = e % (kMmaW / 2);
@@ -248,7 +242,7 @@ __device__ void cta_cholesky_mma(float2 *Ls, float2 *inv, int n, char *dig) {
     }
     __syncthreads();
     trailing_mma<kDigPitch>(Ls, dig, kMmaW, scl, n, j0, &next_item, [&]() {
-      warp_factor_diag<A>(at, inv, j0, min(kNB, n - j0), lane, lsc);
+      warp_factor_diag<A, false>(at, inv, j0, min(kNB, n - j0), lane, lsc);
     });
     __syncthreads();
   }
@@ -283,9 +277,9 @@ __device__ void cta_cholesky_global_mma(float2 *Lg, float2 *inv, int n, char *di
     __syncthreads();
     for (int kk = 0; kk < w; kk += kNB) {
       const int nb = min(kNB, w - kk), c0 = kk + nb;
-      if (warp == (kb / kNB + kk / kNB) % nw) warp_factor_diag<A>(at, inv + kb, kk, nb, lane, lsc);
+      if (warp == (kb / kNB + kk / kNB) % nw) warp_factor_diag<A, false>(at, inv + kb, kk, nb, lane, lsc);
       __syncthreads();
-      for (int i = c0 + tid; i < m; i += blockDim.x) panel_row<A>(at, inv + kb, lsc, kk, nb, i);
+      for (int i = c0 + tid; i < m; i += blockDim.x) panel_row<A>(at, inv + kb, lsc, kk, i);
       __syncthreads();
       if (w > c0) {
         for (int e = tid; e < (m - c0) * kNB; e += blockDim.x) {

@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(32 * kPropWarps) k_propose_warp(ReducedArgs a)
 // memory, and the registers of the tiles halving the warps of the
 // factorisation) both together took 9.85 ms for 512 chains at r = d_y = 400 and
 // 2.95 ms for 4096 at r = 128, d_y = 200; apart, 1.40 + 5.70 ms and 0.65 + 2.02 ms
-// (the factorisation 3.44 and 1.60 ms since its updates run on the tensor cores).
+// (the factorisation 3.40 and 1.52 ms since its updates run on the tensor cores).
 constexpr int kGramB = 64, kGramK = 32, kGramThreads = 128;
 constexpr int kGramFlush = 64;  // rows per FP32 partial sum
 
