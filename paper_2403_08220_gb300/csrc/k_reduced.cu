@@ -459,7 +459,14 @@ __global__ void __launch_bounds__(NT, sizeof(TJ) == 4 && !kBlk
   int *flag = reinterpret_cast<int *>(sm + lay.flag);
   const TJ *J = reinterpret_cast<const TJ *>(a.J) + (size_t)c * dy * r;
   const TJ *f = reinterpret_cast<const TJ *>(a.f) + (size_t)c * dy;
-  const double inv_nv = 1.0 / a.noise_var;
+  const double inv_nv = a.inv_nv;
+  // The thread that takes the accept test; in FP64 it draws log u ahead, a chain of
+  // FP64 operations that would otherwise follow the last sums (64 chains, r = 16,
+  // d_y = 49, with the two changes beside the Gram matrix and the pivots: 47 -> 45 us).
+  const bool judge = threadIdx.x == blockDim.x - 1;
+  double log_u = 0.0;
+  if constexpr (sizeof(TJ) == 8)
+    if (mode == 1 && judge) log_u = draw_log_u(a, c);
   if constexpr (sizeof(TJ) == 4 && !G) {  // the packed I + H by 16-byte copies, all in flight
     const size_t ne = tri_size(r);
     const E *src = reinterpret_cast<const E *>(Lg);
@@ -576,24 +583,27 @@ __global__ void __launch_bounds__(NT, sizeof(TJ) == 4 && !kBlk
     return;
   }
   const E *tb = Ls + tri(r);
-  const double s = a.s, cs = sqrt(1.0 - s * s);
+  const double s = a.s, inv_cs = a.inv_cs;
   double t1 = 0.0, t2 = 0.0, t3 = 0.0;
   for (int i = threadIdx.x; i < r; i += blockDim.x) {
     const double d = vp[i] - A::to(tb[i]);         // L_b^-1 w, w = H_b b - g_b
-    const double mh = (va[i] - s * vb[i]) / cs;    // mhat for b -> a
-    const double u = (vq[i] - s * vp[i]) / cs;     // L_b^T mhat
+    const double mh = (va[i] - s * vb[i]) * inv_cs;  // mhat for b -> a
+    const double u = (vq[i] - s * vp[i]) * inv_cs;   // L_b^T mhat
     t1 += d * d;
     t2 += u * vp[i] - mh * (vb[i] + vg[i]);
     t3 += u * u - mh * mh;
   }
   block_sum3(t1, t2, t3, red);
-  if (threadIdx.x == 0) {
-    const double lq_rev = -a.dt / 8.0 * t1 + sqrt(a.dt) / 2.0 * t2 + hld_b - 0.5 * t3;
-    const double lr = a.phi[c] - phi_b + lq_rev - a.lq_fwd[c];
-    *flag = accept_test(a, c, lr, phi_b, hld_b) ? 1 : 0;
+  double lr = 0.0;
+  if (judge) {
+    if constexpr (sizeof(TJ) == 4) log_u = draw_log_u(a, c);
+    const double lq_rev = -a.dt / 8.0 * t1 + a.sqrt_dt / 2.0 * t2 + hld_b - 0.5 * t3;
+    lr = a.phi[c] - phi_b + lq_rev - a.lq_fwd[c];
+    *flag = accept_decide(lr, log_u) ? 1 : 0;
   }
   __syncthreads();
   const bool accept = *flag != 0;
+  if (judge) accept_record(a, c, lr, log_u, accept, phi_b, hld_b);
   for (int i = threadIdx.x; i < r; i += blockDim.x) {
     a.coef[(size_t)c * r + i] = vb[i] - s * va[i];
     if (accept) {
@@ -675,7 +685,9 @@ static cudaError_t launch_geometry_nt(const ReducedArgs &a, int mode, size_t sme
   auto k = k_geometry<TJ, G, NT, kBlk>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl_n(chain_ctas(a.C), k, a.C, NT, smem, st, a, mode, panel);
+  ReducedArgs b = a;
+  b.derive();
+  return launch_pdl_n(chain_ctas(a.C), k, a.C, NT, smem, st, b, mode, panel);
 }
 
 // CTA size: smaller CTAs let more chains share an SM (the kernel's loops stride
