@@ -463,10 +463,10 @@ __global__ void __launch_bounds__(NT, sizeof(TJ) == 4 && !kBlk
   // The thread that takes the accept test; in FP64 it draws log u ahead, a chain of
   // FP64 operations that would otherwise follow the last sums (64 chains, r = 16,
   // d_y = 49, with the two changes beside the Gram matrix and the pivots: 47 -> 45 us).
-  const bool judge = threadIdx.x == blockDim.x - 1;
+  const bool decider = threadIdx.x == blockDim.x - 1;
   double log_u = 0.0;
   if constexpr (sizeof(TJ) == 8)
-    if (mode == 1 && judge) log_u = draw_log_u(a, c);
+    if (mode == 1 && decider) log_u = draw_log_u(a, c);
   if constexpr (sizeof(TJ) == 4 && !G) {  // the packed I + H by 16-byte copies, all in flight
     const size_t ne = tri_size(r);
     const E *src = reinterpret_cast<const E *>(Lg);
@@ -595,7 +595,7 @@ __global__ void __launch_bounds__(NT, sizeof(TJ) == 4 && !kBlk
   }
   block_sum3(t1, t2, t3, red);
   double lr = 0.0;
-  if (judge) {
+  if (decider) {
     if constexpr (sizeof(TJ) == 4) log_u = draw_log_u(a, c);
     const double lq_rev = -a.dt / 8.0 * t1 + a.sqrt_dt / 2.0 * t2 + hld_b - 0.5 * t3;
     lr = a.phi[c] - phi_b + lq_rev - a.lq_fwd[c];
@@ -603,7 +603,7 @@ __global__ void __launch_bounds__(NT, sizeof(TJ) == 4 && !kBlk
   }
   __syncthreads();
   const bool accept = *flag != 0;
-  if (judge) accept_record(a, c, lr, log_u, accept, phi_b, hld_b);
+  if (decider) accept_record(a, c, lr, log_u, accept, phi_b, hld_b);
   for (int i = threadIdx.x; i < r; i += blockDim.x) {
     a.coef[(size_t)c * r + i] = vb[i] - s * va[i];
     if (accept) {
