@@ -26,7 +26,8 @@
 // Column equilibration: B (weights, laid out once) may carry powers of two
 // f_k with max_j |B_jk| 2^-f_k in [1, 2); A's column k is then scaled by
 // 2^f_k, so that an input that B weighs down cannot push the others' digits
-// out of range.  Rows of A that hold an infinity or a NaN take the plain dot
+// out of range, and an input in a column that is zero in B (kZeroCol) takes no
+// part.  Rows of A that hold an infinity or a NaN take the plain dot
 // product in FP64 instead, element by element.
 //
 // Layout: digit planes [kDigits][rows][ldp] of bf16, TMA boxes of 32 columns
@@ -63,6 +64,7 @@ constexpr int kGemm64Threads = 32 * (2 + kEpiWarps);
 constexpr int kABytes = kDigits * kBM * kKB * 2;
 constexpr int kStgBytes = kEpiWarps * 32 * 16 * 8;  // 32 rows x 16 doubles per warp
 constexpr int kBadRow = INT32_MIN;             // row exponent of a non-finite row
+constexpr int kZeroCol = INT32_MIN;            // column exponent of a zero column of B
 
 // ---- digits -----------------------------------------------------------------
 
@@ -129,17 +131,20 @@ __global__ void __launch_bounds__(256) k_split64(const SplitArgs a) {
       }
     }
   };
-  auto colexp = [&](int k) { return a.fk && k < a.K ? a.fsign * a.fk[k] : 0; };
+  // biased exponent of entry k with its column exponent; 0: takes no part
+  auto entry_exp = [&](int k, double v) {
+    const int ef = exp_field(v), f = a.fk && k < a.K ? a.fk[k] : 0;
+    return ef == 0 || f == kZeroCol ? 0 : ef + 4096 + a.fsign * f;
+  };
   const int ngroups = a.ldp / 4;
   double x[kQ > 0 ? kQ : 1][4];
-  int emax = 0;  // largest exponent field (+ 4096 + column exponent) of a nonzero entry
+  int emax = 0;  // largest entry_exp
   bool bad = false;
   auto scan = [&](int k, const double v[4]) {
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      const int ef = exp_field(v[e]);
-      bad |= ef == 0x7ff;
-      if (ef > 0) emax = max(emax, ef + 4096 + colexp(k + e));
+      bad |= exp_field(v[e]) == 0x7ff;
+      emax = max(emax, entry_exp(k + e, v[e]));
     }
   };
   if constexpr (kQ > 0) {
@@ -163,12 +168,12 @@ __global__ void __launch_bounds__(256) k_split64(const SplitArgs a) {
     uint32_t w[kDigits][2];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      const int ef = exp_field(v[e]);
+      const int ex = entry_exp(4 * grp + e, v[e]);
       long long t = 0;  // the entry in units of 2^(ea - 56), rounded
-      if (ef > 0 && !bad) {
+      if (ex && !bad) {
         const long long bits = __double_as_longlong(v[e]);
         const long long m = (bits & 0xfffffffffffffll) | 0x10000000000000ll;
-        const int s = ef + 4096 + colexp(4 * grp + e) - emax + 3;
+        const int s = ex - emax + 3;
         t = s >= 0 ? m << s : (s > -60 ? (m + (1ll << (-s - 1))) >> -s : 0);
         if (bits < 0) t = -t;
       }
@@ -203,14 +208,19 @@ __global__ void __launch_bounds__(256) k_split64(const SplitArgs a) {
   }
 }
 
-// Column exponents: fk[k] with 2^fk <= max_j |B_jk| < 2^(fk + 1) (0 for a zero column).
+// Column exponents: fk[k] with 2^fk <= max_j |B_jk| < 2^(fk + 1) over the finite
+// entries (-1023 for subnormal ones, kZeroCol for a zero column).
 __global__ void k_col_exp(int rows, int K, const double *__restrict__ B, int ld,
                           int *__restrict__ fk) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= K) return;
-  int m = 0;
-  for (int j = 0; j < rows; ++j) m = max(m, exp_field(B[(size_t)j * ld + k]));
-  fk[k] = m > 0 && m < 0x7ff ? m - 1023 : 0;
+  int m = -1;
+  for (int j = 0; j < rows; ++j) {
+    const double v = B[(size_t)j * ld + k];
+    const int ef = exp_field(v);
+    if (v != 0.0 && ef < 0x7ff) m = max(m, ef);
+  }
+  fk[k] = m < 0 ? kZeroCol : m - 1023;
 }
 
 // ---- product ------------------------------------------------------------------
