@@ -27,8 +27,8 @@
 // f_k with max_j |B_jk| 2^-f_k in [1, 2); A's column k is then scaled by
 // 2^f_k, so that an input that B weighs down cannot push the others' digits
 // out of range, and an input in a column that is zero in B (kZeroCol) takes no
-// part.  Rows of A that hold an infinity or a NaN take the plain dot
-// product in FP64 instead, element by element.
+// part.  Outputs whose row of A or of B holds an infinity or a NaN are plain dot
+// products in FP64 instead.
 //
 // Layout: digit planes [kDigits][rows][ldp] of bf16, TMA boxes of 32 columns
 // x (128 rows of A | BN rows of B) x all eight planes (64-byte swizzle), two
@@ -229,7 +229,7 @@ struct Gemm64Params {
   int M, N, K, row0, nkb;
   int grp;  // Gram products: rows of a group (0: one plain product)
   const int *ea, *eb;
-  const double *A, *W, *der, *B;  // the FP64 operands, for rows of A that are not finite
+  const double *A, *W, *der, *B;  // the FP64 operands, for rows that are not finite
   int lda, g, ldd, ldb;
   uint32_t tmem_cols;
   int *err;
@@ -493,7 +493,7 @@ __global__ void __launch_bounds__(kGemm64Threads, 1)
       }
       if (!ok) break;
       const int ea = row < rows ? p.ea[g0 + row] : 0;
-      bool odd = ea == kBadRow;  // a row or (Gram products) a column that is not finite
+      bool odd = ea == kBadRow;  // a row of A or of B that is not finite
       constexpr int kS = NC < 16 ? NC : 16;  // columns staged at a time
 #pragma unroll
       for (int c0 = 0; c0 < NC; c0 += kS) {
@@ -501,9 +501,10 @@ __global__ void __launch_bounds__(kGemm64Threads, 1)
 #pragma unroll
         for (int c = 0; c < kS; ++c) {
           const int eb = n0 + c0 + c < p.N ? p.eb[g0 + n0 + c0 + c] : 0;
-          if (kGram) odd |= eb == kBadRow;
+          const bool any = ea == kBadRow || eb == kBadRow;
+          odd |= any;
           stg[lane * 16 + ((((c >> 1) ^ (lane & 7)) << 1) | (c & 1))] =
-              scaled_to_f64(acc[c0 + c], low[c0 + c], ea + eb - 35);
+              any ? 0.0 : scaled_to_f64(acc[c0 + c], low[c0 + c], ea + eb - 35);
         }
         const bool plain = __any_sync(0xffffffffu, odd);
         __syncwarp();

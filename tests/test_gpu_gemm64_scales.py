@@ -86,3 +86,23 @@ def test_encode_of_a_field_with_filler_outside_the_basis(dino, precision):
         ctx.close()
     used = m0[:, seen]
     assert np.all(np.abs(m_r - used @ Q) <= 4 * (N + 8) * EPS * (np.abs(used) @ np.abs(Q)))
+
+
+def test_a_row_that_is_not_finite_reaches_every_product_with_it(dino):
+    """A Jacobian column that overflows makes its row and column of J^T J not
+    finite, as in plain arithmetic, and with them every eigenvalue of the
+    derivative-informed basis: no pair may come out as if the column were zero."""
+    rng = np.random.default_rng(13)
+    r, h, dy, n = 140, 150, 30, 20
+    W = [rng.standard_normal((h, r)), 1e10 * rng.standard_normal((dy, h))]
+    W[0][:, 77] = 1e300
+    ctx = dino.dino_init(0)
+    try:
+        sid = dino.dino_load_surrogate(
+            ctx, n_grid=17, prior_gamma=0.1, prior_delta=1.0, r=r, widths=[r, h, dy], activation=0,
+            W=W, b=[np.zeros(h), np.zeros(dy)], basis_kind=dino.DINO_BASIS_KLE, y=np.zeros(dy),
+            noise_var=1.0, precision=dino.DINO_PREC_FP64)
+        out = dino.dino_dis_from_surrogate(ctx, sid, n, 5, 8, r, 17 * 17)
+    finally:
+        ctx.close()
+    assert not np.any(np.isfinite(out["eigvals"]))
