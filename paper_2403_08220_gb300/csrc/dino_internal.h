@@ -165,15 +165,21 @@ cudaError_t gemm_field(int M, int N, int K, const T *A, int lda, const T *B, int
 
 // ---- FP64 GEMMs on the tensor cores (k_gemm64.cu) -------------------------
 // Operands as kDigits64 planes of signed base-128 digits in bf16 (plane s at
-// + s * plane elements, row pitch ldp a multiple of 8) and one exponent a row.
+// + s * plane elements, row pitch ldp a multiple of 8), behind them (not for
+// gram64_slots) a plane of magnitudes, rows padded to 32 columns, and one exponent a row.
 constexpr int kDigits64 = 8;
 int digit_pitch(int K);
+size_t digit_bytes(size_t rows, int K, int group);  // of the planes with the magnitudes
+// The plane of magnitudes: none, each entry's, or one value for four neighbouring
+// columns: their sum (A) or the least (B)
+enum class Magnitudes { kNone, kEach, kSum4, kMin4 };
 struct DigitMat {              // an operand B laid out once (weights, basis)
   const __nv_bfloat16 *d = nullptr;
   const int *ex = nullptr;     // row exponents
   const int *fk = nullptr;     // column exponents taken out of B (nullptr: none)
   int ldp = 0;
   size_t plane = 0;
+  int group = 1;               // columns to a magnitude: 1 (kEach) or 4 (kMin4)
   const double *src = nullptr;  // B itself, rows x K (pitch ld)
   int ld = 0;
 };
@@ -183,11 +189,14 @@ struct DigitMat {              // an operand B laid out once (weights, basis)
 cudaError_t launch_split64(int rows, int K, const double *src, int ld, const double *W,
                            const double *der, int g, int ldd, int row0, const int *fk, int fsign,
                            __nv_bfloat16 *dst, int ldp, size_t plane,
-                           int *ex, cudaStream_t st);
+                           int *ex, cudaStream_t st, Magnitudes mags);
+// *sparse += rows of B (kEach) that are too sparse for kMin4
+cudaError_t launch_count_sparse(int rows, int K, const __nv_bfloat16 *digits, size_t plane,
+                                const int *ex, int *sparse, cudaStream_t st);
 cudaError_t launch_col_exp(int rows, int K, const double *B, int ld, int *fk, cudaStream_t st);
 // out = epilogue(A B^T) for M rows of A (digits A, ea; the values Asrc, pitch
-// lda, or the product form, read only for rows that are not finite); the epilogue's row index
-// starts at row0.  err (device): bit 8 is set when a bounded wait gave up.
+// lda, or the product form, read only where the digits do not do); the epilogue's
+// row index starts at row0.  err (device): bit 8 is set when a bounded wait gave up.
 struct Gemm64Args {
   int M = 0, N = 0, K = 0, row0 = 0;
   const __nv_bfloat16 *A = nullptr;

@@ -495,7 +495,8 @@ static DigitMat make_digits(dino_ctx *ctx, std::vector<std::pair<void *, size_t>
   if ((long)rows * K < kDigitsMinWork || rows < 32 || K < 32) return m;
   const int ldp = digit_pitch(K);
   const size_t plane = (size_t)rows * ldp;
-  const size_t bytes = (plane * kDigits64 * 2 + ((size_t)rows + K) * 4 + 15) & ~(size_t)15;
+  const size_t planes = digit_bytes(rows, K, 1);
+  const size_t bytes = (planes + ((size_t)rows + K + 1) * 4 + 15) & ~(size_t)15;
   if (ctx->used + bytes > ctx->budget) return m;
   void *p = nullptr;
   if (cudaMalloc(&p, bytes) != cudaSuccess) {
@@ -505,10 +506,24 @@ static DigitMat make_digits(dino_ctx *ctx, std::vector<std::pair<void *, size_t>
   ctx->used += bytes;
   allocs.push_back({p, bytes});
   auto *d = (__nv_bfloat16 *)p;
-  int *ex = (int *)(d + plane * kDigits64), *fk = equilibrate ? ex + rows : nullptr;
+  int *ex = (int *)((char *)p + planes), *fk = equilibrate ? ex + rows : nullptr;
+  auto split = [&](Magnitudes mags) {
+    CK(launch_split64(rows, K, B, K, nullptr, nullptr, 1, 0, 0, fk, -1, d, ldp, plane, ex,
+                      ctx->stream, mags));
+  };
   if (fk) CK(launch_col_exp(rows, K, B, K, fk, ctx->stream));
-  CK(launch_split64(rows, K, B, K, nullptr, nullptr, 1, 0, 0, fk, -1, d, ldp, plane, ex,
-                    ctx->stream));
+  split(Magnitudes::kEach);
+  if (fk) {  // an operand of its own: magnitudes by fours unless many rows are sparse
+    int *sparse = fk + K, n = 0;
+    CK(cudaMemsetAsync(sparse, 0, 4, ctx->stream));
+    CK(launch_count_sparse(rows, K, d, plane, ex, sparse, ctx->stream));
+    CK(cudaMemcpyAsync(&n, sparse, 4, cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
+    if ((long)n * 100 <= rows) {
+      split(Magnitudes::kMin4);
+      m.group = 4;
+    }
+  }
   m.d = d;
   m.ex = ex;
   m.fk = fk;
@@ -538,11 +553,13 @@ struct Scratch64 {
   int *err = nullptr;
   void *row = nullptr;
 };
-static size_t digit_row_bytes(int K) { return 16 * (size_t)digit_pitch(K) + 32; }
+static size_t digit_row_bytes(int K) { return digit_bytes(1, K, 1) + 32; }
 
 // Bytes of A's digits worked on at a time: they are written and read again
-// while still in L2 (129 MB).
-constexpr size_t kDigitsChunk = 96u << 20;
+// while still in L2 (129 MB), beside B's.  Smaller chunks fill the last wave of
+// tiles worse (Jacobian and Gram matrices of 1024 chains, r = 200, two steps: 40 MB
+// 8.79 ms, 64 7.42, 80 7.38, 88 6.80, 96 7.02 ms).
+constexpr size_t kDigitsChunk = 88u << 20;
 
 static bool has_digits(const DigitMat &B, const Scratch64 &ws) { return B.d && ws.p && ws.row; }
 
@@ -552,7 +569,7 @@ template <class Tc>
 static void digit_product(dino_ctx *ctx, cudaStream_t st, const char *name, int M, int N, int K,
                           const Left64 &a, const DigitMat &B, const Scratch64 &ws, Tc &&tc) {
   const int ldp = digit_pitch(K);
-  const size_t per = 16 * (size_t)ldp + 4, one = digit_row_bytes(K);
+  const size_t per = digit_bytes(1, K, B.group) + 4, one = digit_row_bytes(K);
   char *scratch = (char *)(ws.bytes >= one ? ws.p : ws.row);
   const size_t bytes = std::max(ws.bytes, one);
   size_t rows = std::min<size_t>({(size_t)M, (bytes - 16) / per,
@@ -564,13 +581,13 @@ static void digit_product(dino_ctx *ctx, cudaStream_t st, const char *name, int 
   }
   auto *d = (__nv_bfloat16 *)scratch;
   const size_t plane = rows * ldp;
-  int *ex = (int *)(d + plane * kDigits64);
+  int *ex = (int *)(scratch + digit_bytes(rows, K, B.group));
   for (size_t r0 = 0; r0 < (size_t)M; r0 += rows) {
     const int m = (int)std::min(rows, (size_t)M - r0);
     const double *A = a.A ? a.A + r0 * a.lda : nullptr;
     launch(ctx, st, "split_f64", [&] {
       return launch_split64(m, K, A, a.lda, a.W, a.der, a.g, a.ldd, (int)r0, B.fk, 1, d, ldp,
-                            plane, ex, st);
+                            plane, ex, st, B.group == 4 ? Magnitudes::kSum4 : Magnitudes::kEach);
     });
     Gemm64Args g;
     g.M = m;
@@ -1518,7 +1535,7 @@ static void gram_of(dino_ctx *ctx, const Pool &p, ReducedArgs &a, int mode, cuda
     const double *J = p.w.J64 + (size_t)c0 * dy * r;
     launch(ctx, st, "split_f64", [&] {
       return launch_split64(n * dy, r, J, r, nullptr, nullptr, 1, 0, 0, nullptr, 1, d, ldp, plane,
-                            ex, st);
+                            ex, st, Magnitudes::kNone);
     });
     launch(ctx, st, "gram_f64", [&] {
       return gram64_slots(n, dy, r, J, r, d, ex, ldp, plane, a.L + (size_t)c0 * ss, a.L_slot, ss,
@@ -2068,7 +2085,7 @@ static int nuclear_terms(dino_ctx *ctx, int d, double *A, double *sig, double *Y
 }
 
 // H = X X^T for a row-major d x K matrix X of the device: on the tensor cores
-// when the rule of make_digits admits X and its digits (16 bytes an entry) fit
+// when the rule of make_digits admits X and its digits (18 bytes an entry) fit
 // the budget for the time of the call.
 static void gram64(dino_ctx *ctx, const char *name, int d, int K, const double *X, double *H,
                    cudaStream_t st) {

@@ -18,30 +18,48 @@
 // (2^24), and levels 6 and 7, which weigh 2^-42 and 2^-49, can round only when
 // nearly all digits align.  The eight level sums are combined in 64-bit
 // integers and rounded to FP64 once, so the result carries no accumulated
-// rounding; its error, about 2^-56 of |a| |b|, is below that of the FP64
-// multiply-add chain that it replaces (2-norm error against extended precision:
-// the Jacobian of widths 200-400-400-100 2.2e-16 against 1.05e-15, its f 1.7e-16 against 9.2e-16,
-// m_r = E m of 4225 nodes with |E| |m| / |E m| = 500 1.0e-15 against 2.6e-15).
+// rounding (2-norm error against extended precision: the Jacobian of widths
+// 200-400-400-100 2.2e-16 against 1.05e-15 of the multiply-add chain, its f
+// 1.7e-16 against 9.2e-16, m_r = E m of 4225 nodes with |E| |m| / |E m| = 500
+// 1.0e-15 against 2.6e-15).
+//
+// Accuracy entry by entry: with a' = a 2^-ea and b' = b 2^-eb the digits leave
+// at most K 11 2^-58 (entries rounded at 2^-57, 7 digit products of s + t = 8),
+// whatever the sum: where A's large entries meet B's small ones that is more
+// than the K 2^-53 sum |a' b'| of the chain.  So a further product is formed,
+// of the entries' magnitudes in bf16 (rounded down, a plane of their own): a
+// lower bound of sum |a' b'|.  An output whose bound is below kLeast = 1/8 is a
+// plain dot product instead; the others are within 2.75 K 2^-53 sum |a b| at
+// most.  With a dense B four neighbouring columns count as one, the sum of A's
+// four magnitudes times the least of B's (Magnitudes): the Jacobian's products
+// of 1024 chains, widths 200-400-400-100, take 2.02 ms, 2.09 with every column on
+// its own, 1.88 without the bound.  The Gram matrices J J^T that are factored
+// next (gram64_slots) go without: their error counts beside |J_i| |J_j|, as the
+// factorisation's own rounding does.
 //
 // Column equilibration: B (weights, laid out once) may carry powers of two
 // f_k with max_j |B_jk| 2^-f_k in [1, 2); A's column k is then scaled by
 // 2^f_k, so that an input that B weighs down cannot push the others' digits
 // out of range, and an input in a column that is zero in B (kZeroCol) takes no
-// part.  Outputs whose row of A or of B holds an infinity or a NaN are plain dot
-// products in FP64 instead.
+// part.  Outputs whose row of A or of B holds an infinity or a NaN, or a
+// subnormal number that counts beside the row's largest, are plain dot products
+// too.
 //
-// Layout: digit planes [kDigits][rows][ldp] of bf16, TMA boxes of 32 columns
-// x (128 rows of A | BN rows of B) x all eight planes (64-byte swizzle), two
-// stages.  The BN rows of consecutive B planes are contiguous in the stage, so
-// one tcgen05.mma multiplies A's plane s with up to 256 / BN planes of B at
-// once and adds into as many neighbouring level accumulators: 12 instructions
-// of mostly N = 256 per 16 columns instead of 36 of N = 64.  The eight
-// accumulators of BN columns fill TMEM at BN = 64.
+// Layout: digit planes [kDigits][rows][ldp] of bf16, then the magnitudes [rows]
+// [check_pitch]; TMA boxes of 32 columns x (128 rows of A | BN rows of B) x
+// all eight planes (64-byte swizzle), two stages; a stage of magnitudes is
+// eight blocks of 32 columns in the place of the eight planes.  The BN rows of
+// consecutive B planes are contiguous in the stage, so one tcgen05.mma
+// multiplies A's plane s with up to 256 / BN planes of B at once and adds into as
+// many neighbouring level accumulators: 12 instructions of mostly N = 256 per 16
+// columns instead of 36 of N = 64.  The eight accumulators of BN columns fill
+// TMEM at BN = 64; the sums of magnitudes take the first one's place when the
+// last chunk has been read.
 //
 // What bounds it: the digit planes' way from L2 (96 KB per 32 columns and
 // tile); the launcher's callers cut M into chunks whose planes stay in L2.
 // 102400 x 400 x 400 and x 200 (the Jacobian of 1024 chains, 98 GFLOP): 46.6 ms
-// on the FP64 pipe, 1.94 ms here and 0.6 ms for the digits of A.
+// on the FP64 pipe, 2.02 ms here and 0.6 ms for the digits of A.
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
 
@@ -63,8 +81,15 @@ constexpr int kEpiWarps = 8;
 constexpr int kGemm64Threads = 32 * (2 + kEpiWarps);
 constexpr int kABytes = kDigits * kBM * kKB * 2;
 constexpr int kStgBytes = kEpiWarps * 32 * 16 * 8;  // 32 rows x 16 doubles per warp
-constexpr int kBadRow = INT32_MIN;             // row exponent of a non-finite row
+constexpr float kLeast = 0.125f;               // sum |a' b'| below which digits do not do
+constexpr int kBadRow = INT32_MIN;             // row exponent: plain dot products
+constexpr int kZeroRow = INT32_MIN + 1;        // row exponent of a row of zeros
 constexpr int kZeroCol = INT32_MIN;            // column exponent of a zero column of B
+
+// Row pitch of the magnitudes of K columns, `group` to a value: whole blocks of 32.
+__host__ __device__ inline int check_pitch(int K, int group) {
+  return ((K + group - 1) / group + kKB - 1) / kKB * kKB;
+}
 
 // ---- digits -----------------------------------------------------------------
 
@@ -77,6 +102,7 @@ struct SplitArgs {
   int g, ldd, row0;   // row0: first row of the product form
   const int *fk;      // column exponents (nullptr: 0), added (A) or subtracted (B)
   int fsign;
+  Magnitudes mags;
   __nv_bfloat16 *dst;
   int *ex;
 };
@@ -93,7 +119,7 @@ __device__ __forceinline__ int exp_field(double x) {
 // (64-bit shifts and integer conversions per digit took 1.6 times as long:
 // 60 us against 37 us for 19456 rows of 400).
 template <int kQ>
-__global__ void __launch_bounds__(256) k_split64(const SplitArgs a) {
+__global__ void __launch_bounds__(256, 4) k_split64(const SplitArgs a) {
   pdl_begin();
   const int lane = threadIdx.x & 31;
   const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -131,20 +157,27 @@ __global__ void __launch_bounds__(256) k_split64(const SplitArgs a) {
       }
     }
   };
-  // biased exponent of entry k with its column exponent; 0: takes no part
-  auto entry_exp = [&](int k, double v) {
-    const int ef = exp_field(v), f = a.fk && k < a.K ? a.fk[k] : 0;
-    return ef == 0 || f == kZeroCol ? 0 : ef + 4096 + a.fsign * f;
-  };
+  const bool four = a.mags == Magnitudes::kSum4 || a.mags == Magnitudes::kMin4;
   const int ngroups = a.ldp / 4;
+  const int ldc = a.mags == Magnitudes::kNone ? 0 : check_pitch(a.K, four ? 4 : 1);
+  uint16_t *chk = reinterpret_cast<uint16_t *>(a.dst + kDigits * a.plane) + (size_t)row * ldc;
   double x[kQ > 0 ? kQ : 1][4];
-  int emax = 0;  // largest entry_exp
+  int emax = 0;        // largest exponent field
+  int tiny = INT32_MIN;  // largest one that an entry left out can have
   bool bad = false;
-  auto scan = [&](int k, const double v[4]) {
+  // Entries k .. k + 3: column exponents into the exponent fields (entries of zero
+  // columns become 0), which leaves out what is subnormal before or after.
+  auto scale = [&](int k, double v[4]) {
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      bad |= exp_field(v[e]) == 0x7ff;
-      emax = max(emax, entry_exp(k + e, v[e]));
+      const int ef = exp_field(v[e]), f = a.fk && k + e < a.K ? a.fk[k + e] : 0;
+      const int es = ef + a.fsign * f, hi = __double2hiint(v[e]), lo = __double2loint(v[e]);
+      bad |= ef == 0x7ff || (es >= 0x7ff && f != kZeroCol);
+      const bool keep = ef > 0 && f != kZeroCol && es > 0;
+      if (!keep && f != kZeroCol && ((hi & 0x7fffffff) | lo))
+        tiny = max(tiny, max(es, 1 + a.fsign * f));
+      emax = max(emax, keep ? es : 0);
+      v[e] = keep ? __hiloint2double(hi + ((es - ef) << 20), lo) : 0.0;
     }
   };
   if constexpr (kQ > 0) {
@@ -152,28 +185,34 @@ __global__ void __launch_bounds__(256) k_split64(const SplitArgs a) {
     for (int q = 0; q < kQ; ++q) {
       const int k = 4 * (lane + 32 * q);
       load4(k, x[q]);
-      scan(k, x[q]);
+      scale(k, x[q]);
     }
   } else {
     for (int grp = lane; grp < ngroups; grp += 32) {
       load4(4 * grp, x[0]);
-      scan(4 * grp, x[0]);
+      scale(4 * grp, x[0]);
     }
   }
 #pragma unroll
   for (int o = 16; o; o >>= 1) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
-  bad = __any_sync(0xffffffffu, bad);
-  if (lane == 0) a.ex[row] = bad ? kBadRow : (emax ? emax - 4096 - 1022 : 0);
+  // what was left out is below 2^-57 of 2^ea, or the row is bad, as is one at the
+  // bottom of the range (fields below 200)
+  bad = __any_sync(0xffffffffu, bad || tiny > (emax ? emax - 58 : INT32_MIN) ||
+                                    (emax > 0 && emax < 200));
+  if (lane == 0) a.ex[row] = bad ? kBadRow : (emax ? emax - 1022 : kZeroRow);
+  const int mbase = (emax - 126) << 7;
   auto emit = [&](int grp, const double v[4]) {
-    uint32_t w[kDigits][2];
+    uint32_t w[kDigits][2], mag[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      const int ex = entry_exp(4 * grp + e, v[e]);
+      const int ef = exp_field(v[e]);
+      // |entry| 2^-ea in bf16, rounded down
+      mag[e] = (uint32_t)max(0, (__double2hiint(v[e]) >> 13 & 0x3ffff) - mbase);
       long long t = 0;  // the entry in units of 2^(ea - 56), rounded
-      if (ex && !bad) {
+      if (ef) {
         const long long bits = __double_as_longlong(v[e]);
         const long long m = (bits & 0xfffffffffffffll) | 0x10000000000000ll;
-        const int s = ex - emax + 3;
+        const int s = ef - emax + 3;
         t = s >= 0 ? m << s : (s > -60 ? (m + (1ll << (-s - 1))) >> -s : 0);
         if (bits < 0) t = -t;
       }
@@ -195,6 +234,15 @@ __global__ void __launch_bounds__(256) k_split64(const SplitArgs a) {
 #pragma unroll
     for (int d = 0; d < kDigits; ++d)
       *reinterpret_cast<uint2 *>(o + d * a.plane) = make_uint2(w[d][0], w[d][1]);
+    if (a.mags == Magnitudes::kEach) {
+      *reinterpret_cast<uint2 *>(chk + 4 * grp) =
+          make_uint2(mag[0] | mag[1] << 16, mag[2] | mag[3] << 16);
+    } else if (a.mags == Magnitudes::kSum4) {
+      auto f = [&](int e) { return __uint_as_float(mag[e] << 16); };
+      chk[grp] = (uint16_t)(__float_as_uint((f(0) + f(1)) + (f(2) + f(3))) >> 16);
+    } else if (a.mags == Magnitudes::kMin4) {
+      chk[grp] = (uint16_t)min(min(mag[0], mag[1]), min(mag[2], mag[3]));
+    }
   };
   if constexpr (kQ > 0) {
 #pragma unroll
@@ -203,9 +251,11 @@ __global__ void __launch_bounds__(256) k_split64(const SplitArgs a) {
   } else {
     for (int grp = lane; grp < ngroups; grp += 32) {
       load4(4 * grp, x[0]);
+      scale(4 * grp, x[0]);
       emit(grp, x[0]);
     }
   }
+  for (int k = (four ? ngroups : a.ldp) + lane; k < ldc; k += 32) chk[k] = 0;
 }
 
 // Column exponents: fk[k] with 2^fk <= max_j |B_jk| < 2^(fk + 1) over the finite
@@ -223,13 +273,28 @@ __global__ void k_col_exp(int rows, int K, const double *__restrict__ B, int ld,
   fk[k] = m < 0 ? kZeroCol : m - 1023;
 }
 
+// *sparse += the nonzero rows whose least magnitudes of four columns (Magnitudes::kEach
+// planes) sum to less than 2: a warp per row
+__global__ void __launch_bounds__(256) k_count_sparse(int rows, int K, const uint16_t *chk,
+                                                      const int *ex, int *sparse) {
+  const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (row >= rows || ex[row] == kZeroRow) return;
+  const uint16_t *c = chk + (size_t)row * check_pitch(K, 1);
+  float s = 0.0f;
+  for (int k = 4 * lane; k < K; k += 128)  // the pitch is a multiple of 32
+    s += __uint_as_float((uint32_t)min(min(c[k], c[k + 1]), min(c[k + 2], c[k + 3])) << 16);
+#pragma unroll
+  for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0 && s < 2.0f) atomicAdd(sparse, 1);
+}
+
 // ---- product ------------------------------------------------------------------
 
 struct Gemm64Params {
-  int M, N, K, row0, nkb;
+  int M, N, K, row0, nkb, ncb;  // nkb: 32-column blocks; ncb: of the magnitudes
   int grp;  // Gram products: rows of a group (0: one plain product)
   const int *ea, *eb;
-  const double *A, *W, *der, *B;  // the FP64 operands, for rows that are not finite
+  const double *A, *W, *der, *B;  // the FP64 operands, for plain dot products
   int lda, g, ldd, ldb;
   uint32_t tmem_cols;
   int *err;
@@ -277,14 +342,26 @@ __device__ __forceinline__ void tmem_wait_ld() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-// The FP64 dot product of one element whose row or column is not finite.
-__device__ __noinline__ double plain_dot(const Gemm64Params &p, int g0, int row, int col) {
-  const double *y = p.B + (size_t)(g0 + col) * p.ldb;
-  const int gr = p.row0 + row;
-  const double *x = p.A ? p.A + (size_t)(g0 + row) * p.lda : p.W + (size_t)(gr % p.g) * p.K;
-  const double *d = p.A ? nullptr : p.der + (size_t)(gr / p.g) * p.ldd;
-  double v = 0.0;
-  for (int k = 0; k < p.K; ++k) v += (d ? x[k] * d[k] : x[k]) * y[k];
+// The plain FP64 dot products of the lanes in `redo` (a warp's outputs, lane l at
+// (row, col) of its own arguments), each by the whole warp: a lone lane's chain of K
+// multiply-adds takes the FP64 pipe as long as 32 of them.  Every lane returns v or
+// its own product.
+__device__ __noinline__ double plain_dots(const Gemm64Params &p, int g0, int row, int col,
+                                          unsigned redo, double v) {
+  const int lane = threadIdx.x & 31;
+  for (; redo; redo &= redo - 1) {
+    const int l = __ffs(redo) - 1;
+    const int r = __shfl_sync(0xffffffffu, row, l), c = __shfl_sync(0xffffffffu, col, l);
+    const double *y = p.B + (size_t)(g0 + c) * p.ldb;
+    const int gr = p.row0 + r;
+    const double *x = p.A ? p.A + (size_t)(g0 + r) * p.lda : p.W + (size_t)(gr % p.g) * p.K;
+    const double *d = p.A ? nullptr : p.der + (size_t)(gr / p.g) * p.ldd;
+    double s = 0.0;
+    for (int k = lane; k < p.K; k += 32) s += (d ? x[k] * d[k] : x[k]) * y[k];
+#pragma unroll
+    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == l) v = s;
+  }
   return v;
 }
 
@@ -304,6 +381,7 @@ __device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t addr) {
 template <int BN, bool kGram, class Epi>
 __global__ void __launch_bounds__(kGemm64Threads, 1)
     k_gemm64(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+             const __grid_constant__ CUtensorMap tmAc, const __grid_constant__ CUtensorMap tmBc,
              const Gemm64Params p, const Epi epi) {
   constexpr int NC = BN / 2;                       // columns of an epilogue warp
   constexpr uint32_t kBBytes = kDigits * BN * kKB * 2;
@@ -333,6 +411,7 @@ __global__ void __launch_bounds__(kGemm64Threads, 1)
     return !kGram || n0 < m0 + kBM;  // false: above the diagonal
   };
   constexpr int kChunkB = kChunkK / kKB;           // stages per exact accumulation
+  const int nck = kGram ? 0 : (p.ncb + kDigits - 1) / kDigits;  // stages of the magnitudes
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
@@ -366,7 +445,7 @@ __global__ void __launch_bounds__(kGemm64Threads, 1)
       for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
         int g0, m0, n0;
         if (!tile(t, g0, m0, n0)) continue;
-        for (int kb = 0; kb < p.nkb; ++kb, ++g) {
+        for (int kb = 0; kb < p.nkb + nck; ++kb, ++g) {
           const int s = g % kStages;
           if (!mbar_wait(smem_u32(&bars[kStages + s]), ((uint32_t)(g / kStages) & 1u) ^ 1u,
                          abort_flag)) {
@@ -377,8 +456,13 @@ __global__ void __launch_bounds__(kGemm64Threads, 1)
           }
           const uint32_t full = smem_u32(&bars[s]), sa = base + s * kStage;
           mbar_expect_tx(full, kStage);
-          tma_load_3d(sa, &tmA, kb * kKB, g0 + m0, 0, full);
-          tma_load_3d(sa + kABytes, &tmB, kb * kKB, g0 + n0, 0, full);
+          if (kb < p.nkb) {
+            tma_load_3d(sa, &tmA, kb * kKB, g0 + m0, 0, full);
+            tma_load_3d(sa + kABytes, &tmB, kb * kKB, g0 + n0, 0, full);
+          } else {
+            tma_load_3d(sa, &tmAc, 0, g0 + m0, (kb - p.nkb) * kDigits, full);
+            tma_load_3d(sa + kABytes, &tmBc, 0, g0 + n0, (kb - p.nkb) * kDigits, full);
+          }
         }
       }
       if (*abort_flag)  // let the copies already issued land
@@ -392,7 +476,8 @@ __global__ void __launch_bounds__(kGemm64Threads, 1)
       for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
         int g0, m0, n0;
         if (!tile(t, g0, m0, n0)) continue;
-        for (int kb0 = 0; kb0 < p.nkb && ok; kb0 += kChunkB, ++j) {
+        // the chunks, then the magnitudes' stages [nkb, nkb + nck)
+        for (int kb0 = 0; kb0 < p.nkb + nck && ok; ++j) {
           if (!mbar_wait(acc_empty, ((uint32_t)j & 1u) ^ 1u, abort_flag)) {
             *abort_flag = 1;
             atomicOr(p.err, 8);
@@ -400,7 +485,8 @@ __global__ void __launch_bounds__(kGemm64Threads, 1)
             break;
           }
           fence_after();
-          const int kb1 = min(p.nkb, kb0 + kChunkB);
+          const bool mags = kb0 >= p.nkb;
+          const int kb1 = mags ? p.nkb + nck : min(p.nkb, kb0 + kChunkB);
           for (int kb = kb0; kb < kb1; ++kb, ++g) {
             const int s = g % kStages;
             if (!mbar_wait(smem_u32(&bars[s]), (uint32_t)(g / kStages) & 1u, abort_flag)) {
@@ -413,6 +499,17 @@ __global__ void __launch_bounds__(kGemm64Threads, 1)
             fence_after();
             const uint32_t sa = base + s * kStage;
             const uint64_t ad = smem_desc_sw64(sa), bd = smem_desc_sw64(sa + kABytes);
+            if (!kGram && mags) {
+              const int nblk = min(kDigits, p.ncb - (kb - p.nkb) * kDigits);
+              for (int i = 0; i < nblk; ++i)
+#pragma unroll
+                for (int kk = 0; kk < kKB / 16; ++kk)
+                  mma_bf16(tmem, ad + (uint64_t)(i * kBM * kKB * 2 / 16 + 2 * kk),
+                           bd + (uint64_t)(i * BN * kKB * 2 / 16 + 2 * kk), idesc_bf16(kBM, BN),
+                           (kb > kb0 || i > 0 || kk > 0) ? 1u : 0u);
+              mma_commit(smem_u32(&bars[kStages + s]));
+              continue;
+            }
 #pragma unroll
             for (int kk = 0; kk < kKB / 16; ++kk) {
 #pragma unroll
@@ -431,6 +528,7 @@ __global__ void __launch_bounds__(kGemm64Threads, 1)
             mma_commit(smem_u32(&bars[kStages + s]));
           }
           if (ok) mma_commit(acc_full);
+          kb0 = kb1;
         }
       }
       if (!ok) {  // drain the MMAs already issued
@@ -456,7 +554,7 @@ __global__ void __launch_bounds__(kGemm64Threads, 1)
         acc[c] = 0;
         low[c] = 0;
       }
-      for (int kb0 = 0; kb0 < p.nkb; kb0 += kChunkB, ++j) {
+      auto wait_acc = [&]() {
         int okl = 0;
         if (lane == 0) okl = mbar_wait(acc_full, (uint32_t)j & 1u, abort_flag) ? 1 : 0;
         if (__shfl_sync(0xffffffffu, okl, 0) == 0) {
@@ -465,10 +563,19 @@ __global__ void __launch_bounds__(kGemm64Threads, 1)
             atomicOr(p.err, 8);
           }
           ok = false;
-          break;
         }
         fence_after();
-        const uint32_t tacc = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(half * NC);
+      };
+      auto free_acc = [&]() {
+        fence_before();
+        __syncwarp();
+        if (lane == 0)
+          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(acc_empty) : "memory");
+      };
+      const uint32_t tacc = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(half * NC);
+      for (int kb0 = 0; kb0 < p.nkb; kb0 += kChunkB, ++j) {
+        wait_acc();
+        if (!ok) break;
 #pragma unroll
         for (int c0 = 0; c0 < NC; c0 += 8) {
           int v[kDigits][8];
@@ -486,36 +593,56 @@ __global__ void __launch_bounds__(kGemm64Threads, 1)
             low[c0 + e] &= 0xfffffffu;
           }
         }
-        fence_before();
-        __syncwarp();
-        if (lane == 0)
-          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(acc_empty) : "memory");
+        free_acc();
       }
       if (!ok) break;
-      const int ea = row < rows ? p.ea[g0 + row] : 0;
-      bool odd = ea == kBadRow;  // a row of A or of B that is not finite
+      uint32_t redo = 0;  // bit c: this row's output in column n0 + c is a plain dot product
+      if constexpr (!kGram) {
+        wait_acc();  // the sums of magnitudes
+        if (!ok) break;
+#pragma unroll
+        for (int c0 = 0; c0 < NC; c0 += 8) {
+          int v[8];
+          tmem_ld8(tacc + (uint32_t)c0, v);
+          tmem_wait_ld();
+#pragma unroll
+          for (int e = 0; e < 8; ++e)
+            redo |= (__int_as_float(v[e]) >= kLeast ? 0u : 1u) << (c0 + e);
+        }
+        free_acc();
+        ++j;
+      }
+      int ea = row < rows ? p.ea[g0 + row] : kZeroRow;
+      if (ea == kZeroRow) redo = ea = 0;
+      const bool bad = ea == kBadRow;
+      if (bad) ea = 0;
       constexpr int kS = NC < 16 ? NC : 16;  // columns staged at a time
 #pragma unroll
       for (int c0 = 0; c0 < NC; c0 += kS) {
         if (n0 + c0 >= p.N) break;
 #pragma unroll
         for (int c = 0; c < kS; ++c) {
-          const int eb = n0 + c0 + c < p.N ? p.eb[g0 + n0 + c0 + c] : 0;
-          const bool any = ea == kBadRow || eb == kBadRow;
-          odd |= any;
+          int eb = n0 + c0 + c < p.N ? p.eb[g0 + n0 + c0 + c] : 0;
+          if (eb == kZeroRow) {
+            redo &= ~(1u << (c0 + c));
+            eb = 0;
+          }
+          if (bad || eb == kBadRow) {
+            redo |= 1u << (c0 + c);
+            eb = 0;
+          }
           stg[lane * 16 + ((((c >> 1) ^ (lane & 7)) << 1) | (c & 1))] =
-              any ? 0.0 : scaled_to_f64(acc[c0 + c], low[c0 + c], ea + eb - 35);
+              scaled_to_f64(acc[c0 + c], low[c0 + c], ea + eb - 35);
         }
-        const bool plain = __any_sync(0xffffffffu, odd);
         __syncwarp();
         for (int q = lane; q < 32 * kS; q += 32) {
           const int r = q / kS, c = q % kS, col = n0 + c0 + c;
-          if (row0 + r < rows && col < p.N && (!kGram || col <= row0 + r)) {
-            double v = stg[r * 16 + ((((c >> 1) ^ (r & 7)) << 1) | (c & 1))];
-            if (plain && (p.ea[g0 + row0 + r] == kBadRow || p.eb[g0 + col] == kBadRow))
-              v = plain_dot(p, g0, row0 + r, col);
-            epi(p.row0 + g0 + row0 + r, col, v);
-          }
+          const bool in = row0 + r < rows && col < p.N && (!kGram || col <= row0 + r);
+          double v = stg[r * 16 + ((((c >> 1) ^ (r & 7)) << 1) | (c & 1))];
+          const uint32_t of_row = __shfl_sync(0xffffffffu, redo, r);
+          const unsigned lanes = __ballot_sync(0xffffffffu, in && (of_row >> (c0 + c) & 1u));
+          if (lanes) v = plain_dots(p, g0, row0 + r, col, lanes, v);
+          if (in) epi(p.row0 + g0 + row0 + r, col, v);
         }
         __syncwarp();
       }
@@ -545,9 +672,9 @@ struct EpiSlot {
   }
 };
 
-// 3D map over digit planes: dims (K, rows, planes), box (32, box_rows, planes).
-bool make_digit_map(CUtensorMap *tm, const __nv_bfloat16 *ptr, int K, int rows, int ldp,
-                    size_t plane, int box_rows) {
+// 3D map with boxes of 32 columns x box_rows x eight
+bool make_map3(CUtensorMap *tm, const __nv_bfloat16 *ptr, const cuuint64_t dims[3],
+               const cuuint64_t strides[2], int box_rows) {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = [] {
     void *f = nullptr;
     cudaDriverEntryPointQueryResult q;
@@ -558,13 +685,29 @@ bool make_digit_map(CUtensorMap *tm, const __nv_bfloat16 *ptr, int K, int rows, 
                : nullptr;
   }();
   if (!fn) return false;
-  cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)rows, (cuuint64_t)kDigits};
-  cuuint64_t strides[2] = {(cuuint64_t)ldp * 2, (cuuint64_t)plane * 2};
   cuuint32_t box[3] = {(cuuint32_t)kKB, (cuuint32_t)box_rows, (cuuint32_t)kDigits};
   cuuint32_t es[3] = {1, 1, 1};
   return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, (void *)ptr, dims, strides, box, es,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// ... over digit planes: dims (K, rows, planes)
+bool make_digit_map(CUtensorMap *tm, const __nv_bfloat16 *ptr, int K, int rows, int ldp,
+                    size_t plane, int box_rows) {
+  const cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)rows, (cuuint64_t)kDigits};
+  const cuuint64_t strides[2] = {(cuuint64_t)ldp * 2, (cuuint64_t)plane * 2};
+  return make_map3(tm, ptr, dims, strides, box_rows);
+}
+
+
+// ... and over the magnitudes behind them, 32 columns to a block: dims (32, rows, blocks)
+// (their rows are whole blocks, padded with zeros), box (32, box_rows, eight blocks).
+bool make_check_map(CUtensorMap *tm, const __nv_bfloat16 *ptr, int ldc, int rows, size_t plane,
+                    int box_rows) {
+  const cuuint64_t dims[3] = {(cuuint64_t)kKB, (cuuint64_t)rows, (cuuint64_t)(ldc / kKB)};
+  const cuuint64_t strides[2] = {(cuuint64_t)ldc * 2, (cuuint64_t)kKB * 2};
+  return make_map3(tm, ptr + kDigits * plane, dims, strides, box_rows);
 }
 
 template <int BN, bool kGram, class Epi>
@@ -576,6 +719,8 @@ cudaError_t run_gemm64_t(const Gemm64Args &a, const Epi &epi, cudaStream_t st) {
   p.K = a.K;
   p.row0 = a.row0;
   p.nkb = (a.K + kKB - 1) / kKB;
+  const int ldc = check_pitch(a.K, a.B.group);
+  p.ncb = ldc / kKB;
   p.ea = a.ea;
   p.eb = a.B.ex;
   p.A = a.Asrc;
@@ -588,10 +733,18 @@ cudaError_t run_gemm64_t(const Gemm64Args &a, const Epi &epi, cudaStream_t st) {
   p.ldb = a.B.ld;
   p.err = a.err;
   p.tmem_cols = kDigits * BN;
-  CUtensorMap tmA, tmB;
+  CUtensorMap tmA, tmB, tmAc, tmBc;
+  const int rows_b = kGram ? a.M : a.N;
   if (!make_digit_map(&tmA, a.A, a.K, a.M, a.ldp, a.plane, kBM) ||
-      !make_digit_map(&tmB, a.B.d, a.K, kGram ? a.M : a.N, a.B.ldp, a.B.plane, BN))
+      !make_digit_map(&tmB, a.B.d, a.K, rows_b, a.B.ldp, a.B.plane, BN))
     return cudaErrorInvalidValue;
+  if (kGram) {  // never used
+    tmAc = tmA;
+    tmBc = tmB;
+  } else if (!make_check_map(&tmAc, a.A, ldc, a.M, a.plane, kBM) ||
+             !make_check_map(&tmBc, a.B.d, ldc, rows_b, a.B.plane, BN)) {
+    return cudaErrorInvalidValue;
+  }
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -604,7 +757,8 @@ cudaError_t run_gemm64_t(const Gemm64Args &a, const Epi &epi, cudaStream_t st) {
   const int ntn = (a.N + BN - 1) / BN;
   const int tiles = kGram ? a.M / a.N * ((a.N + kBM - 1) / kBM) * ntn
                           : ((a.M + kBM - 1) / kBM) * ntn;
-  return launch_pdl_n(tiles, k, std::min(tiles, sms), kGemm64Threads, smem, st, tmA, tmB, p, epi);
+  return launch_pdl_n(tiles, k, std::min(tiles, sms), kGemm64Threads, smem, st, tmA, tmB, tmAc,
+                      tmBc, p, epi);
 }
 
 template <class Epi>
@@ -622,14 +776,17 @@ cudaError_t run_gemm64(const Gemm64Args &a, const Epi &epi, cudaStream_t st) {
 }  // namespace
 
 int digit_pitch(int K) { return (K + 7) & ~7; }
+size_t digit_bytes(size_t rows, int K, int group) {
+  return rows * (2 * ((size_t)kDigits * digit_pitch(K) + check_pitch(K, group)));
+}
 
 cudaError_t launch_split64(int rows, int K, const double *src, int ld, const double *W,
                            const double *der, int g, int ldd, int row0, const int *fk, int fsign,
                            __nv_bfloat16 *dst, int ldp, size_t plane,
-                           int *ex, cudaStream_t st) {
+                           int *ex, cudaStream_t st, Magnitudes mags) {
   if (rows <= 0) return cudaSuccess;
   if (K <= 0 || ldp < K || (ldp & 7) || (plane & 7)) return cudaErrorInvalidValue;
-  SplitArgs a{rows, K, ldp, plane, src, ld, W, der, g, ldd, row0, fk, fsign, dst, ex};
+  SplitArgs a{rows, K, ldp, plane, src, ld, W, der, g, ldd, row0, fk, fsign, mags, dst, ex};
   const int grid = (rows + 7) / 8;
   auto k = ldp <= 128 ? k_split64<1> : ldp <= 256 ? k_split64<2> : ldp <= 512 ? k_split64<4>
                                                                               : k_split64<0>;
@@ -638,6 +795,13 @@ cudaError_t launch_split64(int rows, int K, const double *src, int ld, const dou
 
 cudaError_t launch_col_exp(int rows, int K, const double *B, int ld, int *fk, cudaStream_t st) {
   k_col_exp<<<(K + 127) / 128, 128, 0, st>>>(rows, K, B, ld, fk);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_count_sparse(int rows, int K, const __nv_bfloat16 *digits, size_t plane,
+                                const int *ex, int *sparse, cudaStream_t st) {
+  k_count_sparse<<<(rows + 7) / 8, 256, 0, st>>>(
+      rows, K, reinterpret_cast<const uint16_t *>(digits + kDigits * plane), ex, sparse);
   return cudaGetLastError();
 }
 

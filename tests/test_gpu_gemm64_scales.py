@@ -106,3 +106,76 @@ def test_a_row_that_is_not_finite_reaches_every_product_with_it(dino):
     finally:
         ctx.close()
     assert not np.any(np.isfinite(out["eigvals"]))
+
+
+# Pairs of outputs and inputs whose large entries do not meet: (what, W0, W1, x) of
+# r inputs, h hidden units, dy outputs.
+
+
+def _one_large_input(rng, r, h, dy, size):
+    W = [rng.standard_normal((h, r)), rng.standard_normal((dy, h))]
+    W[0][::2, 3] = 0.0                     # half of the units ignore the large input
+    W[1][::3, 8] = 0.0
+    W[1][:, 8] *= size
+    x = rng.standard_normal((3, r))
+    x[:, 3] = size
+    return W, x
+
+
+def _blocks(rng, r, h, dy, size):
+    W = [rng.standard_normal((h, r)), rng.standard_normal((dy, h))]
+    W[0][: h // 2, r // 2:] = 0.0          # two groups of inputs, three of units
+    W[0][h // 2: h // 2 + 9, : r // 2] = 0.0
+    W[1][: dy // 2, : h // 2] = 0.0
+    W[0][: h // 2] *= size
+    x = rng.standard_normal((3, r))
+    x[:, : r // 2] *= size
+    return W, x
+
+
+def _pruned(rng, r, h, dy, size):
+    W = [rng.standard_normal((h, r)) * (rng.random((h, r)) < 0.05),
+         rng.standard_normal((dy, h)) * (rng.random((dy, h)) < 0.05)]
+    x = rng.standard_normal((3, r)) * size ** rng.uniform(-1, 1, (3, r))
+    return W, x
+
+
+def _all_scales(rng, r, h, dy, size):
+    s = lambda *n: rng.standard_normal(n) * size ** rng.uniform(-1, 1, n)
+    return [s(h, r), s(dy, h)], s(3, r)
+
+
+def _selection(rng, r, h, dy, size):
+    W = [np.zeros((h, r)), np.zeros((dy, h))]
+    W[0][np.arange(h), rng.integers(0, r, h)] = 1.0
+    W[1][np.arange(dy), rng.integers(0, h, dy)] = 1.0
+    return W, rng.standard_normal((3, r)) * size ** rng.uniform(-1, 1, (3, r))
+
+
+@pytest.mark.parametrize("size", [1e2, 1e6, 1e9, 1e40])
+@pytest.mark.parametrize("make", [_one_large_input, _blocks, _pruned, _all_scales, _selection])
+@pytest.mark.parametrize("r,h,dy", [(130, 200, 129), (200, 400, 100), (65, 1030, 40),
+                                    (40, 513, 200)])
+def test_large_entries_that_meet_small_ones(dino, make, r, h, dy, size):
+    W, x = make(np.random.default_rng(14), r, h, dy, size)
+    _check(_eval(dino, W, x), W, x)
+
+
+@pytest.mark.parametrize("tiny", [1e-308, 3e-310, 5e-324])
+def test_subnormal_entries(dino, tiny):
+    """Entries at the bottom of the range, alone in a row and beside others."""
+    rng = np.random.default_rng(15)
+    r, h, dy = 130, 200, 129
+    W = [1e150 * rng.standard_normal((h, r)), rng.standard_normal((dy, h))]
+    x = np.stack([np.full(r, tiny), np.where(np.arange(r) % 2, tiny, 1e-300),
+                  np.where(np.arange(r) % 2, tiny, 1.0)])
+    W[0][:60, ::2] = 0.0                   # units that see only the tiny entries
+    out = _eval(dino, W, x)
+    a0, a1 = np.abs(W[0]), np.abs(W[1])
+    f, fs = (x @ W[0].T) @ W[1].T, (np.abs(x) @ a0.T) @ a1.T
+    assert np.all(np.abs(out["f"] - f) <= 4 * (h + r + 16) * EPS * fs)
+    W[0][:, 7] = 4 * tiny                  # a column of weights
+    W[1][5] *= tiny                        # a row of them
+    out = _eval(dino, W, np.ones((1, r)))
+    J, Js = W[1] @ W[0], np.abs(W[1]) @ np.abs(W[0])
+    assert np.all(np.abs(out["J"][0] - J) <= 4 * (h + 8) * (EPS * Js + 5e-324))
