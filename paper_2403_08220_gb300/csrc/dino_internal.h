@@ -237,7 +237,8 @@ size_t prior_draw_smem_bytes(int n, int elem);
 // caller's, indexed like the Philox ones.  With `only`, chains c with
 // only[c] == 0 draw nothing (their rows keep earlier contents).  With `overlap`
 // the draw may run while the kernel before it on the stream still does (pdl.cuh;
-// it stores after that kernel's end): sqrtlam, S and ext_z must not come from it.
+// it stores, and reads `only`, after that kernel's end): sqrtlam, S and ext_z must
+// not come from it.
 template <typename T>
 cudaError_t launch_prior_draw(int C, int n, const T *sqrtlam, const T *S, uint64_t seed,
                               uint64_t id_base, uint32_t stream, uint32_t step, T *out,

@@ -135,10 +135,10 @@ __global__ void __launch_bounds__(kPriorThreads, sizeof(T) == 4 ? 4 : 2)
     k_prior_draw(int n, const T *__restrict__ sqrtlam, const T *__restrict__ S, uint64_t seed,
                  uint64_t id_base, uint32_t stream, uint32_t step, T *out, int ldo,
                  __nv_bfloat16 *ms, int ldms, size_t ms_plane, int ms_slices,
-                 const double *__restrict__ ext_z, const int *__restrict__ only) {
-  if (only) {
+                 const double *__restrict__ ext_z, const int *only) {
+  if (only) {  // flags of the kernel before this one: read behind the wait
     pdl_wait();
-    if (!only[blockIdx.x]) return;  // the whole CTA: this chain draws nothing
+    if (!pdl_after(only)[blockIdx.x]) return;  // the whole CTA: this chain draws nothing
   }
   extern __shared__ __align__(16) unsigned char smraw[];
   const int ld = prior_ld(n), nt = ld / 4, NN = ld * ld;
