@@ -2090,8 +2090,8 @@ static int nuclear_terms(dino_ctx *ctx, int d, double *A, double *sig, double *Y
 static void gram64(dino_ctx *ctx, const char *name, int d, int K, const double *X, double *H,
                    cudaStream_t st) {
   std::vector<std::pair<void *, size_t>> tmp;
-  const DigitMat g = make_digits(ctx, tmp, X, d, K, false);
   try {
+    const DigitMat g = make_digits(ctx, tmp, X, d, K, false);
     if (g.d) {
       int *err = (int *)dev_alloc(ctx, 16);
       tmp.push_back({err, 16});
