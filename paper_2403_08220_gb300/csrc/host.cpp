@@ -2044,7 +2044,7 @@ static int jacobi(dino_ctx *ctx, int d, double *G, double *Q, double *sig, int *
     if (!any) break;
   }
   launch(ctx, st, "jacobi_norms", [&] { return launch_col_norms(d, G, sig, st); });
-  return sweep + 1;
+  return std::min(sweep + 1, kMaxJacobiSweeps);
 }
 
 // The nuclear norm's terms (sig, d values that sum to |A|_*) of a d x d matrix A

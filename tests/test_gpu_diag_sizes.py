@@ -126,3 +126,25 @@ def test_nuclear_norm_by_polar_factor_or_jacobi(dino, d, span, polar):
     assert (out["jacobi_sweeps"] == 0) == polar
     tol = (1e-9 if span < 10 else 2e-8 * np.sqrt(d)) * np.trace(V)
     assert abs(out["mpsrf_w"] - dg.wasserstein_mpsrf(W, V)) <= tol
+
+
+@pytest.mark.parametrize("d", [4, 7, 520])
+def test_degrees_of_freedom_of_very_different_scales(dino, d):
+    """Scales down to 1e-30, whose column pairs meet at angles below 1e-45: the
+    sweeps reported are at most the sixty that there are, and the result is the
+    oracle's for the others (what the small ones add is below 1e-23 of it)."""
+    rng = np.random.default_rng(d)
+    n_c, n_s = 4, max(40, d)
+    X = rng.standard_normal((n_c, n_s, d)) + 0.3 * rng.standard_normal((n_c, 1, d))
+    X *= 10.0 ** np.where(np.arange(d) % 2, -24.0 - 6.0 * np.arange(d) / d, 0.0)
+    ctx = dino.dino_init(0)
+    try:
+        g = dino.dino_diag_create(ctx, n_c, d, n_s)
+        for j in range(n_s):
+            dino.dino_diag_push(ctx, g, X[:, j, :])
+        out = dino.dino_diag_compute(ctx, g, d, mpsrf=True)
+    finally:
+        ctx.close()
+    W, V = dg.covariance_estimators(X[:, :, ::2])
+    assert abs(out["mpsrf_w"] - dg.wasserstein_mpsrf(W, V)) <= 1e-9 * np.trace(V)
+    assert 1 <= out["jacobi_sweeps"] <= 60
