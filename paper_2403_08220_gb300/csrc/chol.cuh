@@ -690,7 +690,8 @@ __device__ __forceinline__ double warp_sum(double v) {
 // rotation has to be orthogonal in FP64, so c = (1 + t^2)^-1/2 is an FP32
 // estimate y with one third-order step y + y (e / 2 + 3 e^2 / 8), e = 1 - w y^2,
 // and FP64 divisions and square roots, long chains on a pipe of 16 cycles an
-// instruction, are left out.
+// instruction, are left out.  Angles below FP32's range are ga / (be - al) with
+// an FP32 reciprocal, c = 1.
 __device__ __forceinline__ void jacobi_rotation(double al, double be, double ga, double &c,
                                                 double &s, double &t) {
   const double dq = be - al;
@@ -700,7 +701,10 @@ __device__ __forceinline__ void jacobi_rotation(double al, double be, double ga,
   const float fg = (float)(ga * sc);
   c = 1.0;
   s = t = 0.0;
-  if (fg == 0.0f) return;
+  if (fabsf(fg) < 1e-30f) {
+    if (ga != 0.0) s = t = ga * sc * (double)(1.0f / (float)(dq * sc));  // |dq| sc is in [1, 2)
+    return;
+  }
   const float z = (float)(dq * sc) / (2.0f * fg), az = fabsf(z);
   const float ft =
       copysignf(az > 1e8f ? 0.5f / az : 1.0f / (az + sqrtf(1.0f + az * az)), z);

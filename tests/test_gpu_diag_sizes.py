@@ -148,3 +148,22 @@ def test_degrees_of_freedom_of_very_different_scales(dino, d):
     W, V = dg.covariance_estimators(X[:, :, ::2])
     assert abs(out["mpsrf_w"] - dg.wasserstein_mpsrf(W, V)) <= 1e-9 * np.trace(V)
     assert 1 <= out["jacobi_sweeps"] <= 60
+
+
+@pytest.mark.parametrize("d", [4, 520])
+def test_sweeps_end_with_degrees_of_freedom_of_very_different_scales(dino, d):
+    """... and the solve ends by itself (exact angles: 3 and 22 sweeps, against 5
+    and 13 on one scale) instead of turning the same pairs by nothing to the end."""
+    rng = np.random.default_rng(d)
+    n_c, n_s = 4, max(40, d)
+    X = rng.standard_normal((n_c, n_s, d)) + 0.3 * rng.standard_normal((n_c, 1, d))
+    X *= 10.0 ** np.where(np.arange(d) % 2, -24.0 - 6.0 * np.arange(d) / d, 0.0)
+    ctx = dino.dino_init(0)
+    try:
+        g = dino.dino_diag_create(ctx, n_c, d, n_s)
+        for j in range(n_s):
+            dino.dino_diag_push(ctx, g, X[:, j, :])
+        out = dino.dino_diag_compute(ctx, g, d, mpsrf=True)
+    finally:
+        ctx.close()
+    assert 1 <= out["jacobi_sweeps"] < 60
