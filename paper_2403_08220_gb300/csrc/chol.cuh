@@ -132,8 +132,20 @@ struct F64 {
   // r = 1 - x y^2 (y^2 is exact, the square of an FP32 number; the error left is
   // 5 e^3 / 2): four dependent FP64 operations, 64 cycles each, where two Newton
   // steps take eight
-  __device__ static void pivot(T x, T &d, T &id) {
-    const double y = (double)rsqrtf((float)x);
+  __device__ static void pivot(T x, T &d, T &id) { refine(x, (double)rsqrtf((float)x), d, id); }
+  // ... for x beyond FP32's range too, where the estimate is that of x 4^-k, times
+  // 2^-k (in the geometry kernels of small pools, whose pivots are a serial chain, the
+  // question costs 1.6 us of 126 a step)
+  __device__ static void pivot_any(T x, T &d, T &id) {
+    pivot(x, d, id);
+    const int ef = __double2hiint(x) >> 20;
+    if (ef < 897 || ef >= 1150) {
+      const int k = ef > 0 && ef < 0x7ff ? (ef - 1023) >> 1 : 0;  // 0: not positive or not finite
+      const double xs = __hiloint2double(__double2hiint(x) - k * (1 << 21), __double2loint(x));
+      refine(x, (double)rsqrtf((float)xs) * __hiloint2double((1023 - k) << 20, 0), d, id);
+    }
+  }
+  __device__ static void refine(T x, double y, T &d, T &id) {
     const double r = fma(-x, y * y, 1.0);
     id = fma(y * r, fma(0.375, r, 0.5), y);
     d = x * id;

@@ -88,7 +88,7 @@ __device__ bool eig_cholesky(int d, int ld, double *A) {
     const double piv = A[(size_t)q * ld + q];
     ok = ok && piv > 0.0;
     double root, inv;
-    F64::pivot(piv, root, inv);
+    F64::pivot_any(piv, root, inv);
     __syncthreads();  // everyone has read the pivot
     for (int i = q + threadIdx.x; i < d; i += blockDim.x)
       A[(size_t)q * ld + i] = i == q ? root : A[(size_t)q * ld + i] * inv;
