@@ -509,7 +509,8 @@ int dino_kernel_times(dino_ctx *ctx, char *names, double *total_ms, uint64_t *la
  *   (cudaGetSymbolAddress) with that device current, so make that first call
  *   before any stream capture on the device.
  * Every call shares the one array: calls whose kernels can overlap on the GPU
- *   (unordered streams) race on it, so order them on one stream.
+ *   (unordered streams) race on it, so order them on one stream (several host
+ *   threads may share it: a call's kernels are queued together).
  * Returns DINO_OK once the kernels are queued, DINO_ECUDA if a launch fails. */
 #define DINO_NOALLOC_SCRATCH_DOUBLES (1u << 20)
 

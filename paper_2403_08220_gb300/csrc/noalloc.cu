@@ -179,19 +179,19 @@ extern "C" int dino_surrogate_jacobian_noalloc(int n, int n_layers, const int *w
 
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return DINO_ECUDA;
-  double *scratch = nullptr;
-  {
-    std::lock_guard<std::mutex> lk(g_mu);
-    if (!g_addr[dev]) {
-      void *p = nullptr;
-      if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || !p) {
-        cudaGetLastError();
-        return DINO_ECUDA;
-      }
-      g_addr[dev] = (double *)p;
+  // Held to the last launch: the kernels of calls that host threads make on one
+  // stream must not alternate on the scratch, nor one call lower the
+  // shared-memory limit that another has just set.
+  std::lock_guard<std::mutex> lk(g_mu);
+  if (!g_addr[dev]) {
+    void *p = nullptr;
+    if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || !p) {
+      cudaGetLastError();
+      return DINO_ECUDA;
     }
-    scratch = g_addr[dev];
+    g_addr[dev] = (double *)p;
   }
+  double *scratch = g_addr[dev];
   // a point's slab: two activation buffers and every hidden layer's derivatives
   const cudaStream_t st = (cudaStream_t)stream;
   size_t hidden = 0;

@@ -43,3 +43,50 @@ def test_rows_and_chunks(widths, act, n):
     torch.cuda.synchronize()
     assert rel_err(ft.cpu().numpy(), f_ref) <= TOL
     assert rel_err(Jt.cpu().numpy(), J_ref) <= TOL
+
+
+def test_host_threads_share_a_stream():
+    """Calls of several threads on one stream: two networks, different numbers of
+    points (and so of rows per CTA and shared memory); every call's own results."""
+    torch = pytest.importorskip("torch")
+    import threading
+
+    import paper_2403_08220_gb300 as dino
+
+    dev = torch.device("cuda", 0)
+    st = torch.cuda.current_stream().cuda_stream
+    jobs = []
+    for k, (widths, n) in enumerate([([200, 400, 400, 100], 1), ([200, 400, 400, 100], 12),
+                                     ([30, 900, 70], 8), ([30, 900, 70], 2)]):
+        Ws, bs = mlp_weights(widths, 21 + k)
+        x = np.random.default_rng(k).standard_normal((n, widths[0]))
+        f_ref, zs = mlp.forward(Ws, bs, mlp.ACT_TANH, x)
+        t = lambda a: torch.tensor(a, dtype=torch.float64, device=dev).contiguous()
+        jobs.append(dict(widths=widths, n=n, W=[t(a) for a in Ws], b=[t(a) for a in bs], x=t(x),
+                         f=t(np.full((20, n, widths[-1]), np.nan)),
+                         J=t(np.full((20, n, widths[-1], widths[0]), np.nan)), f_ref=f_ref,
+                         J_ref=mlp.jacobian_reverse(Ws, mlp.ACT_TANH, zs)))
+    torch.cuda.synchronize()
+    failed = []
+
+    def work(j):
+        try:
+            for i in range(20):
+                dino.dino_surrogate_jacobian_noalloc(
+                    j["n"], j["widths"], mlp.ACT_TANH, [a.data_ptr() for a in j["W"]],
+                    [a.data_ptr() for a in j["b"]], j["x"].data_ptr(), j["f"][i].data_ptr(),
+                    j["J"][i].data_ptr(), st)
+        except Exception as e:
+            failed.append(e)
+
+    threads = [threading.Thread(target=work, args=(j,)) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not failed
+    for j in jobs:
+        for i in range(20):
+            assert rel_err(j["f"][i].cpu().numpy(), j["f_ref"]) <= TOL
+            assert rel_err(j["J"][i].cpu().numpy(), j["J_ref"]) <= TOL
