@@ -484,6 +484,11 @@ __global__ void k_mpsrf_final(int d, const double *__restrict__ W, const double 
   }
 }
 
+// Limits of the kernels' dynamic shared memory are set to the same value whatever
+// the call's size, so that contexts of several host threads cannot lower one
+// another's between the setting and the launch.
+constexpr int kStagedSmem = 200 * 1024;  // also the two blocks of columns of a Jacobi CTA
+
 int grid_for(size_t n) { return (int)std::min<size_t>((n + 255) / 256, 152 * 8) + 0; }
 
 // out[i r + q] = normal q of Philox (seed, stream, step 0, "chain" i), i < n
@@ -531,7 +536,7 @@ cudaError_t launch_diag_ess(int d, int n_c, int n_s, const double *traj, int max
   if (n_c < 2 || n_s < 2 || (size_t)n_c * 8 > 48 * 1024) return cudaErrorInvalidValue;
   // the centred samples in shared memory where they fit (two CTAs an SM up to 14000)
   const size_t staged = ((size_t)n_c * n_s + n_c) * 8;
-  const bool fits = staged <= 200 * 1024;
+  const bool fits = staged <= kStagedSmem;
   auto kernel = fits ? k_diag_ess<true> : k_diag_ess<false>;
   // More CTAs for a degree of freedom while the chip (two CTAs an SM) has room: the
   // slowest one, which may run all n_s lags, sets the time.  Each CTA of a cluster
@@ -554,7 +559,7 @@ cudaError_t launch_diag_ess(int d, int n_c, int n_s, const double *traj, int max
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)cfg.dynamicSmemBytes);
+                                       fits ? kStagedSmem : 48 * 1024);
   if (e != cudaSuccess) return e;
   return cudaLaunchKernelEx(&cfg, kernel, n_c, n_s, traj, max_s, means, ess, sqjump);
 }
@@ -632,7 +637,7 @@ static cudaError_t jacobi_round(int d, int rnd, double *G, double *Q, int *rotat
   const size_t smem = (size_t)2 * kB * d * sizeof(double) * (Q ? 2 : 1);
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k_jacobi_round<kB>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kStagedSmem);
     if (e != cudaSuccess) return e;
   }
   k_jacobi_round<kB><<<n / 2, kB * kPairThreads, smem, st>>>(d, nb, rnd, G, Q, rotated);
@@ -658,7 +663,7 @@ cudaError_t launch_psd_chol(int d, const double *W, const double *V, double *F, 
                             cudaStream_t st) {
   const size_t smem = (size_t)d * (kCholPanel + 2) * sizeof(double);
   cudaError_t e = cudaFuncSetAttribute(k_psd_chol, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+                                       kStagedSmem);
   if (e != cudaSuccess) return e;
   k_psd_chol<<<2, kCholThreads, smem, st>>>(d, W, V, F, C);
   return cudaGetLastError();

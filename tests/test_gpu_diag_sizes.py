@@ -167,3 +167,40 @@ def test_sweeps_end_with_degrees_of_freedom_of_very_different_scales(dino, d):
     finally:
         ctx.close()
     assert 1 <= out["jacobi_sweeps"] < 60
+
+
+def test_contexts_of_two_threads_with_different_sizes(dino):
+    """Calls of different sizes side by side, each in a context of its own: every
+    call succeeds and gives what it gives alone."""
+    import threading
+
+    runs, errors = {}, []
+
+    def compute(key, n_c, n_s, d, times):
+        try:
+            rng = np.random.default_rng(d)
+            X = rng.standard_normal((n_c, n_s, d))
+            ctx = dino.dino_init(0)
+            try:
+                g = dino.dino_diag_create(ctx, n_c, d, n_s)
+                for j in range(n_s):
+                    dino.dino_diag_push(ctx, g, X[:, j, :])
+                runs[key] = [dino.dino_diag_compute(ctx, g, d, mpsrf=True) for _ in range(times)]
+            finally:
+                ctx.close()
+        except Exception as e:
+            errors.append(e)
+
+    sizes = [(2, 2000, 40), (3, 60, 5), (2, 900, 300)]
+    for i, s in enumerate(sizes):
+        compute(("alone", i), *s, 1)
+    threads = [threading.Thread(target=compute, args=((i,) + s + (60,))) for i, s in enumerate(sizes)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors
+    for i in range(len(sizes)):
+        ref = runs["alone", i][0]
+        for out in runs[i]:
+            assert np.array_equal(out["ess"], ref["ess"]) and out["mpsrf_w"] == ref["mpsrf_w"]
