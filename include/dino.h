@@ -101,7 +101,10 @@ typedef struct dino_ctx dino_ctx;
 
 /* Create a context on CUDA device `device`.
  * hbm_budget_bytes: cap on device memory the context may allocate
- *   (0 = 90% of the device's free memory at init).
+ *   (0 = 90% of the device's free memory at init).  Beside it lie, like the code
+ *   and the CUDA context, the forms in which the tensor cores take the FP64
+ *   products' weights: up to 18 bytes per entry of each W_l and its transpose,
+ *   E and D (of E and E_t alone with DINO_PREC_BF16).
  * stream: a cudaStream_t (as void*) to launch on, or NULL for a new
  *   non-blocking stream owned by the context.  A caller stream stays owned by
  *   the caller and must outlive the context.

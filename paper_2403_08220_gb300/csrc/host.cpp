@@ -486,25 +486,31 @@ static T *sur_upload(dino_ctx *ctx, Surrogate *s, const T *host, size_t n) {
 // on how many chains share the product.
 constexpr long kDigitsMinWork = 16384;
 
-// Digits of a device matrix B, with its column exponents taken out unless the
-// same digits are to serve as A too.  Left empty where the rule above or the
-// HBM budget says no; its products then take the SIMT GEMM.
+// Digits of a device matrix B.  A surrogate's operands (counted = false) are
+// equilibrated by columns and lie beside the HBM budget: what fits it does not
+// depend on them, nor a product's route, and with it its last bits, on what else
+// it holds.  Digits for the time of one call (counted = true), which are to serve as
+// A too, count, and are left out where they do not fit.  Left empty, too, where
+// the rule above says no or the device has no memory left; the products then
+// take the SIMT GEMM.
 static DigitMat make_digits(dino_ctx *ctx, std::vector<std::pair<void *, size_t>> &allocs,
-                            const double *B, int rows, int K, bool equilibrate = true) {
+                            const double *B, int rows, int K, bool counted = false) {
   DigitMat m;
   if ((long)rows * K < kDigitsMinWork || rows < 32 || K < 32) return m;
+  const bool equilibrate = !counted;
   const int ldp = digit_pitch(K);
   const size_t plane = (size_t)rows * ldp;
   const size_t planes = digit_bytes(rows, K, 1);
-  const size_t bytes = (planes + ((size_t)rows + K + 1) * 4 + 15) & ~(size_t)15;
-  if (ctx->used + bytes > ctx->budget) return m;
+  // the planes, the exponents and a word of the caller's at the end
+  const size_t bytes = ((planes + ((size_t)rows + K + 1) * 4 + 15) & ~(size_t)15) + 16;
+  if (counted && ctx->used + bytes > ctx->budget) return m;
   void *p = nullptr;
   if (cudaMalloc(&p, bytes) != cudaSuccess) {
     cudaGetLastError();
     return m;
   }
-  ctx->used += bytes;
-  allocs.push_back({p, bytes});
+  if (counted) ctx->used += bytes;
+  allocs.push_back({p, counted ? bytes : 0});
   auto *d = (__nv_bfloat16 *)p;
   int *ex = (int *)((char *)p + planes), *fk = equilibrate ? ex + rows : nullptr;
   auto split = [&](Magnitudes mags) {
@@ -543,10 +549,10 @@ struct Left64 {
   int g = 1, ldd = 0;
 };
 
-// Scratch for the digits of A: free device memory of the caller's, and the
-// pool's own for a single row, taken where the other does not hold one (a few
-// chains with few observations), so that no product changes its route, and
-// with it its last bits, with the number of chains.
+// Scratch for the digits of A: free device memory of the caller's, and where
+// that may not hold a single row (a few chains with few observations) the pool's
+// own for one, so that no product changes its route, and with it its last bits,
+// with the number of chains.
 struct Scratch64 {
   void *p = nullptr;
   size_t bytes = 0;
@@ -561,7 +567,9 @@ static size_t digit_row_bytes(int K) { return digit_bytes(1, K, 1) + 32; }
 // 8.79 ms, 64 7.42, 80 7.38, 88 6.80, 96 7.02 ms).
 constexpr size_t kDigitsChunk = 88u << 20;
 
-static bool has_digits(const DigitMat &B, const Scratch64 &ws) { return B.d && ws.p && ws.row; }
+static bool has_digits(const DigitMat &B, const Scratch64 &ws) {
+  return B.d && ws.p && (ws.row || ws.bytes >= digit_row_bytes(B.ld));  // B.ld: the reduction
+}
 
 // The product on the tensor cores in chunks of rows: digits of A into the
 // scratch, then tc(args) for those rows.
@@ -1398,7 +1406,11 @@ static void layout_pool(Pool &p, bool assign) {
   int kmax = N;
   for (int x : s->widths) kmax = std::max(kmax, x);
   for (int x : s->tm.widths) kmax = std::max(kmax, x);
-  if (s->L >= 2) p.w.digit_row = take(digit_row_bytes(kmax));
+  // the buffers that hold digits: P, and J for the FP64 products in between
+  const size_t room = s->precision == DINO_PREC_FP64 ? std::min(p.w.p_bytes, p.w.j_bytes)
+                                                     : p.w.p_bytes;
+  const bool small = s->L >= 2 && room < digit_row_bytes(kmax);
+  p.w.digit_row = small ? take(digit_row_bytes(kmax)) : nullptr;
   p.da = s->tm.on;
   if (p.da) {
     const auto &t = s->tm;
@@ -2091,10 +2103,9 @@ static void gram64(dino_ctx *ctx, const char *name, int d, int K, const double *
                    cudaStream_t st) {
   std::vector<std::pair<void *, size_t>> tmp;
   try {
-    const DigitMat g = make_digits(ctx, tmp, X, d, K, false);
+    const DigitMat g = make_digits(ctx, tmp, X, d, K, true);
     if (g.d) {
-      int *err = (int *)dev_alloc(ctx, 16);
-      tmp.push_back({err, 16});
+      int *err = (int *)((char *)tmp[0].first + tmp[0].second - 16);
       CK(cudaMemsetAsync(err, 0, 16, st));
       Gemm64Args a;
       a.M = a.N = d;
