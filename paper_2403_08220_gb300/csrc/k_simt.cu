@@ -36,7 +36,8 @@ __global__ void __launch_bounds__(kGemmThreads)
   B = pdl_after(B);
   __shared__ T out[kT * kT];
   const int o = threadIdx.x / kKG, q = threadIdx.x % kKG;
-  const int row0 = blockIdx.x * kT, col0 = blockIdx.y * kT;
+  const int mt = (M + kT - 1) / kT;  // tiles by columns; one dimension, the others end at 65535
+  const int row0 = (int)(blockIdx.x % mt) * kT, col0 = (int)(blockIdx.x / mt) * kT;
   const T *a = A + (size_t)min(row0 + o / kT, M - 1) * lda;
   const T *b = B + (size_t)min(col0 + o % kT, N - 1) * ldb;
   T s0 = T(0), s1 = T(0);
@@ -63,11 +64,15 @@ cudaError_t run_gemm(int M, int N, int K, const T *A, int lda, const T *B, int l
                      cudaStream_t st) {
   if (M <= 0 || N <= 0) return cudaSuccess;
   if (K > 256) {  // long reductions: 16 threads per output, 4 x 4 tiles
-    dim3 grid((M + 3) / 4, (N + 3) / 4);
-    return launch_pdl(k_gemm<T, 4, 16, Epi>, grid, kGemmThreads, 0, st, M, N, K, A, lda, B, ldb, epi);
+    const long grid = (long)((M + 3) / 4) * ((N + 3) / 4);
+    if (grid > 0x7fffffffL) return cudaErrorInvalidValue;
+    return launch_pdl(k_gemm<T, 4, 16, Epi>, dim3((unsigned)grid), kGemmThreads, 0, st, M, N, K,
+                      A, lda, B, ldb, epi);
   } else {
-    dim3 grid((M + 7) / 8, (N + 7) / 8);
-    return launch_pdl(k_gemm<T, 8, 4, Epi>, grid, kGemmThreads, 0, st, M, N, K, A, lda, B, ldb, epi);
+    const long grid = (long)((M + 7) / 8) * ((N + 7) / 8);
+    if (grid > 0x7fffffffL) return cudaErrorInvalidValue;
+    return launch_pdl(k_gemm<T, 8, 4, Epi>, dim3((unsigned)grid), kGemmThreads, 0, st, M, N, K, A,
+                      lda, B, ldb, epi);
   }
 }
 

@@ -113,3 +113,27 @@ def test_points_do_not_depend_on_their_company(dino):
                 assert np.array_equal(one[q][0], many[q][k]), (k, q)
     finally:
         ctx.close()
+
+
+def test_more_hidden_units_than_a_grid_has_second_rows(dino):
+    """600000 hidden units between 16 inputs and 2 outputs: small products (no
+    digits) whose column tiles outnumber a grid's second dimension."""
+    widths = [16, 600000, 2]
+    W, b, rng = _weights(widths, 8)
+    x = rng.standard_normal((2, 16))
+    ctx = dino.dino_init(0)
+    try:
+        sid = _load(dino, ctx, 9, widths, 1, W, b)
+        out = dino.dino_surrogate_eval(ctx, sid, x, 2, want_L=False)
+    finally:
+        ctx.close()
+    z = x @ W[0].T + b[0]
+    t = np.tanh(z)
+    f = t @ W[1].T + b[1]
+    J = np.einsum("ih,nh,hr->nir", W[1], 1 - t * t, W[0], optimize=True)
+    # sums of 600000 terms of order 1/800: rounding errors of at most K eps of the
+    # sum of their magnitudes
+    tol = 4 * (600000 + 16) * EPS
+    assert np.all(np.abs(out["f"] - f) <= tol * (np.abs(t) @ np.abs(W[1]).T + np.abs(b[1])))
+    Js = np.einsum("ih,nh,hr->nir", np.abs(W[1]), 1 - t * t, np.abs(W[0]), optimize=True)
+    assert np.all(np.abs(out["J"] - J) <= tol * Js)
