@@ -369,7 +369,9 @@ __device__ void wb_store_factor(double *Lg, const typename A::T *Ms, const typen
 // path); this instantiation is kept lean in registers so that 1024 threads (64
 // registers each) fit an SM.
 template <typename TJ, bool kPre, int NT>
-__global__ void __launch_bounds__(NT, kPre ? 1024 / NT : kWbMinBlocks)
+__global__ void __launch_bounds__(NT, kPre               ? 1024 / NT
+                                      : NT > kWbThreads ? 1
+                                                        : kWbMinBlocks)
     k_wb_geometry(ReducedArgs a, int mode) {
   pdl_begin();
   using A = std::conditional_t<sizeof(TJ) == 4, DF, F64>;
@@ -858,6 +860,13 @@ cudaError_t launch_wb_geometry_t(const ReducedArgs &a, int mode, cudaStream_t st
              : nt == 128 ? launch_wb_geometry_k<TJ, true, 128>(a, mode, st)
                          : launch_wb_geometry_k<TJ, true, 256>(a, mode, st);
     }
+  if constexpr (sizeof(TJ) == 4) {
+    // wb_gram_rows holds kHMaxTiles tiles a thread: 128 threads up to d_y = 108, 512
+    // up to 220 (one CTA an SM fits either way)
+    const int nt = (a.d_y + kHT - 1) / kHT;
+    if (!a.G && nt * (nt + 1) / 2 > kHMaxTiles * kWbThreads)
+      return launch_wb_geometry_k<TJ, false, 512>(a, mode, st);
+  }
   return launch_wb_geometry_k<TJ, false, kWbThreads>(a, mode, st);
 }
 
