@@ -621,10 +621,14 @@ __global__ void __launch_bounds__(NT, sizeof(TJ) == 4 && !kBlk
 
 }  // namespace
 
+// What k_geometry may take of dynamic shared memory beside its static variables
+// (304 bytes).
+constexpr size_t kGeoSmem = kSmemLimit - 512;
+
 bool uses_global_factor(int r, int d_y) {
   const Layout lay(r, d_y, false);
   const size_t jc = (size_t)kJChunk * r * sizeof(double);
-  return r > kMaxRSmem || lay.tail * sizeof(double) + jc > kSmemLimit;
+  return r > kMaxRSmem || lay.tail * sizeof(double) + jc > kGeoSmem;
 }
 
 size_t propose_smem_bytes(int r) {
@@ -674,7 +678,7 @@ static int geometry_panel(int r, int d_y, int jf_f32, size_t &smem) {
                        : G     ? std::max(mma_panel_bytes(r + 1), (size_t)32 * r)
                                : mma_digit_bytes(r + 1);
   const size_t need = at * sizeof(double) + bytes;
-  if (need > kSmemLimit) return 0;
+  if (need > kGeoSmem) return 0;
   smem = G && jf_f32 ? need : std::max(smem, need);
   return (int)at;
 }

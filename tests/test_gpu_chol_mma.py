@@ -47,3 +47,33 @@ def test_factor_reproduces_the_matrix(r):
         ref = np.linalg.slogdet(M)[1] / 2
         tol = 2.0 ** -45 * max(r, 4) * np.sum(np.abs(np.linalg.inv(M)) * np.outer(s, s))
         assert abs(o["hld"][c] - ref) <= tol + 1e-13 * abs(ref)
+
+
+@pytest.mark.parametrize("r,dy,precision", [(204, 187, "bf16"), (204, 224, "bf16"),
+                                            (202, 690, "bf16"), (888, 40, "bf16"),
+                                            (885, 140, "bf16"), (200, 3630, "fp64")])
+def test_sizes_whose_shared_memory_ends_at_the_limit(r, dy, precision):
+    """The blocked factorisation's digits, or the staged rows of J, would end within
+    the last 304 bytes of a CTA's shared memory, which static variables hold."""
+    import paper_2403_08220_gb300 as dino
+
+    rng = np.random.default_rng(r)
+    h = 16
+    W = [rng.integers(-1, 2, size=(h, r)).astype(float),
+         rng.integers(-1, 2, size=(dy, h)).astype(float)]
+    n = int(np.ceil(np.sqrt(r))) + 1
+    ctx = dino.dino_init(0)
+    try:
+        sid = dino.dino_load_surrogate(
+            ctx, n_grid=n, prior_gamma=0.1, prior_delta=1.0, r=r, widths=[r, h, dy],
+            activation=0, W=W, b=[np.zeros(h), np.zeros(dy)], basis_kind=dino.DINO_BASIS_KLE,
+            y=np.zeros(dy), noise_var=64.0 * h * dy,
+            precision=dino.DINO_PREC_BF16 if precision == "bf16" else dino.DINO_PREC_FP64,
+            noise_map=dino.DINO_NOISE_CHOLESKY)
+        o = dino.dino_surrogate_eval(ctx, sid, rng.standard_normal((1, r)), dy, want_L=False)
+    finally:
+        ctx.close()
+    J = W[1] @ W[0]
+    assert np.array_equal(o["J"][0], J)
+    ref = np.linalg.slogdet(np.eye(r) + J.T @ J / (64.0 * h * dy))[1] / 2
+    assert abs(o["hld"][0] - ref) <= 1e-9 * max(1.0, abs(ref))
