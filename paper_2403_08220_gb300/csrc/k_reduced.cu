@@ -658,11 +658,15 @@ cudaError_t launch_propose(const ReducedArgs &a, cudaStream_t st) {
   return launch_pdl_n(chain_ctas(a.C), k_propose, a.C, kThreads, smem, st, a);
 }
 
-// r from which the smem-resident factor of an FP32 Jacobian takes the blocked
-// factorisation: at r = 128 it is the faster (1.60 against 2.02 ms for 4096 chains),
-// at r = 73 the slower (the four CTAs an SM of the plain one hide its chains of
-// dependent operations better: 2.85 against 2.60 ms for a step of 4089 chains).
-constexpr int kBlkMinR = 112;
+// Whether the smem-resident factor of an FP32 Jacobian takes the blocked
+// factorisation, by the CTAs an SM that either leaves room for (plain, blk).  The
+// plain one's chains of dependent operations need company: four CTAs of 256
+// threads, or two of 512, are the faster against fewer blocked ones; otherwise the
+// blocked one is.  2048 chains, d_y = r + 20, geometry in us, plain and blocked:
+// r = 106 (4, 2 CTAs) 522 653, 108 (3, 2) 727 649, 134 (2, 2) 999 875, 136 (2, 1)
+// 1045 1391, 156 (2, 1) 1323 1614, 160 (1, 1) 2062 1732, 200 (1, 1) 3079 2349.
+static bool takes_blocked(size_t plain, size_t blk) { return blk >= 2 ? plain < 4 : plain < 2; }
+static size_t ctas_an_sm(size_t smem) { return kSmemLimit / (smem + 1024); }
 
 // Where the blocked factorisations keep their digits or panel (elements from the
 // start of shared memory; 0 where they do not apply or fit), with smem raised
@@ -672,13 +676,14 @@ constexpr int kBlkMinR = 112;
 // with by then).
 static int geometry_panel(int r, int d_y, int jf_f32, size_t &smem) {
   const bool G = uses_global_factor(r, d_y);
-  if (!G && (!jf_f32 || r < kBlkMinR)) return 0;
+  if (!G && !jf_f32) return 0;
   const size_t at = Layout(r, d_y, G, G && jf_f32).tail;
   const size_t bytes = !jf_f32 ? (size_t)(r + 1) * kPanelLd * sizeof(double)
                        : G     ? std::max(mma_panel_bytes(r + 1), (size_t)32 * r)
                                : mma_digit_bytes(r + 1);
   const size_t need = at * sizeof(double) + bytes;
   if (need > kGeoSmem) return 0;
+  if (!G && !takes_blocked(ctas_an_sm(smem), ctas_an_sm(std::max(smem, need)))) return 0;
   smem = G && jf_f32 ? need : std::max(smem, need);
   return (int)at;
 }
@@ -704,7 +709,7 @@ template <typename TJ, bool G>
 static cudaError_t launch_geometry_t(const ReducedArgs &a, int mode, size_t smem,
                                      cudaStream_t st) {
   const int panel = geometry_panel(a.r, a.d_y, a.jf_f32, smem);
-  const size_t ctas = kSmemLimit / (smem + 1024);
+  const size_t ctas = ctas_an_sm(smem);
   if constexpr (G) {
     if (panel) return launch_geometry_nt<TJ, G, 256, true>(a, mode, smem, panel, st);
     return launch_geometry_nt<TJ, G, kThreads, false>(a, mode, smem, 0, st);
