@@ -491,11 +491,10 @@ int dino_kernel_times(dino_ctx *ctx, char *names, double *total_ms, uint64_t *la
  * It is meant for host code that must not call cudaMalloc: for example a
  * plugin inside a framework that owns every device byte through its own
  * pool, or a latency-critical loop in which the synchronisation that
- * cudaMalloc/cudaFree can imply is not acceptable.  The layers'
- * activations and derivatives live in a fixed device array of
+ * cudaMalloc/cudaFree can imply is not acceptable.  Intermediate values
+ * live in shared memory and in a fixed device array of
  * DINO_NOALLOC_SCRATCH_DOUBLES doubles (8 MiB) that every GPU loading the
- * library keeps until the process exits; the rows of the Jacobian's products
- * in shared memory.
+ * library keeps until the process exits.
  *
  * widths: host array of n_layers + 1 entries (widths[0] = r, widths[n_layers]
  *   = d_y), 1 <= n_layers <= 16; activation as in dino_surrogate_desc.
@@ -514,6 +513,8 @@ int dino_kernel_times(dino_ctx *ctx, char *names, double *total_ms, uint64_t *la
  * Every call shares the one array: calls whose kernels can overlap on the GPU
  *   (unordered streams) race on it, so order them on one stream (several host
  *   threads may share it: a call's kernels are queued together).
+ * Whether points take a CTA each or spread over the GPU depends on n, and with it
+ *   the order of their sums (the last bits).
  * Returns DINO_OK once the kernels are queued, DINO_ECUDA if a launch fails. */
 #define DINO_NOALLOC_SCRATCH_DOUBLES (1u << 20)
 

@@ -5,9 +5,8 @@
 // device byte through its own pool, or a latency-critical loop in which the
 // device-wide synchronisation that cudaMalloc/cudaFree may imply is not
 // acceptable.  The entry point below therefore never allocates.  Inputs and
-// outputs are device buffers the caller owns.  The activations and their
-// derivatives live in one file-scope device array of fixed size, the products
-// of the reverse-mode Jacobian in shared memory.
+// outputs are device buffers the caller owns.  Intermediate values live in one
+// file-scope device array of fixed size and in shared memory.
 // Every GPU that loads this library holds that array until the process exits.
 //
 // Set-up: the host cannot use the array's name as a device address (in host
@@ -33,7 +32,8 @@ namespace {
 
 constexpr int kMaxLayers = 16;
 constexpr int kMaxDevices = 64;
-constexpr int kJacThreads = 512;
+constexpr int kThreads = 256;     // a CTA of k_jac_point
+constexpr int kJacThreads = 512;  // ... of k_jac_rows
 
 static __device__ __align__(256) double g_noalloc_scratch[DINO_NOALLOC_SCRATCH_DOUBLES];
 
@@ -59,6 +59,77 @@ __device__ __forceinline__ double act_deriv(int kind, double z) {
     return 0.5 * (1.0 + erf(z * 0.70710678118654752440)) +
            z * exp(-0.5 * z * z) * 0.39894228040143267794;
   return 1.0;
+}
+
+// One CTA per point, for many points or a small network (spread_rows).  Shared
+// memory holds the activations and the activation derivatives; the d_y x w
+// products of the reverse sweep go to a per-point slab of the scratch array (two
+// ping-pong buffers of d_y * wmax doubles).
+__global__ void __launch_bounds__(kThreads)
+    k_jac_point(const Net net, int wmax, const double *__restrict__ x, double *__restrict__ f,
+                double *__restrict__ J, double *__restrict__ scratch) {
+  extern __shared__ double sm[];
+  const int p = blockIdx.x, L = net.L, r = net.w[0], dy = net.w[L];
+  double *a[kMaxLayers + 1];
+  double *d[kMaxLayers];
+  int off = 0;
+  for (int l = 0; l < L; ++l) {  // a[0..L-1]: layer inputs; d[0..L-2]: derivatives
+    a[l] = sm + off;
+    off += net.w[l];
+  }
+  for (int l = 0; l + 1 < L; ++l) {
+    d[l] = sm + off;
+    off += net.w[l + 1];
+  }
+  for (int i = threadIdx.x; i < r; i += blockDim.x) a[0][i] = x[(size_t)p * r + i];
+  __syncthreads();
+  for (int l = 0; l < L; ++l) {
+    const int wi = net.w[l], wo = net.w[l + 1];
+    const double *W = net.W[l];
+    for (int o = threadIdx.x; o < wo; o += blockDim.x) {
+      double z = net.b[l][o];
+      for (int i = 0; i < wi; ++i) z += W[(size_t)o * wi + i] * a[l][i];
+      if (l + 1 < L) {
+        a[l + 1][o] = act_fn(net.act, z);
+        d[l][o] = act_deriv(net.act, z);
+      } else {
+        f[(size_t)p * dy + o] = z;
+      }
+    }
+    __syncthreads();
+  }
+  double *Jp = J + (size_t)p * dy * r;
+  if (L == 1) {
+    for (int e = threadIdx.x; e < dy * r; e += blockDim.x) Jp[e] = net.W[0][e];
+    return;
+  }
+  double *P = scratch + (size_t)p * 2 * dy * wmax;
+  double *Q = P + (size_t)dy * wmax;
+  const int wl = net.w[L - 1];
+  for (int e = threadIdx.x; e < dy * wl; e += blockDim.x)
+    P[e] = net.W[L - 1][e] * d[L - 2][e % wl];
+  __syncthreads();
+  for (int l = L - 2; l >= 1; --l) {  // P <- (P W_l) .* d_{l-1}
+    const int wi = net.w[l], wo = net.w[l + 1];
+    const double *W = net.W[l];
+    for (int e = threadIdx.x; e < dy * wi; e += blockDim.x) {
+      const int i = e / wi, j = e % wi;
+      double acc = 0.0;
+      for (int k = 0; k < wo; ++k) acc += P[(size_t)i * wo + k] * W[(size_t)k * wi + j];
+      Q[e] = acc * d[l - 1][j];
+    }
+    __syncthreads();
+    double *t = P;
+    P = Q;
+    Q = t;
+  }
+  const int w1 = net.w[1];
+  for (int e = threadIdx.x; e < dy * r; e += blockDim.x) {  // J = P W_0
+    const int i = e / r, j = e % r;
+    double acc = 0.0;
+    for (int k = 0; k < w1; ++k) acc += P[(size_t)i * w1 + k] * net.W[0][(size_t)k * r + j];
+    Jp[e] = acc;
+  }
 }
 
 // One layer of the forward pass for every point of the chunk: a warp per
@@ -102,12 +173,7 @@ __global__ void __launch_bounds__(kJacThreads)
   extern __shared__ double sm[];
   const int p = blockIdx.y, L = net.L, r = net.w[0], dy = net.w[L];
   const int i0 = blockIdx.x * rows, nr = min(rows, dy - i0);
-  double *Jp = J + ((size_t)p * dy + i0) * r;
-  if (L == 1) {
-    for (int e = threadIdx.x; e < nr * r; e += blockDim.x)
-      Jp[e] = net.W[0][(size_t)i0 * r + e];
-    return;
-  }
+  double *Jp = J + ((size_t)p * dy + i0) * r;  // L >= 2
   const double *der = scratch + (size_t)p * slab + 2 * (size_t)wmax;
   int off = 0;  // of d_{l - 1} (layer widths w_1 .. w_{L - 1})
   for (int l = 1; l < L - 1; ++l) off += net.w[l];
@@ -136,6 +202,34 @@ __global__ void __launch_bounds__(kJacThreads)
     P = Q;
     Q = t;
   }
+}
+
+// Whether n points spread their outputs over all SMs (k_layer and k_jac_rows)
+// instead of taking a CTA each (k_jac_point): by the times of both, in us.  A
+// point's CTA runs its layers as chains of w multiply-adds (0.167 each) and the
+// Jacobian's multiply-adds on the FP64 pipe of its SM (0.31 per 1000), the same for
+// every point while each has an SM of its own.  Spread, a layer costs a launch, its
+// values and derivatives come from one lane a warp (1.16, 3.1 and 7.1 per 1000 hidden
+// units and point for the identity, tanh and GELU) and the Jacobian's multiply-adds
+// run on all SMs (0.0036 per 1000).  Fitted to 450 measured calls (16 networks of 1
+// to 11 layers, 4 to 3200 wide, 1 to 2000 points): the way taken is at most 9% slower
+// than a CTA per point, and at most 27% slower than the other way (at 150 points
+// of 200-400-400-1 with the identity, 257 against 203).  16-64-64-49, GELU, a CTA each
+// and spread: 1 point 96 and 45, 24 points 95 and 78, 48 points 96 and 116, 150 points 97
+// and 238; 12-30-7: 1 point 16 and 26, 1000 points 32 and 259; 200-400-400-100: 1 point
+// 8164 and 113, 8 points 8160 and 444.
+bool spread_rows(const Net &net, int n, int sms) {
+  const int L = net.L;
+  if (L < 2 || n > sms) return false;
+  double hidden = 0.0, macs = 0.0;  // multiply-adds of one point's Jacobian, in thousands
+  for (int l = 1; l < L; ++l) hidden += net.w[l];
+  for (int l = 0; l + 1 < L; ++l) macs += 1e-3 * net.w[L] * net.w[l] * net.w[l + 1];
+  const bool gelu = net.act == DINO_ACT_GELU, tanh = net.act == DINO_ACT_TANH;
+  const double value = gelu ? 7.1e-3 : tanh ? 3.1e-3 : 1.16e-3, layer = gelu ? 7.7 : tanh ? 2.4 : 0.0;
+  const double point = 9.8 + 0.31 * macs + 0.167 * (net.w[0] + hidden);
+  const double spread = 1.7 + 7.2 * L + 0.056 * hidden + layer * (L - 1) +
+                        n * (value * hidden + 0.0036 * macs);
+  return spread < point;
 }
 
 std::mutex g_mu;
@@ -192,23 +286,30 @@ extern "C" int dino_surrogate_jacobian_noalloc(int n, int n_layers, const int *w
     g_addr[dev] = (double *)p;
   }
   double *scratch = g_addr[dev];
-  // a point's slab: two activation buffers and every hidden layer's derivatives
   const cudaStream_t st = (cudaStream_t)stream;
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+    return DINO_ECUDA;
+  if (!spread_rows(net, n, sms)) {
+    if (smem > 48 * 1024 &&
+        cudaFuncSetAttribute(k_jac_point, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)smem) != cudaSuccess)
+      return DINO_ECUDA;
+    k_jac_point<<<n, kThreads, smem, st>>>(net, wmax, x, f, J, scratch);
+    return cudaGetLastError() == cudaSuccess ? DINO_OK : DINO_ECUDA;
+  }
+  // a point's slab: two activation buffers and every hidden layer's derivatives
   size_t hidden = 0;
   for (int l = 1; l < n_layers; ++l) hidden += widths[l];
   const int r = widths[0], dy = widths[n_layers];
   const size_t slab = 2 * (size_t)wmax + hidden;
-  const size_t most = slab ? (size_t)DINO_NOALLOC_SCRATCH_DOUBLES / slab : (size_t)n;
   // blockIdx.y runs over the points of a chunk
-  const int chunk = (int)std::min({most, (size_t)n, (size_t)65535});
-  int sms = 0;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
-    return DINO_ECUDA;
+  const int chunk = (int)std::min((size_t)DINO_NOALLOC_SCRATCH_DOUBLES / slab, (size_t)n);
   // rows per CTA: one CTA on every SM, within the shared memory of one CTA
   // (two buffers of rows x wmax; one row always fits, since the widths' sums do)
   const size_t row_bytes = 2 * (size_t)wmax * sizeof(double);
   size_t rows = ((size_t)std::min(n, chunk) * dy + sms - 1) / sms;
-  if (row_bytes) rows = std::min(rows, (size_t)(200 * 1024) / row_bytes);
+  rows = std::min(rows, (size_t)(200 * 1024) / row_bytes);
   rows = std::max<size_t>(1, std::min(rows, (size_t)dy));
   const size_t jsm = rows * row_bytes;
   if (jsm > 48 * 1024 &&

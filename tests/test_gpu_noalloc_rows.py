@@ -90,3 +90,16 @@ def test_host_threads_share_a_stream():
         for i in range(20):
             assert rel_err(j["f"][i].cpu().numpy(), j["f_ref"]) <= TOL
             assert rel_err(j["J"][i].cpu().numpy(), j["J_ref"]) <= TOL
+
+
+@pytest.mark.parametrize("widths,act,n", [
+    ([20, 9], mlp.ACT_TANH, 700),                    # a CTA per point: one layer,
+    ([3, 4, 2], mlp.ACT_GELU, 3000),                 # a small network,
+    ([16, 64, 64, 49], mlp.ACT_GELU, 48),            # many points;
+    ([16, 64, 64, 49], mlp.ACT_GELU, 24),            # rows over all SMs: fewer,
+    ([16, 64, 64, 49], mlp.ACT_IDENTITY, 90),        # cheaper activations,
+    ([20, 6000, 6000, 1], mlp.ACT_TANH, 60),         # more points than scratch slabs
+])
+def test_both_ways_of_taking_the_points(widths, act, n):
+    """... a CTA per point, or every point's outputs over all SMs."""
+    test_rows_and_chunks(widths, act, n)
