@@ -581,7 +581,7 @@ __device__ void cta_cholesky_panels(typename A::T *Ls, typename A::T *inv, int n
 }
 
 // The same factorisation for a packed matrix in global memory (r-sized path,
-// factors beyond one CTA's shared memory), blocked so that the trailing matrix
+// double-float factors too large for chol_mma.cuh's panel), blocked so that the trailing matrix
 // is read and written once per kWide columns: the panel of kWide columns lives
 // in shared memory (rows of kPanelLd elements), is factored there in 8-column
 // steps and written back, and the warps apply its rank-kWide update to 32-column

@@ -248,8 +248,8 @@ __device__ void cta_cholesky_mma(float2 *Ls, float2 *inv, int n, char *dig) {
   }
 }
 
-// The same for a packed matrix in global memory (the counterpart of
-// cta_cholesky_global, which serves FP64): the panel's rows live in shared
+// The same for a packed matrix in global memory (cta_cholesky_global is for those whose
+// panel of digits does not fit): the panel's rows live in shared
 // memory at a pitch of kDigTight bytes, are written back when solved, and their
 // digits take their place.  dig: n kDigTight bytes and the scales.
 __host__ __device__ inline size_t mma_panel_bytes(int n) {

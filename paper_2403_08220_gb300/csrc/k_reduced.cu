@@ -428,13 +428,13 @@ __global__ void __launch_bounds__(kGramThreads, 4) k_gram_f32(ReducedArgs a, int
 // an accepted chain to b: its factor slot (written only then, into the other
 // slot, which becomes current) and its state vectors.  The complement
 // coefficient b - s a is written for every chain.
-// The FP32-Jacobian instantiations find I + H in the slot (k_gram_f32).  kBlk: a
-// blocked factorisation, whose digits or panel lie at sm + panel (FP32
-// Jacobian: trailing updates on the tensor cores; FP64: factors in global
-// memory).  Otherwise 8-column panels, and with an FP32 Jacobian 64 registers a
-// thread, 32 warps an SM where shared memory allows.
-template <typename TJ, bool G, int NT, bool kBlk>
-__global__ void __launch_bounds__(NT, sizeof(TJ) == 4 && !kBlk
+// The FP32-Jacobian instantiations find I + H in the slot (k_gram_f32).  kFac: the
+// factorisation.  The blocked ones (FP32 Jacobian) keep their digits or panel at sm +
+// panel; the plain one has 64 registers a thread with an FP32 Jacobian, 32 warps an
+// SM where shared memory allows.
+enum Factor { kPlain, kMma, kPanels };  // 8-column panels; chol_mma.cuh; cta_cholesky_global
+template <typename TJ, bool G, int NT, Factor kFac>
+__global__ void __launch_bounds__(NT, sizeof(TJ) == 4 && kFac == kPlain
                                           ? 1024 / NT
                                           : (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
     k_geometry(ReducedArgs a, int mode, int panel) {
@@ -446,7 +446,8 @@ __global__ void __launch_bounds__(NT, sizeof(TJ) == 4 && !kBlk
   extern __shared__ __align__(16) double sm[];
   const int c = blockIdx.x, r = a.r, dy = a.d_y;
   const size_t ldL = slot_stride(r), lsz = tri_size(r + 1);
-  constexpr bool kLean = G && sizeof(TJ) == 4 && kBlk;
+  static_assert(kFac == kPlain || sizeof(TJ) == 4, "FP64 factors are plain");
+  constexpr bool kLean = G && kFac != kPlain;
   const Layout lay(r, dy, G, kLean);
   const int slot = mode == 0 ? a.cur[c] : 1 - a.cur[c];
   double *Lg = a.L + (size_t)slot * a.L_slot + (size_t)c * ldL;
@@ -537,9 +538,9 @@ __global__ void __launch_bounds__(NT, sizeof(TJ) == 4 && !kBlk
   vv = block_sum(vv, red);
   if (threadIdx.x == 0) Ls[tri(r) + r] = A::from(1.0 + vv);
   __syncthreads();
-  if constexpr (!kBlk)
+  if constexpr (kFac == kPlain)
     cta_cholesky_panels<A>(Ls, inv, r + 1);
-  else if constexpr (sizeof(TJ) == 8)
+  else if constexpr (kFac == kPanels)
     cta_cholesky_global<A>(Ls, inv, r + 1, reinterpret_cast<E *>(sm + panel));
   else if constexpr (G)
     cta_cholesky_global_mma(Ls, inv, r + 1, reinterpret_cast<char *>(sm + panel));
@@ -668,30 +669,38 @@ cudaError_t launch_propose(const ReducedArgs &a, cudaStream_t st) {
 static bool takes_blocked(size_t plain, size_t blk) { return blk >= 2 ? plain < 4 : plain < 2; }
 static size_t ctas_an_sm(size_t smem) { return kSmemLimit / (smem + 1024); }
 
-// Where the blocked factorisations keep their digits or panel (elements from the
-// start of shared memory; 0 where they do not apply or fit), with smem raised
-// to hold them.  FP32 Jacobian: behind the layout; for a factor in global memory
-// the vectors vp, vq, be, ae, formed after it, take the panel's place.  FP64 with
-// the factor in global memory: after the vectors (the staged rows of J are done
-// with by then).
-static int geometry_panel(int r, int d_y, int jf_f32, size_t &smem) {
+// The factorisation of an FP32 Jacobian's I + H, and where its digits or panel lie
+// (elements from the start of shared memory), with smem raised to hold them.
+// Digits behind the layout for a factor in shared memory; for one in global
+// memory the panel, in whose place the vectors vp, vq, be, ae are formed afterwards:
+// of 224 bytes a row with the digits, or where that does not fit (r from about 890)
+// of 136 without them (152 chains, d_y = 60, plain and in panels: r = 890 24.0 and 11.3
+// ms, 1024 36.9 and 16.7).
+//
+// FP64 factors take the plain one wherever they lie.  (r = 209 to 900 in global
+// memory, blocked in panels with 256 threads: 1.05 to 1.23 times the time, with 512 1.02
+// to 1.15; the FP64 pipe bounds both.)
+static Factor geometry_factor(int r, int d_y, size_t &smem, int &panel) {
   const bool G = uses_global_factor(r, d_y);
-  if (!G && !jf_f32) return 0;
-  const size_t at = Layout(r, d_y, G, G && jf_f32).tail;
-  const size_t bytes = !jf_f32 ? (size_t)(r + 1) * kPanelLd * sizeof(double)
-                       : G     ? std::max(mma_panel_bytes(r + 1), (size_t)32 * r)
-                               : mma_digit_bytes(r + 1);
-  const size_t need = at * sizeof(double) + bytes;
-  if (need > kGeoSmem) return 0;
-  if (!G && !takes_blocked(ctas_an_sm(smem), ctas_an_sm(std::max(smem, need)))) return 0;
-  smem = G && jf_f32 ? need : std::max(smem, need);
-  return (int)at;
+  const size_t at = Layout(r, d_y, G, G).tail, n = r + 1, after = 32 * (size_t)r;
+  panel = (int)at;
+  if (!G) {
+    const size_t need = std::max(smem, at * sizeof(double) + mma_digit_bytes((int)n));
+    if (need > kGeoSmem || !takes_blocked(ctas_an_sm(smem), ctas_an_sm(need))) return kPlain;
+    smem = need;
+    return kMma;
+  }
+  const size_t mma = at * sizeof(double) + std::max(mma_panel_bytes((int)n), after);
+  const size_t plain = at * sizeof(double) + std::max(n * kPanelLd * sizeof(double), after);
+  if (std::min(mma, plain) > kGeoSmem) return kPlain;
+  smem = mma <= kGeoSmem ? mma : plain;
+  return mma <= kGeoSmem ? kMma : kPanels;
 }
 
-template <typename TJ, bool G, int NT, bool kBlk>
+template <typename TJ, bool G, int NT, Factor kFac>
 static cudaError_t launch_geometry_nt(const ReducedArgs &a, int mode, size_t smem, int panel,
                                       cudaStream_t st) {
-  auto k = k_geometry<TJ, G, NT, kBlk>;
+  auto k = k_geometry<TJ, G, NT, kFac>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   ReducedArgs b = a;
@@ -708,22 +717,26 @@ static cudaError_t launch_geometry_nt(const ReducedArgs &a, int mode, size_t sme
 template <typename TJ, bool G>
 static cudaError_t launch_geometry_t(const ReducedArgs &a, int mode, size_t smem,
                                      cudaStream_t st) {
-  const int panel = geometry_panel(a.r, a.d_y, a.jf_f32, smem);
-  const size_t ctas = ctas_an_sm(smem);
-  if constexpr (G) {
-    if (panel) return launch_geometry_nt<TJ, G, 256, true>(a, mode, smem, panel, st);
-    return launch_geometry_nt<TJ, G, kThreads, false>(a, mode, smem, 0, st);
-  } else if constexpr (sizeof(TJ) == 4) {
-    if (panel)
-      return ctas >= 2 ? launch_geometry_nt<TJ, G, 256, true>(a, mode, smem, panel, st)
-                       : launch_geometry_nt<TJ, G, kThreads, true>(a, mode, smem, panel, st);
-    if (a.r <= 64) return launch_geometry_nt<TJ, G, 128, false>(a, mode, smem, 0, st);
-    if (ctas >= 4) return launch_geometry_nt<TJ, G, 256, false>(a, mode, smem, 0, st);
-    return launch_geometry_nt<TJ, G, kThreads, false>(a, mode, smem, 0, st);
+  if constexpr (sizeof(TJ) == 8) {
+    if (!G && a.r <= 64) return launch_geometry_nt<TJ, G, 128, kPlain>(a, mode, smem, 0, st);
+    if (!G && a.r <= 128) return launch_geometry_nt<TJ, G, 256, kPlain>(a, mode, smem, 0, st);
+    return launch_geometry_nt<TJ, G, kThreads, kPlain>(a, mode, smem, 0, st);
   } else {
-    if (a.r <= 64) return launch_geometry_nt<TJ, G, 128, false>(a, mode, smem, 0, st);
-    if (a.r <= 128) return launch_geometry_nt<TJ, G, 256, false>(a, mode, smem, 0, st);
-    return launch_geometry_nt<TJ, G, kThreads, false>(a, mode, smem, 0, st);
+    int panel;
+    const Factor fac = geometry_factor(a.r, a.d_y, smem, panel);
+    const size_t ctas = ctas_an_sm(smem);
+    if constexpr (G) {
+      if (fac == kMma) return launch_geometry_nt<TJ, G, 256, kMma>(a, mode, smem, panel, st);
+      if (fac == kPanels)
+        return launch_geometry_nt<TJ, G, kThreads, kPanels>(a, mode, smem, panel, st);
+    } else {
+      if (fac == kMma)
+        return ctas >= 2 ? launch_geometry_nt<TJ, G, 256, kMma>(a, mode, smem, panel, st)
+                         : launch_geometry_nt<TJ, G, kThreads, kMma>(a, mode, smem, panel, st);
+      if (a.r <= 64) return launch_geometry_nt<TJ, G, 128, kPlain>(a, mode, smem, 0, st);
+      if (ctas >= 4) return launch_geometry_nt<TJ, G, 256, kPlain>(a, mode, smem, 0, st);
+    }
+    return launch_geometry_nt<TJ, G, kThreads, kPlain>(a, mode, smem, 0, st);
   }
 }
 

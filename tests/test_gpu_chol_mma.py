@@ -83,3 +83,31 @@ def test_sizes_whose_shared_memory_ends_at_the_limit(r, dy, precision):
 def test_both_sides_of_the_rule_for_the_blocked_factorisation(r):
     """... by the CTAs an SM (d_y = r + 11)."""
     test_factor_reproduces_the_matrix(r)
+
+
+@pytest.mark.parametrize("r,dy", [(887, 30), (895, 902), (1024, 40)])
+def test_global_factor_beyond_the_panel_of_digits(r, dy):
+    """The largest factors: the panel holds no digits (r from about 890)."""
+    import paper_2403_08220_gb300 as dino
+
+    rng = np.random.default_rng(r)
+    h = 30
+    W1 = rng.integers(-1, 2, size=(h, r)) * 2.0 ** rng.integers(-6, 7, size=r)
+    W2 = rng.integers(-1, 2, size=(dy, h)).astype(float)
+    ctx = dino.dino_init(0)
+    try:
+        sid = dino.dino_load_surrogate(
+            ctx, n_grid=33, prior_gamma=0.1, prior_delta=1.0, r=r, widths=[r, h, dy],
+            activation=0, W=[W1, W2], b=[np.zeros(h), np.zeros(dy)],
+            basis_kind=dino.DINO_BASIS_KLE, y=np.zeros(dy), noise_var=1.0,
+            precision=dino.DINO_PREC_BF16, noise_map=dino.DINO_NOISE_CHOLESKY)
+        o = dino.dino_surrogate_eval(ctx, sid, rng.standard_normal((1, r)), dy)
+    finally:
+        ctx.close()
+    J = o["J"][0]
+    assert np.array_equal(J, W2 @ W1)
+    M = np.eye(r) + J.T @ J
+    s = np.sqrt(np.diag(M))
+    L = o["L"][0]
+    err = np.abs(L @ L.T - M) / np.outer(s, s)   # the product's own rounding is below r 2^-53
+    assert err.max() <= (2.0 ** -44 + 2.0 ** -53) * r, err.max()
