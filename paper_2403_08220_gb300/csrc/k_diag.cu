@@ -192,7 +192,8 @@ __global__ void __launch_bounds__(kEssThreads)
         for (int j = j0 + lane; j < j1; j += 32) {
           const double x = kStaged ? xk[j] : xk[j] - m;
 #pragma unroll
-          for (int q = 0; q < kLags; ++q) acc[q] += x * (kStaged ? xk[j + t0 + q] : xk[j + t0 + q] - m);
+          for (int q = 0; q < kLags; ++q)
+            acc[q] += x * (kStaged ? xk[j + t0 + q] : xk[j + t0 + q] - m);
         }
       } else {
         for (int j = j0 + lane; j < j1; j += 32) {
@@ -538,14 +539,18 @@ cudaError_t launch_diag_ess(int d, int n_c, int n_s, const double *traj, int max
   const size_t staged = ((size_t)n_c * n_s + n_c) * 8;
   const bool fits = staged <= kStagedSmem;
   auto kernel = fits ? k_diag_ess<true> : k_diag_ess<false>;
-  // More CTAs for a degree of freedom while the chip (two CTAs an SM) has room: the
-  // slowest one, which may run all n_s lags, sets the time.  Each CTA of a cluster
-  // stages all samples and a pass forms 8 lags in each, so a cluster costs where
-  // the lags are few: 10 chains of 1000 samples, 1 / 2 / 4 / 8 CTAs, correlation
-  // 0.9: d = 8 0.51 / 0.31 / 0.21 / 0.16 ms, d = 200 1.23 / 0.85 / 0.70 / 0.77,
-  // d = 2000 3.80 / 3.61 / 4.74 / 6.95; correlation 0.5, d = 200: 0.25 / 0.25 /
-  // 0.35 / 0.65; 50 samples, d = 100: 0.08 / 0.09 / 0.09 / 0.13.
-  int cs = d * 8 <= 304 ? kEssMaxCluster : d * 4 <= 800 ? 4 : d <= 1000 ? 2 : 1;
+  // More CTAs for a degree of freedom: the slowest one, which may run all n_s lags,
+  // sets the time, but each CTA of a cluster reads all samples and a pass forms 8 lags
+  // in each, which costs where few lags are needed and the CTAs take several
+  // rounds of the chip (two an SM, 304).  Eight in one round, four in up to three, two in
+  // up to seven.  Clusters of 1 / 2 / 4 / 8, us, 10 chains of 1000 samples, correlation 0.5,
+  // 0.9, 0.99: d = 38 137 92 110 171, 466 266 180 190, 2413 1309 1016 798; d = 100 158 173 212
+  // 316, 606 493 366 413, 2414 1778 1477 1606; d = 200 241 219 333 616, 862 562 558 720, 3358 2632
+  // 2585 2956; d = 400 338 358 620 1151, 1192 832 961 1403, 4949 4496 4761 5737; d = 1000 576 762
+  // 1436 2821, 3428 2599 2690 3486, 10259 10043 11194 13907; d = 2000 1047 1502, 3630 3523, 18545
+  // 18952.
+  constexpr int kRound = 304;
+  int cs = d * 8 <= kRound ? kEssMaxCluster : d * 4 <= 3 * kRound ? 4 : d * 2 <= 7 * kRound ? 2 : 1;
   while (cs > 1 && n_s < 64 * cs) cs /= 2;
   cudaLaunchAttribute attr = {};
   attr.id = cudaLaunchAttributeClusterDimension;
