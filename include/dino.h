@@ -366,8 +366,8 @@ int dino_dis_from_surrogate(dino_ctx *ctx, int surrogate_id, int n_samples, uint
  *   the Wasserstein MPSRF Tr(W + V - 2 (W^1/2 V W^1/2)^1/2) of the within-
  *     chain and pooled covariance estimators (eq:covariance_estimator), whose
  *     last term is the nuclear norm of C^T F for V = C C^T, W = F F^T: from the
- *     polar factor, or one-sided Jacobi where that is nearly singular
- *     (n_dof <= 1024);
+ *     polar factor, or one-sided Jacobi where that is nearly singular and for
+ *     n_dof below 8 or above 512 (n_dof <= 1024);
  *   the mean squared jump MSJ = 1/(n_s - 1) sum_j |x_{j+1} - x_j|^2, averaged
  *     over chains (the acceptance rate comes with dino_chains_step's stats).
  * The trajectory takes n_dof n_chains max_samples doubles of device memory. */

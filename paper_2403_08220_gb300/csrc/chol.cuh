@@ -611,7 +611,8 @@ __device__ void cta_cholesky_global(typename A::T *Lg, typename A::T *inv, int n
     __syncthreads();
     for (int kk = 0; kk < w; kk += kNB) {
       const int nb = min(kNB, w - kk);
-      if (warp == (kb / kNB + kk / kNB) % nw) warp_factor_diag<A, false>(at, inv + kb, kk, nb, lane, lsc);
+      if (warp == (kb / kNB + kk / kNB) % nw)
+        warp_factor_diag<A, false>(at, inv + kb, kk, nb, lane, lsc);
       __syncthreads();
       for (int i = kk + nb + tid; i < m; i += blockDim.x)
         panel_row<A>(at, inv + kb, lsc, kk, i);

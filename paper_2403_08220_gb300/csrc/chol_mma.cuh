@@ -19,9 +19,10 @@
 // scheduler; here 28 mma.sync.m16n8k16 per 128 entries (8 cycles each on
 // GB300) run beside about 42 instructions per entry that join the levels.
 // Geometry of 512 chains at r = 400 (factor in global memory): 4.61 -> 3.44 ms;
-// of 4096 chains at r = 128: 2.02 -> 1.60 ms (3.40 and 1.52 since the diagonal blocks take less).  The d_y-sized factors of the Woodbury path (101
-// rows, four chains an SM) gain nothing: 3.32 against 3.20 ms for 16384 chains,
-// their time is in the panels and barriers.
+// of 4096 chains at r = 128: 2.02 -> 1.60 ms (3.38 and 1.50 since the diagonal
+// blocks take less).  The d_y-sized factors of the Woodbury path (101 rows, four
+// chains an SM) gain nothing: 3.32 against 3.20 ms for 16384 chains, their time is
+// in the panels and barriers.
 #pragma once
 #include "chol.cuh"
 
@@ -277,7 +278,8 @@ __device__ void cta_cholesky_global_mma(float2 *Lg, float2 *inv, int n, char *di
     __syncthreads();
     for (int kk = 0; kk < w; kk += kNB) {
       const int nb = min(kNB, w - kk), c0 = kk + nb;
-      if (warp == (kb / kNB + kk / kNB) % nw) warp_factor_diag<A, false>(at, inv + kb, kk, nb, lane, lsc);
+      if (warp == (kb / kNB + kk / kNB) % nw)
+        warp_factor_diag<A, false>(at, inv + kb, kk, nb, lane, lsc);
       __syncthreads();
       for (int i = c0 + tid; i < m; i += blockDim.x) panel_row<A>(at, inv + kb, lsc, kk, i);
       __syncthreads();

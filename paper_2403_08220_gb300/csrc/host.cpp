@@ -482,8 +482,8 @@ static T *sur_upload(dino_ctx *ctx, Surrogate *s, const T *host, size_t n) {
 // B's digits are laid out once, and the product runs on the tensor cores, when
 // B has at least kDigitsMinWork entries and neither side is short (a tile has 32
 // columns, a stage 32 of the reduction); below that the SIMT GEMM is as fast or
-// faster (64 rows by 16 x 1089: 18 us against 70 us).  The rule looks at B alone, so that an output's bits do not depend
-// on how many chains share the product.
+// faster (64 rows by 16 x 1089: 18 us against 70 us).  The rule looks at B alone,
+// so that an output's bits do not depend on how many chains share the product.
 constexpr long kDigitsMinWork = 16384;
 
 // Digits of a device matrix B.  A surrogate's operands (counted = false) are
@@ -1521,9 +1521,11 @@ static ReducedArgs reduced_args(const Pool &p) {
 // Tensor path, r-sized: I + J^T J / noise_var.  FP64 Woodbury path: J J^T on the
 // tensor cores, J's digits in the Jacobian's two product buffers (not in use any
 // more) for as many chains at a time as they hold; below 24 observations the
-// geometry kernel forms it as fast itself, and where the hidden layers are not
-// wider than r the buffers hold less than one chain.  The rule looks at the
-// surrogate alone, so that a chain's bits do not depend on the pool.
+// geometry kernel forms it as fast itself (1024 chains, r = 200, geometry with
+// the digits and products and by itself: d_y = 16 427 and 395 us, 20 451 and 444, 24
+// 505 and 523, 32 621 and 714), and where the hidden layers are not wider than r the
+// buffers hold less than one chain.  The rule looks at the surrogate alone, so
+// that a chain's bits do not depend on the pool.
 static void gram_of(dino_ctx *ctx, const Pool &p, ReducedArgs &a, int mode, cudaStream_t st) {
   const Surrogate *s = p.s;
   if (!p.wb) {
@@ -2063,8 +2065,10 @@ static int jacobi(dino_ctx *ctx, int d, double *G, double *Q, double *sig, int *
 // held by columns: Newton-Schulz for the polar factor while the matrix is
 // regular enough, at most kNsSteps steps (each can make a singular value 1.5
 // times larger: 4e-9 of |A|_F reaches 1), the host looking at max |X^T X - I|
-// every kNsBatch steps; else, and at a d outside the range where it is the
-// faster one, the column norms of one-sided Jacobi, in place.  Y, X, X2, P: d d
+// every kNsBatch steps; else, and at d outside kNsMinD .. kNsMaxD, the column norms
+// of one-sided Jacobi, in place.  (A computation by Newton-Schulz and by Jacobi:
+// d = 6 0.59 and 0.44 ms, 8 0.59 and 0.58, 10 0.61 and 0.71, 24 0.73 and 1.48, 512 23.8 and
+// 56.7, 600 36.3 and 70.6, 1024 176 and 227: the range could end later.)  Y, X, X2, P: d d
 // doubles each; flags: kMaxJacobiSweeps doubles.  Returns Jacobi sweeps.
 constexpr int kNsSteps = 48, kNsBatch = 4, kNsMinD = 8, kNsMaxD = 512;
 static int nuclear_terms(dino_ctx *ctx, int d, double *A, double *sig, double *Y, double *X,

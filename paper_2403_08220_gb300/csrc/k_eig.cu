@@ -214,7 +214,8 @@ __global__ void __launch_bounds__(NT) k_eig_geometry(ReducedArgs a, int mode) {
   const EigLayout lay(r, dy);
   const EigSlot sl(dy);
   const int ld = eig_ld(dy);
-  double *Md = sm + lay.Md, *nu = sm + lay.nu, *Kb = sm + lay.Kb, *Ka = sm + lay.Ka, *u = sm + lay.u, *wv = sm + lay.w, *vv = sm + lay.vv,
+  double *Md = sm + lay.Md, *nu = sm + lay.nu, *Kb = sm + lay.Kb, *Ka = sm + lay.Ka,
+         *u = sm + lay.u, *wv = sm + lay.w, *vv = sm + lay.vv,
          *ys = sm + lay.ys, *vb = sm + lay.vb, *va = sm + lay.va, *red = sm + lay.red;
   int *flag = reinterpret_cast<int *>(sm + lay.flag);
   const size_t ldS = (((size_t)dy * dy + 3 * (size_t)dy + 1) + 1) & ~(size_t)1;

@@ -767,7 +767,10 @@ cudaError_t run_gemm64(const Gemm64Args &a, const Epi &epi, cudaStream_t st) {
   if (a.K <= 0 || a.K > (1 << 28) || (a.ldp & 7) || (a.plane & 7) || (a.B.ldp & 7) ||
       (a.B.plane & 7) || ((uintptr_t)a.A & 15) || ((uintptr_t)a.B.d & 15) || !a.err)
     return cudaErrorInvalidValue;
-  // 64 columns a tile; 32 where those tiles would leave SMs idle
+  // 64 columns a tile; 32 where those tiles would leave SMs idle (M x 200 x 1089, 64 and
+  // 32 columns: 32 tiles of 64 228 and 194 us, 64 236 and 223, 96 281 and 296, 256 576 and 606;
+  // a layer with GELU, whose FP64 epilogue gains from more CTAs at any size: three of 400,
+  // 56 tiles 514 and 340, 112 644 and 614, 448 2013 and 1977)
   const long t64 = (long)((a.M + kBM - 1) / kBM) * ((a.N + 63) / 64);
   if (a.N <= 32 || t64 < 100) return run_gemm64_t<32, false>(a, epi, st);
   return run_gemm64_t<64, false>(a, epi, st);

@@ -425,8 +425,9 @@ __global__ void __launch_bounds__(kGramThreads, 4) k_gram_f32(ReducedArgs a, int
 //
 // Mode 0 makes b the chain state (slot cur[c]).  Mode 1 evaluates
 // log rho_r^(1) against the current state a, takes the accept test and moves
-// an accepted chain to b: its factor slot (written only then, into the other
-// slot, which becomes current) and its state vectors.  The complement
+// an accepted chain to b: its factor (stored only then, into the other slot,
+// which becomes current; factors in global memory and k_gram_f32 work in that
+// slot every time) and its state vectors.  The complement
 // coefficient b - s a is written for every chain.
 // The FP32-Jacobian instantiations find I + H in the slot (k_gram_f32).  kFac: the
 // factorisation.  The blocked ones (FP32 Jacobian) keep their digits or panel at sm +
@@ -749,8 +750,8 @@ cudaError_t launch_gram_f32(const ReducedArgs &a, int mode, cudaStream_t st) {
     b.cur = a.cur + o;
     b.L = a.L + o * slot_stride(a.r);
     b.J = reinterpret_cast<const float *>(a.J) + o * a.d_y * a.r;
-    const cudaError_t e = launch_pdl(k_gram_f32, dim3(nb * (nb + 1) / 2, b.C), kGramThreads, 0, st, b,
-                                     mode);
+    const cudaError_t e = launch_pdl(k_gram_f32, dim3(nb * (nb + 1) / 2, b.C), kGramThreads, 0, st,
+                                     b, mode);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

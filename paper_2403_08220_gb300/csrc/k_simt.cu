@@ -372,11 +372,13 @@ __global__ void __launch_bounds__(256)
   const size_t off = (size_t)blockIdx.y * a * b;
 #pragma unroll
   for (int k = 0; k < 32; k += 8)
-    if (i0 + ty + k < a && j0 + tx < b) tile[ty + k][tx] = __ldg(src + off + (size_t)(i0 + ty + k) * b + j0 + tx);
+    if (i0 + ty + k < a && j0 + tx < b)
+      tile[ty + k][tx] = __ldg(src + off + (size_t)(i0 + ty + k) * b + j0 + tx);
   __syncthreads();
 #pragma unroll
   for (int k = 0; k < 32; k += 8)
-    if (j0 + ty + k < b && i0 + tx < a) dst[off + (size_t)(j0 + ty + k) * a + i0 + tx] = tile[tx][ty + k];
+    if (j0 + ty + k < b && i0 + tx < a)
+      dst[off + (size_t)(j0 + ty + k) * a + i0 + tx] = tile[tx][ty + k];
 }
 
 cudaError_t launch_batched_transpose(int C, int a, int b, const void *src, int f32, void *dst,
@@ -472,8 +474,8 @@ cudaError_t launch_prior_draw(int C, int n, const T *sqrtlam, const T *S, uint64
 template <typename T>
 cudaError_t launch_jac_init(int C, int d_y, int w, const T *WL, const T *der, int ldd, T *P,
                             cudaStream_t st) {
-  return launch_pdl(k_jac_init<T>, grid_for((size_t)C * d_y * w), 256, 0, st, C, d_y, w, WL, der, ldd,
-                    P);
+  return launch_pdl(k_jac_init<T>, grid_for((size_t)C * d_y * w), 256, 0, st, C, d_y, w, WL, der,
+                    ldd, P);
 }
 
 template <typename T>

@@ -1068,13 +1068,14 @@ cudaError_t launch_tc_gemm(const TcGemmArgs &a, cudaStream_t st) {
   cudaError_t e =
       cudaFuncSetAttribute(k_tc_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const cudaError_t e2 = launch_pdl_n((long)total * p.ksplit, k_tc_gemm, std::min(total * p.ksplit, sms), kThreads, smem, st,
-                                    tmA, tmB, tmO, tmS, p);
+  const cudaError_t e2 =
+      launch_pdl_n((long)total * p.ksplit, k_tc_gemm, std::min(total * p.ksplit, sms), kThreads,
+                   smem, st, tmA, tmB, tmO, tmS, p);
   if (e2 != cudaSuccess || p.ksplit == 1) return e2;
   const size_t n = (size_t)a.M * a.N;
   const int grid = (int)std::min<size_t>((n + 255) / 256, 152 * 32);
-  return launch_pdl(k_coef_finish, grid, 256, 0, st, (uint32_t)n, a.N, p.ksplit, p.ws, a.coef, a.ldc,
-                    a.cs, a.out_bf, a.ldo, a.out_plane, a.out_slices);
+  return launch_pdl(k_coef_finish, grid, 256, 0, st, (uint32_t)n, a.N, p.ksplit, p.ws, a.coef,
+                    a.ldc, a.cs, a.out_bf, a.ldo, a.out_plane, a.out_slices);
 }
 
 cudaError_t launch_tc_gram(int C, int g, int K, const __nv_bfloat16 *J, int ldj, size_t plane,
@@ -1120,7 +1121,8 @@ cudaError_t launch_tc_gram(int C, int g, int K, const __nv_bfloat16 *J, int ldj,
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
     return cudaErrorInvalidValue;
-  return launch_pdl_n(C / p.batch, k_tc_gram, std::min((C + p.batch - 1) / p.batch, sms), kThreads, smem, st, tm, p);
+  return launch_pdl_n(C / p.batch, k_tc_gram, std::min((C + p.batch - 1) / p.batch, sms), kThreads,
+                      smem, st, tm, p);
 }
 
 cudaError_t launch_split_bf16_f64(int rows, int cols, const double *src, int lds,
@@ -1138,8 +1140,8 @@ cudaError_t launch_jac_init_bf16(int C, int d_y, int w, const float *WL, const f
   const size_t items = (size_t)C * d_y * ((w + 7) / 8);  // 8 columns per thread
   if (items >= 0xffffffffull - 152ull * 16 * 256) return cudaErrorInvalidValue;
   const int grid = (int)std::min<size_t>((items + 255) / 256, 152 * 16);
-  return launch_pdl(k_jac_init_bf16, grid > 0 ? grid : 1, 256, 0, st, C, d_y, w, WL, der, ldd, P, ldp,
-                    plane, nslice);
+  return launch_pdl(k_jac_init_bf16, grid > 0 ? grid : 1, 256, 0, st, C, d_y, w, WL, der, ldd, P,
+                    ldp, plane, nslice);
 }
 
 }  // namespace dino

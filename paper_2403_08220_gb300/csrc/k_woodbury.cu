@@ -822,8 +822,9 @@ size_t wb_geometry_smem(int r, int dy) {
 
 template <typename TJ, bool kPre, int NT>
 cudaError_t launch_wb_geometry_k(const ReducedArgs &a, int mode, cudaStream_t st) {
-  const size_t smem = a.gram_in_slot ? WbLayout(a.r, a.d_y).tail * sizeof(double)  // no rows of J staged
-                            : wb_geometry_smem<TJ>(a.r, a.d_y);
+  const size_t smem = a.gram_in_slot
+                          ? WbLayout(a.r, a.d_y).tail * sizeof(double)  // no rows of J staged
+                          : wb_geometry_smem<TJ>(a.r, a.d_y);
   cudaError_t e = cudaFuncSetAttribute(k_wb_geometry<TJ, kPre, NT>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;

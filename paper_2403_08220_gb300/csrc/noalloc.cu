@@ -225,7 +225,8 @@ bool spread_rows(const Net &net, int n, int sms) {
   for (int l = 1; l < L; ++l) hidden += net.w[l];
   for (int l = 0; l + 1 < L; ++l) macs += 1e-3 * net.w[L] * net.w[l] * net.w[l + 1];
   const bool gelu = net.act == DINO_ACT_GELU, tanh = net.act == DINO_ACT_TANH;
-  const double value = gelu ? 7.1e-3 : tanh ? 3.1e-3 : 1.16e-3, layer = gelu ? 7.7 : tanh ? 2.4 : 0.0;
+  const double value = gelu ? 7.1e-3 : tanh ? 3.1e-3 : 1.16e-3;
+  const double layer = gelu ? 7.7 : tanh ? 2.4 : 0.0;
   const double point = 9.8 + 0.31 * macs + 0.167 * (net.w[0] + hidden);
   const double spread = 1.7 + 7.2 * L + 0.056 * hidden + layer * (L - 1) +
                         n * (value * hidden + 0.0036 * macs);

@@ -79,7 +79,8 @@ def test_sizes_whose_shared_memory_ends_at_the_limit(r, dy, precision):
     assert abs(o["hld"][0] - ref) <= 1e-9 * max(1.0, abs(ref))
 
 
-@pytest.mark.parametrize("r", [106, 107, 108, 109, 133, 134, 135, 136, 157, 158, 159, 160, 203, 204])
+@pytest.mark.parametrize("r", [106, 107, 108, 109, 133, 134, 135, 136, 157, 158, 159, 160, 203,
+                               204])
 def test_both_sides_of_the_rule_for_the_blocked_factorisation(r):
     """... by the CTAs an SM (d_y = r + 11)."""
     test_factor_reproduces_the_matrix(r)

@@ -194,7 +194,7 @@ def test_contexts_of_two_threads_with_different_sizes(dino):
     sizes = [(2, 2000, 40), (3, 60, 5), (2, 900, 300)]
     for i, s in enumerate(sizes):
         compute(("alone", i), *s, 1)
-    threads = [threading.Thread(target=compute, args=((i,) + s + (60,))) for i, s in enumerate(sizes)]
+    threads = [threading.Thread(target=compute, args=(i, *s, 60)) for i, s in enumerate(sizes)]
     for t in threads:
         t.start()
     for t in threads:
