@@ -173,7 +173,14 @@ __global__ void __launch_bounds__(kJacThreads)
   extern __shared__ double sm[];
   const int p = blockIdx.y, L = net.L, r = net.w[0], dy = net.w[L];
   const int i0 = blockIdx.x * rows, nr = min(rows, dy - i0);
-  double *Jp = J + ((size_t)p * dy + i0) * r;  // L >= 2
+  double *Jp = J + ((size_t)p * dy + i0) * r;
+  // A single layer: spread_rows sends it to k_jac_point, but without this branch the
+  // compiler's inner loop is the slower one (one point of 100-200-200-20 49.5 -> 53.7 us).
+  if (L == 1) {
+    for (int e = threadIdx.x; e < nr * r; e += blockDim.x)
+      Jp[e] = net.W[0][(size_t)i0 * r + e];
+    return;
+  }
   const double *der = scratch + (size_t)p * slab + 2 * (size_t)wmax;
   int off = 0;  // of d_{l - 1} (layer widths w_1 .. w_{L - 1})
   for (int l = 1; l < L - 1; ++l) off += net.w[l];
