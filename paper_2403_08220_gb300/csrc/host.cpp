@@ -2068,13 +2068,14 @@ static int jacobi(dino_ctx *ctx, int d, double *G, double *Q, double *sig, int *
 // every kNsBatch steps; else, and at d outside kNsMinD .. kNsMaxD, the column norms
 // of one-sided Jacobi, in place.  (A computation by Newton-Schulz and by Jacobi:
 // d = 6 0.59 and 0.44 ms, 8 0.59 and 0.58, 10 0.61 and 0.71, 24 0.73 and 1.48, 512 23.8 and
-// 56.7, 600 36.3 and 70.6, 1024 176 and 227: the range could end later.)  Y, X, X2, P: d d
-// doubles each; flags: kMaxJacobiSweeps doubles.  Returns Jacobi sweeps.
+// 56.7, 600 36.3 and 70.6, 1024 176 and 227: the range could end later.)  rank: A's at
+// most; a singular A would take all the steps and come to Jacobi after all.  Y, X,
+// X2, P: d d doubles each; flags: kMaxJacobiSweeps doubles.  Returns Jacobi sweeps.
 constexpr int kNsSteps = 48, kNsBatch = 4, kNsMinD = 8, kNsMaxD = 512;
-static int nuclear_terms(dino_ctx *ctx, int d, double *A, double *sig, double *Y, double *X,
-                         double *X2, double *P, double *flags, cudaStream_t st) {
+static int nuclear_terms(dino_ctx *ctx, int d, size_t rank, double *A, double *sig, double *Y,
+                         double *X, double *X2, double *P, double *flags, cudaStream_t st) {
   static_assert(kNsSteps / kNsBatch <= kMaxJacobiSweeps, "a residual per batch");
-  if (d >= kNsMinD && d <= kNsMaxD) {
+  if (d >= kNsMinD && d <= kNsMaxD && rank >= (size_t)d) {
     auto *res = (unsigned long long *)flags;
     CK(cudaMemsetAsync(res, 0, kNsSteps / kNsBatch * sizeof(*res), st));
     launch(ctx, st, "ns_start", [&] { return launch_ns_start(d, A, Y, X, st); });
@@ -2347,7 +2348,7 @@ static void diag_compute(dino_ctx *ctx, Diag *g, int want_mpsrf, double *ess_out
       // the singular values of C^T F, W = F F^T, V = C C^T (k_diag.cu)
       launch(ctx, st, "psd_chol", [&] { return launch_psd_chol(d, W, V, F, Cv, st); });
       launch(ctx, st, "ct_f", [&] { return launch_ct_f(d, Cv, F, G, st); });
-      sweeps = nuclear_terms(ctx, d, G, sig, Wr, Br, F, Cv, o + 4, st);
+      sweeps = nuclear_terms(ctx, d, K - n_c, G, sig, Wr, Br, F, Cv, o + 4, st);
       launch(ctx, st, "mpsrf_final", [&] { return launch_mpsrf_final(d, W, V, sig, o, st); });
       CK(cudaMemcpyAsync(out, o, 24, cudaMemcpyDeviceToHost, st));
       CK(cudaStreamSynchronize(st));
