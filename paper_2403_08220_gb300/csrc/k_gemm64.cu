@@ -54,7 +54,8 @@
 // many neighbouring level accumulators: 12 instructions of mostly N = 256 per 16
 // columns instead of 36 of N = 64.  The eight accumulators of BN columns fill
 // TMEM at BN = 64; the sums of magnitudes take the first one's place when the
-// last chunk has been read.
+// last chunk has been read.  At BN = 32 they have columns of their own and come with
+// the last chunk, without a second round between the MMAs and the epilogue.
 //
 // What bounds it: the chain from tile to tile.  One set of accumulators means that
 // the next tile's MMAs wait for the epilogue's reads, and two stages (96 KB per 32
@@ -80,6 +81,7 @@ constexpr int kDigits = kDigits64;
 constexpr int kBM = 128, kKB = 32;             // tile rows, columns per stage
 constexpr int kChunkK = 512;                   // columns per exact accumulation
 constexpr int kStages = 2;
+constexpr int kTmemCols = 512;
 constexpr int kEpiWarps = 8;
 constexpr int kGemm64Threads = 32 * (2 + kEpiWarps);
 constexpr int kABytes = kDigits * kBM * kKB * 2;
@@ -387,6 +389,9 @@ __global__ void __launch_bounds__(kGemm64Threads, 1)
              const __grid_constant__ CUtensorMap tmAc, const __grid_constant__ CUtensorMap tmBc,
              const Gemm64Params p, const Epi epi) {
   constexpr int NC = BN / 2;                       // columns of an epilogue warp
+  // the sums of magnitudes beside the levels (TMEM column kMagCol), in the last chunk's round
+  constexpr bool kBeside = !kGram && (kDigits + 1) * BN <= kTmemCols;
+  constexpr int kMagCol = kBeside ? kDigits * BN : 0;
   constexpr uint32_t kBBytes = kDigits * BN * kKB * 2;
   constexpr uint32_t kStage = kABytes + kBBytes;
   extern __shared__ __align__(1024) unsigned char smraw[];
@@ -488,8 +493,8 @@ __global__ void __launch_bounds__(kGemm64Threads, 1)
             break;
           }
           fence_after();
-          const bool mags = kb0 >= p.nkb;
-          const int kb1 = mags ? p.nkb + nck : min(p.nkb, kb0 + kChunkB);
+          int kb1 = kb0 >= p.nkb ? p.nkb + nck : min(p.nkb, kb0 + kChunkB);
+          if (kBeside && kb1 == p.nkb) kb1 += nck;
           for (int kb = kb0; kb < kb1; ++kb, ++g) {
             const int s = g % kStages;
             if (!mbar_wait(smem_u32(&bars[s]), (uint32_t)(g / kStages) & 1u, abort_flag)) {
@@ -502,14 +507,14 @@ __global__ void __launch_bounds__(kGemm64Threads, 1)
             fence_after();
             const uint32_t sa = base + s * kStage;
             const uint64_t ad = smem_desc_sw64(sa), bd = smem_desc_sw64(sa + kABytes);
-            if (!kGram && mags) {
+            if (!kGram && kb >= p.nkb) {
               const int nblk = min(kDigits, p.ncb - (kb - p.nkb) * kDigits);
               for (int i = 0; i < nblk; ++i)
 #pragma unroll
                 for (int kk = 0; kk < kKB / 16; ++kk)
-                  mma_bf16(tmem, ad + (uint64_t)(i * kBM * kKB * 2 / 16 + 2 * kk),
+                  mma_bf16(tmem + kMagCol, ad + (uint64_t)(i * kBM * kKB * 2 / 16 + 2 * kk),
                            bd + (uint64_t)(i * BN * kKB * 2 / 16 + 2 * kk), idesc_bf16(kBM, BN),
-                           (kb > kb0 || i > 0 || kk > 0) ? 1u : 0u);
+                           (kb > p.nkb || i > 0 || kk > 0) ? 1u : 0u);
               mma_commit(smem_u32(&bars[kStages + s]));
               continue;
             }
@@ -576,6 +581,18 @@ __global__ void __launch_bounds__(kGemm64Threads, 1)
           asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(acc_empty) : "memory");
       };
       const uint32_t tacc = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(half * NC);
+      uint32_t redo = 0;  // bit c: this row's output in column n0 + c is a plain dot product
+      auto read_magnitudes = [&]() {
+#pragma unroll
+        for (int c0 = 0; c0 < NC; c0 += 8) {
+          int v[8];
+          tmem_ld8(tacc + (uint32_t)(kMagCol + c0), v);
+          tmem_wait_ld();
+#pragma unroll
+          for (int e = 0; e < 8; ++e)
+            redo |= (__int_as_float(v[e]) >= kLeast ? 0u : 1u) << (c0 + e);
+        }
+      };
       for (int kb0 = 0; kb0 < p.nkb; kb0 += kChunkB, ++j) {
         wait_acc();
         if (!ok) break;
@@ -596,22 +613,14 @@ __global__ void __launch_bounds__(kGemm64Threads, 1)
             low[c0 + e] &= 0xfffffffu;
           }
         }
+        if (kBeside && kb0 + kChunkB >= p.nkb) read_magnitudes();
         free_acc();
       }
       if (!ok) break;
-      uint32_t redo = 0;  // bit c: this row's output in column n0 + c is a plain dot product
-      if constexpr (!kGram) {
-        wait_acc();  // the sums of magnitudes
+      if constexpr (!kGram && !kBeside) {
+        wait_acc();
         if (!ok) break;
-#pragma unroll
-        for (int c0 = 0; c0 < NC; c0 += 8) {
-          int v[8];
-          tmem_ld8(tacc + (uint32_t)c0, v);
-          tmem_wait_ld();
-#pragma unroll
-          for (int e = 0; e < 8; ++e)
-            redo |= (__int_as_float(v[e]) >= kLeast ? 0u : 1u) << (c0 + e);
-        }
+        read_magnitudes();
         free_acc();
         ++j;
       }
@@ -637,14 +646,17 @@ __global__ void __launch_bounds__(kGemm64Threads, 1)
           stg[lane * 16 + ((((c >> 1) ^ (lane & 7)) << 1) | (c & 1))] =
               scaled_to_f64(acc[c0 + c], low[c0 + c], ea + eb - 35);
         }
+        const bool some = __any_sync(0xffffffffu, redo >> c0 & ((1u << kS) - 1u));
         __syncwarp();
         for (int q = lane; q < 32 * kS; q += 32) {
           const int r = q / kS, c = q % kS, col = n0 + c0 + c;
           const bool in = row0 + r < rows && col < p.N && (!kGram || col <= row0 + r);
           double v = stg[r * 16 + ((((c >> 1) ^ (r & 7)) << 1) | (c & 1))];
-          const uint32_t of_row = __shfl_sync(0xffffffffu, redo, r);
-          const unsigned lanes = __ballot_sync(0xffffffffu, in && (of_row >> (c0 + c) & 1u));
-          if (lanes) v = plain_dots(p, g0, row0 + r, col, lanes, v);
+          if (some) {
+            const uint32_t of_row = __shfl_sync(0xffffffffu, redo, r);
+            const unsigned lanes = __ballot_sync(0xffffffffu, in && (of_row >> (c0 + c) & 1u));
+            if (lanes) v = plain_dots(p, g0, row0 + r, col, lanes, v);
+          }
           if (in) epi(p.row0 + g0 + row0 + r, col, v);
         }
         __syncwarp();
@@ -735,7 +747,7 @@ cudaError_t run_gemm64_t(const Gemm64Args &a, const Epi &epi, cudaStream_t st) {
   p.B = a.B.src;
   p.ldb = a.B.ld;
   p.err = a.err;
-  p.tmem_cols = kDigits * BN;
+  p.tmem_cols = kGram ? kDigits * BN : kTmemCols;
   CUtensorMap tmA, tmB, tmAc, tmBc;
   const int rows_b = kGram ? a.M : a.N;
   if (!make_digit_map(&tmA, a.A, a.K, a.M, a.ldp, a.plane, kBM) ||
